@@ -70,11 +70,14 @@
 
 namespace regione {
 
-constexpr int kAttnThreads = 384;        // 2 softmax warpgroups + 1 of producer / issuers
+constexpr int kSoftmaxWarps = 16;        // 4 softmax warpgroups: [query tile][64-key chunk]
+constexpr int kWarpLoad = kSoftmaxWarps, kWarpPv = kSoftmaxWarps + 1, kWarpS = kSoftmaxWarps + 3;   // (two P*V issuers)
+constexpr int kAttnThreads = 32 * (kSoftmaxWarps + 4);
 constexpr int kBM = 128;                 // query rows per tile
 constexpr int kBN = 128;                 // key rows per shared-memory tile
-constexpr int kBH = 64;                  // key rows per P chunk (half a tile)
-constexpr int kPolyEvery = 4;             // one pair in kPolyEvery computes one of its two exponentials on the FMA pipe
+constexpr int kBH = 64;                  // key rows per chunk (half a tile): the logits one thread holds
+constexpr float kOutgrownSum = 1.152921504606846976e18f;   // 2^60: chunk sum at which a reference maximum is renewed
+constexpr int kCopySlots = 4;             // cache refresh: units of rows in flight beside the walk of a segment
 constexpr int kHalfBytes = 128 * 64 * 2; // one 128-row x 64-column bf16 box (128-byte rows)
 constexpr long long kTimeoutCycles = 4000000000LL;   // default bound of every wait (about 2 s)
 
@@ -86,9 +89,30 @@ struct AttnCfg {
     // 2 query tiles + the ring + one more stage that only a lone query tile uses (its ring is that
     // stage, the ordinary ring and the idle second query tile: kStages + 2 stages)
     static constexpr int kSmemTiles = (2 + kStages + 1) * kTileBytes;
-    static constexpr int kCtrlBytes = 256;
-    static constexpr int kSmemBytes = kSmemTiles + 1024 /*alignment slack*/ + kCtrlBytes +
-                                      kBM * 8 /*(max, sum) of a lone tile's second half*/;
+    static constexpr int kCtrlBytes = 512;
+    static constexpr int kExchBytes = 4 * kBM * 4;         // exchange of the chunks' maxima and sums
+    static constexpr int kExtraAt = kSmemTiles + kCtrlBytes + kExchBytes;
+    // D = 128 fills shared memory: the epilogue stages its rows (4 KB per softmax warp) in the idle query
+    // tiles, and a launch that refreshes the cache copies rows through the extra stage, which a lone query
+    // tile then does without.  D = 64 has room for both.
+    static constexpr int kStageAt = (D == 128) ? 0 : kExtraAt;
+    static constexpr int kCopySlotBytes = (D == 128) ? 8192 : 4096;
+    static constexpr int kCopyAt = (D == 128) ? (2 + kStages) * kTileBytes : kExtraAt + kSoftmaxWarps * 4096;
+    static constexpr int kSmemBytes = kExtraAt + (D == 128 ? 0 : kSoftmaxWarps * 4096 + kCopySlots * kCopySlotBytes);
+    static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
+    __host__ __device__ static constexpr int lone_stages(bool store) { return kStages + (D == 128 && store ? 1 : 2); }
+    // slots of the copies that are left when the walks are over and all tiles are idle
+    static constexpr int kTailSlots = 3, kTailSlotBytes = (D == 128) ? 65536 : 40960;
+    static_assert(kTailSlots * kTailSlotBytes <= kSmemTiles, "tail slots");
+};
+
+// The part of one item that a CTA works on, as its roles need it (shared memory).
+struct SegInfo {
+    int live;                   // 0: the share ends here
+    int b, h, q0, nq;           // request, head, first query row, live query rows of the request
+    int j_first, n_tiles;       // key tiles [j_first, j_first + n_tiles) of the item
+    int nt_c, nt, nc, nf;       // cached key tiles, all key tiles, live keys of the two segments
+    int item, slot, n_slots;    // item index within the launch, slot among the shares that touch it
 };
 
 struct AttnCtrl {
@@ -98,22 +122,29 @@ struct AttnCtrl {
     uint64_t s_full[2];         // [query tile]
     uint64_t p_full[2][2];      // [query tile][chunk of 64 keys]
     uint64_t o_final[2];        // completes once, after the tile's last P*V product
-    uint64_t pv_done[2];        // [query tile] completes after every key tile's last product: P may be
-                                // overwritten and O rescaled
+    uint64_t pv_done[2];        // [query tile] completes after every key tile's last product: the second chunk's P
+                                // may be overwritten
+    uint64_t pv_half[2];        // [query tile] ... after every key tile's first product: the first chunk's P may be
     uint64_t s_free;            // the shared S buffer has been read by the softmax warps it was computed for
-    uint64_t half_done;         // lone query tile: the odd key tiles' (max, sum) are in shared memory
     uint32_t tmem_base;
     int abort_flag;
+    int redo;                   // a row outgrew the reference maximum of its first key tile
+    SegInfo seg[2];
+    // cache refresh: a slot's rows have landed; where they go, and which of them are to be stored
+    uint64_t copy_full[kCopySlots];
+    uint8_t* copy_dst[kCopySlots];
+    int copy_item[kCopySlots];
+    uint32_t copy_valid[kCopySlots];
 };
 
 // The barriers of AttnCtrl as one array starting at q_full.
-constexpr int kBarKvEmpty = 9, kBarSFull = 17, kBarPFull = 19, kBarOFinal = 23, kBarPvDone = 25, kBarSFree = 27,
-              kBarHalfDone = 28, kNumBarriers = 29;
+constexpr int kBarKvEmpty = 9, kBarSFull = 17, kBarPFull = 19, kBarOFinal = 23, kBarPvDone = 25, kBarPvHalf = 27,
+              kBarSFree = 29, kNumBarriers = 30;
 static_assert(offsetof(AttnCtrl, kv_empty) == kBarKvEmpty * 8 && offsetof(AttnCtrl, s_full) == kBarSFull * 8 &&
               offsetof(AttnCtrl, p_full) == kBarPFull * 8 && offsetof(AttnCtrl, o_final) == kBarOFinal * 8 &&
-              offsetof(AttnCtrl, pv_done) == kBarPvDone * 8 && offsetof(AttnCtrl, s_free) == kBarSFree * 8 &&
-              offsetof(AttnCtrl, half_done) == kBarHalfDone * 8 && offsetof(AttnCtrl, tmem_base) == kNumBarriers * 8,
-              "barrier layout");
+              offsetof(AttnCtrl, pv_done) == kBarPvDone * 8 && offsetof(AttnCtrl, pv_half) == kBarPvHalf * 8 &&
+              offsetof(AttnCtrl, s_free) == kBarSFree * 8 && offsetof(AttnCtrl, tmem_base) == kNumBarriers * 8 &&
+              sizeof(AttnCtrl) <= 512, "barrier layout");
 
 // What share c tells the merge kernel: the item that the boundary between shares c - 1 and c
 // cuts, if c is the second share of that item (so every cut item is named exactly once).
@@ -139,17 +170,16 @@ struct AttnParams {
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
 };
 
-// Cache refresh fused into a full step: the rows keep_rows[b, 0..n_keep[b]) (ascending) of the fresh
-// K and V are also written to k_store / v_store [B, store_cap, H, D].  A parameter of its own, of
-// the kernel that refreshes the cache only: the plain attention kernel's parameters do not grow.
+// Cache refresh fused into a full step: the rows keep_rows[b, 0..n_keep[b]) (ascending) of the K and V
+// that the launch attends over are also written to k_store / v_store [B, store_cap, H, D].  A parameter of
+// its own, of the kernel that refreshes the cache only: the plain attention kernel's parameters do not grow.
 struct StoreParams {
     const int32_t* keep_rows;
     const int32_t* n_keep;
-    int store_cap;
-    uint16_t* k_store;
-    uint16_t* v_store;
+    int store_cap, src_cap;             // rows per request of the cache and of the sources
+    const uint8_t* src[2];              // K, V [B, src_cap, H, D]
+    uint8_t* dst[2];
 };
-
 
 // ---- the plan every CTA (and the merge kernel) derives from the device-side counts ------------
 // Shares are cut on a cost axis measured in ticks, not in steps, so that they take about the same
@@ -171,11 +201,9 @@ struct ReqShape {
     long long ticks_full, ticks_last, head_ticks, ticks;   // per full-pair item, last item, head, request
 };
 
-// NO_CACHE: the launch has no cached segment at all (p.n_cache is not read).
-template <bool NO_CACHE>
 __device__ __forceinline__ ReqShape req_shape(const AttnParams& p, int b, bool* bad = nullptr) {
     ReqShape r;
-    int nq = p.n_q[b], nf = p.n_fresh[b], nc = NO_CACHE ? 0 : p.n_cache[b];
+    int nq = p.n_q[b], nf = p.n_fresh[b], nc = p.n_cache == nullptr ? 0 : p.n_cache[b];      // (nullptr: no cached segment)
     if (nq < 0 || nq > p.Nq_cap || nf < 0 || nf > p.Nf_cap || nc < 0 || nc > p.Nc_cap) {
         if (bad) *bad = true;
         nq = max(0, min(nq, p.Nq_cap));
@@ -207,12 +235,11 @@ struct Plan {
     long long total, chunk;
 };
 
-template <bool NO_CACHE>
 __device__ __forceinline__ Plan plan_shares(const AttnParams& p, int grid, bool* bad = nullptr) {
     Plan pl;
     long long items = 0, ticks = 0, span = 0;      // span: first tick of an item's last step, at most
     for (int b = 0; b < p.B; ++b) {
-        const ReqShape r = req_shape<NO_CACHE>(p, b, bad);
+        const ReqShape r = req_shape(p, b, bad);
         items += r.items;
         ticks += r.ticks;
         if (r.np > 0) span = max(span, (long long)(r.np > 1 ? kTickPair : r.w_last) * (r.steps - 1));
@@ -259,16 +286,15 @@ __device__ __forceinline__ void item_slots(const Plan& pl, long long first_tick,
 }
 
 // Whole-item plan: the item with index `idx`.
-template <bool NO_CACHE>
 __device__ __forceinline__ Segment segment_whole(const AttnParams& p, long long idx) {
     Segment sg;
     long long base = 0;
     int b = 0;
-    ReqShape r = req_shape<NO_CACHE>(p, 0);
+    ReqShape r = req_shape(p, 0);
     while (idx >= base + r.items && b + 1 < p.B) {
         base += r.items;
         ++b;
-        r = req_shape<NO_CACHE>(p, b);
+        r = req_shape(p, b);
     }
     const long long item = idx - base;
     sg.b = b; sg.r = r;
@@ -282,17 +308,16 @@ __device__ __forceinline__ Segment segment_whole(const AttnParams& p, long long 
 }
 
 // Tick plan: the item that contains tick `pos`, and the steps of it that share `c` owns.
-template <bool NO_CACHE>
 __device__ __forceinline__ Segment segment_ticks(const AttnParams& p, const Plan& pl, long long pos,
                                                  int c) {
     Segment sg;
     long long base = 0;
     int b = 0;
-    ReqShape r = req_shape<NO_CACHE>(p, 0);
+    ReqShape r = req_shape(p, 0);
     while (pos >= base + r.ticks && b + 1 < p.B) {
         base += r.ticks;
         ++b;
-        r = req_shape<NO_CACHE>(p, b);
+        r = req_shape(p, b);
     }
     sg.b = b; sg.r = r;
     if (r.np == 0) {                                  // nothing left behind the last live request
@@ -359,450 +384,164 @@ __device__ __forceinline__ float chunk_max(const uint32_t* s) {
     return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
 }
 
-// 2^x for x <= 0 on the FMA pipe: x = n + f with n = round(x) (the magic-number addition leaves n in
-// the low mantissa bits of t), 2^f by a cubic on [-0.5, 0.5] (relative error 7.5e-5, far below the
-// bf16 rounding of the probabilities), n added to the exponent field.  Used for part of the
-// exponentials so that they do not all queue on the special-function unit.
-__device__ __forceinline__ float poly_exp2(float x) {
-    x = fmaxf(x, -126.f);
-    const float t = x + 12582912.f;
-    const float f = x - (t - 12582912.f);
-    float p = fmaf(f, 0.0551716f, 0.2426111f);
-    p = fmaf(p, f, 0.6932610f);
-    p = fmaf(p, f, 0.9999281f);
-    return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
+// Barrier `id` of the CTA's named barriers, for `n` threads.
+__device__ __forceinline__ void named_barrier(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// p = 2^(s*c - m) for 64 logits, written to tensor memory at `tP` (32 columns) as packed bf16;
-// returns their fp32 sum.
-__device__ __forceinline__ float chunk_probabilities(uint32_t tP, const uint32_t* s, float c, float m) {
-    float sum[4] = {0.f, 0.f, 0.f, 0.f};
-    uint32_t pk[kBH / 2];
+// Two fp32 values in one 64-bit register pair, and the packed operations on them.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// p = 2^(s*c - m) for 64 logits, written to tensor memory at `tP` (32 columns) as packed bf16; returns
+// their fp32 sum.  The exponentials replace the logits in place and leave in pieces of 8 columns, so that
+// a thread's 104 registers hold the chunk.  All of them run on the special-function unit: with four softmax
+// warps per scheduler it is busy 70 % of the time, and moving a quarter or an eighth of them to the FMA pipe
+// (a cubic) made the call 4 % and 0 % slower.
+__device__ __forceinline__ float chunk_probabilities(uint32_t tP, uint32_t* s, float c, float m) {
+    const uint64_t c2 = pack2(c, c), m2 = pack2(-m, -m);
+    uint64_t sum[2] = {0, 0};
 #pragma unroll
-    for (int i = 0; i < kBH / 2; ++i) {
-        const float p0 = fast_exp2(fmaf(__uint_as_float(s[2 * i]), c, -m));
-        const float p1 = (i % kPolyEvery == 1) ? poly_exp2(fmaf(__uint_as_float(s[2 * i + 1]), c, -m))
-                                               : fast_exp2(fmaf(__uint_as_float(s[2 * i + 1]), c, -m));
-        sum[i & 3] += p0 + p1;
-        pk[i] = pack_bf16x2(p0, p1);
+    for (int i = 0; i < kBH; i += 2) {
+        float a, b;
+        unpack2(fma2(pack2(__uint_as_float(s[i]), __uint_as_float(s[i + 1])), c2, m2), a, b);
+        s[i] = __float_as_uint(fast_exp2(a));
+        s[i + 1] = __float_as_uint(fast_exp2(b));
     }
-    ptx::tmem_st32(tP, pk);
-    return (sum[0] + sum[1]) + (sum[2] + sum[3]);
+#pragma unroll
+    for (int g = 0; g < kBH; g += 16) {
+        uint32_t pk[8];
+#pragma unroll
+        for (int i = g; i < g + 16; i += 2) {
+            const float a = __uint_as_float(s[i]), b = __uint_as_float(s[i + 1]);
+            sum[(i >> 1) & 1] = add2(sum[(i >> 1) & 1], pack2(a, b));
+            pk[(i - g) >> 1] = pack_bf16x2(a, b);
+        }
+        ptx::tmem_st8(tP + (g >> 1), pk);
+    }
+    float a, b;
+    unpack2(add2(sum[0], sum[1]), a, b);
+    return a + b;
 }
 
-// The segments of one CTA's share, for one of the two kinds of warpgroup: the softmax warpgroups
-// (SOFTMAX_WG, many registers) or the producer / issuer warpgroup (few).  The two instantiations
-// are called from the two sides of the setmaxnreg split so that each is compiled for its own
-// register budget; both execute the same sequence of CTA-wide barriers.
-// STORE: the instantiation for the full step that also refreshes the cache (warp 11 writes the
-// retained K / V rows); the plain instantiation contains none of that code.
-template <int D, bool SOFTMAX_WG, bool STORE>
-__device__ __forceinline__ void run_share(const CUtensorMap* tm_q_, const CUtensorMap* tm_kf_,
-                                          const CUtensorMap* tm_vf_, const CUtensorMap* tm_kc_,
-                                          const CUtensorMap* tm_vc_, const AttnParams& p,
-                                          const StoreParams& sp,
-                                          long long pos, const long long hi, const Plan pl,
-                                          AttnCtrl* ctrl, uint8_t* smem_gen, const uint32_t sQ,
-                                          const uint32_t sKV, const int warp, const int lane) {
+// Live keys of the key tiles of a segment: kBN but for the last tile of either part of the KV sequence.
+struct TileKeys {
+    int jc, vc, jf, vf;     // segment-relative index and live keys of the last cached / last fresh tile
+    __device__ __forceinline__ explicit TileKeys(const SegInfo& it) {
+        jc = it.nt_c - 1 - it.j_first; vc = it.nc - (it.nt_c - 1) * kBN;
+        jf = it.nt - 1 - it.j_first;   vf = it.nf - (it.nt - it.nt_c - 1) * kBN;
+    }
+    __device__ __forceinline__ int operator()(int jl) const { return jl == jc ? vc : jl == jf ? vf : kBN; }
+};
+
+// What one walk over a segment does.  kWalk: one pass, the reference maximum of a row is its maximum over
+// the segment's first key tile.  If a row outgrows that (AttnCtrl::redo) the segment is walked twice more:
+// kMaxOnly finds the rows' maxima, kExact repeats the pass with them.
+enum WalkMode { kWalk, kMaxOnly, kExact };
+
+// ---- softmax / epilogue of one segment: thread = (query row, 64-key chunk) ----------------------------
+template <int D, bool STORE>
+__device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it, uint8_t* smem_gen,
+                                                const uint32_t tmem, const int warp, const int lane, const int mode,
+                                                float& m_known) {
     using Cfg = AttnCfg<D>;
-    constexpr int kStages = Cfg::kStages;
     constexpr int kTileBytes = Cfg::kTileBytes;
     volatile int* abort_flag = &ctrl->abort_flag;
-    const CUtensorMap& tm_q = *tm_q_;
-    const CUtensorMap& tm_kf = *tm_kf_;
-    const CUtensorMap& tm_vf = *tm_vf_;
-    const CUtensorMap& tm_kc = *tm_kc_;
-    const CUtensorMap& tm_vc = *tm_vc_;
-    bool first_segment = true;
-    while (pos < hi) {
-    // ---- the segment: key tiles [j_first, j_first + n_tiles) of item (b, h, query pair) ----
-    const Segment it = pl.whole_items ? segment_whole<STORE>(p, pos)
-                                      : segment_ticks<STORE>(p, pl, pos, (int)blockIdx.x);
-    if (first_segment && SOFTMAX_WG && threadIdx.x == 0) {
-        // tell the merge kernel which item the start of this share cuts
-        CutItem ci;
-        ci.valid = (!pl.whole_items && it.r.np > 0 && it.n_slots >= 2 && it.slot == 1) ? 1 : 0;
-        ci.b = it.b; ci.h = it.h; ci.qp = it.qp; ci.n_slots = it.n_slots; ci.nq = it.r.nq;
-        ci.pad0 = ci.pad1 = 0;
-        p.cut[blockIdx.x] = ci;
-    }
-    first_segment = false;
-    if (it.n_steps == 0) {                              // (uniform for the CTA)
-        pos = pl.whole_items ? pos + gridDim.x : it.next;
-        continue;
-    }
-    const int b = it.b, h = it.h;
-    const int q0 = it.qp * (2 * kBM);
-    const int nq = it.r.nq, nf = it.r.nf, nc = it.r.nc, nt_c = it.r.nt_c;
-    const int ntq = (nq - q0 > kBM) ? 2 : 1;            // live query tiles of this segment
-    const int j_first = it.j_first;
-    const int n_tiles = it.r.nt == 0 ? 0 : it.n_steps;
-    // slot of this segment among the shares that touch the item; a lone segment writes the output
-    const int slot = it.slot;
-    const bool direct = it.n_slots == 1;
-    // A lone query tile would leave half of the CTA idle and run at the speed of its dependency
-    // chain.  Instead the roles of "tile 1" work on the same query tile against the odd key tiles
-    // of the segment while "tile 0" takes the even ones; the two halves (own accumulator, maximum
-    // and sum) are merged in the epilogue.  `lanes` = query-tile roles at work.
-    const bool split = ntq == 1 && n_tiles >= 2;
-    const int lanes = split ? 2 : ntq;
-    // a lone tile's ring starts at the idle second query tile and runs over the extra stage: two
-    // stages more, because its two halves consume K/V tiles at twice the rate per chain
-    const int n_stages = split ? kStages + 2 : kStages;
-    // cache refresh: every item walks all key tiles of its (request, head); key tile j is written to
-    // the cache by the item of query pair j mod np, so every (request, head, key tile) is written
-    // exactly once and the copies are spread evenly over the thread blocks
-    const bool store_item = STORE && n_tiles > 0;
-    const uint32_t ring = split ? sQ + kTileBytes : sKV;
-    uint8_t* const ring_gen = smem_gen + (split ? 1 : 2) * kTileBytes;
-
-    // thread i sets barrier i of the control block up (and takes it down after the segment)
-    if (threadIdx.x < kNumBarriers) {
-        const int i = threadIdx.x;
-        int count = 1;                                               // q_full, kv_full, s_full, o_final
-        if (i >= kBarKvEmpty && i < kBarSFull) count = (split ? 1 : ntq) + (store_item ? 1 : 0);   // commits per stage (+ the cache writer)
-        else if ((i >= kBarPFull && i < kBarOFinal) || i >= kBarSFree) count = kBM / 32;   // one arrival per warp
-        ptx::mbar_init(ptx::smem_addr(&ctrl->q_full + i), count);
-        ptx::fence_barrier_init();
-    }
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
-    const uint32_t tmem = ctrl->tmem_base;
-
-    // key tile jl of this segment -> (segment of the KV sequence, first row, live rows); a tile
-    // yields one P chunk when at most 64 of its keys are live, else two
-    auto tile_seg = [&](int jl, bool& cached, int& row0, int& valid) {
-        const int j = j_first + jl;
-        cached = j < nt_c;
-        const int jj = cached ? j : j - nt_c;
-        row0 = jj * kBN;
-        valid = min(kBN, (cached ? nc : nf) - row0);
-    };
-    auto tile_chunks = [&](int jl) {
-        bool cached; int row0, valid;
-        tile_seg(jl, cached, row0, valid);
-        return valid > kBH ? 2 : 1;
-    };
-    // key tiles of query-tile role t: all of them, or every second one of a lone query tile
-    auto role_tiles = [&](int t) { return split ? (n_tiles + 1 - t) >> 1 : n_tiles; };
-    auto role_tile = [&](int t, int j) { return split ? 2 * j + t : j; };
-
-    if constexpr (!SOFTMAX_WG) {
-    if (warp == 8) {
-        // ================= TMA producer (and, in the cache-refreshing kernel, the cache writer) =================
-        if (n_tiles > 0) {
-            if (lane == 0) {
-                ptx::prefetch_tensormap(&tm_q);
-                ptx::prefetch_tensormap(j_first < nt_c ? &tm_kc : &tm_kf);
-                ptx::prefetch_tensormap(j_first < nt_c ? &tm_vc : &tm_vf);
-                const uint32_t qbar = ptx::smem_addr(&ctrl->q_full);
-                ptx::mbar_arrive_expect_tx(qbar, ntq * kTileBytes);
-                for (int t = 0; t < ntq; ++t)
-                    for (int hf = 0; hf < Cfg::kHalves; ++hf)
-                        ptx::tma_load_4d(sQ + t * kTileBytes + hf * kHalfBytes, &tm_q, qbar, hf * 64, h,
-                                         q0 + t * kBM, b);
-            }
-            // ---- cache writer state (whole warp; used by the cache-refreshing kernel only) ----
-            // The retained rows of every K / V tile this segment stages are copied from shared memory
-            // to their slots in the cache, two ring items behind the loads (an item has landed by
-            // then), before its stage is given back.
-            constexpr int kCpr = D / 8;                 // 16-byte chunks per row of one head
-            constexpr int kRowsPer = 32 / kCpr;         // rows a warp instruction moves
-            constexpr int kLag = 2;
-            const int32_t* keep = nullptr;
-            int nk = 0, lo = 0, cnt = 0;
-            bool mine = false;                          // the key tile being written belongs to this item
-            int r[kBN / 32];
-            if (STORE && store_item) {
-                keep = sp.keep_rows + (size_t)b * sp.store_cap;
-                nk = sp.n_keep[b];
-                if (nk < 0 || nk > sp.store_cap) {
-                    record_status(p.dev_status, REGIONE_DEV_BOUNDS);
-                    nk = max(0, min(nk, sp.store_cap));
-                }
-            }
-            // number of retained rows below `row_first` (the list is ascending): 32-ary search, one
-            // coalesced probe per level
-            auto rows_below = [&](int row_first) {
-                int at0 = 0, len = nk;
-                while (len > 0) {
-                    const int step = (len + 31) / 32;
-                    const int at = at0 + min(lane * step, len - 1);
-                    const bool below = (lane * step < len) && keep[at] < row_first;
-                    const int nb = __popc(__ballot_sync(0xffffffffu, below));   // probes below the target
-                    // the answer lies behind probe nb - 1 and at or before probe nb
-                    const int new_lo = nb == 0 ? at0 : at0 + (nb - 1) * step + 1;
-                    const int new_hi = nb == 0 ? at0 : min(at0 + nb * step, at0 + len);
-                    len = (step == 1) ? 0 : new_hi - new_lo;
-                    at0 = (step == 1) ? at0 + nb : new_lo;
-                }
-                return at0;
-            };
-            // copies ring item x (K of key tile x / 2, or V) to the cache if that tile is this item's to
-            // write, and releases its stage
-            auto write_item = [&](int x) -> bool {
-                const int jl = x >> 1, is_v = x & 1, stage = x % n_stages;
-                bool cached; int row0, valid;
-                tile_seg(jl, cached, row0, valid);
-                if (!is_v) {
-                    mine = (j_first + jl) % it.r.np == it.qp;
-                    if (mine) {
-                        // retained rows of this tile: at most kBN consecutive entries of the ascending list
-                        lo = rows_below(row0);
-                        cnt = 0;                        // length of the run of entries inside this tile
-                        bool run_open = true;
-#pragma unroll
-                        for (int k = 0; k < kBN / 32; ++k) {
-                            const int i = lo + k * 32 + lane;
-                            r[k] = i < nk ? keep[i] - row0 : kBN;
-                            if (r[k] < 0) {             // the list is not ascending
-                                record_status(p.dev_status, REGIONE_DEV_BOUNDS);
-                                r[k] = kBN;
-                            }
-                            const uint32_t inside = __ballot_sync(0xffffffffu, r[k] < valid);
-                            if (run_open) cnt += inside == 0xffffffffu ? 32 : __ffs(~inside) - 1;
-                            run_open = run_open && inside == 0xffffffffu;
-                        }
-                        // entries left over behind the last key tile name rows that do not exist
-                        if (j_first + jl == it.r.nt - 1 && lo + cnt < nk)
-                            record_status(p.dev_status, REGIONE_DEV_BOUNDS);
-                    }
-                }
-                if (mine) {
-                    if (!wait_bar(ptx::smem_addr(&ctrl->kv_full[stage]), (x / n_stages) & 1, abort_flag,
-                                  p.dev_status, p.timeout_cycles))
-                        return false;
-                    const uint8_t* tile = ring_gen + stage * kTileBytes;
-                    uint16_t* dst_base = (is_v ? sp.v_store : sp.k_store) +
-                                         (((size_t)b * sp.store_cap + lo) * p.H + h) * D;
-                    const int q = lane % kCpr;          // this lane's 16-byte chunk of the row
-#pragma unroll
-                    for (int k = 0; k < kBN / 32; ++k) {
-                        if (k * 32 >= cnt) break;                       // (uniform)
-#pragma unroll 1
-                        for (int e0 = 0; e0 < 32; e0 += 4 * kRowsPer) {
-                            // four warp-wide moves at a time: all loads are issued before the first store
-                            uint4 x4[4];
-                            int el[4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                el[u] = e0 + u * kRowsPer + lane / kCpr;    // entry of the tile's run: k * 32 + el
-                                const int rr = __shfl_sync(0xffffffffu, r[k], el[u]);
-                                if (k * 32 + el[u] < cnt)
-                                    x4[u] = *reinterpret_cast<const uint4*>(
-                                        tile + (q >> 3) * kHalfBytes + rr * 128 + (((q & 7) ^ (rr & 7)) << 4));
-                            }
-#pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                if (k * 32 + el[u] < cnt)
-                                    *reinterpret_cast<uint4*>(dst_base + (size_t)(k * 32 + el[u]) * p.H * D + q * 8) = x4[u];
-                        }
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->kv_empty[stage]));
-                return true;
-            };
-            bool ok = true;
-            const int n_items = 2 * n_tiles;
-            for (int i = 0; i < n_items + (STORE && store_item ? kLag : 0) && ok; ++i) {
-                if (STORE && store_item && i >= kLag) ok = write_item(i - kLag);
-                if (i < n_items && ok) {
-                    if (lane == 0) {
-                        const int j = i >> 1, is_v = i & 1;
-                        const int stage = i % n_stages, use = i / n_stages;
-                        if (use > 0)
-                            ok = wait_bar(ptx::smem_addr(&ctrl->kv_empty[stage]), (use - 1) & 1, abort_flag,
-                                          p.dev_status, p.timeout_cycles);
-                        if (ok) {
-                            bool cached; int row0, valid;
-                            tile_seg(j, cached, row0, valid);
-                            const CUtensorMap* map = cached ? (is_v ? &tm_vc : &tm_kc) : (is_v ? &tm_vf : &tm_kf);
-                            const uint32_t bar = ptx::smem_addr(&ctrl->kv_full[stage]);
-                            ptx::mbar_arrive_expect_tx(bar, kTileBytes);
-                            for (int hf = 0; hf < Cfg::kHalves; ++hf)
-                                ptx::tma_load_4d(ring + stage * kTileBytes + hf * kHalfBytes, map, bar, hf * 64, h,
-                                                 row0, b);
-                        }
-                    }
-                    if (STORE) ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;     // (the writer's lanes follow lane 0)
-                }
-            }
-        }
-    } else if (warp == 11) {
-        // ================= issuer of the S products of both query tiles =================
-        // S = Q_t K_j^T goes to ONE staging buffer in tensor memory that the two query tiles share:
-        // a product is issued as soon as its K tile has landed and the buffer's previous contents
-        // have been read into registers by the softmax warps they were computed for.  It does not
-        // have to wait for the P*V products of its own tile, which read P from a place of their own.
-        if (n_tiles > 0) {
-            constexpr uint32_t idesc_s = ptx::idesc_bf16_f32(kBM, kBN, false);
-            constexpr uint32_t hi_k = ptx::smem_desc_hi_sw128(1024);   // 8-row groups 1024 B apart
-            const uint32_t k_lo = ptx::smem_desc_lo(ring, 16);
-            bool ok = wait_bar(ptx::smem_addr(&ctrl->q_full), 0, abort_flag, p.dev_status, p.timeout_cycles);
-            int n_issued = 0;                                   // products so far = uses of the staging buffer
-            for (int jl = 0; jl < n_tiles && ok; ++jl) {
-                const int ik = 2 * jl, sk = ik % n_stages;
-                ok = wait_bar(ptx::smem_addr(&ctrl->kv_full[sk]), (ik / n_stages) & 1, abort_flag,
-                              p.dev_status, p.timeout_cycles);
-                // the roles this key tile feeds: both query tiles, or one half of a lone query tile
-                const int t_first = split ? (jl & 1) : 0, t_last = split ? (jl & 1) : ntq - 1;
-                for (int t = t_first; t <= t_last && ok; ++t) {
-                    if (n_issued > 0)
-                        ok = wait_bar(ptx::smem_addr(&ctrl->s_free), (n_issued - 1) & 1, abort_flag,
-                                      p.dev_status, p.timeout_cycles);
-                    if (!ok) break;
-                    ptx::tc_fence_after_sync();
-                    if (ptx::elect_one()) {
-                        const uint32_t q_lo = ptx::smem_desc_lo(sQ + (split ? 0 : t) * kTileBytes, 16);
-                        const uint32_t b0 = k_lo + ((sk * kTileBytes) >> 4);
-#pragma unroll
-                        for (int kk = 0; kk < D / 16; ++kk) {
-                            const uint32_t off = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
-                            ptx::mma_ss(tmem, ptx::smem_desc_join(q_lo + off, hi_k),
-                                        ptx::smem_desc_join(b0 + off, hi_k), idesc_s, kk > 0);
-                        }
-                        ptx::mma_commit(ptx::smem_addr(&ctrl->s_full[t]));
-                        ptx::mma_commit(ptx::smem_addr(&ctrl->kv_empty[sk]));
-                    }
-                    __syncwarp();
-                    ++n_issued;
-                }
-            }
-        }
-    } else if (warp == 9 || warp == 10) {
-        // ================= issuers of the P*V products: warp 9 for query tile 0, warp 10 for query tile 1 ========
-        // Each whole warp walks its loop and waits on the barriers; one elected lane issues.
-        const int t = warp - 9;
-        if (t < lanes && n_tiles > 0) {
-            const int n_my = role_tiles(t);
-            constexpr uint32_t idesc_pv = ptx::idesc_bf16_f32(kBM, D, true);
-            constexpr uint32_t hi_k = ptx::smem_desc_hi_sw128(1024);   // 8-key groups 1024 B apart
-            // V is MN-major: 64-column boxes kHalfBytes apart (LBO), 8-key groups 1024 B apart (SBO)
-            const uint32_t v_lo = ptx::smem_desc_lo(ring, kHalfBytes);
-            const uint32_t tPt = tmem + kBN + t * (kBN / 2), tOt = tmem + 256 + t * D;
-            // O_t (+)= P_t[chunk] V[64 chunk .. 64 chunk + 64) : A from tensor memory (bf16 pairs,
-            // 8 columns per 16 keys)
-            auto issue_pv = [&](int stage, int chunk, bool accumulate) {
-                const uint32_t b0 = v_lo + ((stage * kTileBytes + chunk * (kBH / 16) * 2048) >> 4);
-#pragma unroll
-                for (int kk = 0; kk < kBH / 16; ++kk)
-                    ptx::mma_ts(tOt, tPt + chunk * (kBH / 2) + kk * 8,
-                                ptx::smem_desc_join(b0 + ((kk * 2048) >> 4), hi_k), idesc_pv,
-                                (accumulate || kk > 0) ? 1u : 0u);
-            };
-            bool ok = true;
-            int nb = 0;                                     // second chunks seen so far
-            for (int j = 0; j < n_my && ok; ++j) {
-                const int jl = role_tile(t, j);
-                const int iv = 2 * jl + 1, sv = iv % n_stages;
-                const bool more = (j + 1 < n_my);
-                const int chunks = tile_chunks(jl);
-                ok = wait_bar(ptx::smem_addr(&ctrl->kv_full[sv]), (iv / n_stages) & 1, abort_flag,
-                              p.dev_status, p.timeout_cycles);
-                if (ok)
-                    ok = wait_bar(ptx::smem_addr(&ctrl->p_full[t][0]), j & 1, abort_flag,
-                                  p.dev_status, p.timeout_cycles);
-                if (!ok) break;
-                if (chunks == 2) {
-                    ptx::tc_fence_after_sync();
-                    if (ptx::elect_one()) issue_pv(sv, 0, j > 0);
-                    __syncwarp();
-                    ok = wait_bar(ptx::smem_addr(&ctrl->p_full[t][1]), nb & 1, abort_flag,
-                                  p.dev_status, p.timeout_cycles);
-                    ++nb;
-                    if (!ok) break;
-                }
-                ptx::tc_fence_after_sync();
-                if (ptx::elect_one()) {
-                    issue_pv(sv, chunks - 1, j > 0 || chunks == 2);
-                    ptx::mma_commit(ptx::smem_addr(&ctrl->pv_done[t]));
-                    if (!more) ptx::mma_commit(ptx::smem_addr(&ctrl->o_final[t]));
-                    ptx::mma_commit(ptx::smem_addr(&ctrl->kv_empty[sv]));
-                }
-                __syncwarp();
-            }
-        }
-    }
-    } else if (warp < 4 * lanes) {
-        // ================= softmax / correction / epilogue =================
-        const int t = warp >> 2;
-        const int row = ((warp & 3) << 5) + lane;                  // row of the query tile
-        const uint32_t lane_sel = (uint32_t)((warp & 3) << 5) << 16;
-        const uint32_t tS = tmem + lane_sel;                       // the S staging buffer both tiles share
-        const uint32_t tP = tmem + lane_sel + kBN + t * (kBN / 2); // this tile's probabilities (bf16 pairs)
-        const uint32_t tO = tmem + lane_sel + 256 + t * D;
-        const float c = p.scale_log2e;
-        float m = -INFINITY, l = 0.f;
-        bool ok = true;
-
-        const int n_my = n_tiles > 0 ? role_tiles(t) : 0;
+    const int t = warp >> 3, ck = (warp >> 2) & 1;
+    const int n_tiles = it.n_tiles;
+    const bool pair = it.nq - it.q0 > kBM;
+    const bool split = !pair && n_tiles >= 2;
+    if (t == 1 && !pair && !split) return;
+    const int row = ((warp & 3) << 5) + lane;                  // row of the query tile
+    const uint32_t lane_sel = (uint32_t)((warp & 3) << 5) << 16;
+    const uint32_t tS = tmem + lane_sel + ck * kBH;            // this chunk of the S staging buffer
+    const uint32_t tP = tmem + lane_sel + kBN + t * (kBN / 2) + ck * (kBH / 2);   // its probabilities (bf16 pairs)
+    // [tile][chunk][row]: maxima at the first key tile, sums at the end
+    float* const exch = reinterpret_cast<float*>(smem_gen + Cfg::kSmemTiles + Cfg::kCtrlBytes) + t * 2 * kBM + row;
+    const float c = p.scale_log2e;
+    float m = -INFINITY, l = 0.f;
+    bool ok = true, outgrown = false;
+    {
+        const TileKeys keys(it);
+        const int n_my = split ? (n_tiles + 1 - t) >> 1 : n_tiles;
+        const uint32_t bar_s = ptx::smem_addr(&ctrl->s_full[t]), bar_free = ptx::smem_addr(&ctrl->s_free);
+        const uint32_t bar_p = ptx::smem_addr(&ctrl->p_full[t][ck]);
+        const uint32_t bar_pv = ptx::smem_addr(ck == 0 ? &ctrl->pv_half[t] : &ctrl->pv_done[t]);
         for (int j = 0; j < n_my; ++j) {
-            bool cached; int row0, valid;
-            tile_seg(role_tile(t, j), cached, row0, valid);
-            const int chunks = valid > kBH ? 2 : 1;
-            ok = wait_bar(ptx::smem_addr(&ctrl->s_full[t]), j & 1, abort_flag, p.dev_status, p.timeout_cycles);
+            const int jl = split ? 2 * j + t : j;
+            const int valid = keys(jl);
+            const int live_keys = valid - ck * kBH;                // live keys of this chunk (<= 0: none)
+            ok = wait_bar(bar_s, j & 1, abort_flag, p.dev_status, p.timeout_cycles);
+            uint32_t s[kBH];
+            if (ok) {
+                ptx::tc_fence_after_sync();
+                if (live_keys > 0) {
+                    ptx::tmem_ld32(tS, s);
+                    ptx::tmem_ld32(tS + 32, s + 32);
+                    ptx::tmem_wait_ld();
+                }
+                // the logits are in registers: the staging buffer may take the next product (of the other
+                // query tile, or of this tile's next key tile)
+                ptx::tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar_free);
+                if (live_keys > 0 && live_keys < kBH) mask_dead_keys(s, live_keys);
+            }
+            if (mode == kMaxOnly) {
+                if (!ok) break;
+                if (live_keys > 0) m = fmaxf(m, chunk_max(s) * c);
+                continue;
+            }
+            // The reference maximum of a row is its maximum over the first key tile (any reference within a
+            // factor of 2^60 of the true maximum gives the same relative accuracy): the two chunks' threads
+            // of a row agree on it once and then run independently of each other.
+            if (j == 0) {
+                if (mode == kExact) {
+                    m = m_known;
+                } else {
+                    exch[ck * kBM] = (ok && live_keys > 0) ? chunk_max(s) * c : -INFINITY;
+                    named_barrier(1 + t, 2 * kBM);
+                    m = fmaxf(exch[0], exch[kBM]);
+                    named_barrier(1 + t, 2 * kBM);                 // (the sums go to the same place at the end)
+                }
+            }
             if (!ok) break;
-            ptx::tc_fence_after_sync();
-            uint32_t s[kBN];
-            ptx::tmem_ld32(tS, s);
-            ptx::tmem_ld32(tS + 32, s + 32);
-            if (chunks == 2) {
-                ptx::tmem_ld32(tS + 64, s + 64);
-                ptx::tmem_ld32(tS + 96, s + 96);
-            }
-            ptx::tmem_wait_ld();
-            // the logits are in registers: the staging buffer may take the next product (of the other
-            // query tile, or of this tile's next key tile)
-            ptx::tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->s_free));
-            float mt;
-            if (chunks == 2) {
-                if (valid < kBN) mask_dead_keys(s + kBH, valid - kBH);
-                mt = fmaxf(chunk_max(s), chunk_max(s + kBH));
-            } else {
-                if (valid < kBH) mask_dead_keys(s, valid);
-                mt = chunk_max(s);
-            }
-            mt *= c;
-            // P_t and O_t belong to the products of the key tile before this one until they have
-            // completed (they run in the shadow of this tile's wait for S and of its row maximum)
+            if (live_keys <= 0) continue;                          // (a last tile with one live chunk)
+            // the chunk's place in tensor memory belongs to the previous key tile's product until that has completed
             if (j > 0) {
-                ok = wait_bar(ptx::smem_addr(&ctrl->pv_done[t]), (j - 1) & 1, abort_flag, p.dev_status,
-                              p.timeout_cycles);
+                ok = wait_bar(bar_pv, (j - 1) & 1, abort_flag, p.dev_status, p.timeout_cycles);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
             }
-            if (j == 0) {
-                m = mt;
-            } else if (__any_sync(0xffffffffu, mt > m + 8.f)) {
-                const float m_new = fmaxf(m, mt);
-                const float alpha = fast_exp2(m - m_new);
-                uint32_t r[32];
-#pragma unroll 1
-                for (int ch = 0; ch < D / 32; ++ch) {
-                    ptx::tmem_ld32(tO + ch * 32, r);
-                    ptx::tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-                    ptx::tmem_st32(tO + ch * 32, r);
-                }
-                l *= alpha;
-                m = m_new;
-            }
-            // first chunk of probabilities (keys 0..63 of the tile)
-            l += chunk_probabilities(tP, s, c, m);
+            const float sum = chunk_probabilities(tP, s, c, m);
+            outgrown |= !(sum < kOutgrownSum);
+            l += sum;
             ptx::tmem_wait_st();
-            if (valid < kBN) {
-                // last tile of a segment: zero the V rows behind the live prefix (0 * NaN = NaN)
-                const int iv = 2 * role_tile(t, j) + 1, sv = iv % n_stages;
+            if (valid < kBN && ck == 0) {
+                // last tile of a part: zero the V rows behind the live prefix (0 * NaN = NaN)
+                const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
+                const int iv = 2 * jl + 1, sv = iv % n_stages;
                 ok = wait_bar(ptx::smem_addr(&ctrl->kv_full[sv]), (iv / n_stages) & 1, abort_flag,
                               p.dev_status, p.timeout_cycles);
                 if (!ok) break;
                 if (row >= valid) {
-                    uint8_t* vrow = ring_gen + sv * kTileBytes + row * 128;
+                    uint8_t* vrow = smem_gen + ((split ? 1 : 2) + sv) * kTileBytes + row * 128;
 #pragma unroll
                     for (int hf = 0; hf < Cfg::kHalves; ++hf)
 #pragma unroll
@@ -813,160 +552,482 @@ __device__ __forceinline__ void run_share(const CUtensorMap* tm_q_, const CUtens
             }
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->p_full[t][0]));
-            if (chunks == 2) {
-                // second chunk (keys 64..127) while the first chunk's product runs
-                l += chunk_probabilities(tP + kBH / 2, s + kBH, c, m);
-                ptx::tmem_wait_st();
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->p_full[t][1]));
-            }
+            if (lane == 0) ptx::mbar_arrive(bar_p);
         }
-        // epilogue (rows past n_q are not written).  A thread holds one row, so storing straight
-        // from registers would touch 32 different rows per warp instruction; instead each warp
-        // passes 128-byte row pieces through its own 4 KB corner of the (now idle) query tile in
-        // shared memory and stores four whole pieces per instruction.
-        const int wrow0 = q0 + (split ? 0 : t) * kBM + ((warp & 3) << 5);   // first query row of this warp
-        const int live_rows = min(max(nq - wrow0, 0), 32);
-        const bool live = lane < live_rows;
-        // where this thread's query row goes in `out` (-1: the row is dead); the lookup is issued
-        // ahead of the wait for the last product and used after it
-        int dst_row = -1;
-        if (live && direct)
-            dst_row = p.out_rows != nullptr ? p.out_rows[(size_t)b * p.Nq_cap + wrow0 + lane] : wrow0 + lane;
-        if (n_tiles > 0 && ok) {
-            ok = wait_bar(ptx::smem_addr(&ctrl->o_final[t]), 0, abort_flag, p.dev_status, p.timeout_cycles);
-            if (ok) ptx::tc_fence_after_sync();
-        }
-        // lone query tile: role 1 leaves its (max, sum) in shared memory (its accumulator stays in
-        // tensor memory) and is done; role 0 merges the halves
-        float2* const half_ml = reinterpret_cast<float2*>(smem_gen + Cfg::kSmemTiles + Cfg::kCtrlBytes);
-        float w_own = 1.f, w_other = 0.f;                   // weights of the two accumulators
-        if (split && t == 1) {
-            half_ml[row] = make_float2(m, l);
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->half_done));
-        } else if (split && ok) {
-            ok = wait_bar(ptx::smem_addr(&ctrl->half_done), 0, abort_flag, p.dev_status, p.timeout_cycles);
-            if (ok) ok = wait_bar(ptx::smem_addr(&ctrl->o_final[1]), 0, abort_flag, p.dev_status, p.timeout_cycles);
-            if (ok) {
-                ptx::tc_fence_after_sync();
-                const float2 other = half_ml[row];
-                const float m_all = fmaxf(m, other.x);
-                w_own = fast_exp2(m - m_all);
-                w_other = other.y > 0.f ? fast_exp2(other.x - m_all) : 0.f;
-                l = w_own * l + w_other * other.y;
-                m = m_all;
-            }
-        }
-        // lone tile: 32 columns of this row's two accumulators, weighted and added
-        auto load_merged = [&](int col, uint32_t* r) {
-            uint32_t r1[32];
-            ptx::tmem_ld32(tO + col, r);
-            ptx::tmem_ld32(tO + D + col, r1);
-            ptx::tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                r[i] = __float_as_uint(fmaf(w_own, __uint_as_float(r[i]), w_other * __uint_as_float(r1[i])));
-        };
-        if (!(split && t == 1)) {
-        uint8_t* const stage = smem_gen + t * kTileBytes + (warp & 3) * (kTileBytes / 4);
-        // `to` = this lane's destination row (counted from g_row0), -1 to drop the row
-        auto store_pieces = [&](const uint4 (&v)[8], uint8_t* g_row0, size_t row_stride, int to) {
-            // piece q of row r sits at 16-byte column q ^ (r & 7): both the row-wise writes and
-            // the piece-wise reads are free of bank conflicts without padding
-            uint4* dst = reinterpret_cast<uint4*>(stage + lane * 128);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) dst[q ^ (lane & 7)] = v[q];
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int rr = i * 4 + (lane >> 3);
-                const uint4 x = *reinterpret_cast<const uint4*>(stage + rr * 128 +
-                                                                 (((lane & 7) ^ (rr & 7)) << 4));
-                const int to_rr = __shfl_sync(0xffffffffu, to, rr);
-                if (to_rr >= 0)
-                    *reinterpret_cast<uint4*>(g_row0 + to_rr * row_stride + (lane & 7) * 16) = x;
-            }
-            __syncwarp();
-        };
-        if (direct) {
-            // O / l -> bf16 -> out
-            if (dst_row >= p.out_cap || (dst_row < 0 && live)) {     // destination out of range: dropped
-                record_status(p.dev_status, REGIONE_DEV_BOUNDS);
-                dst_row = -1;
-            }
-            const size_t row_stride = (size_t)p.H * D * 2;
-            uint8_t* g_row0 = reinterpret_cast<uint8_t*>(p.out) +
-                              (((size_t)b * p.out_cap) * p.H + h) * D * 2;      // row 0 of the request
-            if (n_tiles == 0) {
-                if (dst_row >= 0)
-                    for (int q = 0; q < D / 8; ++q)
-                        reinterpret_cast<uint4*>(g_row0 + dst_row * row_stride)[q] = make_uint4(0, 0, 0, 0);
-            } else if (ok) {
-                const float inv = l > 0.f ? 1.f / l : 0.f;
-#pragma unroll 1
-                for (int c64 = 0; c64 < D / 64; ++c64) {
-                    uint32_t r[64];
-                    if (!split) {
-                        ptx::tmem_ld32(tO + c64 * 64, r);
-                        ptx::tmem_ld32(tO + c64 * 64 + 32, r + 32);
-                        ptx::tmem_wait_ld();
-                    } else {
-                        load_merged(c64 * 64, r);
-                        load_merged(c64 * 64 + 32, r + 32);
-                    }
-                    uint4 v[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        v[q].x = pack_bf16x2(__uint_as_float(r[8 * q + 0]) * inv, __uint_as_float(r[8 * q + 1]) * inv);
-                        v[q].y = pack_bf16x2(__uint_as_float(r[8 * q + 2]) * inv, __uint_as_float(r[8 * q + 3]) * inv);
-                        v[q].z = pack_bf16x2(__uint_as_float(r[8 * q + 4]) * inv, __uint_as_float(r[8 * q + 5]) * inv);
-                        v[q].w = pack_bf16x2(__uint_as_float(r[8 * q + 6]) * inv, __uint_as_float(r[8 * q + 7]) * inv);
-                    }
-                    store_pieces(v, g_row0 + c64 * 128, row_stride, dst_row);
-                }
-            }
-        } else {
-            // unnormalised O and (m, l) of this segment -> its workspace slot
-            const size_t item_idx = ((size_t)b * p.H + h) * p.P_cap + it.qp;
-            const size_t prow_w = (item_idx * p.max_slots + slot) * (2 * kBM) + (split ? 0 : t) * kBM +
-                                  ((warp & 3) << 5);
-            if (n_tiles == 0) {
-                if (live) p.part_ml[prow_w + lane] = make_float2(-INFINITY, 0.f);
-            } else if (ok) {
-                uint8_t* g_row0 = reinterpret_cast<uint8_t*>(p.part_o + prow_w * D);
-#pragma unroll 1
-                for (int ch = 0; ch < D / 32; ++ch) {
-                    uint32_t r[32];
-                    if (!split) {
-                        ptx::tmem_ld32(tO + ch * 32, r);
-                        ptx::tmem_wait_ld();
-                    } else {
-                        load_merged(ch * 32, r);
-                    }
-                    uint4 v[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) v[q] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-                    store_pieces(v, g_row0 + ch * 128, (size_t)D * 4, live ? lane : -1);
-                }
-                if (live) p.part_ml[prow_w + lane] = make_float2(m, l);
-            }
-        }
-        }   // all roles but the second half of a lone tile
-        ptx::fence_proxy_async_smem();      // the next segment's query tile arrives by TMA
     }
+    if (mode == kMaxOnly) {
+        exch[ck * kBM] = m;
+        named_barrier(1 + t, 2 * kBM);
+        m_known = fmaxf(exch[0], exch[kBM]);
+        return;
+    }
+    if (outgrown && mode == kWalk) ctrl->redo = 1;
 
-    // ---- end of the segment: every role is done with shared and tensor memory ----
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
-    if (threadIdx.x < kNumBarriers) ptx::mbar_inval(ptx::smem_addr(&ctrl->q_full + threadIdx.x));
-    pos = pl.whole_items ? pos + gridDim.x : it.next;
-    if (*abort_flag) break;
-    }   // segments
+    // ---- epilogue (rows past n_q are not written).  A thread holds one row, so storing straight
+    // from registers would touch 32 different rows per warp instruction; instead each warp
+    // passes row pieces of 32 columns through its own 4 KB corner of the (now idle) query tiles in
+    // shared memory and stores whole pieces.  The columns of a query tile are dealt to the
+    // warpgroups at work on it: two, or all four of a lone tile.
+    const int qt = split ? 0 : t;
+    const int wrow0 = it.q0 + qt * kBM + ((warp & 3) << 5);     // first query row of this warp
+    const bool live = wrow0 + lane < it.nq;
+    const bool direct = it.n_slots == 1;
+    // where this thread's query row goes in `out` (-1: the row is dead); the lookup is issued
+    // ahead of the wait for the last product and used after it
+    int dst_row = -1;
+    if (live && direct)
+        dst_row = p.out_rows != nullptr ? p.out_rows[(size_t)it.b * p.Nq_cap + wrow0 + lane] : wrow0 + lane;
+    if (n_tiles > 0 && ok) {
+        ok = wait_bar(ptx::smem_addr(&ctrl->o_final[t]), 0, abort_flag, p.dev_status, p.timeout_cycles);
+        if (split && ok)
+            ok = wait_bar(ptx::smem_addr(&ctrl->o_final[1 - t]), 0, abort_flag, p.dev_status, p.timeout_cycles);
+        if (ok) ptx::tc_fence_after_sync();
+    }
+    float w0 = 1.f, w1 = 0.f;                           // weights of the two accumulators (lone tile)
+    if (n_tiles > 0) {
+        exch[ck * kBM] = l;
+        if (split) {
+            // the ring is idle by now: the maxima of the two halves go there
+            float* const ms = reinterpret_cast<float*>(smem_gen + 2 * kTileBytes) + row;
+            if (ck == 0) ms[t * kBM] = m;
+            named_barrier(3, 4 * kBM);
+            const float* const e0 = exch - t * 2 * kBM;
+            const float m0 = ms[0], m1 = ms[kBM], l0 = e0[0] + e0[kBM], l1 = e0[2 * kBM] + e0[3 * kBM];
+            m = fmaxf(m0, m1);
+            w0 = l0 > 0.f ? fast_exp2(m0 - m) : 0.f;
+            w1 = l1 > 0.f ? fast_exp2(m1 - m) : 0.f;
+            l = w0 * l0 + w1 * l1;
+        } else {
+            named_barrier(1 + t, 2 * kBM);
+            l = exch[0] + exch[kBM];
+        }
+    }
+    // this warp's 32-column pieces of the row: [pc0, pc1)
+    constexpr int kPieces = D / 32;
+    const int per = split ? (kPieces >= 4 ? 1 : (t == 0 ? 1 : 0)) : kPieces / 2;
+    const int pc0 = split ? (kPieces >= 4 ? 2 * ck + t : ck) : ck * per, pc1 = pc0 + per;
+    const uint32_t tO = tmem + lane_sel + 256 + (split ? 0 : t * D);
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    uint8_t* const stage = smem_gen + Cfg::kStageAt + warp * 4096;
+    const size_t out_stride = (size_t)p.H * D * 2;
+    uint8_t* const out0 = reinterpret_cast<uint8_t*>(p.out) + (((size_t)it.b * p.out_cap) * p.H + it.h) * D * 2;
+    const size_t prow_w = ((size_t)it.item * p.max_slots + it.slot) * (2 * kBM) + qt * kBM + ((warp & 3) << 5);
+    if (direct && (dst_row >= p.out_cap || (dst_row < 0 && live))) {     // destination out of range: dropped
+        record_status(p.dev_status, REGIONE_DEV_BOUNDS);
+        dst_row = -1;
+    }
+    if (n_tiles == 0) {
+        // no keys: zero rows, or an empty slot
+        if (ck == 0 && direct && dst_row >= 0)
+            for (int q = 0; q < D / 8; ++q)
+                reinterpret_cast<uint4*>(out0 + dst_row * out_stride)[q] = make_uint4(0, 0, 0, 0);
+        if (ck == 0 && !direct && live) p.part_ml[prow_w + lane] = make_float2(-INFINITY, 0.f);
+    } else if (ok) {
+#pragma unroll 1
+        for (int pc = pc0; pc < pc1; ++pc) {
+            uint32_t r[32];
+            ptx::tmem_ld32(tO + pc * 32, r);
+            if (split) {
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    uint32_t r1[16];
+                    ptx::tmem_ld16(tO + D + pc * 32 + hf * 16, r1);
+                    ptx::tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        r[hf * 16 + i] = __float_as_uint(fmaf(w0, __uint_as_float(r[hf * 16 + i]), w1 * __uint_as_float(r1[i])));
+                }
+            } else {
+                ptx::tmem_wait_ld();
+            }
+            // 16-byte chunk q of row r sits at column q ^ (r & 7): both the row-wise writes and
+            // the piece-wise reads are free of bank conflicts without padding
+            uint4* const mine = reinterpret_cast<uint4*>(stage + lane * 128);
+            if (direct) {
+                // O / l -> bf16 -> out: 64-byte pieces, 8 rows per instruction
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint4 v;
+                    v.x = pack_bf16x2(__uint_as_float(r[8 * q + 0]) * inv, __uint_as_float(r[8 * q + 1]) * inv);
+                    v.y = pack_bf16x2(__uint_as_float(r[8 * q + 2]) * inv, __uint_as_float(r[8 * q + 3]) * inv);
+                    v.z = pack_bf16x2(__uint_as_float(r[8 * q + 4]) * inv, __uint_as_float(r[8 * q + 5]) * inv);
+                    v.w = pack_bf16x2(__uint_as_float(r[8 * q + 6]) * inv, __uint_as_float(r[8 * q + 7]) * inv);
+                    mine[q ^ (lane & 7)] = v;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int rr = i * 8 + (lane >> 2), q = lane & 3;
+                    const uint4 x = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((q ^ (rr & 7)) << 4));
+                    const int to = __shfl_sync(0xffffffffu, dst_row, rr);
+                    if (to >= 0) *reinterpret_cast<uint4*>(out0 + to * out_stride + pc * 64 + q * 16) = x;
+                }
+            } else {
+                // unnormalised O of this segment -> its workspace slot: 128-byte pieces, 4 rows per instruction
+#pragma unroll
+                for (int q = 0; q < 8; ++q) mine[q ^ (lane & 7)] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                __syncwarp();
+                uint8_t* const g0 = reinterpret_cast<uint8_t*>(p.part_o + prow_w * D) + pc * 128;
+                const int n_live = it.nq - wrow0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = i * 4 + (lane >> 3), q = lane & 7;
+                    const uint4 x = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((q ^ (rr & 7)) << 4));
+                    if (rr < n_live) *reinterpret_cast<uint4*>(g0 + (size_t)rr * D * 4 + q * 16) = x;
+                }
+            }
+            __syncwarp();
+        }
+        if (!direct && live && ck == 0 && (!split || t == 0)) p.part_ml[prow_w + lane] = make_float2(m, l);
+    }
+    ptx::fence_proxy_async_smem();      // the next segment's query tile arrives by TMA
 }
+
+// ---- cache refresh: copies of retained rows, done by the producer warp while it has nothing to load ---------
+// The rows travel as bulk copies (one per lane: global -> slot of shared memory -> cache), so the copies
+// take no registers, no issue slots to speak of and no time of the tensor cores.  The launch's rows
+// (K of every request, then V) are cut into equal contiguous shares, one per CTA, whatever attention work
+// the CTA has.  An item is one row, or a slot's length of it where a row is longer than that; a unit is up
+// to `per_unit` consecutive items of one request, lane i moving item i.
+struct CachePump {
+    const StoreParams* sp;
+    const int32_t* n_rows;
+    AttnCtrl* ctrl;
+    int32_t* dev_status;
+    int row_bytes, item_bytes, per_row; // items per row
+    uint32_t slots;                     // shared-memory address of slot 0
+    int n_slots, slot_bytes, per_unit;
+    int x, b, i, run, live_rows;        // cursor of the loads: tensor, request, item, items of the run, source rows
+    int left;                           // items not yet loaded
+    int head, tail;                     // units loaded / stored through the present slots
+    int row, before;                    // list entry of this lane's next item, and the one ahead of it
+
+    __device__ __forceinline__ int kept(int req, bool report) const {
+        const int nk = sp->n_keep[req];
+        if (nk >= 0 && nk <= sp->store_cap) return nk;
+        if (report && blockIdx.x == 0) record_status(dev_status, REGIONE_DEV_BOUNDS);
+        return nk < 0 ? 0 : sp->store_cap;
+    }
+    // from an item index behind the runs x, b to the run that holds it (a request without rows stores nothing)
+    __device__ __forceinline__ void open_run(int B) {
+        for (;;) {
+            live_rows = min(n_rows[b], sp->src_cap);
+            run = live_rows > 0 ? kept(b, false) * per_row : 0;
+            if (i < run) return;
+            i -= run;
+            if (++b == B) { b = 0; ++x; }
+        }
+    }
+    // list entries of the next unit's items, fetched one unit ahead of their use
+    __device__ __forceinline__ void fetch(int lane) {
+        row = before = -1;
+        if (lane < min(per_unit, min(run - i, left))) {
+            const int32_t* keep = sp->keep_rows + (size_t)b * sp->store_cap;
+            const int j = (i + lane) / per_row;
+            row = keep[j];
+            if (j > 0) before = keep[j - 1];
+        }
+    }
+    __device__ __forceinline__ void use_slots(uint32_t at, int n, int bytes, int lane) {
+        slots = at; n_slots = n; slot_bytes = bytes;
+        per_unit = min(32, bytes / item_bytes);
+        head = tail = 0;
+        if (lane < n) ptx::mbar_init(ptx::smem_addr(&ctrl->copy_full[lane]), 1);
+        ptx::fence_barrier_init();
+        __syncwarp();
+        if (left > 0) fetch(lane);
+    }
+    __device__ __forceinline__ void begin(const AttnParams& p, const StoreParams& s, AttnCtrl* c, int d, uint32_t at, int slot,
+                                          int lane) {
+        sp = &s; n_rows = p.n_fresh; ctrl = c; dev_status = p.dev_status;
+        row_bytes = p.H * d * 2;
+        per_row = (row_bytes + slot - 1) / slot;
+        item_bytes = min(row_bytes, slot);
+        long long total = 0;
+        for (int r = 0; r < p.B; ++r) {
+            const int nk = kept(r, lane == 0);
+            if (n_rows[r] > 0) total += 2LL * nk * per_row;
+        }
+        const long long per = (total + gridDim.x - 1) / gridDim.x, first = per * blockIdx.x;
+        left = (int)max(0LL, min(per, total - first));
+        x = b = 0;
+        i = (int)first;
+        if (left > 0) open_run(p.B);
+        use_slots(at, kCopySlots, slot, lane);
+    }
+    __device__ __forceinline__ bool busy() const { return left > 0 || tail < head; }
+    // One step of the pump (whole warp): stores the oldest unit if it has landed, then loads the next one
+    // if its slot is free.
+    __device__ __forceinline__ void poll(int B, int lane) {
+        if (tail < head) {
+            const int slot = tail % n_slots;
+            const bool landed = ptx::mbar_test_wait(ptx::smem_addr(&ctrl->copy_full[slot]), (tail / n_slots) & 1);
+            if (__any_sync(0xffffffffu, landed)) {
+                if ((ctrl->copy_valid[slot] >> lane) & 1u) {
+                    const int at = ctrl->copy_item[slot] + lane, j = at / per_row, off = (at - j * per_row) * item_bytes;
+                    ptx::bulk_store(ctrl->copy_dst[slot] + (size_t)j * row_bytes + off,
+                                    slots + slot * slot_bytes + lane * item_bytes, min(item_bytes, row_bytes - off));
+                }
+                ptx::bulk_commit();
+                ++tail;
+            }
+        }
+        // (one slot of slack: all but the latest store have been read out of shared memory)
+        if (left > 0 && head - tail < n_slots - 1) {
+            ptx::bulk_wait_read<1>();
+            __syncwarp();
+            const int n = min(per_unit, min(run - i, left));
+            const bool ok = row >= 0 && row < live_rows && row > before;
+            if (lane < n && !ok) record_status(dev_status, REGIONE_DEV_BOUNDS);
+            const uint32_t valid = __ballot_sync(0xffffffffu, lane < n && ok);
+            const int slot = head % n_slots;
+            const uint32_t bar = ptx::smem_addr(&ctrl->copy_full[slot]);
+            const int off = ((i + lane) % per_row) * item_bytes;
+            const int bytes = (valid >> lane) & 1u ? min(item_bytes, row_bytes - off) : 0;
+            const int unit_bytes = __reduce_add_sync(0xffffffffu, bytes);
+            if (lane == 0) {
+                ctrl->copy_valid[slot] = valid;
+                ctrl->copy_item[slot] = i;
+                ctrl->copy_dst[slot] = sp->dst[x] + (size_t)b * sp->store_cap * row_bytes;
+                ptx::mbar_arrive_expect_tx(bar, unit_bytes);
+            }
+            __syncwarp();
+            if (bytes > 0)
+                ptx::bulk_load(slots + slot * slot_bytes + lane * item_bytes,
+                               sp->src[x] + ((size_t)b * sp->src_cap + row) * row_bytes + off, bytes, bar);
+            ++head;
+            left -= n;
+            i += n;
+            if (left > 0) {
+                if (i >= run) open_run(B);
+                fetch(lane);
+            }
+        }
+    }
+    // Stores everything that is left; false when a load did not land within `limit` cycles.
+    __device__ __forceinline__ bool drain(int B, int lane, long long limit) {
+        long long t0 = clock64();
+        int last = tail;
+        while (busy()) {
+            poll(B, lane);
+            if (tail != last) { last = tail; t0 = clock64(); }
+            if (__any_sync(0xffffffffu, clock64() - t0 > limit)) {
+                record_status(dev_status, REGIONE_DEV_TIMEOUT);
+                return false;
+            }
+        }
+        return true;
+    }
+};
+
+// ---- TMA producer of one segment (whole warp; lane 0 issues) ----------------------------------------------
+template <int D, bool STORE>
+__device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUtensorMap* tm_kf, const CUtensorMap* tm_vf,
+                                             const CUtensorMap* tm_kc, const CUtensorMap* tm_vc, const AttnParams& p,
+                                             AttnCtrl* ctrl, const SegInfo& it, const uint32_t smem, const int lane,
+                                             CachePump& pump) {
+    using Cfg = AttnCfg<D>;
+    constexpr int kTileBytes = Cfg::kTileBytes;
+    const int n_tiles = it.n_tiles;
+    if (n_tiles == 0) return;
+    const int ntq = it.nq - it.q0 > kBM ? 2 : 1;
+    const bool split = ntq == 1 && n_tiles >= 2;
+    const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
+    const uint32_t ring = smem + (split ? 1 : 2) * kTileBytes;
+    const int nt_c = it.nt_c, j_first = it.j_first, h = it.h, b = it.b;
+    if (lane == 0) {
+        ptx::prefetch_tensormap(tm_q);
+        ptx::prefetch_tensormap(j_first < nt_c ? tm_kc : tm_kf);
+        ptx::prefetch_tensormap(j_first < nt_c ? tm_vc : tm_vf);
+        const uint32_t qbar = ptx::smem_addr(&ctrl->q_full);
+        ptx::mbar_arrive_expect_tx(qbar, ntq * kTileBytes);
+        for (int t = 0; t < ntq; ++t)
+            for (int hf = 0; hf < Cfg::kHalves; ++hf)
+                ptx::tma_load_4d(smem + t * kTileBytes + hf * kHalfBytes, tm_q, qbar, hf * 64, h, it.q0 + t * kBM, b);
+    }
+    int stage = 0, use = 0;
+    for (int i = 0; i < 2 * n_tiles; ++i) {
+        const int j = j_first + (i >> 1), is_v = i & 1;
+        if (use > 0) {
+            const uint32_t bar = ptx::smem_addr(&ctrl->kv_empty[stage]);
+            if constexpr (STORE) {
+                // rows of the cache are copied while the stage is not free yet
+                while (pump.busy() && !__any_sync(0xffffffffu, ptx::mbar_test_wait(bar, (use - 1) & 1)) && !ctrl->abort_flag)
+                    pump.poll(p.B, lane);
+            }
+            if (!wait_bar(bar, (use - 1) & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
+        }
+        if (lane == 0) {
+            const bool cached = j < nt_c;
+            const CUtensorMap* map = cached ? (is_v ? tm_vc : tm_kc) : (is_v ? tm_vf : tm_kf);
+            const uint32_t bar = ptx::smem_addr(&ctrl->kv_full[stage]);
+            ptx::mbar_arrive_expect_tx(bar, kTileBytes);
+            for (int hf = 0; hf < Cfg::kHalves; ++hf)
+                ptx::tma_load_4d(ring + stage * kTileBytes + hf * kHalfBytes, map, bar, hf * 64, h,
+                                 (cached ? j : j - nt_c) * kBN, b);
+        }
+        __syncwarp();
+        if (++stage == n_stages) { stage = 0; ++use; }
+    }
+    if constexpr (STORE) {
+        // ... and while the segment's last products run
+        while (pump.busy() && !__any_sync(0xffffffffu, ptx::mbar_test_wait(ptx::smem_addr(&ctrl->o_final[0]), 0)) &&
+               !ctrl->abort_flag)
+            pump.poll(p.B, lane);
+    }
+}
+
+// ---- issuer of the S products of both query tiles (whole warp, one elected lane issues) ------------------
+// S = Q_t K_j^T goes to ONE staging buffer in tensor memory that the two query tiles share: a product is
+// issued as soon as its K tile has landed and the buffer's previous contents have been read into registers
+// by the softmax warps they were computed for.  It does not have to wait for the P*V products of its own
+// tile, which read P from a place of their own.
+template <int D, bool STORE>
+__device__ __forceinline__ void issue_s_segment(const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it, const uint32_t smem,
+                                                const uint32_t tmem) {
+    using Cfg = AttnCfg<D>;
+    constexpr int kTileBytes = Cfg::kTileBytes;
+    const int n_tiles = it.n_tiles;
+    if (n_tiles == 0) return;
+    const int ntq = it.nq - it.q0 > kBM ? 2 : 1;
+    const bool split = ntq == 1 && n_tiles >= 2;
+    const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
+    constexpr uint32_t idesc_s = ptx::idesc_bf16_f32(kBM, kBN, false);
+    constexpr uint32_t hi_k = ptx::smem_desc_hi_sw128(1024);   // 8-row groups 1024 B apart
+    const uint32_t k_lo = ptx::smem_desc_lo(smem + (split ? 1 : 2) * kTileBytes, 16);
+    const uint32_t q_base = ptx::smem_desc_lo(smem, 16);
+    if (!wait_bar(ptx::smem_addr(&ctrl->q_full), 0, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
+    int n_issued = 0;                                   // products so far = uses of the staging buffer
+    int sk = 0, use = 0;
+    for (int jl = 0; jl < n_tiles; ++jl) {
+        if (!wait_bar(ptx::smem_addr(&ctrl->kv_full[sk]), use & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
+        // the roles this key tile feeds: both query tiles, or one half of a lone query tile
+        const int t_first = split ? (jl & 1) : 0, t_last = split ? (jl & 1) : ntq - 1;
+        for (int t = t_first; t <= t_last; ++t) {
+            if (n_issued > 0 && !wait_bar(ptx::smem_addr(&ctrl->s_free), (n_issued - 1) & 1, &ctrl->abort_flag,
+                                          p.dev_status, p.timeout_cycles))
+                return;
+            ptx::tc_fence_after_sync();
+            if (ptx::elect_one()) {
+                const uint32_t q_lo = q_base + (((split ? 0 : t) * kTileBytes) >> 4);
+                const uint32_t b0 = k_lo + ((sk * kTileBytes) >> 4);
+#pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk) {
+                    const uint32_t off = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
+                    ptx::mma_ss(tmem, ptx::smem_desc_join(q_lo + off, hi_k),
+                                ptx::smem_desc_join(b0 + off, hi_k), idesc_s, kk > 0);
+                }
+                ptx::mma_commit(ptx::smem_addr(&ctrl->s_full[t]));
+                ptx::mma_commit(ptx::smem_addr(&ctrl->kv_empty[sk]));
+            }
+            __syncwarp();
+            ++n_issued;
+        }
+        sk += 2;
+        if (sk >= n_stages) { sk -= n_stages; ++use; }
+    }
+}
+
+// ---- issuer of the P*V products of query-tile role t (whole warp, one elected lane issues) ----------------
+template <int D, bool STORE>
+__device__ __forceinline__ void issue_pv_segment(const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it, const uint32_t smem,
+                                                 const uint32_t tmem, const int t, const int lane, const int mode) {
+    using Cfg = AttnCfg<D>;
+    constexpr int kTileBytes = Cfg::kTileBytes;
+    const int n_tiles = it.n_tiles;
+    const int ntq = it.nq - it.q0 > kBM ? 2 : 1;
+    const bool split = ntq == 1 && n_tiles >= 2;
+    if (n_tiles == 0 || t >= (split ? 2 : ntq)) return;
+    const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
+    const TileKeys keys(it);
+    const int n_my = split ? (n_tiles + 1 - t) >> 1 : n_tiles;
+    constexpr uint32_t idesc_pv = ptx::idesc_bf16_f32(kBM, D, true);
+    constexpr uint32_t hi_k = ptx::smem_desc_hi_sw128(1024);   // 8-key groups 1024 B apart
+    // V is MN-major: 64-column boxes kHalfBytes apart (LBO), 8-key groups 1024 B apart (SBO)
+    const uint32_t v_lo = ptx::smem_desc_lo(smem + (split ? 1 : 2) * kTileBytes, kHalfBytes);
+    const uint32_t tPt = tmem + kBN + t * (kBN / 2), tOt = tmem + 256 + t * D;
+    // O_t (+)= P_t[chunk] V[64 chunk .. 64 chunk + 64) : A from tensor memory (bf16 pairs,
+    // 8 columns per 16 keys)
+    auto issue_pv = [&](int stage, int chunk, bool accumulate) {
+        const uint32_t b0 = v_lo + ((stage * kTileBytes + chunk * (kBH / 16) * 2048) >> 4);
+#pragma unroll
+        for (int kk = 0; kk < kBH / 16; ++kk)
+            ptx::mma_ts(tOt, tPt + chunk * (kBH / 2) + kk * 8,
+                        ptx::smem_desc_join(b0 + ((kk * 2048) >> 4), hi_k), idesc_pv,
+                        (accumulate || kk > 0) ? 1u : 0u);
+    };
+    int nb = 0;                                     // second chunks seen so far
+    for (int j = 0; j < n_my; ++j) {
+        const int jl = split ? 2 * j + t : j;
+        const int iv = 2 * jl + 1, sv = iv % n_stages;
+        const bool more = (j + 1 < n_my);
+        const int chunks = keys(jl) > kBH ? 2 : 1;
+        if (!wait_bar(ptx::smem_addr(&ctrl->kv_full[sv]), (iv / n_stages) & 1, &ctrl->abort_flag, p.dev_status,
+                      p.timeout_cycles))
+            return;
+        if (mode == kMaxOnly) {                     // no products in this pass: the stage is given back
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->kv_empty[sv]));
+            continue;
+        }
+        if (!wait_bar(ptx::smem_addr(&ctrl->p_full[t][0]), j & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
+        if (chunks == 2) {
+            ptx::tc_fence_after_sync();
+            if (ptx::elect_one()) {
+                issue_pv(sv, 0, j > 0);
+                ptx::mma_commit(ptx::smem_addr(&ctrl->pv_half[t]));
+            }
+            __syncwarp();
+            if (!wait_bar(ptx::smem_addr(&ctrl->p_full[t][1]), nb & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
+            ++nb;
+        }
+        ptx::tc_fence_after_sync();
+        if (ptx::elect_one()) {
+            issue_pv(sv, chunks - 1, j > 0 || chunks == 2);
+            if (chunks == 1) ptx::mma_commit(ptx::smem_addr(&ctrl->pv_half[t]));
+            ptx::mma_commit(ptx::smem_addr(&ctrl->pv_done[t]));
+            if (!more) ptx::mma_commit(ptx::smem_addr(&ctrl->o_final[t]));
+            ptx::mma_commit(ptx::smem_addr(&ctrl->kv_empty[sv]));
+        }
+        __syncwarp();
+    }
+}
+
+// ---- the share of one CTA: plan and next segment (one warp computes them, the others read SegInfo) --------
+struct ShareCursor {
+    Plan pl;
+    long long pos, hi;
+    bool first;
+    // The next live segment of the share into *out (out->live = 0 when the share ends).
+    __device__ __forceinline__ void next(const AttnParams& p, SegInfo* out, const int lane) {
+        while (pos < hi) {
+            const Segment it = pl.whole_items ? segment_whole(p, pos) : segment_ticks(p, pl, pos, (int)blockIdx.x);
+            if (first && lane == 0) {
+                // tell the merge kernel which item the start of this share cuts
+                CutItem ci;
+                ci.valid = (!pl.whole_items && it.r.np > 0 && it.n_slots >= 2 && it.slot == 1) ? 1 : 0;
+                ci.b = it.b; ci.h = it.h; ci.qp = it.qp; ci.n_slots = it.n_slots; ci.nq = it.r.nq;
+                ci.pad0 = ci.pad1 = 0;
+                p.cut[blockIdx.x] = ci;
+            }
+            first = false;
+            pos = pl.whole_items ? pos + gridDim.x : it.next;
+            if (it.n_steps == 0) continue;
+            if (lane == 0) {
+                out->b = it.b; out->h = it.h; out->q0 = it.qp * (2 * kBM); out->nq = it.r.nq;
+                out->j_first = it.j_first; out->n_tiles = it.r.nt == 0 ? 0 : it.n_steps;
+                out->nt_c = it.r.nt_c; out->nt = it.r.nt; out->nc = it.r.nc; out->nf = it.r.nf;
+                out->item = (it.b * p.H + it.h) * p.P_cap + it.qp; out->slot = it.slot; out->n_slots = it.n_slots;
+                out->live = 1;
+            }
+            return;
+        }
+        if (lane == 0) {
+            if (first) p.cut[blockIdx.x].valid = 0;
+            out->live = 0;
+        }
+        first = false;
+    }
+};
 
 template <int D, bool STORE>
 __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, const CUtensorMap& tm_kf,
@@ -974,45 +1035,103 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
                                                       const CUtensorMap& tm_vc, const AttnParams& p,
                                                       const StoreParams& sp) {
     using Cfg = AttnCfg<D>;
-    constexpr int kTileBytes = Cfg::kTileBytes;
-
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
-    uint8_t* smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
-    const uint32_t sQ = smem_base;                      // 2 query tiles
-    const uint32_t sKV = smem_base + 2 * kTileBytes;    // ring of K/V stages
-    AttnCtrl* ctrl = reinterpret_cast<AttnCtrl*>(smem_gen + Cfg::kSmemTiles);
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t smem = ptx::smem_addr(smem_raw);     // 2 query tiles, then the ring of K/V stages
+    AttnCtrl* ctrl = reinterpret_cast<AttnCtrl*>(smem_raw + Cfg::kSmemTiles);
     volatile int* abort_flag = &ctrl->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    grid_dependency_wait();                             // (everything below reads the launch's inputs)
-    // this CTA's share [pos, hi) of the item sequence or of the cost axis
-    bool bad = false;
-    const Plan pl = plan_shares<STORE>(p, gridDim.x, &bad);
-    if (bad && blockIdx.x == 0 && threadIdx.x == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
-    // (whole items are dealt round-robin, so that the CTAs running at any one time work on
-    // neighbouring items, which share K/V tiles in L2; a share of steps is one contiguous range)
-    long long pos = pl.whole_items ? (long long)blockIdx.x : (long long)blockIdx.x * pl.chunk;
-    const long long hi = pl.whole_items ? pl.total : min(pos + pl.chunk, pl.total);
-    if (pos >= hi) {                                    // uniform for the CTA
-        if (threadIdx.x == 0) p.cut[blockIdx.x].valid = 0;
-        return;
-    }
-
-    grid_launch_dependents();                      // the merge kernel may queue up behind this CTA
-    if (threadIdx.x == 0) ctrl->abort_flag = 0;
-    if (warp == 9) {
+    if (warp == kWarpPv) {
         ptx::tmem_alloc(ptx::smem_addr(&ctrl->tmem_base), 512);
         ptx::tmem_relinquish();
     }
-    if (warp >= 8) {
-        ptx::reg_dealloc<56>();                         // producer / issuer warpgroup gives registers up
-        run_share<D, false, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, p, sp, pos, hi, pl, ctrl, smem_gen,
-                                   sQ, sKV, warp, lane);
+    grid_dependency_wait();                             // (everything below reads the launch's inputs)
+    grid_launch_dependents();                           // the merge kernel may queue up behind this CTA
+    ShareCursor cur;
+    if (warp == kWarpS) {
+        // this CTA's share [pos, hi) of the item sequence or of the cost axis
+        // (whole items are dealt round-robin, so that the CTAs running at any one time work on
+        // neighbouring items, which share K/V tiles in L2; a share of steps is one contiguous range)
+        bool bad = false;
+        cur.pl = plan_shares(p, gridDim.x, &bad);
+        if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
+        cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)blockIdx.x * cur.pl.chunk;
+        cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
+        cur.first = true;
+        cur.next(p, &ctrl->seg[0], lane);
+        if (lane == 0) ctrl->abort_flag = 0;
+    }
+
+    // The two sides of the register split walk the same segments: the softmax warpgroups hold a chunk of 64
+    // logits per thread, the producer / issuer warpgroup gives registers up.  CTA-wide barriers around a
+    // segment: `set-up` (control block's barriers initialised, next segment known) and `end` (every role is
+    // done with shared and tensor memory).
+    auto set_up = [&](const SegInfo& it) {
+        // thread i sets barrier i of the control block up
+        const int ntq = it.nq - it.q0 > kBM ? 2 : 1;
+        const bool split = ntq == 1 && it.n_tiles >= 2;
+        if (threadIdx.x < kNumBarriers) {
+            const int i = threadIdx.x;
+            int count = 1;                                               // q_full, kv_full, s_full, commits
+            if (i >= kBarKvEmpty && i < kBarSFull) count = split ? 1 : ntq;      // commits per stage
+            else if (i >= kBarPFull && i < kBarOFinal) count = kBM / 32;         // one arrival per warp
+            else if (i == kBarSFree) count = 2 * (kBM / 32);
+            ptx::mbar_init(ptx::smem_addr(&ctrl->q_full + i), count);
+            ptx::fence_barrier_init();
+        }
+        if (threadIdx.x == 0) ctrl->redo = 0;
+        ptx::tc_fence_before_sync();
+        __syncthreads();
+        ptx::tc_fence_after_sync();
+    };
+    auto tear_down = [&]() {
+        ptx::tc_fence_before_sync();
+        __syncthreads();
+        ptx::tc_fence_after_sync();
+        if (threadIdx.x < kNumBarriers) ptx::mbar_inval(ptx::smem_addr(&ctrl->q_full + threadIdx.x));
+    };
+    // what to do after a walk: repeat the segment (new mode) or go on
+    auto repeat = [&](int& mode) {
+        const bool redo = mode == kWalk && *reinterpret_cast<volatile int*>(&ctrl->redo) != 0;
+        const int next_mode = redo ? kMaxOnly : mode == kMaxOnly ? kExact : kWalk;
+        const bool again = next_mode != kWalk;
+        mode = next_mode;
+        __syncthreads();                                // (redo has been read by everyone)
+        return again;
+    };
+    __syncthreads();
+    const uint32_t tmem = ctrl->tmem_base;
+    CachePump pump;
+    int k = 0, mode = kWalk;
+    if (warp >= kSoftmaxWarps) {
+        ptx::reg_dealloc<64>();
+        if constexpr (STORE) {
+            if (warp == kWarpLoad) pump.begin(p, sp, ctrl, D, smem + Cfg::kCopyAt, Cfg::kCopySlotBytes, lane);
+        }
+        while (ctrl->seg[k].live && !*abort_flag) {
+            const SegInfo& it = ctrl->seg[k];
+            set_up(it);
+            if (warp == kWarpLoad) {
+                load_segment<D, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, p, ctrl, it, smem, lane, pump);
+            } else if (warp == kWarpS) {
+                issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
+                // (the next segment is planned behind the last product, ahead of the end of this one)
+                if (mode == kWalk) cur.next(p, &ctrl->seg[k ^ 1], lane);
+            } else {
+                issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, warp - kWarpPv, lane, mode);
+            }
+            tear_down();
+            if (!repeat(mode)) k ^= 1;
+        }
     } else {
-        ptx::reg_alloc<224>();                          // a row of 128 logits stays in registers
-        run_share<D, true, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, p, sp, pos, hi, pl, ctrl, smem_gen,
-                                  sQ, sKV, warp, lane);
+        ptx::reg_alloc<104>();
+        float m_known = -INFINITY;
+        while (ctrl->seg[k].live && !*abort_flag) {
+            set_up(ctrl->seg[k]);
+            softmax_segment<D, STORE>(p, ctrl, ctrl->seg[k], smem_raw, tmem, warp, lane, mode, m_known);
+            tear_down();
+            if (!repeat(mode)) k ^= 1;
+        }
     }
 
     // ================= teardown =================
@@ -1024,9 +1143,34 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
-    if (warp == 9) {
+    if (warp == kWarpPv) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(ctrl->tmem_base, 512);
+        ptx::tmem_dealloc(tmem, 512);
+    }
+    if constexpr (STORE) {
+        // the rows that the walks left no time for: every tile is idle now, so that enough of them are in
+        // flight to run at the speed of memory
+        if (warp == kWarpLoad && !*abort_flag && pump.busy()) {
+            bool ok = pump.left == 0;
+            if (!ok) {
+                // what is in the small slots first, then all of shared memory
+                const int left = pump.left;
+                pump.left = 0;
+                ok = pump.drain(p.B, lane, p.timeout_cycles);
+                pump.left = left;
+                ptx::bulk_wait_read<0>();
+                __syncwarp();
+                if (lane < kCopySlots) ptx::mbar_inval(ptx::smem_addr(&ctrl->copy_full[lane]));
+                __syncwarp();
+                pump.use_slots(smem, Cfg::kTailSlots, Cfg::kTailSlotBytes, lane);
+            }
+            if (ok) ok = pump.drain(p.B, lane, p.timeout_cycles);
+            if (!ok) {
+                const long long t0 = clock64();
+                while (clock64() - t0 < 2000000LL) __nanosleep(1000);
+            }
+        }
+        if (warp == kWarpLoad) ptx::bulk_wait_all();
     }
 }
 
@@ -1048,7 +1192,7 @@ region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_vf,
                               const __grid_constant__ CUtensorMap tm_kc,
                               const __grid_constant__ CUtensorMap tm_vc, const AttnParams p,
-                              const StoreParams sp) {
+                              const __grid_constant__ StoreParams sp) {
     attention_kernel_body<D, true>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, sp);
 }
 
@@ -1322,8 +1466,9 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
     prm.timeout_cycles = kTimeoutCycles;
     StoreParams sp = {};
     if (store != nullptr) {
-        sp.keep_rows = store->keep_rows; sp.n_keep = store->n_keep; sp.store_cap = store->cap;
-        sp.k_store = store->k_cache; sp.v_store = store->v_cache;
+        sp.keep_rows = store->keep_rows; sp.n_keep = store->n_keep; sp.store_cap = store->cap; sp.src_cap = Nf_cap;
+        sp.src[0] = reinterpret_cast<const uint8_t*>(k_fresh); sp.src[1] = reinterpret_cast<const uint8_t*>(v_fresh);
+        sp.dst[0] = reinterpret_cast<uint8_t*>(store->k_cache); sp.dst[1] = reinterpret_cast<uint8_t*>(store->v_cache);
     }
     const size_t rows = slot_rows(lp, B, H);
     prm.part_o = reinterpret_cast<float*>(workspace);
