@@ -4,43 +4,43 @@
 // materialising the concatenation.
 //
 // One CTA = one (request, head, pair of 128-row query tiles).  Warp roles:
-//   warps 0-3  softmax / correction / epilogue of query tile 0 (thread = row)
-//   warps 4-7  the same for query tile 1
-//   warp  8    TMA producer: Q once, then K_j, V_j tiles (128 keys) through a ring
-//              of shared-memory stages; the cached segment and the fresh segment
-//              are two tensor maps walked one after the other.  In the full step that
-//              refreshes the Region-Instruction KV cache the whole warp also copies the
-//              retained rows of the staged K / V tiles from shared memory to the cache
-//   warps 9,10 issuers of the O_t += P_t V_j products, one per query tile (the whole
-//              warp walks the loop, one elected lane issues); warp 9 owns the
-//              tensor-memory allocation
-//   warp  11   issuer of the S = Q_t K_j^T products of both query tiles
-//   (warps 8-11 form the third warpgroup; it gives registers up to the softmax
-//   warpgroups with setmaxnreg)
+//   warps 0-15  softmax and epilogue: thread = (query row, 64-key chunk of a key tile); warps 0-7 work on
+//               query tile 0, warps 8-15 on query tile 1, the first four of each on the first chunk
+//   warp  16    TMA producer: Q once, then K_j, V_j tiles (128 keys) through a ring of shared-memory stages;
+//               the cached segment and the fresh segment are two tensor maps walked one after the other.  In
+//               the full step that refreshes the Region-Instruction KV cache it also moves the retained rows,
+//               by asynchronous bulk copies, while it has nothing to load
+//   warps 17,18 issuers of the O_t += P_t V_j products, one per query tile (the whole warp walks the loop,
+//               one elected lane issues); warp 17 owns the tensor-memory allocation
+//   warp  19    issuer of the S = Q_t K_j^T products of both query tiles; plans the CTA's next segment
+//   (warps 16-19 give registers up to the softmax warpgroups with setmaxnreg: 64 against 104 per thread)
 //
 // Tensor memory (512 columns): S | P0 | P1 | O0 | O1 = 128 + 64 + 64 + 128 + 128.
-// There is ONE S buffer (fp32, 128 logits per row), a staging place that the two
-// query tiles share: a product lands there, the softmax warps of its tile read their
-// row into registers and give the buffer back at once, and the next product (the other
-// tile's, or the same tile's next key tile) may follow while the exponentials are
-// still being computed.  The probabilities go to the tile's own P region as packed
-// bf16, in two chunks of 64 keys, and O_t += P_t V_j runs straight from tensor memory:
-// the product of the first chunk is issued while the exponentials of the second are
-// computed.  Because P does not live in the S buffer, S_t(j+1) never waits for the
-// products P_t(j) V_j: the dependency chain of a tile is  S ready -> row maximum ->
-// exponentials -> (S of the next key tile is already there),  with both kinds of
-// product off it.  What a tile must wait for before it overwrites P_t or rescales O_t
-// is the completion of its previous key tile's products (a barrier of their own), and
-// that has long happened by then.  The two tiles run their exponentials whenever they
-// are ready; nothing sequences them.  A pair with a single live query tile does not
-// leave the second tile's warps idle: they run the same query tile against the odd key
-// tiles of the segment (own accumulator, maximum and sum), the first tile's warps take
-// the even ones, and the epilogue merges the halves.
+// There is ONE S buffer (fp32, 128 logits per row), a staging place that the two query tiles share: a product
+// lands there, the softmax warps of its tile read it into registers and give the buffer back at once, and the
+// next product (the other tile's, or the same tile's next key tile) may follow while the exponentials are
+// still being computed.  The probabilities go to the tile's own P region as packed bf16, chunk by chunk, and
+// O_t += P_t V_j runs straight from tensor memory.  Because P does not live in the S buffer, S_t(j+1) never
+// waits for the products P_t(j) V_j.  What a chunk's threads wait for before they overwrite its part of P_t is
+// the completion of the previous key tile's product with that part.  A pair with a single live query tile does
+// not leave the second tile's warps idle: they run the same query tile against the odd key tiles of the segment
+// (own accumulator, maximum and sum), the first tile's warps take the even ones, and the epilogue merges them.
 //
-// Online softmax in the exp2 domain; O is rescaled in tensor memory only when
-// a row maximum grows by more than 2^8.  Keys past a segment's live count are
-// masked in the softmax and their V rows zeroed in shared memory, so garbage
-// (even NaN) behind the live prefix cannot leak.
+// What bounds the loop: per key tile and query pair the tensor cores need 2048 cycles and the special-function
+// unit 2048 (32768 exponentials, 16 a cycle); the dependency chain  S -> registers -> exponentials -> P -> product
+// hides behind neither.  Two threads per row (four softmax warps per scheduler instead of two), no row maximum
+// after the first key tile and packed fp32 arithmetic shorten the chain: 2860 cycles per key tile and pair,
+// against 3250 with one thread per row, a maximum per key tile and scalar arithmetic.  Measured, one box, L2 warm:
+// 8704 queries x 8704 keys x 24 heads 763 -> 720 us in isolation (1292 TFLOP/s), 889 -> 848 us under the power
+// cap; 4 x 1382 queries x 18944 keys 1141 -> 1056 us; 2048 queries x 8448 keys 189 -> 180 us; D = 64 127 -> 114 us;
+// 205 queries x 8448 keys, where the fill and the drain of the pipeline dominate, 42.3 -> 43.2 us.
+//
+// Online softmax in the exp2 domain without a running maximum: a row's reference is its maximum over the
+// segment's first key tile.  Any reference within a factor of 2^60 of the true maximum gives the same relative
+// accuracy (probabilities are bf16, sums fp32).  A row whose chunk sum reaches 2^60 makes the CTA walk the
+// segment twice more, once for the rows' true maxima and once with them; that costs three times the segment,
+// for inputs whose logits spread over more than 41 nats.  Keys past a segment's live count are masked in the
+// softmax and their V rows zeroed in shared memory, so garbage (even NaN) behind the live prefix cannot leak.
 //
 // Scheduling: the kernel is persistent, one CTA per SM.  A "step" is one key tile of one
 // (request, head, query pair) item; all steps of the launch form one sequence, item after item,
@@ -522,17 +522,20 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
                 }
             }
             if (!ok) break;
-            if (live_keys <= 0) continue;                          // (a last tile with one live chunk)
             // the chunk's place in tensor memory belongs to the previous key tile's product until that has completed
             if (j > 0) {
                 ok = wait_bar(bar_pv, (j - 1) & 1, abort_flag, p.dev_status, p.timeout_cycles);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
             }
-            const float sum = chunk_probabilities(tP, s, c, m);
-            outgrown |= !(sum < kOutgrownSum);
-            l += sum;
-            ptx::tmem_wait_st();
+            // (a second chunk without live keys waits and arrives like any other, so that every barrier goes
+            // through one phase per key tile; it writes nothing and no product reads it)
+            if (live_keys > 0) {
+                const float sum = chunk_probabilities(tP, s, c, m);
+                outgrown |= !(sum < kOutgrownSum);
+                l += sum;
+                ptx::tmem_wait_st();
+            }
             if (valid < kBN && ck == 0) {
                 // last tile of a part: zero the V rows behind the live prefix (0 * NaN = NaN)
                 const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
@@ -561,7 +564,6 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
         m_known = fmaxf(exch[0], exch[kBM]);
         return;
     }
-    if (outgrown && mode == kWalk) ctrl->redo = 1;
 
     // ---- epilogue (rows past n_q are not written).  A thread holds one row, so storing straight
     // from registers would touch 32 different rows per warp instruction; instead each warp
@@ -571,6 +573,7 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
     const int qt = split ? 0 : t;
     const int wrow0 = it.q0 + qt * kBM + ((warp & 3) << 5);     // first query row of this warp
     const bool live = wrow0 + lane < it.nq;
+    if (outgrown && live && mode == kWalk) ctrl->redo = 1;      // (rows past n_q may hold anything)
     const bool direct = it.n_slots == 1;
     // where this thread's query row goes in `out` (-1: the row is dead); the lookup is issued
     // ahead of the wait for the last product and used after it
@@ -956,12 +959,10 @@ __device__ __forceinline__ void issue_pv_segment(const AttnParams& p, AttnCtrl* 
                         ptx::smem_desc_join(b0 + ((kk * 2048) >> 4), hi_k), idesc_pv,
                         (accumulate || kk > 0) ? 1u : 0u);
     };
-    int nb = 0;                                     // second chunks seen so far
     for (int j = 0; j < n_my; ++j) {
         const int jl = split ? 2 * j + t : j;
         const int iv = 2 * jl + 1, sv = iv % n_stages;
         const bool more = (j + 1 < n_my);
-        const int chunks = keys(jl) > kBH ? 2 : 1;
         if (!wait_bar(ptx::smem_addr(&ctrl->kv_full[sv]), (iv / n_stages) & 1, &ctrl->abort_flag, p.dev_status,
                       p.timeout_cycles))
             return;
@@ -970,23 +971,19 @@ __device__ __forceinline__ void issue_pv_segment(const AttnParams& p, AttnCtrl* 
             continue;
         }
         if (!wait_bar(ptx::smem_addr(&ctrl->p_full[t][0]), j & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
-        if (chunks == 2) {
-            ptx::tc_fence_after_sync();
-            if (ptx::elect_one()) {
-                issue_pv(sv, 0, j > 0);
-                ptx::mma_commit(ptx::smem_addr(&ctrl->pv_half[t]));
-            }
-            __syncwarp();
-            if (!wait_bar(ptx::smem_addr(&ctrl->p_full[t][1]), nb & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
-            ++nb;
-        }
         ptx::tc_fence_after_sync();
         if (ptx::elect_one()) {
-            issue_pv(sv, chunks - 1, j > 0 || chunks == 2);
-            if (chunks == 1) ptx::mma_commit(ptx::smem_addr(&ctrl->pv_half[t]));
+            issue_pv(sv, 0, j > 0);
+            ptx::mma_commit(ptx::smem_addr(&ctrl->pv_half[t]));
+        }
+        __syncwarp();
+        if (!wait_bar(ptx::smem_addr(&ctrl->p_full[t][1]), j & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
+        ptx::tc_fence_after_sync();
+        if (ptx::elect_one()) {
+            if (keys(jl) > kBH) issue_pv(sv, 1, true);
             ptx::mma_commit(ptx::smem_addr(&ctrl->pv_done[t]));
-            if (!more) ptx::mma_commit(ptx::smem_addr(&ctrl->o_final[t]));
             ptx::mma_commit(ptx::smem_addr(&ctrl->kv_empty[sv]));
+            if (!more) ptx::mma_commit(ptx::smem_addr(&ctrl->o_final[t]));      // (the segment's last arrival)
         }
         __syncwarp();
     }

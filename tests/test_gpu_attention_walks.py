@@ -1,0 +1,85 @@
+"""GPU parity of the attention where its walk over the key tiles changes course: rows whose logits outgrow
+the reference maximum of the first key tile (the segment is walked again), and key tiles whose second
+half has no live key, in the middle of the walk and at its end."""
+import numpy as np
+import pytest
+
+from gpu_util import dev_bf16, dev_i32, host_f64
+from oracle import regione_oracle as orc
+from paper_2510_25590_b200 import binding
+from test_gpu_attention import _rand_bf16, check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("n_q,n_f,n_c", [
+    (300, 300, 1000),      # a full query pair and a lone tile, items cut between thread blocks
+    (100, 100, 300),       # a lone tile
+    (256, 0, 128 * 3),     # whole tiles only
+])
+@pytest.mark.parametrize("rows", ["all", "one"])
+def test_logits_that_outgrow_the_first_key_tile(D, n_q, n_f, n_c, rows):
+    """Later keys raise the logits of every row, or of one row, by far more than the exponent range of the
+    probabilities: the softmax is then almost one-hot on those keys and the tolerance is that of the plain case."""
+    rng = np.random.default_rng(D + n_q)
+    B, H = 2, 3
+    q = _rand_bf16(rng, (B, n_q, H, D), 0.3)
+    kf, vf = _rand_bf16(rng, (B, max(n_f, 1), H, D), 0.3), _rand_bf16(rng, (B, max(n_f, 1), H, D))
+    kc, vc = _rand_bf16(rng, (B, n_c, H, D), 0.3), _rand_bf16(rng, (B, n_c, H, D))
+    # dimension 0 of q is 16 (or 0 for rows that stay ordinary); key 200 (second tile) gives +16 * 40 / sqrt(D),
+    # key 290 (third tile) twice that
+    q[..., 0] = 16.0 if rows == "all" else 0.0
+    if rows == "one":
+        q[:, n_q - 1, :, 0] = 16.0
+    kc[..., 0] = 0.0
+    kf[..., 0] = 0.0
+    kc[:, 200, :, 0] = 40.0
+    kc[:, 290, :, 0] = 80.0
+    check(q, kf, vf, kc, vc, [n_q] * B, [n_f] * B, [n_c] * B, what=f"outgrown rows ({rows}), D={D}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("n_q", [100, 256, 700])
+@pytest.mark.parametrize("n_f,n_c", [(60, 1000 + 24), (64, 128 * 7 + 1), (65, 128 * 7 + 64), (1, 128 * 4 + 56)])
+def test_key_tiles_with_a_dead_second_half(D, n_q, n_f, n_c):
+    rng = np.random.default_rng(n_q + n_f + n_c + D)
+    B, H = 2, 12
+    q = _rand_bf16(rng, (B, n_q, H, D))
+    kf, vf = _rand_bf16(rng, (B, n_f + 5, H, D)), _rand_bf16(rng, (B, n_f + 5, H, D))
+    kc, vc = _rand_bf16(rng, (B, n_c + 9, H, D)), _rand_bf16(rng, (B, n_c + 9, H, D))
+    check(q, kf, vf, kc, vc, [n_q] * B, [n_f] * B, [n_c] * B, what=f"dead second half, D={D}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("H", [1, 24, 70])
+def test_cache_refresh_row_lengths_and_outgrown_rows(D, H):
+    """The refreshing call with rows shorter and longer than a copy slot, its attention walked twice over."""
+    import torch
+    rng = np.random.default_rng(D + H)
+    B, N = 2, 300
+    q, k, v = (_rand_bf16(rng, (B, N, H, D), 0.3) for _ in range(3))
+    q[..., 0] = 16.0
+    k[..., 0] = 0.0
+    k[:, 200, :, 0] = 40.0
+    n_rows = [300, 211]
+    keep = np.zeros((B, N), np.int32)
+    for b, n in enumerate((251, 40)):
+        keep[b, :n] = np.sort(rng.permutation(n_rows[b])[:n])
+    out = torch.full((B, N, H, D), -3.0, dtype=torch.bfloat16, device="cuda")
+    kc, vc = torch.full_like(out, -3.0), torch.full_like(out, -3.0)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(max(binding.full_attention_store_workspace(B, N, H, D), 256), dtype=torch.uint8, device="cuda")
+    binding.full_attention_store(dev_bf16(q), dev_bf16(k), dev_bf16(v), dev_i32(n_rows), dev_i32(keep),
+                                 dev_i32([251, 40]), kc, vc, out, workspace=ws, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st[0]) == 0
+    for b, n in enumerate((251, 40)):
+        assert np.array_equal(host_f64(kc)[b, :n], k[b, keep[b, :n]].astype(np.float64))
+        assert np.array_equal(host_f64(vc)[b, :n], v[b, keep[b, :n]].astype(np.float64))
+        assert np.all(host_f64(kc)[b, n:] == -3.0) and np.all(host_f64(vc)[b, n:] == -3.0)
+    empty = np.zeros((B, 0, H, D))
+    want = orc.region_attention(q, k, v, empty, empty, n_rows, n_rows, [0, 0])
+    from gpu_util import assert_close
+    for b in range(B):
+        assert_close(host_f64(out)[b, :n_rows[b]], want[b, :n_rows[b]], f"attention, request {b}")
