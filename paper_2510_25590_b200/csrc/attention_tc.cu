@@ -87,20 +87,21 @@ struct AttnCfg {
     static constexpr int kTileBytes = kHalves * kHalfBytes;
     static constexpr int kStages = (D == 128) ? 4 : 6;
     // 2 query tiles + the ring + one more stage that only a lone query tile uses (its ring is that
-    // stage, the ordinary ring and the idle second query tile: kStages + 2 stages)
+    // stage, the ordinary ring and the idle second query tile: kStages + 2 stages, an even number: K tiles and
+    // V tiles have stages of their own)
     static constexpr int kSmemTiles = (2 + kStages + 1) * kTileBytes;
     static constexpr int kCtrlBytes = 512;
     static constexpr int kExchBytes = 4 * kBM * 4;         // exchange of the chunks' maxima and sums
     static constexpr int kExtraAt = kSmemTiles + kCtrlBytes + kExchBytes;
     // D = 128 fills shared memory: the epilogue stages its rows (4 KB per softmax warp) in the idle query
-    // tiles, and a launch that refreshes the cache copies rows through the extra stage, which a lone query
-    // tile then does without.  D = 64 has room for both.
+    // tiles, and a launch that refreshes the cache copies rows through the extra stage, a lone query tile
+    // then keeps to the ordinary number of stages.  D = 64 has room for both.
     static constexpr int kStageAt = (D == 128) ? 0 : kExtraAt;
     static constexpr int kCopySlotBytes = (D == 128) ? 8192 : 4096;
     static constexpr int kCopyAt = (D == 128) ? (2 + kStages) * kTileBytes : kExtraAt + kSoftmaxWarps * 4096;
     static constexpr int kSmemBytes = kExtraAt + (D == 128 ? 0 : kSoftmaxWarps * 4096 + kCopySlots * kCopySlotBytes);
     static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
-    __host__ __device__ static constexpr int lone_stages(bool store) { return kStages + (D == 128 && store ? 1 : 2); }
+    __host__ __device__ static constexpr int lone_stages(bool store) { return kStages + (D == 128 && store ? 0 : 2); }
     // slots of the copies that are left when the walks are over and all tiles are idle
     static constexpr int kTailSlots = 3, kTailSlotBytes = (D == 128) ? 65536 : 40960;
     static_assert(kTailSlots * kTailSlotBytes <= kSmemTiles, "tail slots");
@@ -126,6 +127,7 @@ struct AttnCtrl {
                                 // may be overwritten
     uint64_t pv_half[2];        // [query tile] ... after every key tile's first product: the first chunk's P may be
     uint64_t s_free;            // the shared S buffer has been read by the softmax warps it was computed for
+    uint64_t v_full[4];         // [V stage] key tiles of role 1 of a lone query tile (see v_landing)
     uint32_t tmem_base;
     int abort_flag;
     int redo;                   // a row outgrew the reference maximum of its first key tile
@@ -139,11 +141,12 @@ struct AttnCtrl {
 
 // The barriers of AttnCtrl as one array starting at q_full.
 constexpr int kBarKvEmpty = 9, kBarSFull = 17, kBarPFull = 19, kBarOFinal = 23, kBarPvDone = 25, kBarPvHalf = 27,
-              kBarSFree = 29, kNumBarriers = 30;
+              kBarSFree = 29, kNumBarriers = 34;
 static_assert(offsetof(AttnCtrl, kv_empty) == kBarKvEmpty * 8 && offsetof(AttnCtrl, s_full) == kBarSFull * 8 &&
               offsetof(AttnCtrl, p_full) == kBarPFull * 8 && offsetof(AttnCtrl, o_final) == kBarOFinal * 8 &&
               offsetof(AttnCtrl, pv_done) == kBarPvDone * 8 && offsetof(AttnCtrl, pv_half) == kBarPvHalf * 8 &&
-              offsetof(AttnCtrl, s_free) == kBarSFree * 8 && offsetof(AttnCtrl, tmem_base) == kNumBarriers * 8 &&
+              offsetof(AttnCtrl, s_free) == kBarSFree * 8 && offsetof(AttnCtrl, v_full) == (kBarSFree + 1) * 8 &&
+              offsetof(AttnCtrl, tmem_base) == kNumBarriers * 8 &&
               sizeof(AttnCtrl) <= 512, "barrier layout");
 
 // What share c tells the merge kernel: the item that the boundary between shares c - 1 and c
@@ -450,6 +453,19 @@ struct TileKeys {
     __device__ __forceinline__ int operator()(int jl) const { return jl == jc ? vc : jl == jf ? vf : kBN; }
 };
 
+// The barrier on which V of key tile jl lands, and the phase of it.  A barrier's waiter must see every phase of
+// it, or a wait for a phase could be answered by the one two phases back.  With 4 or 8 stages a lone query tile's
+// two roles never share a V stage; with 6 they take turns on it, so each role has a barrier of its own there.
+struct VLanding {
+    uint32_t bar;
+    int phase;
+};
+__device__ __forceinline__ VLanding v_landing(AttnCtrl* ctrl, bool split, int n_stages, int jl) {
+    const int iv = 2 * jl + 1, sv = iv % n_stages, use = iv / n_stages;
+    if (split && n_stages % 4 != 0) return {ptx::smem_addr(jl & 1 ? &ctrl->v_full[sv >> 1] : &ctrl->kv_full[sv]), use >> 1};
+    return {ptx::smem_addr(&ctrl->kv_full[sv]), use};
+}
+
 // What one walk over a segment does.  kWalk: one pass, the reference maximum of a row is its maximum over
 // the segment's first key tile.  If a row outgrows that (AttnCtrl::redo) the segment is walked twice more:
 // kMaxOnly finds the rows' maxima, kExact repeats the pass with them.
@@ -539,9 +555,9 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             if (valid < kBN && ck == 0) {
                 // last tile of a part: zero the V rows behind the live prefix (0 * NaN = NaN)
                 const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
-                const int iv = 2 * jl + 1, sv = iv % n_stages;
-                ok = wait_bar(ptx::smem_addr(&ctrl->kv_full[sv]), (iv / n_stages) & 1, abort_flag,
-                              p.dev_status, p.timeout_cycles);
+                const int sv = (2 * jl + 1) % n_stages;
+                const VLanding vl = v_landing(ctrl, split, n_stages, jl);
+                ok = wait_bar(vl.bar, vl.phase & 1, abort_flag, p.dev_status, p.timeout_cycles);
                 if (!ok) break;
                 if (row >= valid) {
                     uint8_t* vrow = smem_gen + ((split ? 1 : 2) + sv) * kTileBytes + row * 128;
@@ -863,7 +879,7 @@ __device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUte
         if (lane == 0) {
             const bool cached = j < nt_c;
             const CUtensorMap* map = cached ? (is_v ? tm_vc : tm_kc) : (is_v ? tm_vf : tm_kf);
-            const uint32_t bar = ptx::smem_addr(&ctrl->kv_full[stage]);
+            const uint32_t bar = is_v ? v_landing(ctrl, split, n_stages, i >> 1).bar : ptx::smem_addr(&ctrl->kv_full[stage]);
             ptx::mbar_arrive_expect_tx(bar, kTileBytes);
             for (int hf = 0; hf < Cfg::kHalves; ++hf)
                 ptx::tma_load_4d(ring + stage * kTileBytes + hf * kHalfBytes, map, bar, hf * 64, h,
@@ -961,11 +977,10 @@ __device__ __forceinline__ void issue_pv_segment(const AttnParams& p, AttnCtrl* 
     };
     for (int j = 0; j < n_my; ++j) {
         const int jl = split ? 2 * j + t : j;
-        const int iv = 2 * jl + 1, sv = iv % n_stages;
+        const int sv = (2 * jl + 1) % n_stages;
+        const VLanding vl = v_landing(ctrl, split, n_stages, jl);
         const bool more = (j + 1 < n_my);
-        if (!wait_bar(ptx::smem_addr(&ctrl->kv_full[sv]), (iv / n_stages) & 1, &ctrl->abort_flag, p.dev_status,
-                      p.timeout_cycles))
-            return;
+        if (!wait_bar(vl.bar, vl.phase & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
         if (mode == kMaxOnly) {                     // no products in this pass: the stage is given back
             if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->kv_empty[sv]));
             continue;
@@ -1072,7 +1087,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             int count = 1;                                               // q_full, kv_full, s_full, commits
             if (i >= kBarKvEmpty && i < kBarSFull) count = split ? 1 : ntq;      // commits per stage
             else if (i >= kBarPFull && i < kBarOFinal) count = kBM / 32;         // one arrival per warp
-            else if (i == kBarSFree) count = 2 * (kBM / 32);
+            else if (i == kBarSFree) count = 2 * (kBM / 32);             // (v_full: one, like kv_full)
             ptx::mbar_init(ptx::smem_addr(&ctrl->q_full + i), count);
             ptx::fence_barrier_init();
         }
