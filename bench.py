@@ -4,8 +4,8 @@
 A "step" is one pass of the whole hot path over one batch of synthetic input of
 the FLUX-Kontext-shaped workload (4096 image + 4096 reference + 512 text tokens,
 24 heads x 128, two-ellipse 20 % edit mask): partition, row lists, gathers, RIKV
-store, region attention with its rows scattered back, velocity decay + Euler, merge (7 library calls,
-8 kernel launches on two streams).
+store, region attention with its rows scattered back, velocity decay + Euler, merge (one library call,
+4 kernel launches).
 
 Prints ONE JSON line (rank 0).  `value` = region-attention FLOPs of the step
 divided by the whole step's device time (inputs resident in HBM).  `roofline`
@@ -282,7 +282,7 @@ def hbm_sweep(torch, binding, step, d, flush_l2, peak_gbs, iters=10):
 
 def ratio_sweep(torch, binding, synth, flush_l2, to_dev, steps=20):
     """Denoise-step time against the edit-mask ratio on the Qwen-Image-Edit-shaped workload (config 3):
-    one region step (7 library calls, 8 launches) and its attention call per ratio, CUDA events, L2
+    one region step (one library call, 4 launches) and its attention call per ratio, CUDA events, L2
     flushed per step."""
     from paper_2510_25590_b200.step import RegionStep, StepShapes, plan_capacity
     wl = synth.WORKLOADS[3]
@@ -756,7 +756,7 @@ def run_ours(args):
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(steps)]
     aev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(steps)]
     sampler = ClockSampler(local)
-    launches0 = step.launches
+    launches0 = step.kernel_launches
     if world > 1:
         dist.barrier()
     torch.cuda.synchronize()
@@ -774,7 +774,7 @@ def run_ours(args):
     wall = time.perf_counter() - wall0
     clocks = sampler.stop()
     step.attention_events = None
-    launches = step.launches - launches0
+    launches = step.kernel_launches - launches0
     step_ms = np.array([a.elapsed_time(b) for a, b in ev])
     attn_ms = np.array([a.elapsed_time(b) for a, b in aev])
     total_ms = float(step_ms.sum())

@@ -323,6 +323,42 @@ int regione_region_attention_scatter(const regione_bf16* q,
                                      int32_t* dev_status, void* stream);
 
 /*
+ * One whole region-aware step of one attention layer: regione_partition_rows, the gather of X^E and v,
+ * regione_velocity_decay, regione_merge, the gather of Q / K / V, regione_rikv_store (with store_cache) and
+ * regione_region_attention_scatter, with the results those calls leave, in four kernel launches.
+ * The plan names the sizes and the buffers that the step owns (device pointers; layouts as in those
+ * calls, c_cap = n_full = n_text + N + n_ref, q_cap = ne_cap, plus n_text under REGIONE_ROWS_PAPER):
+ *   mask u8 [B, N]; edit_idx, keep_idx, slot i32 [B, N]; n_edit, n_q, n_cache i32 [B];
+ *   query_rows i32 [B, q_cap]; cache_rows i32 [B, n_full]; n_rows i32 [B], every entry n_full;
+ *   x_e, v_e, v_avd bf16 [B, ne_cap, C]; x_out bf16 [B, N, C]; q_e, k_fresh, v_fresh bf16 [B, q_cap, H, D];
+ *   k_cache, v_cache, o_full bf16 [B, n_full, H, D]; workspace 256-byte aligned, at least
+ *   regione_region_step_workspace(plan) bytes; dev_status i32 [1] or NULL.
+ * x_t, v, ref bf16 [B, N, C]; q_full, k_full, v_full bf16 [B, n_full, H, D]; t, scale, dt, dt_unedited host
+ * arrays [B] (NaN: the request sits that operation out, as in the single calls).
+ * store_cache != 0: the attention reads K and V where they are (fresh and cached rows together are all of
+ * them), the cache receives its rows in the same launch, k_fresh and v_fresh are not written.
+ * parts: REGIONE_STEP_MOVES (everything up to the attention) | REGIONE_STEP_ATTENTION.
+ */
+typedef struct {
+    int B, N, n_text, n_ref, C, H, D, ne_cap, metric, membership;
+    float threshold;
+    uint8_t* mask;
+    int32_t *edit_idx, *keep_idx, *slot, *n_edit, *query_rows, *n_q, *cache_rows, *n_cache;
+    const int32_t* n_rows;
+    regione_bf16 *x_e, *v_e, *v_avd, *x_out, *q_e, *k_fresh, *v_fresh, *k_cache, *v_cache, *o_full;
+    void* workspace;
+    size_t workspace_bytes;
+    int32_t* dev_status;
+} regione_step_plan;
+#define REGIONE_STEP_MOVES 1
+#define REGIONE_STEP_ATTENTION 2
+size_t regione_region_step_workspace(const regione_step_plan* plan);
+int regione_region_step(const regione_step_plan* plan, const regione_bf16* x_t, const regione_bf16* v,
+                        const regione_bf16* ref, const regione_bf16* q_full, const regione_bf16* k_full,
+                        const regione_bf16* v_full, const float* t, const float* scale, const float* dt,
+                        const float* dt_unedited, int store_cache, int parts, void* stream);
+
+/*
  * Full attention step that refreshes the Region-Instruction KV cache in passing (Sec. 4,
  * "Stabilization Stage": the last full step saves K and V of every attention layer; end of the
  * "Adaptive Velocity Decay Cache" paragraph: forced full-image steps update the cache; Algorithm 1,

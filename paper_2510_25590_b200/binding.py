@@ -20,6 +20,19 @@ METRIC_COSINE, METRIC_L2 = 0, 1
 ROWS_EDITED_QUERIES, ROWS_PAPER = 0, 1
 ROPE_INTERLEAVED, ROPE_HALF = 0, 1
 
+STEP_MOVES, STEP_ATTENTION = 1, 2
+
+
+class StepPlan(ctypes.Structure):
+    """``regione_step_plan``: sizes and buffers of one region-aware step."""
+    _fields_ = ([(n, c_int) for n in ("B", "N", "n_text", "n_ref", "C", "H", "D", "ne_cap", "metric", "membership")] +
+                [("threshold", c_float)] +
+                [(n, c_void_p) for n in ("mask", "edit_idx", "keep_idx", "slot", "n_edit", "query_rows", "n_q", "cache_rows",
+                                         "n_cache", "n_rows", "x_e", "v_e", "v_avd", "x_out", "q_e", "k_fresh", "v_fresh",
+                                         "k_cache", "v_cache", "o_full", "workspace")] +
+                [("workspace_bytes", c_size_t), ("dev_status", c_void_p)])
+
+
 # every symbol include/regione.h declares: name -> (restype, argtypes)
 _P = c_void_p
 SIGNATURES = {
@@ -43,6 +56,8 @@ SIGNATURES = {
     "regione_region_attention_workspace": (c_size_t, [c_int] * 6),
     "regione_region_attention": (c_int, [_P] * 8 + [c_int] * 6 + [c_float, _P, _P, c_size_t, _P, _P]),
     "regione_region_attention_scatter": (c_int, [_P] * 8 + [c_int] * 6 + [c_float, _P, c_int, _P, _P, c_size_t, _P, _P]),
+    "regione_region_step_workspace": (c_size_t, [POINTER(StepPlan)]),
+    "regione_region_step": (c_int, [POINTER(StepPlan)] + [_P] * 10 + [c_int, c_int, _P]),
     "regione_full_attention_store_workspace": (c_size_t, [c_int] * 4),
     "regione_full_attention_store": (c_int, [_P] * 4 + [c_int] * 4 + [c_float, _P, _P, c_int, _P, _P, _P, _P,
                                              c_size_t, _P, _P]),
@@ -92,40 +107,50 @@ def _check(code: int, what: str) -> None:
         raise RegionEError(f"{what} failed: {status_string(code)} ({code})")
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _ptr(t, dtype=None, name="tensor"):
+    """Device address of a contiguous CUDA tensor (an int: ctypes converts it), None for None."""
     if t is None:
         return None
-    torch = _torch()
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise RegionEError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise RegionEError(f"{name} must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise RegionEError(f"{name} must have dtype {dtype}, got {t.dtype}")
-    return c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    torch = _torch()
-    s = torch.cuda.current_stream() if stream is None else stream
-    return c_void_p(s.cuda_stream)
+    s = _torch().cuda.current_stream() if stream is None else stream
+    return s.cuda_stream
+
+
+_FLOATS = {}                      # array type per length
 
 
 def _per_request(value, B, name):
     """A sampler scalar for the batch: one number (shared by every request) or B numbers (each
     request at its own sampler step) -> a host float array of length B."""
+    if B == 1 and value.__class__ is float:
+        return (_FLOATS.get(1) or _FLOATS.setdefault(1, c_float * 1))(value)
     try:
         vals = [float(value)] * B
     except (TypeError, ValueError):
         vals = [float(x) for x in value]
         if len(vals) != B:
             raise RegionEError(f"{name} must be one number or {B} numbers, got {len(vals)}")
-    return (c_float * max(B, 1))(*vals)
+    return (_FLOATS.get(B) or _FLOATS.setdefault(B, c_float * max(B, 1)))(*vals)
 
 
 def version() -> int:
@@ -213,8 +238,8 @@ def gather_multi(srcs, idx, n, dsts, dev_status=None, stream=None):
     for s_, d_ in zip(srcs, dsts):
         if s_.shape != srcs[0].shape or d_.shape != dsts[0].shape or s_.dtype != d_.dtype:
             raise RegionEError("gather_multi: tensors must share shape and dtype")
-    sp = (c_void_p * k)(*[_ptr(t, None, "src").value for t in srcs])
-    dp = (c_void_p * k)(*[_ptr(t, None, "dst").value for t in dsts])
+    sp = (c_void_p * k)(*[_ptr(t, None, "src") for t in srcs])
+    dp = (c_void_p * k)(*[_ptr(t, None, "dst") for t in dsts])
     _check(load().regione_gather_multi(
         sp, dp, k, _ptr(idx, torch.int32, "idx"), _ptr(n, torch.int32, "n"), srcs[0].shape[0],
         srcs[0].shape[1], idx.shape[1], dsts[0].shape[1], _row_bytes(srcs[0]),
@@ -329,6 +354,30 @@ def region_attention_scatter(q, k_fresh, v_fresh, k_cache, v_cache, n_q, n_fresh
         _ptr(out_full, bf, "out_full"), out_full.shape[1], _ptr(out_rows, i32, "out_rows"),
         _ptr(workspace, None, "workspace"), ws_bytes, _ptr(dev_status, i32), _stream(stream)),
         "regione_region_attention_scatter")
+
+
+def region_step_workspace(plan: StepPlan) -> int:
+    return int(load().regione_region_step_workspace(ctypes.byref(plan)))
+
+
+def _shaped(t, shape, name):
+    """Address of a contiguous bf16 CUDA tensor of the given shape."""
+    p = _ptr(t, _torch().bfloat16, name)
+    if t.shape != shape:
+        raise RegionEError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
+    return p
+
+
+def region_step(plan: StepPlan, x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, store_cache=True,
+                parts=STEP_MOVES | STEP_ATTENTION, stream=None):
+    """One region-aware step in one call (see ``RegionStep``, which owns the plan and its buffers)."""
+    B, lat = plan.B, (plan.B, plan.N, plan.C)
+    full = (B, plan.n_text + plan.N + plan.n_ref, plan.H, plan.D)
+    _check(load().regione_region_step(
+        plan, _shaped(x_t, lat, "x_t"), _shaped(v, lat, "v"), _shaped(ref, lat, "ref"), _shaped(q_full, full, "q_full"),
+        _shaped(k_full, full, "k_full"), _shaped(v_full, full, "v_full"), _per_request(t, B, "t"),
+        _per_request(scale, B, "scale"), _per_request(dt, B, "dt"), _per_request(dt_unedited, B, "dt_unedited"),
+        1 if store_cache else 0, parts, _stream(stream)), "regione_region_step")
 
 
 def full_attention_store_workspace(B, N_cap, H, D) -> int:

@@ -9,11 +9,6 @@ int launch_region_attention_simt(const uint16_t*, const uint16_t*, const uint16_
                                  const uint16_t*, const int32_t*, const int32_t*, const int32_t*,
                                  int, int, int, int, int, int, float, uint16_t*, int32_t*,
                                  cudaStream_t);
-size_t region_attention_tc_workspace(int B, int Nq_cap, int Nf_cap, int Nc_cap, int H, int D);
-int launch_region_attention_tc(const uint16_t*, const uint16_t*, const uint16_t*, const uint16_t*,
-                               const uint16_t*, const int32_t*, const int32_t*, const int32_t*, int,
-                               int, int, int, int, int, float, uint16_t*, const int32_t*, int, void*,
-                               size_t, int32_t*, cudaStream_t, const CacheStore*);
 }  // namespace regione
 
 using namespace regione;

@@ -34,6 +34,15 @@ __device__ __forceinline__ uint4 ldg128(const void* p) {
     return __ldg(reinterpret_cast<const uint4*>(p));
 }
 
+__device__ __forceinline__ uint4 axpy8(uint4 x, uint4 v, float a) {   // x + a * v, per bf16 lane
+    uint4 o;
+    o.x = pack_bf16x2(fmaf(a, bf16_lo(v.x), bf16_lo(x.x)), fmaf(a, bf16_hi(v.x), bf16_hi(x.x)));
+    o.y = pack_bf16x2(fmaf(a, bf16_lo(v.y), bf16_lo(x.y)), fmaf(a, bf16_hi(v.y), bf16_hi(x.y)));
+    o.z = pack_bf16x2(fmaf(a, bf16_lo(v.z), bf16_lo(x.z)), fmaf(a, bf16_hi(v.z), bf16_hi(x.z)));
+    o.w = pack_bf16x2(fmaf(a, bf16_lo(v.w), bf16_lo(x.w)), fmaf(a, bf16_hi(v.w), bf16_hi(x.w)));
+    return o;
+}
+
 // Streaming 128-bit load for data that is read exactly once (bypasses L1 allocation).
 __device__ __forceinline__ uint4 ld_stream128(const void* p) {
     uint4 r;
@@ -89,6 +98,15 @@ struct CacheStore {
     uint16_t* k_cache;          // dev [B, cap, H, D]
     uint16_t* v_cache;
 };
+
+// The attention's host side (defined in attention_tc.cu).  n_cache = nullptr: no cached rows in any request;
+// store != nullptr: the rows store->keep_rows of k_fresh / v_fresh go to the cache in the same launch.
+int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const uint16_t* v_fresh, const uint16_t* k_cache,
+                               const uint16_t* v_cache, const int32_t* n_q, const int32_t* n_fresh, const int32_t* n_cache,
+                               int B, int Nq_cap, int Nf_cap, int Nc_cap, int H, int D, float scale, uint16_t* out,
+                               const int32_t* out_rows, int out_cap, void* workspace, size_t workspace_bytes,
+                               int32_t* dev_status, cudaStream_t st, const CacheStore* store);
+size_t region_attention_tc_workspace(int B, int Nq_cap, int Nf_cap, int Nc_cap, int H, int D);
 
 // Host-side argument checks shared by every region-attention entry point (defined in api.cu).
 // Returns REGIONE_OK when the call may proceed; *nothing_to_do is set for B == 0 or Nq_cap == 0.

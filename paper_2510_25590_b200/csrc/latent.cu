@@ -11,15 +11,6 @@ namespace regione {
 
 constexpr int kLatThreads = 256;
 
-__device__ __forceinline__ uint4 axpy8(uint4 x, uint4 v, float a) {   // x + a * v, per bf16 lane
-    uint4 o;
-    o.x = pack_bf16x2(fmaf(a, bf16_lo(v.x), bf16_lo(x.x)), fmaf(a, bf16_hi(v.x), bf16_hi(x.x)));
-    o.y = pack_bf16x2(fmaf(a, bf16_lo(v.y), bf16_lo(x.y)), fmaf(a, bf16_hi(v.y), bf16_hi(x.y)));
-    o.z = pack_bf16x2(fmaf(a, bf16_lo(v.z), bf16_lo(x.z)), fmaf(a, bf16_hi(v.z), bf16_hi(x.z)));
-    o.w = pack_bf16x2(fmaf(a, bf16_lo(v.w), bf16_lo(x.w)), fmaf(a, bf16_hi(v.w), bf16_hi(x.w)));
-    return o;
-}
-
 // x_e <- x_e - dt * (scale * v_in); optionally v_cache_out <- v_in.  One thread = 8 channels.
 __global__ void __launch_bounds__(kLatThreads)
 velocity_decay_kernel(const uint4* __restrict__ v_in, const PerRequestF neg_dt_scale_v, int b0,

@@ -1,31 +1,12 @@
 // Indexed row copies: token gather / scatter (Algorithm 1: X[E_index] and the
 // re-gathering by spatial position) and the Region-Instruction KV cache store
 // (Sec. 4 "Stabilization Stage": K and V of every attention layer are saved).
-//
-// All three are pure HBM traffic.  Rows are byte strings whose length is a
-// multiple of 16; a thread moves kUnroll 16-byte chunks that are blockDim
-// apart, so a warp always touches 512 contiguous bytes per request, all loads
-// of a thread are issued before its first store, and source data (read once)
-// bypasses L1.
-#include "common.cuh"
+// All three are pure HBM traffic.
+#include "rowcopy.cuh"
 
 namespace regione {
 
-constexpr int kCopyThreads = 256;
-constexpr int kUnroll = 8;
-
-struct RowCopyPair {
-    const uint4* src;
-    uint4* dst;
-};
-
-constexpr int kMaxPairs = 4;                 // tensors sharing one index list in one launch
-struct RowCopyPairs {
-    RowCopyPair p[kMaxPairs];
-};
-
-// GATHER: dst[b, j] = src[b, idx[b, j]];  !GATHER: dst[b, idx[b, j]] = src[b, j].
-// `idx_rows` bounds the indexed side, `cap` the dense side.  blockIdx.z picks the tensor pair.
+// blockIdx.z picks the tensor pair.
 template <bool GATHER>
 __global__ void __launch_bounds__(kCopyThreads)
 row_copy_kernel(const RowCopyPairs pairs, const int32_t* __restrict__ idx,
@@ -33,50 +14,7 @@ row_copy_kernel(const RowCopyPairs pairs, const int32_t* __restrict__ idx,
                 long long cap, int cpr, int32_t* dev_status) {
     grid_dependency_wait();
     grid_launch_dependents();
-    const int b = blockIdx.y;
-    const RowCopyPair p = pairs.p[blockIdx.z];
-    long long live = n[b];
-    if (live < 0 || live > cap) {
-        if (threadIdx.x == 0 && blockIdx.x == 0) record_status(dev_status, REGIONE_DEV_BOUNDS);
-        live = live < 0 ? 0 : cap;
-    }
-    // 32-bit chunk arithmetic: the host guarantees cap * cpr < 2^31.
-    const unsigned total = (unsigned)live * (unsigned)cpr;
-    const unsigned base = blockIdx.x * (unsigned)(kCopyThreads * kUnroll) + threadIdx.x;
-    if (base >= total) return;
-    const uint4* __restrict__ src = p.src + (size_t)b * (GATHER ? idx_rows : cap) * cpr;
-    uint4* __restrict__ dst = p.dst + (size_t)b * (GATHER ? cap : idx_rows) * cpr;
-    const int32_t* __restrict__ my_idx = idx + (size_t)b * idx_stride;
-
-    // (row j, chunk c) of the first element; later elements advance by kCopyThreads chunks.
-    unsigned j = base / (unsigned)cpr;
-    unsigned c = base - j * (unsigned)cpr;
-    const unsigned step_rows = (unsigned)kCopyThreads / (unsigned)cpr;
-    const unsigned step_chunks = (unsigned)kCopyThreads - step_rows * (unsigned)cpr;
-
-    uint4 val[kUnroll];
-    long long to[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-        const unsigned e = base + (unsigned)u * kCopyThreads;
-        to[u] = -1;
-        if (e < total) {
-            const long long r = my_idx[j];
-            if (r < 0 || r >= idx_rows) {
-                record_status(dev_status, REGIONE_DEV_BOUNDS);
-            } else {
-                const long long from = (GATHER ? r : (long long)j) * cpr + c;
-                to[u] = (GATHER ? (long long)j : r) * cpr + c;
-                val[u] = ld_stream128(src + from);
-            }
-        }
-        j += step_rows;
-        c += step_chunks;
-        if (c >= (unsigned)cpr) { c -= (unsigned)cpr; ++j; }
-    }
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u)
-        if (to[u] >= 0) dst[to[u]] = val[u];
+    copy_rows<GATHER>(pairs.p[blockIdx.z], blockIdx.y, blockIdx.x, idx, n, idx_rows, idx_stride, cap, cpr, dev_status);
 }
 
 template <bool GATHER>

@@ -1,15 +1,13 @@
-"""One region-aware denoising step for one attention layer, as a fixed sequence of C-ABI calls.
+"""One region-aware denoising step for one attention layer, as one C-ABI call.
 
-This is call sequencing and buffer ownership only (torch tensors are device
-buffers): every operation runs in the library's kernels.  The sequence follows
-Algorithm 1 of the paper for one layer:
+This is buffer ownership only (torch tensors are device buffers): every operation runs in the
+library's kernels.  The sequence follows Algorithm 1 of the paper for one layer:
 
-  partition with the joint-sequence row lists (one launch) -> two independent branches, joined
-  before the step returns:
-    attention branch: RIKV store -> gather Q/K/V of the recomputed rows (one launch) ->
-                      region attention writing its rows back at their joint-sequence positions
-    latent branch   : gather X^E, v^E (one launch) -> velocity decay + Euler update -> merge with
-                      the one-step-predicted unedited tokens (on a side stream)
+  partition with the joint-sequence row lists -> gather X^E, v^E; velocity decay + Euler update; merge with
+  the one-step-predicted unedited tokens; gather of the recomputed rows of Q (K, V) -> region attention
+  writing its rows back at their joint-sequence positions, the RIKV store in the same launch
+
+(four kernel launches: partition, moves, attention, merge of the attention's shared items).
 
 No step needs a host round trip: per-request counts stay in device memory.
 Capacities are host integers chosen by the caller (``plan_capacity`` reads the
@@ -82,52 +80,48 @@ class RegionStep:
         self.o_full = z(B, shp.n_full, H, D)
         self.x_out = z(B, N, C)
         self.dev_status = z(1, dt=i32)
-        ws = binding.region_attention_workspace(B, shp.q_cap, shp.q_cap, shp.c_cap, H, D)
-        self.workspace = torch.empty(max(ws, 256), dtype=torch.uint8, device=device)
-        self.launches = 0
-        self._side = torch.cuda.Stream(device=device)
-        self._fork, self._join = torch.cuda.Event(), torch.cuda.Event()
+        self.n_rows = torch.full((B,), shp.n_full, dtype=i32, device=device)
+        self.workspace = None
+        self.workspace = torch.empty(max(binding.region_step_workspace(self._step_plan()), 256), dtype=torch.uint8,
+                                     device=device)
+        self.launches = 0                 # operations of the sequence run so far (8 per step, 7 without the store)
+        self.kernel_launches = 0          # kernels launched so far (batches of up to 128 requests)
         self.attention_events = None      # optional (start, stop) pair recorded around the attention
+
+    _BUFFERS = ("mask", "edit_idx", "keep_idx", "slot", "n_edit", "query_rows", "n_q", "cache_rows", "n_cache", "n_rows",
+                "x_e", "v_e", "v_avd", "x_out", "q_e", "k_fresh", "v_fresh", "k_cache", "v_cache", "o_full", "workspace",
+                "dev_status")
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        if name in self._BUFFERS or name == "shp":
+            object.__setattr__(self, "_plan", None)      # the plan names this object's buffers: made anew
+
+    def _step_plan(self):
+        if self._plan is None:
+            s = self.shp
+            p = binding.StepPlan(s.B, s.N, s.n_text, s.n_ref, s.C, s.H, s.D, s.ne_cap, int(s.metric), int(s.membership),
+                                 float(s.threshold))
+            for name in self._BUFFERS:
+                t = getattr(self, name)
+                setattr(p, name, None if t is None else t.data_ptr())
+            p.workspace_bytes = 0 if self.workspace is None else self.workspace.numel()
+            object.__setattr__(self, "_plan", p)
+        self._plan.metric, self._plan.threshold = int(self.shp.metric), self.shp.threshold
+        return self._plan
 
     def run(self, x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, stream=None,
             store_cache=True):
         """One region-aware step.  ``store_cache=False`` leaves the cache as the last storing call wrote
         it (Algorithm 1 refreshes it at full steps only; valid while the partition is unchanged)."""
-        import torch
-        s = self.shp
-        st = self.dev_status
-        b = binding
-        b.partition_rows(x_t, v, ref, t, s.metric, s.threshold, self.mask, self.edit_idx,
-                         self.keep_idx, self.slot, self.n_edit, s.n_text, s.n_ref, s.membership,
-                         self.query_rows, self.n_q, self.cache_rows, self.n_cache, dev_status=st,
-                         stream=stream)
-        # Two independent branches hang off the partition: the latent branch (gather of X^E and v,
-        # velocity decay, merge: small latency-bound kernels) and the attention branch (cache store,
-        # gather of Q/K/V, attention, scatter).  The latent branch runs on a side stream so that it
-        # falls into the shadow of the cache store; both join before the step returns.
-        main = torch.cuda.current_stream() if stream is None else stream
-        self._fork.record(main)
-        self._side.wait_event(self._fork)
-        side = self._side
-        b.gather_multi([x_t, v], self.edit_idx, self.n_edit, [self.x_e, self.v_e], dev_status=st,
-                       stream=side)
-        b.velocity_decay(self.v_e, scale, dt, self.x_e, self.n_edit, v_cache_out=self.v_avd,
-                         dev_status=st, stream=side)
-        b.merge(x_t, v, self.x_e, self.slot, dt_unedited, self.x_out, dev_status=st, stream=side)
-        self._join.record(side)
-        if store_cache:
-            b.rikv_store(k_full, v_full, self.cache_rows, self.n_cache, self.k_cache, self.v_cache,
-                         dev_status=st, stream=stream)
-        b.gather_multi([q_full, k_full, v_full], self.query_rows, self.n_q,
-                       [self.q_e, self.k_fresh, self.v_fresh], dev_status=st, stream=stream)
-        if self.attention_events is not None:
+        args = (self._step_plan(), x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, store_cache)
+        if self.attention_events is None:
+            binding.region_step(*args, stream=stream)
+        else:
+            binding.region_step(*args, parts=binding.STEP_MOVES, stream=stream)
             self.attention_events[0].record(stream)
-        # the attention rows go straight to their positions in the joint sequence (o_full)
-        b.region_attention_scatter(self.q_e, self.k_fresh, self.v_fresh, self.k_cache, self.v_cache,
-                                   self.n_q, self.n_q, self.n_cache, self.o_full, self.query_rows,
-                                   workspace=self.workspace, dev_status=st, stream=stream)
-        if self.attention_events is not None:
+            binding.region_step(*args, parts=binding.STEP_ATTENTION, stream=stream)
             self.attention_events[1].record(stream)
-        main.wait_event(self._join)
-        self.launches += 8 if store_cache else 7     # kernels launched (the attention call launches two)
+        self.launches += 8 if store_cache else 7
+        self.kernel_launches += 4
         return self.x_out
