@@ -21,8 +21,8 @@ conditional / unconditional pair of one guided request, which is simply two batc
 ``offsets`` request b takes its step k at tick ``offsets[b] + k``; at every tick the Euler updates of
 all requests share their launches, each request with its own time, step length and decay product,
 and a request that has nothing to do in a launch sits it out (NaN scalar, see the header).  The
-calls that happen once per run of region steps (partition, gather of X^E, merge) are made per
-request on its slice of the batch.
+gather of X^E at the beginning of a run of region steps is made per request on its slice of the batch
+when the requests are shifted, the merge at the end too when a hook watches the loop.
 
 When the requests of a tick differ in time the model callbacks receive lists:
     model.full(x, [t_b or None], [store_b])          None = request b is not at a full step
@@ -85,7 +85,11 @@ class LoopTrace:
 
 
 @dataclass
-class _RequestState:
+class _Group:
+    """Requests with the same offset: they take the same steps at the same ticks."""
+    offset: int
+    requests: list
+    k: int = -1                      # the step taken at the present tick
     partitioned: bool = False
     in_run: bool = False
     t_run: float = 0.0
@@ -98,7 +102,11 @@ _NAN = float("nan")
 
 class RegionELoop:
     """Buffers and call sequence of one edit (a batch of B independent requests; same schedule,
-    optionally shifted against each other by ``offsets``)."""
+    optionally shifted against each other by ``offsets``).
+
+    The loop's own work is launch-bound (kernels of 2 to 3 us), so its host side is kept short: addresses
+    and the stream are looked up once per run, requests that move together share their bookkeeping and
+    their calls, and a full step's velocity is kept by the Euler update that reads it."""
 
     def __init__(self, B, N, C, cfg: LoopConfig, device="cuda"):
         import torch
@@ -110,147 +118,188 @@ class RegionELoop:
         self.n_edit = z(B, dt=i32)
         self.n_all = torch.full((B,), N, dtype=i32, device=device)
         self.x_e, self.v_cache = z(B, N, C), z(B, N, C)      # capacity N: no host read-back needed
-        self.x_run_start, self.v_last_full = z(B, N, C), z(B, N, C)
+        self.v_last_full = z(B, N, C)
         self.dev_status = z(1, dt=i32)
         self.hook = None             # optional callable(event: str, k: int, tensors: dict)
-
-    @staticmethod
-    def _copy(dst, src, stream):
-        """Device-to-device copy ordered on the same stream as the library calls around it."""
-        import torch
-        if stream is None:
-            dst.copy_(src)
-        else:
-            with torch.cuda.stream(stream):
-                dst.copy_(src)
-
-    def _emit(self, event, k, **tensors):
-        if self.hook is not None:
-            self.hook(event, k, tensors)
 
     def run(self, x, ref, model, stream=None, offsets=None):
         """Runs all steps on ``x`` [B, N, C] bf16 (updated in place); returns (x, trace).
 
         ``offsets`` [B]: request b takes step k at tick offsets[b] + k (default: all zero)."""
-        cfg, b, st = self.cfg, binding, self.dev_status
-        ts, T, B = cfg.timesteps, len(cfg.kinds), self.B
+        import torch
+        cfg, b, st, hook = self.cfg, binding, self.dev_status, self.hook
+        kinds, T, B, N, C = cfg.kinds, len(cfg.kinds), self.B, self.N, self.C
+        ts = [float(t) for t in cfg.timesteps[:T + 1]]
         offsets = [0] * B if offsets is None else [int(o) for o in offsets]
         if len(offsets) != B or min(offsets) < 0:
-            raise binding.RegionEError("offsets must hold one non-negative tick per request")
-        uniform = len(set(offsets)) == 1
+            raise b.RegionEError("offsets must hold one non-negative tick per request")
+        groups = [_Group(o, [r for r in range(B) if offsets[r] == o]) for o in sorted(set(offsets))]
+        uniform = len(groups) == 1
         tr = LoopTrace(per_request=[[] for _ in range(B)])
-        state = [_RequestState() for _ in range(B)]
-        sl = lambda t_, r: t_[r:r + 1]                     # request r's slice of a batch tensor
 
-        def merge_request(r, k, t_to):
-            # end of a run of region steps: edited tokens from X^E, unedited tokens by one step of
-            # the last full velocity over the whole run
-            s_ = state[r]
-            self._emit("merge_in", k, r=r, x=sl(self.x_run_start, r), v=sl(self.v_last_full, r),
-                       x_e=sl(self.x_e, r), slot=sl(self.slot, r), dt_unedited=s_.t_run - t_to)
-            b.merge(sl(self.x_run_start, r), sl(self.v_last_full, r), sl(self.x_e, r), sl(self.slot, r),
-                    s_.t_run - t_to, sl(x, r), dev_status=st, stream=stream)
-            self._emit("merge_out", k, r=r, x=sl(x, r))
+        # ---- the library calls of the loop, over the whole batch (NaN scalar: a request sits a call out) ----
+        lib, check, ptr, floats = b.load(), b._check, b._ptr, b._per_request
+        bf, shape, s = torch.bfloat16, (B, N, C), b._stream(stream)
+        p_x, p_xe, p_vl, p_vc = ptr(x, bf, "x"), self.x_e.data_ptr(), self.v_last_full.data_ptr(), self.v_cache.data_ptr()
+        p_idx, p_slot, p_ne = self.edit_idx.data_ptr(), self.slot.data_ptr(), self.n_edit.data_ptr()
+        p_all, p_st = self.n_all.data_ptr(), st.data_ptr()
+        if x.shape != shape:
+            raise b.RegionEError(f"x must have shape {shape}, got {tuple(x.shape)}")
+
+        def velocity(v, name):
+            p = ptr(v, bf, name)
+            if v.shape != shape:
+                raise b.RegionEError(f"{name} must have shape {shape}, got {tuple(v.shape)}")
+            return p
+
+        def decay(p_v, scale, dts, p_target, p_keep, p_n):
+            check(lib.regione_velocity_decay(p_v, floats(scale, B, "scale"), floats(dts, B, "dt"), p_target, p_keep, p_n,
+                                             B, N, C, p_st, s), "regione_velocity_decay")
             tr.launches += 1
-            s_.in_run = False
+
+        def spread(values):
+            """(group, value) pairs -> one value per request, NaN for the others; a number when all share it."""
+            if uniform:
+                return values[0][1]
+            out = [_NAN] * B
+            for g, val in values:
+                for r in g.requests:
+                    out[r] = val
+            return out
+
+        def listed(value):                                  # (for the hook: always one value per request)
+            return value if isinstance(value, list) else [value] * B
+
+        def members(gs):
+            return sorted(r for g in gs for r in g.requests)
+
+        one = lambda t_, r: t_[r:r + 1]                     # request r's slice of a batch tensor
+
+        def merge(ending, at_end=False):
+            # end of runs of region steps: edited tokens from X^E, unedited tokens by one step of the last full
+            # velocity over the whole run (x has not changed since the run began, so it is merged in place)
+            if hook is None:
+                check(lib.regione_merge(p_x, p_vl, p_xe, p_slot, floats(spread([(g, g.t_run - t) for g, t in ending]), B, "dt"),
+                                        B, N, N, C, p_x, p_st, s), "regione_merge")
+                tr.launches += 1
+            for g, t in ending:
+                g.in_run = False
+                for r in g.requests if hook is not None else ():
+                    k = T if at_end else g.k
+                    hook("merge_in", k, dict(r=r, x=one(x, r), v=one(self.v_last_full, r), x_e=one(self.x_e, r),
+                                             slot=one(self.slot, r), dt_unedited=g.t_run - t))
+                    b.merge(one(x, r), one(self.v_last_full, r), one(self.x_e, r), one(self.slot, r), g.t_run - t, one(x, r),
+                            dev_status=st, stream=stream)
+                    hook("merge_out", k, dict(r=r, x=one(x, r)))
+                    tr.launches += 1
+
+        def start_runs(starting):
+            if uniform:
+                check(lib.regione_gather(p_x, p_idx, p_ne, B, N, N, N, 2 * C, p_xe, p_st, s), "regione_gather")
+                tr.launches += 1
+            for g in starting:
+                g.in_run, g.t_run, g.product, g.have_cache = True, ts[g.k], 1.0, False
+                for r in g.requests if not uniform else ():
+                    b.gather(one(x, r), one(self.edit_idx, r), one(self.n_edit, r), one(self.x_e, r), dev_status=st,
+                             stream=stream)
+                    tr.launches += 1
 
         for tick in range(T + max(offsets)):
-            ks = [tick - o if 0 <= tick - o < T else None for o in offsets]     # step of each request
-            full = [r for r in range(B) if ks[r] is not None and cfg.kinds[ks[r]] == "F"]
-            region = [r for r in range(B) if ks[r] is not None and cfg.kinds[ks[r]] == "R"]
-            t_cur = [float(ts[k]) if k is not None else None for k in ks]
-            dt = [float(ts[k]) - float(ts[k + 1]) if k is not None else None for k in ks]
-            k0 = ks[0] if uniform else tick
+            full, region = [], []
+            for g in groups:
+                k = tick - g.offset
+                if 0 <= k < T:
+                    g.k = k
+                    (full if kinds[k] == "F" else region).append(g)
+            k0 = groups[0].k if uniform else tick
 
             # ---- full steps ----
             if full:
-                for r in full:
-                    if state[r].in_run:
-                        merge_request(r, ks[r], t_cur[r])
-                store = [ks[r] is not None and (state[r].partitioned or ks[r] + 1 == cfg.partition_after)
-                         for r in range(B)]
+                ending = [(g, ts[g.k]) for g in full if g.in_run]
+                if ending:
+                    merge(ending)
                 if uniform:
-                    v = model.full(x, t_cur[0], store[0])
+                    g = full[0]
+                    v = model.full(x, ts[g.k], g.partitioned or g.k + 1 == cfg.partition_after)
                 else:
-                    v = model.full(x, [t_cur[r] if r in full else None for r in range(B)], store)
+                    t_full, store = [None] * B, [False] * B
+                    for g in groups:
+                        live = 0 <= tick - g.offset < T
+                        for r in g.requests:
+                            store[r] = live and (g.partitioned or g.k + 1 == cfg.partition_after)
+                            if g in full:
+                                t_full[r] = ts[g.k]
+                    v = model.full(x, t_full, store)
                 tr.model_full_calls += 1
-                if len(full) == B:
-                    self._copy(self.v_last_full, v, stream)
-                else:
-                    for r in full:
-                        self._copy(sl(self.v_last_full, r), sl(v, r), stream)
-                dts = [dt[r] if r in full else _NAN for r in range(B)]
-                self._emit("euler_in", k0, x=x, v=v, dt=dts, active=full)
-                b.velocity_decay(v, 1.0, dts, x, self.n_all, dev_status=st, stream=stream)
-                self._emit("euler_out", k0, x=x, active=full)
-                tr.launches += 1
-                part = [r for r in full if ks[r] + 1 == cfg.partition_after]
+                p_v = velocity(v, "v")
+                dts = spread([(g, ts[g.k] - ts[g.k + 1]) for g in full])
+                if hook is not None:
+                    hook("euler_in", k0, dict(x=x, v=v, dt=listed(dts), active=members(full)))
+                decay(p_v, 1.0, dts, p_x, p_vl, p_all)       # (keeps v as the last full velocity in passing)
+                if hook is not None:
+                    hook("euler_out", k0, dict(x=x, active=members(full)))
+                part = [g for g in full if g.k + 1 == cfg.partition_after]
                 if part:
-                    t_part = [float(ts[ks[r] + 1]) if r in part else _NAN for r in range(B)]
-                    self._emit("partition_in", k0, x=x, v=v, ref=ref, t=t_part, active=part)
+                    t_part = spread([(g, ts[g.k + 1]) for g in part])
+                    if hook is not None:
+                        hook("partition_in", k0, dict(x=x, v=v, ref=ref, t=listed(t_part), active=members(part)))
                     b.partition(x, v, ref, t_part, cfg.metric, cfg.threshold, self.mask, self.edit_idx,
                                 self.keep_idx, self.slot, self.n_edit, dev_status=st, stream=stream)
-                    self._emit("partition_out", k0, mask=self.mask, edit_idx=self.edit_idx, slot=self.slot,
-                               n_edit=self.n_edit, active=part)
+                    if hook is not None:
+                        hook("partition_out", k0, dict(mask=self.mask, edit_idx=self.edit_idx, slot=self.slot,
+                                                       n_edit=self.n_edit, active=members(part)))
                     tr.launches += 1
-                    for r in part:
-                        state[r].partitioned = True
-                for r in full:
-                    tr.per_request[r].append((ks[r], "F", "full", 1.0))
+                    for g in part:
+                        g.partitioned = True
+                for g in full:
+                    for r in g.requests:
+                        tr.per_request[r].append((g.k, "F", "full", 1.0))
 
             # ---- region steps ----
             if region:
+                starting = [g for g in region if not g.in_run]
+                if any(not g.partitioned for g in starting):
+                    raise b.RegionEError("a region step was scheduled before the partition")
+                if starting:
+                    start_runs(starting)
                 reuse, compute = [], []
-                for r in region:
-                    s_ = state[r]
-                    if not s_.partitioned:
-                        raise binding.RegionEError("a region step was scheduled before the partition")
-                    if not s_.in_run:
-                        self._copy(sl(self.x_run_start, r), sl(x, r), stream)
-                        b.gather(sl(x, r), sl(self.edit_idx, r), sl(self.n_edit, r), sl(self.x_e, r),
-                                 dev_status=st, stream=stream)
-                        tr.launches += 1
-                        s_.in_run, s_.t_run = True, t_cur[r]
-                        s_.product, s_.have_cache = 1.0, False
+                for g in region:
                     again = False
-                    if s_.have_cache:
-                        k = ks[r]
-                        s_.product, again = b.avd_step(s_.product, float(ts[k - 1]) - t_cur[r],
-                                                       float(cfg.gammas[k]), cfg.delta)
-                    (reuse if again else compute).append(r)
-                if reuse:
-                    scale = [state[r].product if r in reuse else _NAN for r in range(B)]
-                    dts = [dt[r] if r in reuse else _NAN for r in range(B)]
-                    self._emit("decay_in", k0, v=self.v_cache, x_e=self.x_e, scale=scale, dt=dts,
-                               n_edit=self.n_edit, active=reuse)
-                    b.velocity_decay(self.v_cache, scale, dts, self.x_e, self.n_edit, dev_status=st,
-                                     stream=stream)
-                    self._emit("decay_out", k0, x_e=self.x_e, active=reuse)
-                    tr.launches += 1
-                    for r in reuse:
-                        tr.per_request[r].append((ks[r], "R", "reuse", state[r].product))
-                if compute:
-                    if uniform:
-                        v_e = model.region(self.x_e, t_cur[0], self.edit_idx, self.n_edit)
-                    else:
-                        v_e = model.region(self.x_e, [t_cur[r] if r in compute else None for r in range(B)],
-                                           self.edit_idx, self.n_edit)
-                    tr.model_region_calls += 1
-                    scale = [1.0 if r in compute else _NAN for r in range(B)]
-                    dts = [dt[r] if r in compute else _NAN for r in range(B)]
-                    self._emit("decay_in", k0, v=v_e, x_e=self.x_e, scale=scale, dt=dts, n_edit=self.n_edit,
-                               active=compute)
-                    b.velocity_decay(v_e, scale, dts, self.x_e, self.n_edit, v_cache_out=self.v_cache,
-                                     dev_status=st, stream=stream)
-                    self._emit("decay_out", k0, x_e=self.x_e, active=compute)
-                    tr.launches += 1
-                    for r in compute:
-                        state[r].product, state[r].have_cache = 1.0, True
-                        tr.per_request[r].append((ks[r], "R", "compute", 1.0))
+                    if g.have_cache:
+                        g.product, again = b.avd_step(g.product, ts[g.k - 1] - ts[g.k], float(cfg.gammas[g.k]), cfg.delta)
+                    (reuse if again else compute).append(g)
+                for gs, kind in ((reuse, "reuse"), (compute, "compute")):
+                    if not gs:
+                        continue
+                    scale = spread([(g, g.product if kind == "reuse" else 1.0) for g in gs])
+                    dts = spread([(g, ts[g.k] - ts[g.k + 1]) for g in gs])
+                    v_e, p_v, p_keep = self.v_cache, p_vc, None
+                    if kind == "compute":
+                        if uniform:
+                            v_e = model.region(self.x_e, ts[gs[0].k], self.edit_idx, self.n_edit)
+                        else:
+                            t_e = [None] * B
+                            for g in gs:
+                                for r in g.requests:
+                                    t_e[r] = ts[g.k]
+                            v_e = model.region(self.x_e, t_e, self.edit_idx, self.n_edit)
+                        tr.model_region_calls += 1
+                        p_v, p_keep = velocity(v_e, "v_e"), p_vc
+                    if hook is not None:
+                        hook("decay_in", k0, dict(v=v_e, x_e=self.x_e, scale=listed(scale), dt=listed(dts),
+                                                  n_edit=self.n_edit, active=members(gs)))
+                    decay(p_v, scale, dts, p_xe, p_keep, p_ne)
+                    if hook is not None:
+                        hook("decay_out", k0, dict(x_e=self.x_e, active=members(gs)))
+                    for g in gs:
+                        if kind == "compute":
+                            g.product, g.have_cache = 1.0, True
+                        for r in g.requests:
+                            tr.per_request[r].append((g.k, "R", kind, g.product))
 
-            # a request whose last step was a region step ends with the merge
-            for r in range(B):
-                if ks[r] == T - 1 and state[r].in_run:
-                    merge_request(r, T, float(ts[T]))
+            # requests whose last step was a region step end with the merge
+            ending = [(g, ts[T]) for g in region if g.k == T - 1]
+            if ending:
+                merge(ending, at_end=True)
         tr.steps = tr.per_request[0]
         return x, tr
