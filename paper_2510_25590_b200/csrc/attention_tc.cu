@@ -7,11 +7,11 @@
 //   warps 0-15  softmax and epilogue: thread = (query row, 64-key chunk of a key tile); warps 0-7 work on
 //               query tile 0, warps 8-15 on query tile 1, the first four of each on the first chunk
 //   warp  16    TMA producer: Q once, then K_j, V_j tiles (128 keys) through a ring of shared-memory stages;
-//               the cached segment and the fresh segment are two tensor maps walked one after the other.  In
-//               the full step that refreshes the Region-Instruction KV cache it also moves the retained rows,
-//               by asynchronous bulk copies, while it has nothing to load
-//   warps 17,18 issuers of the O_t += P_t V_j products, one per query tile (the whole warp walks the loop,
-//               one elected lane issues); warp 17 owns the tensor-memory allocation
+//               the cached segment and the fresh segment are two tensor maps walked one after the other
+//   warp  17    issuer of the O_t += P_t V_j products of both query tiles (the whole warp walks the loop, one
+//               elected lane issues); owns the tensor-memory allocation
+//   warp  18    in the launch that also refreshes the Region-Instruction KV cache: moves the retained rows by
+//               asynchronous bulk copies; idle otherwise
 //   warp  19    issuer of the S = Q_t K_j^T products of both query tiles; plans the CTA's next segment
 //   (warps 16-19 give registers up to the softmax warpgroups with setmaxnreg: 64 against 104 per thread)
 //
@@ -71,13 +71,15 @@
 namespace regione {
 
 constexpr int kSoftmaxWarps = 16;        // 4 softmax warpgroups: [query tile][64-key chunk]
-constexpr int kWarpLoad = kSoftmaxWarps, kWarpPv = kSoftmaxWarps + 1, kWarpS = kSoftmaxWarps + 3;   // (two P*V issuers)
+constexpr int kWarpLoad = kSoftmaxWarps, kWarpPv = kSoftmaxWarps + 1, kWarpCopy = kSoftmaxWarps + 2,
+              kWarpS = kSoftmaxWarps + 3;
 constexpr int kAttnThreads = 32 * (kSoftmaxWarps + 4);
+constexpr int kWalkBarrier = 4, kWalkThreads = kAttnThreads - 32;   // named barrier of the warps that walk the segments
 constexpr int kBM = 128;                 // query rows per tile
 constexpr int kBN = 128;                 // key rows per shared-memory tile
 constexpr int kBH = 64;                  // key rows per chunk (half a tile): the logits one thread holds
 constexpr float kOutgrownSum = 1.152921504606846976e18f;   // 2^60: chunk sum at which a reference maximum is renewed
-constexpr int kCopySlots = 4;             // cache refresh: units of rows in flight beside the walk of a segment
+constexpr int kCopySlots = 8;             // cache refresh: at most so many units of rows in flight
 constexpr int kHalfBytes = 128 * 64 * 2; // one 128-row x 64-column bf16 box (128-byte rows)
 constexpr long long kTimeoutCycles = 4000000000LL;   // default bound of every wait (about 2 s)
 
@@ -90,21 +92,21 @@ struct AttnCfg {
     // stage, the ordinary ring and the idle second query tile: kStages + 2 stages, an even number: K tiles and
     // V tiles have stages of their own)
     static constexpr int kSmemTiles = (2 + kStages + 1) * kTileBytes;
-    static constexpr int kCtrlBytes = 512;
+    static constexpr int kCtrlBytes = 640;
     static constexpr int kExchBytes = 4 * kBM * 4;         // exchange of the chunks' maxima and sums
     static constexpr int kExtraAt = kSmemTiles + kCtrlBytes + kExchBytes;
     // D = 128 fills shared memory: the epilogue stages its rows (4 KB per softmax warp) in the idle query
     // tiles, and a launch that refreshes the cache copies rows through the extra stage, a lone query tile
     // then keeps to the ordinary number of stages.  D = 64 has room for both.
     static constexpr int kStageAt = (D == 128) ? 0 : kExtraAt;
-    static constexpr int kCopySlotBytes = (D == 128) ? 8192 : 4096;
+    static constexpr int kCopyBytes = (D == 128) ? kTileBytes : 16384;
     static constexpr int kCopyAt = (D == 128) ? (2 + kStages) * kTileBytes : kExtraAt + kSoftmaxWarps * 4096;
-    static constexpr int kSmemBytes = kExtraAt + (D == 128 ? 0 : kSoftmaxWarps * 4096 + kCopySlots * kCopySlotBytes);
+    static constexpr int kSmemBytes = kExtraAt + (D == 128 ? 0 : kSoftmaxWarps * 4096 + kCopyBytes);
     static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
     __host__ __device__ static constexpr int lone_stages(bool store) { return kStages + (D == 128 && store ? 0 : 2); }
     // slots of the copies that are left when the walks are over and all tiles are idle
-    static constexpr int kTailSlots = 3, kTailSlotBytes = (D == 128) ? 65536 : 40960;
-    static_assert(kTailSlots * kTailSlotBytes <= kSmemTiles, "tail slots");
+    static constexpr int kTailBytes = (D == 128) ? 3 * 65536 : 3 * 40960;
+    static_assert(kTailBytes <= kSmemTiles, "tail slots");
 };
 
 // The part of one item that a CTA works on, as its roles need it (shared memory).
@@ -132,6 +134,7 @@ struct AttnCtrl {
     int abort_flag;
     int redo;                   // a row outgrew the reference maximum of its first key tile
     SegInfo seg[2];
+    int walks_done;             // cache refresh: the walks are over, every tile of shared memory is idle
     // cache refresh: a slot's rows have landed; where they go, and which of them are to be stored
     uint64_t copy_full[kCopySlots];
     uint8_t* copy_dst[kCopySlots];
@@ -147,7 +150,7 @@ static_assert(offsetof(AttnCtrl, kv_empty) == kBarKvEmpty * 8 && offsetof(AttnCt
               offsetof(AttnCtrl, pv_done) == kBarPvDone * 8 && offsetof(AttnCtrl, pv_half) == kBarPvHalf * 8 &&
               offsetof(AttnCtrl, s_free) == kBarSFree * 8 && offsetof(AttnCtrl, v_full) == (kBarSFree + 1) * 8 &&
               offsetof(AttnCtrl, tmem_base) == kNumBarriers * 8 &&
-              sizeof(AttnCtrl) <= 512, "barrier layout");
+              sizeof(AttnCtrl) <= 640, "barrier layout");
 
 // What share c tells the merge kernel: the item that the boundary between shares c - 1 and c
 // cuts, if c is the second share of that item (so every cut item is named exactly once).
@@ -702,17 +705,19 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
     ptx::fence_proxy_async_smem();      // the next segment's query tile arrives by TMA
 }
 
-// ---- cache refresh: copies of retained rows, done by the producer warp while it has nothing to load ---------
-// The rows travel as bulk copies (one per lane: global -> slot of shared memory -> cache), so the copies
-// take no registers, no issue slots to speak of and no time of the tensor cores.  The launch's rows
-// (K of every request, then V) are cut into equal contiguous shares, one per CTA, whatever attention work
-// the CTA has.  An item is one row, or a slot's length of it where a row is longer than that; a unit is up
-// to `per_unit` consecutive items of one request, lane i moving item i.
+// ---- cache refresh: copies of the retained rows, by a warp of their own ------------------------------------
+// The rows travel as bulk copies (one per lane: global -> slot of shared memory -> cache), so the copies take
+// no registers, few issue slots and no time of the tensor cores, and the warp may block on them.  (A first version
+// ran them from the producer warp between its loads: every wait for a slot delayed a key tile, and 194 MB of copies
+// cost the attention of 819 queries as much as a store kernel ahead of it.)  The launch's rows (K of every request,
+// then V) are cut into equal contiguous shares, one per CTA, whatever attention work the CTA has.  An item is one
+// row, or a slot's length of it where a row is longer than that; a unit is up to `per_unit` consecutive items of one
+// request, lane i moving item i.
 struct CachePump {
     const StoreParams* sp;
     const int32_t* n_rows;
     AttnCtrl* ctrl;
-    int32_t* dev_status;
+    const AttnParams* p;
     int row_bytes, item_bytes, per_row; // items per row
     uint32_t slots;                     // shared-memory address of slot 0
     int n_slots, slot_bytes, per_unit;
@@ -724,17 +729,17 @@ struct CachePump {
     __device__ __forceinline__ int kept(int req, bool report) const {
         const int nk = sp->n_keep[req];
         if (nk >= 0 && nk <= sp->store_cap) return nk;
-        if (report && blockIdx.x == 0) record_status(dev_status, REGIONE_DEV_BOUNDS);
+        if (report && blockIdx.x == 0) record_status(p->dev_status, REGIONE_DEV_BOUNDS);
         return nk < 0 ? 0 : sp->store_cap;
     }
     // from an item index behind the runs x, b to the run that holds it (a request without rows stores nothing)
-    __device__ __forceinline__ void open_run(int B) {
+    __device__ __forceinline__ void open_run() {
         for (;;) {
             live_rows = min(n_rows[b], sp->src_cap);
             run = live_rows > 0 ? kept(b, false) * per_row : 0;
             if (i < run) return;
             i -= run;
-            if (++b == B) { b = 0; ++x; }
+            if (++b == p->B) { b = 0; ++x; }
         }
     }
     // list entries of the next unit's items, fetched one unit ahead of their use
@@ -747,23 +752,25 @@ struct CachePump {
             if (j > 0) before = keep[j - 1];
         }
     }
-    __device__ __forceinline__ void use_slots(uint32_t at, int n, int bytes, int lane) {
-        slots = at; n_slots = n; slot_bytes = bytes;
-        per_unit = min(32, bytes / item_bytes);
+    // slots of one item each for long rows, of `unit` bytes for short ones, in `bytes` of shared memory
+    __device__ __forceinline__ void use_slots(uint32_t at, int bytes, int unit, int lane) {
+        slots = at;
+        slot_bytes = max(unit, (item_bytes + 127) & ~127);
+        n_slots = min(kCopySlots, bytes / slot_bytes);
+        per_unit = min(32, slot_bytes / item_bytes);
         head = tail = 0;
-        if (lane < n) ptx::mbar_init(ptx::smem_addr(&ctrl->copy_full[lane]), 1);
+        if (lane < n_slots) ptx::mbar_init(ptx::smem_addr(&ctrl->copy_full[lane]), 1);
         ptx::fence_barrier_init();
         __syncwarp();
         if (left > 0) fetch(lane);
     }
-    __device__ __forceinline__ void begin(const AttnParams& p, const StoreParams& s, AttnCtrl* c, int d, uint32_t at, int slot,
-                                          int lane) {
-        sp = &s; n_rows = p.n_fresh; ctrl = c; dev_status = p.dev_status;
-        row_bytes = p.H * d * 2;
-        per_row = (row_bytes + slot - 1) / slot;
-        item_bytes = min(row_bytes, slot);
+    __device__ __forceinline__ void begin(const AttnParams& prm, const StoreParams& s, AttnCtrl* c, int d, int longest, int lane) {
+        sp = &s; n_rows = prm.n_fresh; ctrl = c; p = &prm;
+        row_bytes = prm.H * d * 2;
+        per_row = (row_bytes + longest - 1) / longest;
+        item_bytes = min(row_bytes, longest);
         long long total = 0;
-        for (int r = 0; r < p.B; ++r) {
+        for (int r = 0; r < prm.B; ++r) {
             const int nk = kept(r, lane == 0);
             if (n_rows[r] > 0) total += 2LL * nk * per_row;
         }
@@ -771,70 +778,78 @@ struct CachePump {
         left = (int)max(0LL, min(per, total - first));
         x = b = 0;
         i = (int)first;
-        if (left > 0) open_run(p.B);
-        use_slots(at, kCopySlots, slot, lane);
+        if (left > 0) open_run();
     }
-    __device__ __forceinline__ bool busy() const { return left > 0 || tail < head; }
-    // One step of the pump (whole warp): stores the oldest unit if it has landed, then loads the next one
-    // if its slot is free.
-    __device__ __forceinline__ void poll(int B, int lane) {
-        if (tail < head) {
-            const int slot = tail % n_slots;
-            const bool landed = ptx::mbar_test_wait(ptx::smem_addr(&ctrl->copy_full[slot]), (tail / n_slots) & 1);
-            if (__any_sync(0xffffffffu, landed)) {
-                if ((ctrl->copy_valid[slot] >> lane) & 1u) {
-                    const int at = ctrl->copy_item[slot] + lane, j = at / per_row, off = (at - j * per_row) * item_bytes;
-                    ptx::bulk_store(ctrl->copy_dst[slot] + (size_t)j * row_bytes + off,
-                                    slots + slot * slot_bytes + lane * item_bytes, min(item_bytes, row_bytes - off));
-                }
-                ptx::bulk_commit();
-                ++tail;
-            }
+    __device__ __forceinline__ bool store_oldest(int lane) {
+        const int slot = tail % n_slots;
+        const bool landed = wait_bar(ptx::smem_addr(&ctrl->copy_full[slot]), (tail / n_slots) & 1, &ctrl->abort_flag,
+                                     p->dev_status, p->timeout_cycles);
+        if (!__all_sync(0xffffffffu, landed)) return false;
+        if ((ctrl->copy_valid[slot] >> lane) & 1u) {
+            const int at = ctrl->copy_item[slot] + lane, j = at / per_row, off = (at - j * per_row) * item_bytes;
+            ptx::bulk_store(ctrl->copy_dst[slot] + (size_t)j * row_bytes + off, slots + slot * slot_bytes + lane * item_bytes,
+                            min(item_bytes, row_bytes - off));
         }
+        ptx::bulk_commit();
+        ++tail;
+        return true;
+    }
+    __device__ __forceinline__ void load_next(int lane) {
         // (one slot of slack: all but the latest store have been read out of shared memory)
-        if (left > 0 && head - tail < n_slots - 1) {
-            ptx::bulk_wait_read<1>();
-            __syncwarp();
-            const int n = min(per_unit, min(run - i, left));
-            const bool ok = row >= 0 && row < live_rows && row > before;
-            if (lane < n && !ok) record_status(dev_status, REGIONE_DEV_BOUNDS);
-            const uint32_t valid = __ballot_sync(0xffffffffu, lane < n && ok);
-            const int slot = head % n_slots;
-            const uint32_t bar = ptx::smem_addr(&ctrl->copy_full[slot]);
-            const int off = ((i + lane) % per_row) * item_bytes;
-            const int bytes = (valid >> lane) & 1u ? min(item_bytes, row_bytes - off) : 0;
-            const int unit_bytes = __reduce_add_sync(0xffffffffu, bytes);
-            if (lane == 0) {
-                ctrl->copy_valid[slot] = valid;
-                ctrl->copy_item[slot] = i;
-                ctrl->copy_dst[slot] = sp->dst[x] + (size_t)b * sp->store_cap * row_bytes;
-                ptx::mbar_arrive_expect_tx(bar, unit_bytes);
-            }
-            __syncwarp();
-            if (bytes > 0)
-                ptx::bulk_load(slots + slot * slot_bytes + lane * item_bytes,
-                               sp->src[x] + ((size_t)b * sp->src_cap + row) * row_bytes + off, bytes, bar);
-            ++head;
-            left -= n;
-            i += n;
-            if (left > 0) {
-                if (i >= run) open_run(B);
-                fetch(lane);
-            }
+        ptx::bulk_wait_read<1>();
+        __syncwarp();
+        const int n = min(per_unit, min(run - i, left));
+        const bool ok = row >= 0 && row < live_rows && row > before;
+        if (lane < n && !ok) record_status(p->dev_status, REGIONE_DEV_BOUNDS);
+        const uint32_t valid = __ballot_sync(0xffffffffu, lane < n && ok);
+        const int slot = head % n_slots;
+        const uint32_t bar = ptx::smem_addr(&ctrl->copy_full[slot]);
+        const int off = ((i + lane) % per_row) * item_bytes;
+        const int bytes = (valid >> lane) & 1u ? min(item_bytes, row_bytes - off) : 0;
+        const int unit_bytes = __reduce_add_sync(0xffffffffu, bytes);
+        if (lane == 0) {
+            ctrl->copy_valid[slot] = valid;
+            ctrl->copy_item[slot] = i;
+            ctrl->copy_dst[slot] = sp->dst[x] + (size_t)b * sp->store_cap * row_bytes;
+            ptx::mbar_arrive_expect_tx(bar, unit_bytes);
+        }
+        __syncwarp();
+        if (bytes > 0)
+            ptx::bulk_load(slots + slot * slot_bytes + lane * item_bytes,
+                           sp->src[x] + ((size_t)b * sp->src_cap + row) * row_bytes + off, bytes, bar);
+        ++head;
+        left -= n;
+        i += n;
+        if (left > 0) {
+            if (i >= run) open_run();
+            fetch(lane);
         }
     }
-    // Stores everything that is left; false when a load did not land within `limit` cycles.
-    __device__ __forceinline__ bool drain(int B, int lane, long long limit) {
-        long long t0 = clock64();
-        int last = tail;
-        while (busy()) {
-            poll(B, lane);
-            if (tail != last) { last = tail; t0 = clock64(); }
-            if (__any_sync(0xffffffffu, clock64() - t0 > limit)) {
-                record_status(dev_status, REGIONE_DEV_TIMEOUT);
-                return false;
+    // Moves the CTA's rows: through a corner of shared memory beside the walks, through the idle tiles once they are
+    // over.  False when a copy did not land within the bound of the waits.
+    template <int D>
+    __device__ __forceinline__ bool run_all(uint32_t smem, int lane) {
+        using Cfg = AttnCfg<D>;
+        bool wide = false;
+        if (left > 0) use_slots(smem + Cfg::kCopyAt, Cfg::kCopyBytes, Cfg::kCopyBytes / kCopySlots, lane);
+        while (left > 0) {
+            if (!wide && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&ctrl->walks_done) != 0)) {
+                while (tail < head)
+                    if (!store_oldest(lane)) return false;
+                ptx::bulk_wait_read<0>();
+                __threadfence_block();
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane < n_slots) ptx::mbar_inval(ptx::smem_addr(&ctrl->copy_full[lane]));
+                __syncwarp();
+                use_slots(smem, Cfg::kTailBytes, Cfg::kTailBytes / kCopySlots, lane);
+                wide = true;
             }
+            if (head - tail < n_slots - 1) load_next(lane);
+            else if (!store_oldest(lane)) return false;
         }
+        while (tail < head)
+            if (!store_oldest(lane)) return false;
         return true;
     }
 };
@@ -843,8 +858,7 @@ struct CachePump {
 template <int D, bool STORE>
 __device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUtensorMap* tm_kf, const CUtensorMap* tm_vf,
                                              const CUtensorMap* tm_kc, const CUtensorMap* tm_vc, const AttnParams& p,
-                                             AttnCtrl* ctrl, const SegInfo& it, const uint32_t smem, const int lane,
-                                             CachePump& pump) {
+                                             AttnCtrl* ctrl, const SegInfo& it, const uint32_t smem, const int lane) {
     using Cfg = AttnCfg<D>;
     constexpr int kTileBytes = Cfg::kTileBytes;
     const int n_tiles = it.n_tiles;
@@ -869,11 +883,6 @@ __device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUte
         const int j = j_first + (i >> 1), is_v = i & 1;
         if (use > 0) {
             const uint32_t bar = ptx::smem_addr(&ctrl->kv_empty[stage]);
-            if constexpr (STORE) {
-                // rows of the cache are copied while the stage is not free yet
-                while (pump.busy() && !__any_sync(0xffffffffu, ptx::mbar_test_wait(bar, (use - 1) & 1)) && !ctrl->abort_flag)
-                    pump.poll(p.B, lane);
-            }
             if (!wait_bar(bar, (use - 1) & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
         }
         if (lane == 0) {
@@ -887,12 +896,6 @@ __device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUte
         }
         __syncwarp();
         if (++stage == n_stages) { stage = 0; ++use; }
-    }
-    if constexpr (STORE) {
-        // ... and while the segment's last products run
-        while (pump.busy() && !__any_sync(0xffffffffu, ptx::mbar_test_wait(ptx::smem_addr(&ctrl->o_final[0]), 0)) &&
-               !ctrl->abort_flag)
-            pump.poll(p.B, lane);
     }
 }
 
@@ -947,58 +950,58 @@ __device__ __forceinline__ void issue_s_segment(const AttnParams& p, AttnCtrl* c
     }
 }
 
-// ---- issuer of the P*V products of query-tile role t (whole warp, one elected lane issues) ----------------
+// ---- issuer of the P*V products of both query-tile roles (whole warp, one elected lane issues) --------------
+// The roles take turns, as their logits do in the shared S buffer: a pair's tiles on every key tile, a lone tile's
+// roles on alternate key tiles.
 template <int D, bool STORE>
 __device__ __forceinline__ void issue_pv_segment(const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it, const uint32_t smem,
-                                                 const uint32_t tmem, const int t, const int lane, const int mode) {
+                                                 const uint32_t tmem, const int lane, const int mode) {
     using Cfg = AttnCfg<D>;
     constexpr int kTileBytes = Cfg::kTileBytes;
     const int n_tiles = it.n_tiles;
-    const int ntq = it.nq - it.q0 > kBM ? 2 : 1;
-    const bool split = ntq == 1 && n_tiles >= 2;
-    if (n_tiles == 0 || t >= (split ? 2 : ntq)) return;
+    const bool pair = it.nq - it.q0 > kBM;
+    const bool split = !pair && n_tiles >= 2;
     const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
     const TileKeys keys(it);
-    const int n_my = split ? (n_tiles + 1 - t) >> 1 : n_tiles;
+    const int n_turns = pair ? 2 * n_tiles : n_tiles;
     constexpr uint32_t idesc_pv = ptx::idesc_bf16_f32(kBM, D, true);
     constexpr uint32_t hi_k = ptx::smem_desc_hi_sw128(1024);   // 8-key groups 1024 B apart
     // V is MN-major: 64-column boxes kHalfBytes apart (LBO), 8-key groups 1024 B apart (SBO)
     const uint32_t v_lo = ptx::smem_desc_lo(smem + (split ? 1 : 2) * kTileBytes, kHalfBytes);
-    const uint32_t tPt = tmem + kBN + t * (kBN / 2), tOt = tmem + 256 + t * D;
-    // O_t (+)= P_t[chunk] V[64 chunk .. 64 chunk + 64) : A from tensor memory (bf16 pairs,
-    // 8 columns per 16 keys)
-    auto issue_pv = [&](int stage, int chunk, bool accumulate) {
-        const uint32_t b0 = v_lo + ((stage * kTileBytes + chunk * (kBH / 16) * 2048) >> 4);
-#pragma unroll
-        for (int kk = 0; kk < kBH / 16; ++kk)
-            ptx::mma_ts(tOt, tPt + chunk * (kBH / 2) + kk * 8,
-                        ptx::smem_desc_join(b0 + ((kk * 2048) >> 4), hi_k), idesc_pv,
-                        (accumulate || kk > 0) ? 1u : 0u);
-    };
-    for (int j = 0; j < n_my; ++j) {
-        const int jl = split ? 2 * j + t : j;
+    for (int n = 0; n < n_turns; ++n) {
+        const int t = n & 1, j = n >> 1, jl = pair ? j : n;
         const int sv = (2 * jl + 1) % n_stages;
         const VLanding vl = v_landing(ctrl, split, n_stages, jl);
-        const bool more = (j + 1 < n_my);
-        if (!wait_bar(vl.bar, vl.phase & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
+        if ((!pair || t == 0) && !wait_bar(vl.bar, vl.phase & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
         if (mode == kMaxOnly) {                     // no products in this pass: the stage is given back
             if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctrl->kv_empty[sv]));
             continue;
         }
+        const uint32_t tPt = tmem + kBN + t * (kBN / 2), tOt = tmem + 256 + t * D;
+        // O_t (+)= P_t[chunk] V[64 chunk .. 64 chunk + 64) : A from tensor memory (bf16 pairs,
+        // 8 columns per 16 keys)
+        auto issue_pv = [&](int chunk, bool accumulate) {
+            const uint32_t b0 = v_lo + ((sv * kTileBytes + chunk * (kBH / 16) * 2048) >> 4);
+#pragma unroll
+            for (int kk = 0; kk < kBH / 16; ++kk)
+                ptx::mma_ts(tOt, tPt + chunk * (kBH / 2) + kk * 8,
+                            ptx::smem_desc_join(b0 + ((kk * 2048) >> 4), hi_k), idesc_pv,
+                            (accumulate || kk > 0) ? 1u : 0u);
+        };
         if (!wait_bar(ptx::smem_addr(&ctrl->p_full[t][0]), j & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
         ptx::tc_fence_after_sync();
         if (ptx::elect_one()) {
-            issue_pv(sv, 0, j > 0);
+            issue_pv(0, j > 0);
             ptx::mma_commit(ptx::smem_addr(&ctrl->pv_half[t]));
         }
         __syncwarp();
         if (!wait_bar(ptx::smem_addr(&ctrl->p_full[t][1]), j & 1, &ctrl->abort_flag, p.dev_status, p.timeout_cycles)) return;
         ptx::tc_fence_after_sync();
         if (ptx::elect_one()) {
-            if (keys(jl) > kBH) issue_pv(sv, 1, true);
+            if (keys(jl) > kBH) issue_pv(1, true);
             ptx::mma_commit(ptx::smem_addr(&ctrl->pv_done[t]));
             ptx::mma_commit(ptx::smem_addr(&ctrl->kv_empty[sv]));
-            if (!more) ptx::mma_commit(ptx::smem_addr(&ctrl->o_final[t]));      // (the segment's last arrival)
+            if (n + 2 >= n_turns) ptx::mma_commit(ptx::smem_addr(&ctrl->o_final[t]));      // (the role's last arrival)
         }
         __syncwarp();
     }
@@ -1078,6 +1081,9 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     // logits per thread, the producer / issuer warpgroup gives registers up.  CTA-wide barriers around a
     // segment: `set-up` (control block's barriers initialised, next segment known) and `end` (every role is
     // done with shared and tensor memory).
+    auto walk_sync = [&]() {
+        asm volatile("bar.sync %0, %1;" ::"n"(kWalkBarrier), "n"(kWalkThreads) : "memory");
+    };
     auto set_up = [&](const SegInfo& it) {
         // thread i sets barrier i of the control block up
         const int ntq = it.nq - it.q0 > kBM ? 2 : 1;
@@ -1093,12 +1099,12 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         }
         if (threadIdx.x == 0) ctrl->redo = 0;
         ptx::tc_fence_before_sync();
-        __syncthreads();
+        walk_sync();
         ptx::tc_fence_after_sync();
     };
     auto tear_down = [&]() {
         ptx::tc_fence_before_sync();
-        __syncthreads();
+        walk_sync();
         ptx::tc_fence_after_sync();
         if (threadIdx.x < kNumBarriers) ptx::mbar_inval(ptx::smem_addr(&ctrl->q_full + threadIdx.x));
     };
@@ -1108,29 +1114,39 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         const int next_mode = redo ? kMaxOnly : mode == kMaxOnly ? kExact : kWalk;
         const bool again = next_mode != kWalk;
         mode = next_mode;
-        __syncthreads();                                // (redo has been read by everyone)
+        walk_sync();                                // (redo has been read by everyone)
         return again;
     };
+    if (STORE && threadIdx.x == 0) ctrl->walks_done = 0;
     __syncthreads();
     const uint32_t tmem = ctrl->tmem_base;
-    CachePump pump;
     int k = 0, mode = kWalk;
     if (warp >= kSoftmaxWarps) {
         ptx::reg_dealloc<64>();
-        if constexpr (STORE) {
-            if (warp == kWarpLoad) pump.begin(p, sp, ctrl, D, smem + Cfg::kCopyAt, Cfg::kCopySlotBytes, lane);
+        if (warp == kWarpCopy) {
+            if constexpr (STORE) {
+                CachePump pump;
+                pump.begin(p, sp, ctrl, D, Cfg::kCopyBytes / 4, lane);
+                if (!pump.run_all<D>(smem, lane)) {
+                    // give copies that are still in flight time to land before shared memory is given back
+                    const long long t0 = clock64();
+                    while (clock64() - t0 < 2000000LL) __nanosleep(1000);
+                }
+                ptx::bulk_wait_all();
+            }
+            return;
         }
         while (ctrl->seg[k].live && !*abort_flag) {
             const SegInfo& it = ctrl->seg[k];
             set_up(it);
             if (warp == kWarpLoad) {
-                load_segment<D, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, p, ctrl, it, smem, lane, pump);
+                load_segment<D, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, p, ctrl, it, smem, lane);
             } else if (warp == kWarpS) {
                 issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
                 // (the next segment is planned behind the last product, ahead of the end of this one)
                 if (mode == kWalk) cur.next(p, &ctrl->seg[k ^ 1], lane);
             } else {
-                issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, warp - kWarpPv, lane, mode);
+                issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, lane, mode);
             }
             tear_down();
             if (!repeat(mode)) k ^= 1;
@@ -1154,35 +1170,15 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         while (clock64() - t0 < 2000000LL) __nanosleep(1000);
     }
     ptx::tc_fence_before_sync();
-    __syncthreads();
+    walk_sync();
     if (warp == kWarpPv) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem, 512);
     }
-    if constexpr (STORE) {
-        // the rows that the walks left no time for: every tile is idle now, so that enough of them are in
-        // flight to run at the speed of memory
-        if (warp == kWarpLoad && !*abort_flag && pump.busy()) {
-            bool ok = pump.left == 0;
-            if (!ok) {
-                // what is in the small slots first, then all of shared memory
-                const int left = pump.left;
-                pump.left = 0;
-                ok = pump.drain(p.B, lane, p.timeout_cycles);
-                pump.left = left;
-                ptx::bulk_wait_read<0>();
-                __syncwarp();
-                if (lane < kCopySlots) ptx::mbar_inval(ptx::smem_addr(&ctrl->copy_full[lane]));
-                __syncwarp();
-                pump.use_slots(smem, Cfg::kTailSlots, Cfg::kTailSlotBytes, lane);
-            }
-            if (ok) ok = pump.drain(p.B, lane, p.timeout_cycles);
-            if (!ok) {
-                const long long t0 = clock64();
-                while (clock64() - t0 < 2000000LL) __nanosleep(1000);
-            }
-        }
-        if (warp == kWarpLoad) ptx::bulk_wait_all();
+    // (every role's writes to the tiles are ordered before this by its proxy fence and the barrier above)
+    if (STORE && threadIdx.x == 0) {
+        __threadfence_block();
+        *reinterpret_cast<volatile int*>(&ctrl->walks_done) = 1;
     }
 }
 
