@@ -52,6 +52,11 @@
 // slot of the caller's workspace and a small second kernel merges the slots of such items (the
 // attention kernel leaves it a table of the items that its share boundaries cut).  The share
 // length is bounded below so that no item is spread over more slots than the workspace holds.
+// Where the capacities allow only few items (choose_cluster), an item is shared by a cluster of 2 to 8 CTAs instead, an
+// equal run of its key tiles each; they leave their partial rows in shared memory, where the cluster's CTAs read
+// them (distributed shared memory) and write the output: no workspace, no second kernel, no plan to derive.  Measured,
+// shares of the cost axis -> clusters: 3 x 333 queries x 261 keys x 5 heads 20.9 -> 17.9 us (D = 64 17.4 -> 14.4),
+// 2 x 700 x 3700 x 12 47.8 -> 44.0 (D = 64 41.6 -> 35.3), 256 x 2112 x 4, D = 64 17.1 -> 15.5, one row 14.2 -> 10.6.
 // Counts live in device memory, so every CTA derives the same plan from them.  Output rows go to
 // out[b, i] or, with a row list, to out[b, out_rows[b, i]] (the scatter of the attention rows back
 // into the joint sequence, done by whichever kernel writes the row).
@@ -75,6 +80,7 @@ constexpr int kWarpLoad = kSoftmaxWarps, kWarpPv = kSoftmaxWarps + 1, kWarpCopy 
               kWarpS = kSoftmaxWarps + 3;
 constexpr int kAttnThreads = 32 * (kSoftmaxWarps + 4);
 constexpr int kWalkBarrier = 4, kWalkThreads = kAttnThreads - 32;   // named barrier of the warps that walk the segments
+constexpr int kMaxCluster = 8;           // CTAs that may share an item through their shared memories
 constexpr int kBM = 128;                 // query rows per tile
 constexpr int kBN = 128;                 // key rows per shared-memory tile
 constexpr int kBH = 64;                  // key rows per chunk (half a tile): the logits one thread holds
@@ -105,6 +111,9 @@ struct AttnCfg {
     static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
     __host__ __device__ static constexpr int lone_stages(bool store) { return kStages + (D == 128 && store ? 0 : 2); }
     // slots of the copies that are left when the walks are over and all tiles are idle
+    // an item shared by a cluster: its CTAs leave their partial rows, chunk by chunk, and (max, sum) pairs here
+    static constexpr int kPartialMlAt = 2 * kBM * D * 4;
+    static_assert(kPartialMlAt + 2 * kBM * 8 <= kSmemTiles, "partial rows");
     static constexpr int kTailBytes = (D == 128) ? 3 * 65536 : 3 * 40960;
     static_assert(kTailBytes <= kSmemTiles, "tail slots");
 };
@@ -134,6 +143,8 @@ struct AttnCtrl {
     int abort_flag;
     int redo;                   // a row outgrew the reference maximum of its first key tile
     SegInfo seg[2];
+    uint64_t peers_ready;       // item shared by a cluster: every CTA's partial rows are in its shared memory
+    uint64_t peers_done;        // ... and have been read by every CTA
     int walks_done;             // cache refresh: the walks are over, every tile of shared memory is idle
     // cache refresh: a slot's rows have landed; where they go, and which of them are to be stored
     uint64_t copy_full[kCopySlots];
@@ -172,6 +183,7 @@ struct AttnParams {
     int32_t* dev_status;
     float* part_o;       // [B, H, P_cap, max_slots, 256, D] unnormalised outputs
     float2* part_ml;     // [B, H, P_cap, max_slots, 256]    (running max in the exp2 domain, sum)
+    int cluster;         // > 0: every item is shared by a cluster of so many CTAs, no workspace, no merge kernel
     CutItem* cut;        // [grid] the item that the start of each share cuts, for the merge kernel
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
 };
@@ -372,6 +384,20 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
     }
 }
 
+// The same for phase 0 of a barrier that the CTAs of a cluster arrive on.
+__device__ __forceinline__ bool wait_bar_cluster(uint32_t bar, volatile int* abort_flag, int32_t* dev_status, long long limit) {
+    const long long t0 = clock64();
+    while (!ptx::mbar_try_wait_cluster(bar, 0)) {
+        if (*abort_flag) return false;
+        if (clock64() - t0 > limit) {
+            *abort_flag = 1;
+            record_status(dev_status, REGIONE_DEV_TIMEOUT);
+            return false;
+        }
+    }
+    return true;
+}
+
 // Keys >= valid of a 64-logit chunk are dead (behind a segment's live prefix): their logits become
 // -inf, after which the chunk goes through the same code as a full one (maximum unaffected,
 // probability 0 or, on the polynomial path, 2^-126).  A short separate pass instead of masked
@@ -475,7 +501,7 @@ __device__ __forceinline__ VLanding v_landing(AttnCtrl* ctrl, bool split, int n_
 enum WalkMode { kWalk, kMaxOnly, kExact };
 
 // ---- softmax / epilogue of one segment: thread = (query row, 64-key chunk) ----------------------------
-template <int D, bool STORE>
+template <int D, bool STORE, bool CLUSTER>
 __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it, uint8_t* smem_gen,
                                                 const uint32_t tmem, const int warp, const int lane, const int mode,
                                                 float& m_known) {
@@ -624,6 +650,12 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             l = exch[0] + exch[kBM];
         }
     }
+    constexpr bool shared = CLUSTER;
+    if (shared && n_tiles > 0 && pair && ok) {
+        // (the partial rows go over the tiles that the other query tile's products may still read)
+        ok = wait_bar(ptx::smem_addr(&ctrl->o_final[1 - t]), 0, abort_flag, p.dev_status, p.timeout_cycles);
+        if (ok) ptx::tc_fence_after_sync();
+    }
     // this warp's 32-column pieces of the row: [pc0, pc1)
     constexpr int kPieces = D / 32;
     const int per = split ? (kPieces >= 4 ? 1 : (t == 0 ? 1 : 0)) : kPieces / 2;
@@ -638,7 +670,12 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
         record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         dst_row = -1;
     }
-    if (n_tiles == 0) {
+    if (shared) {
+        float2* const ml = reinterpret_cast<float2*>(smem_gen + Cfg::kPartialMlAt) + qt * kBM + row;
+        if (ck == 0 && (!split || t == 0)) *ml = n_tiles > 0 && ok ? make_float2(m, l) : make_float2(-INFINITY, 0.f);
+    }
+    if (shared && n_tiles == 0) {
+    } else if (n_tiles == 0) {
         // no keys: zero rows, or an empty slot
         if (ck == 0 && direct && dst_row >= 0)
             for (int q = 0; q < D / 8; ++q)
@@ -665,7 +702,12 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             // 16-byte chunk q of row r sits at column q ^ (r & 7): both the row-wise writes and
             // the piece-wise reads are free of bank conflicts without padding
             uint4* const mine = reinterpret_cast<uint4*>(stage + lane * 128);
-            if (direct) {
+            if (shared) {
+                // unnormalised O of this rank, 16-byte chunk by chunk with the 32 rows of the warp side by side
+                uint4* const col = reinterpret_cast<uint4*>(smem_gen) + ((qt * 4 + (warp & 3)) * (D / 4) + pc * 8) * 32 + lane;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) col[q * 32] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+            } else if (direct) {
                 // O / l -> bf16 -> out: 64-byte pieces, 8 rows per instruction
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -700,9 +742,75 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             }
             __syncwarp();
         }
-        if (!direct && live && ck == 0 && (!split || t == 0)) p.part_ml[prow_w + lane] = make_float2(m, l);
+        if (!shared && !direct && live && ck == 0 && (!split || t == 0)) p.part_ml[prow_w + lane] = make_float2(m, l);
     }
     ptx::fence_proxy_async_smem();      // the next segment's query tile arrives by TMA
+}
+
+// ---- item shared by a cluster: merge of the ranks' partial rows (softmax warps) ------------------------------------
+//     out = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s
+// straight from the CTAs' shared memories.  A unit is 8 columns of 32 rows, dealt over the ranks' warps; a lane
+// owns one row, all ranks' loads are issued before the first use.
+template <int D>
+__device__ __forceinline__ void merge_cluster(const AttnParams& p, const SegInfo& it, const uint32_t smem, const int warp,
+                                              const int lane) {
+    using Cfg = AttnCfg<D>;
+    const int n = p.cluster, rows = min(it.nq - it.q0, 2 * kBM);
+    const int n_units = ((rows + 31) >> 5) * (D / 8);
+    for (int u = it.slot + n * warp; u < n_units; u += n * kSoftmaxWarps) {
+        const int rb = u / (D / 8), col = (u - rb * (D / 8)) * 8;
+        const int row = rb * 32 + lane, qrow = it.q0 + row;
+        const bool live = row < rows;
+        int dst_row = -1;
+        if (live) dst_row = p.out_rows != nullptr ? p.out_rows[(size_t)it.b * p.Nq_cap + qrow] : qrow;
+        const uint32_t at_ml = smem + Cfg::kPartialMlAt + row * 8, at_o = smem + ((rb * (D / 4) + (col >> 2)) * 32 + lane) * 16;
+        float w[kMaxCluster];                         // the ranks' maxima, then their weights
+        float M = -INFINITY, L = 0.f;
+        {
+            float2 ml[kMaxCluster];
+#pragma unroll
+            for (int s = 0; s < kMaxCluster; ++s)
+                if (s < n) ml[s] = ptx::ld_cluster_f2(ptx::map_rank(at_ml, s));
+#pragma unroll
+            for (int s = 0; s < kMaxCluster; ++s)
+                if (s < n && ml[s].y > 0.f) M = fmaxf(M, ml[s].x);
+#pragma unroll
+            for (int s = 0; s < kMaxCluster; ++s) {
+                w[s] = s < n && ml[s].y > 0.f ? fast_exp2(ml[s].x - M) : 0.f;     // a rank without keys carries no weight
+                if (w[s] > 0.f) L = fmaf(w[s], ml[s].y, L);
+            }
+        }
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int s0 = 0; s0 < kMaxCluster; s0 += 4) {
+            if (s0 >= n) break;
+            float4 o[4][2];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                if (s0 + s < n) {
+                    o[s][0] = ptx::ld_cluster_f4(ptx::map_rank(at_o, s0 + s));
+                    o[s][1] = ptx::ld_cluster_f4(ptx::map_rank(at_o + 512, s0 + s));
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                if (s0 + s < n && w[s0 + s] > 0.f) {
+                    const float v[8] = {o[s][0].x, o[s][0].y, o[s][0].z, o[s][0].w, o[s][1].x, o[s][1].y, o[s][1].z, o[s][1].w};
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[e] = fmaf(w[s0 + s], v[e], acc[e]);
+                }
+            }
+        }
+        const float inv = L > 0.f ? 1.f / L : 0.f;
+        if (live && (dst_row < 0 || dst_row >= p.out_cap)) {   // destination out of range: dropped
+            if (col == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
+        } else if (live) {
+            uint4 o;
+            o.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); o.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+            o.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); o.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+            *reinterpret_cast<uint4*>(p.out + (((size_t)it.b * p.out_cap + dst_row) * p.H + it.h) * D + col) = o;
+        }
+    }
 }
 
 // ---- cache refresh: copies of the retained rows, by a warp of their own ------------------------------------
@@ -1012,6 +1120,30 @@ struct ShareCursor {
     Plan pl;
     long long pos, hi;
     bool first;
+    // The only segment of a CTA whose item is shared by a cluster: rank r of n takes the key tiles
+    // [r * nt / n, (r + 1) * nt / n) (possibly none) and reads back its part of the rows.
+    __device__ __forceinline__ void of_cluster(const AttnParams& p, SegInfo* out, const int lane, bool* bad) {
+        int idx = blockIdx.x / p.cluster;
+        const int rank = blockIdx.x - idx * p.cluster;
+        ReqShape r = req_shape(p, 0, bad);
+        int b = 0;
+        while (b + 1 < p.B && idx >= p.H * r.np) {
+            idx -= p.H * r.np;
+            r = req_shape(p, ++b, bad);
+        }
+        pos = hi = 0;
+        first = false;
+        if (lane != 0) return;
+        out->live = idx < p.H * r.np;
+        if (!out->live) return;
+        out->b = b;
+        out->h = idx / r.np;
+        out->q0 = (idx - out->h * r.np) * (2 * kBM);
+        out->nq = r.nq; out->nt_c = r.nt_c; out->nt = r.nt; out->nc = r.nc; out->nf = r.nf;
+        out->j_first = rank * r.nt / p.cluster;
+        out->n_tiles = (rank + 1) * r.nt / p.cluster - out->j_first;
+        out->item = 0; out->slot = rank; out->n_slots = p.cluster;
+    }
     // The next live segment of the share into *out (out->live = 0 when the share ends).
     __device__ __forceinline__ void next(const AttnParams& p, SegInfo* out, const int lane) {
         while (pos < hi) {
@@ -1044,7 +1176,7 @@ struct ShareCursor {
     }
 };
 
-template <int D, bool STORE>
+template <int D, bool STORE, bool CLUSTER>
 __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, const CUtensorMap& tm_kf,
                                                       const CUtensorMap& tm_vf, const CUtensorMap& tm_kc,
                                                       const CUtensorMap& tm_vc, const AttnParams& p,
@@ -1068,12 +1200,22 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         // (whole items are dealt round-robin, so that the CTAs running at any one time work on
         // neighbouring items, which share K/V tiles in L2; a share of steps is one contiguous range)
         bool bad = false;
+        if constexpr (CLUSTER) {
+            cur.of_cluster(p, &ctrl->seg[0], lane, &bad);
+            if (lane == 0) {
+                ctrl->seg[1].live = 0;
+                ptx::mbar_init(ptx::smem_addr(&ctrl->peers_ready), p.cluster);
+                ptx::mbar_init(ptx::smem_addr(&ctrl->peers_done), p.cluster);
+                ptx::fence_barrier_init();
+            }
+        } else {
         cur.pl = plan_shares(p, gridDim.x, &bad);
-        if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)blockIdx.x * cur.pl.chunk;
         cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
         cur.first = true;
         cur.next(p, &ctrl->seg[0], lane);
+        }
+        if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         if (lane == 0) ctrl->abort_flag = 0;
     }
 
@@ -1118,6 +1260,8 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         return again;
     };
     if (STORE && threadIdx.x == 0) ctrl->walks_done = 0;
+    __syncwarp();
+    if (CLUSTER) ptx::cluster_sync();             // (the peers' barriers are initialised)
     __syncthreads();
     const uint32_t tmem = ctrl->tmem_base;
     int k = 0, mode = kWalk;
@@ -1144,7 +1288,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             } else if (warp == kWarpS) {
                 issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
                 // (the next segment is planned behind the last product, ahead of the end of this one)
-                if (mode == kWalk) cur.next(p, &ctrl->seg[k ^ 1], lane);
+                if (!CLUSTER && mode == kWalk) cur.next(p, &ctrl->seg[k ^ 1], lane);
             } else {
                 issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, lane, mode);
             }
@@ -1156,10 +1300,26 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         float m_known = -INFINITY;
         while (ctrl->seg[k].live && !*abort_flag) {
             set_up(ctrl->seg[k]);
-            softmax_segment<D, STORE>(p, ctrl, ctrl->seg[k], smem_raw, tmem, warp, lane, mode, m_known);
+            softmax_segment<D, STORE, CLUSTER>(p, ctrl, ctrl->seg[k], smem_raw, tmem, warp, lane, mode, m_known);
             tear_down();
             if (!repeat(mode)) k ^= 1;
         }
+    }
+
+    // ================= item shared by a cluster =================
+    if (CLUSTER && ctrl->seg[0].live) {
+        // (tear_down's barrier has ordered every warp's partial rows before this)
+        const uint32_t ready = ptx::smem_addr(&ctrl->peers_ready), done = ptx::smem_addr(&ctrl->peers_done);
+        if (warp == 0 && lane < p.cluster && !*abort_flag) ptx::mbar_arrive_cluster(ptx::map_rank(ready, lane));
+        bool ok = !*abort_flag;
+        if (warp < kSoftmaxWarps) {
+            if (ok) ok = wait_bar_cluster(ready, abort_flag, p.dev_status, p.timeout_cycles);
+            if (ok) merge_cluster<D>(p, ctrl->seg[0], smem, warp, lane);
+        }
+        walk_sync();
+        if (warp == 0 && lane < p.cluster && !*abort_flag) ptx::mbar_arrive_cluster(ptx::map_rank(done, lane));
+        // (a CTA's shared memory stays until every peer has read it)
+        if (!*abort_flag) wait_bar_cluster(done, abort_flag, p.dev_status, p.timeout_cycles);
     }
 
     // ================= teardown =================
@@ -1182,8 +1342,9 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     }
 }
 
-// The attention kernel, and the one that also refreshes the cache (one parameter more).
-template <int D>
+// The attention kernel, and the one that also refreshes the cache (one parameter more); each also in the form
+// whose items are shared by clusters (instantiations of their own: the code of one form costs the other 1 %).
+template <int D, bool CLUSTER>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 region_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                            const __grid_constant__ CUtensorMap tm_kf,
@@ -1191,9 +1352,9 @@ region_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                            const __grid_constant__ CUtensorMap tm_kc,
                            const __grid_constant__ CUtensorMap tm_vc, const AttnParams p) {
     const StoreParams none = {};
-    attention_kernel_body<D, false>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, none);
+    attention_kernel_body<D, false, CLUSTER>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, none);
 }
-template <int D>
+template <int D, bool CLUSTER>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_kf,
@@ -1201,7 +1362,7 @@ region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_kc,
                               const __grid_constant__ CUtensorMap tm_vc, const AttnParams p,
                               const __grid_constant__ StoreParams sp) {
-    attention_kernel_body<D, true>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, sp);
+    attention_kernel_body<D, true, CLUSTER>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, sp);
 }
 
 // Merges the workspace slots of the items that were spread over several shares:
@@ -1393,45 +1554,104 @@ size_t region_attention_tc_workspace(int B, int Nq_cap, int Nf_cap, int Nc_cap, 
            ((rows * sizeof(float2) + 255) & ~(size_t)255) + (size_t)lp.grid * sizeof(CutItem);
 }
 
+template <int D, bool STORE, bool CLUSTER>
+static auto main_kernel() {
+    if constexpr (STORE) return region_attention_store_kernel<D, CLUSTER>;
+    else return region_attention_tc_kernel<D, CLUSTER>;
+}
+
+// Once per device: the opt-in to large dynamic shared memory, and how many clusters of each size fit the GPU.
 template <int D, bool STORE>
-static int launch_main(const CUtensorMap* maps, const AttnParams& prm, const StoreParams& sp, int grid,
-                       cudaStream_t st) {
-    using Cfg = AttnCfg<D>;
-    // the opt-in to large dynamic shared memory is a per-device attribute of the kernel
+static int prepare_kernel(const int** fitting) {
     static int configured[kMaxDevices] = {};
+    static int clusters[kMaxDevices][kMaxCluster + 1] = {};
     const int dev = current_device();
     if (dev < 0) return REGIONE_CUDA_ERROR;
     if (!__atomic_load_n(&configured[dev], __ATOMIC_ACQUIRE)) {
-        const cudaError_t e =
-            STORE ? cudaFuncSetAttribute(region_attention_store_kernel<D>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes)
-                  : cudaFuncSetAttribute(region_attention_tc_kernel<D>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes);
-        if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
+        if (cudaFuncSetAttribute(main_kernel<D, STORE, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 AttnCfg<D>::kSmemBytes) != cudaSuccess ||
+            cudaFuncSetAttribute(main_kernel<D, STORE, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 AttnCfg<D>::kSmemBytes) != cudaSuccess)
+            return REGIONE_CUDA_ERROR;
+        for (int n = 2; n <= kMaxCluster; ++n) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(n * 148);
+            cfg.blockDim = dim3(kAttnThreads);
+            cfg.dynamicSmemBytes = AttnCfg<D>::kSmemBytes;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = n; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, main_kernel<D, STORE, true>(), &cfg) != cudaSuccess) {
+                (void)cudaGetLastError();
+                fit = 0;
+            }
+            clusters[dev][n] = fit;
+        }
         __atomic_store_n(&configured[dev], 1, __ATOMIC_RELEASE);
     }
-    cudaError_t e;
-    if constexpr (STORE)
-        e = launch_overlapped(region_attention_store_kernel<D>, dim3(grid), dim3(kAttnThreads),
-                              Cfg::kSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], prm, sp);
-    else
-        e = launch_overlapped(region_attention_tc_kernel<D>, dim3(grid), dim3(kAttnThreads),
-                              Cfg::kSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
-    return e == cudaSuccess ? REGIONE_OK : REGIONE_CUDA_ERROR;
+    *fitting = clusters[dev];
+    return REGIONE_OK;
 }
 
-template <int D>
-static int launch_tc(const CUtensorMap* maps, const AttnParams& prm, const StoreParams* sp, int grid,
-                     cudaStream_t st) {
-    const StoreParams none = {};
-    const int rc = sp != nullptr ? launch_main<D, true>(maps, prm, *sp, grid, st)
-                                 : launch_main<D, false>(maps, prm, none, grid, st);
+// How many CTAs share an item through a cluster, 0: shares of the cost axis with a merge kernel behind them.
+// Few items (at most one cluster of two per pair of SMs) are better off in clusters: the shares of the cost axis are
+// balanced to a step, but every cut item's rows go through the workspace (7300 cycles per pair of tiles, all
+// CTAs at once) and a second kernel (8 us behind the attention's last block), about kTickMerge ticks in all against
+// kTickCluster for a merge through distributed shared memory.  Both sides' ticks from the capacities:
+constexpr int kTickMerge = 125, kTickCluster = 45;
+static int choose_cluster(const int* fitting, const AttnParams& p, int nt) {
+    const long long items = (long long)p.B * p.H * p.P_cap;
+    const bool lone_last = ((p.Nq_cap + kBM - 1) / kBM) % 2 == 1;
+    const long long w_max = p.P_cap == 1 && lone_last ? kTickSingle : kTickPair;
+    const long long ticks = (long long)p.B * p.H * ((p.P_cap - 1) * (kTickStart + (long long)kTickPair * nt) + kTickStart +
+                                                    (long long)(lone_last ? kTickSingle : kTickPair) * nt);
+    // (a share is at least as long as the slots of an item allow, and pays for a start of its own where it begins
+    // inside an item)
+    long long best = std::max((ticks + sm_count() - 1) / sm_count(), w_max * (nt - 1) / (p.max_slots - 1)) + kTickStart +
+                     kTickMerge;
+    int n_best = 0;
+    for (int n = 2; n <= kMaxCluster && n <= nt; ++n) {
+        if (items > fitting[n]) continue;
+        const long long cost = kTickStart + w_max * ((nt + n - 1) / n) + kTickCluster;
+        if (cost < best) { best = cost; n_best = n; }
+    }
+    return n_best;
+}
+
+template <int D, bool STORE>
+static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams& sp, int grid, int nt_cap, cudaStream_t st) {
+    const int* fitting = nullptr;
+    const int rc = prepare_kernel<D, STORE>(&fitting);
     if (rc != REGIONE_OK) return rc;
+    prm.cluster = choose_cluster(fitting, prm, nt_cap);
+    if (prm.cluster > 0) grid = prm.B * prm.H * prm.P_cap * prm.cluster;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kAttnThreads);
+    cfg.dynamicSmemBytes = AttnCfg<D>::kSmemBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see grid_dependency_wait
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = prm.cluster > 0 ? prm.cluster : 1;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = prm.cluster > 0 ? 2 : 1;
+    cudaError_t e;
+    auto launch = [&](auto kernel) {
+        if constexpr (STORE) return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm, sp);
+        else return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
+    };
+    e = prm.cluster > 0 ? launch(main_kernel<D, STORE, true>()) : launch(main_kernel<D, STORE, false>());
+    if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
     // the merge kernel may become resident while the attention kernel drains (it waits for that
     // kernel's completion before it reads a slot)
-    if (grid < 2) return launch_status(cudaGetLastError());     // a single share cuts nothing
+    if (grid < 2 || prm.cluster > 0) return launch_status(cudaGetLastError());     // nothing is cut
     const dim3 cgrid((unsigned)(grid - 1), (2 * kBM) / 8, 1);
-    cudaError_t e;
     if (prm.max_slots <= 2)
         e = launch_overlapped(region_attention_combine_kernel<D, 2>, cgrid, dim3(256), 0, st, prm);
     else if (prm.max_slots <= 3)
@@ -1484,8 +1704,13 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
     const size_t off_ml = (rows * D * sizeof(float) + 255) & ~(size_t)255;
     prm.part_ml = reinterpret_cast<float2*>(ws + off_ml);
     prm.cut = reinterpret_cast<CutItem*>(ws + off_ml + ((rows * sizeof(float2) + 255) & ~(size_t)255));
-    const StoreParams* spp = store != nullptr ? &sp : nullptr;
-    return D == 64 ? launch_tc<64>(maps, prm, spp, lp.grid, st) : launch_tc<128>(maps, prm, spp, lp.grid, st);
+    prm.cluster = 0;
+    const int nt_cap = std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN);
+    if (store != nullptr)
+        return D == 64 ? launch_tc<64, true>(maps, prm, sp, lp.grid, nt_cap, st)
+                       : launch_tc<128, true>(maps, prm, sp, lp.grid, nt_cap, st);
+    return D == 64 ? launch_tc<64, false>(maps, prm, sp, lp.grid, nt_cap, st)
+                   : launch_tc<128, false>(maps, prm, sp, lp.grid, nt_cap, st);
 }
 
 // ---- variant with library-owned scratch -----------------------------------------------------

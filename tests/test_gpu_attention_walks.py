@@ -19,11 +19,12 @@ pytestmark = pytest.mark.gpu
     (256, 0, 128 * 3),     # whole tiles only
 ])
 @pytest.mark.parametrize("rows", ["all", "one"])
-def test_logits_that_outgrow_the_first_key_tile(D, n_q, n_f, n_c, rows):
+@pytest.mark.parametrize("H", [3, 40])     # items shared by clusters; items cut between the shares of the cost axis
+def test_logits_that_outgrow_the_first_key_tile(D, n_q, n_f, n_c, rows, H):
     """Later keys raise the logits of every row, or of one row, by far more than the exponent range of the
     probabilities: the softmax is then almost one-hot on those keys and the tolerance is that of the plain case."""
     rng = np.random.default_rng(D + n_q)
-    B, H = 2, 3
+    B = 2
     q = _rand_bf16(rng, (B, n_q, H, D), 0.3)
     kf, vf = _rand_bf16(rng, (B, max(n_f, 1), H, D), 0.3), _rand_bf16(rng, (B, max(n_f, 1), H, D))
     kc, vc = _rand_bf16(rng, (B, n_c, H, D), 0.3), _rand_bf16(rng, (B, n_c, H, D))
@@ -42,9 +43,10 @@ def test_logits_that_outgrow_the_first_key_tile(D, n_q, n_f, n_c, rows):
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("n_q", [100, 256, 700])
 @pytest.mark.parametrize("n_f,n_c", [(60, 1000 + 24), (64, 128 * 7 + 1), (65, 128 * 7 + 64), (1, 128 * 4 + 56)])
-def test_key_tiles_with_a_dead_second_half(D, n_q, n_f, n_c):
+@pytest.mark.parametrize("H", [12, 38])
+def test_key_tiles_with_a_dead_second_half(D, n_q, n_f, n_c, H):
     rng = np.random.default_rng(n_q + n_f + n_c + D)
-    B, H = 2, 12
+    B = 2
     q = _rand_bf16(rng, (B, n_q, H, D))
     kf, vf = _rand_bf16(rng, (B, n_f + 5, H, D)), _rand_bf16(rng, (B, n_f + 5, H, D))
     kc, vc = _rand_bf16(rng, (B, n_c + 9, H, D)), _rand_bf16(rng, (B, n_c + 9, H, D))
@@ -83,3 +85,21 @@ def test_cache_refresh_row_lengths_and_outgrown_rows(D, H):
     from gpu_util import assert_close
     for b in range(B):
         assert_close(host_f64(out)[b, :n_rows[b]], want[b, :n_rows[b]], f"attention, request {b}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("counts", [
+    [(1, 1, 0)],                                        # one key tile: nothing to share
+    [(200, 100, 128 * 2 + 5), (0, 3, 40), (130, 0, 128)],   # fewer key tiles than ranks, an empty request
+    [(256, 256, 3000)],                                 # more key tiles than ranks
+    [(40, 0, 0), (40, 10, 1000)],                       # a request without keys beside one with them
+])
+def test_items_shared_by_clusters(D, counts):
+    """Capacities of few items: ranks without key tiles, rows of one and of two query tiles, dead items."""
+    rng = np.random.default_rng(D + len(counts))
+    B, H = len(counts), 4
+    cap_q, cap_f, cap_c = (max(c[i] for c in counts) + 7 for i in range(3))
+    q = _rand_bf16(rng, (B, cap_q, H, D))
+    kf, vf = _rand_bf16(rng, (B, cap_f, H, D)), _rand_bf16(rng, (B, cap_f, H, D))
+    kc, vc = _rand_bf16(rng, (B, cap_c, H, D)), _rand_bf16(rng, (B, cap_c, H, D))
+    check(q, kf, vf, kc, vc, [c[0] for c in counts], [c[1] for c in counts], [c[2] for c in counts], what=f"clusters {counts}")
