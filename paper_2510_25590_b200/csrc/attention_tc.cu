@@ -832,7 +832,9 @@ struct CachePump {
     int x, b, i, run, live_rows;        // cursor of the loads: tensor, request, item, items of the run, source rows
     int left;                           // items not yet loaded
     int head, tail;                     // units loaded / stored through the present slots
-    int row, before;                    // list entry of this lane's next item, and the one ahead of it
+    int win;                            // first item of the window of list entries held, one per lane:
+    int row, before;                    // the entry of item win + lane and the one ahead of it,
+    int row_next, before_next;          // the same for the window behind it (fetched long before it is needed)
 
     __device__ __forceinline__ int kept(int req, bool report) const {
         const int nk = sp->n_keep[req];
@@ -850,15 +852,20 @@ struct CachePump {
             if (++b == p->B) { b = 0; ++x; }
         }
     }
-    // list entries of the next unit's items, fetched one unit ahead of their use
-    __device__ __forceinline__ void fetch(int lane) {
-        row = before = -1;
-        if (lane < min(per_unit, min(run - i, left))) {
+    // list entries of the 32 items from `first` on (those of the present run and share)
+    __device__ __forceinline__ void fetch(int first, int lane, int& r, int& ahead) const {
+        r = ahead = -1;
+        if (first + lane < min(run, i + left)) {
             const int32_t* keep = sp->keep_rows + (size_t)b * sp->store_cap;
-            const int j = (i + lane) / per_row;
-            row = keep[j];
-            if (j > 0) before = keep[j - 1];
+            const int j = (first + lane) / per_row;
+            r = keep[j];
+            if (j > 0) ahead = keep[j - 1];
         }
+    }
+    __device__ __forceinline__ void open_window(int lane) {
+        win = i;
+        fetch(win, lane, row, before);
+        fetch(win + 32, lane, row_next, before_next);
     }
     // slots of one item each for long rows, of `unit` bytes for short ones, in `bytes` of shared memory
     __device__ __forceinline__ void use_slots(uint32_t at, int bytes, int unit, int lane) {
@@ -870,7 +877,6 @@ struct CachePump {
         if (lane < n_slots) ptx::mbar_init(ptx::smem_addr(&ctrl->copy_full[lane]), 1);
         ptx::fence_barrier_init();
         __syncwarp();
-        if (left > 0) fetch(lane);
     }
     __device__ __forceinline__ void begin(const AttnParams& prm, const StoreParams& s, AttnCtrl* c, int d, int longest, int lane) {
         sp = &s; n_rows = prm.n_fresh; ctrl = c; p = &prm;
@@ -886,7 +892,10 @@ struct CachePump {
         left = (int)max(0LL, min(per, total - first));
         x = b = 0;
         i = (int)first;
-        if (left > 0) open_run();
+        if (left > 0) {
+            open_run();
+            open_window(lane);
+        }
     }
     __device__ __forceinline__ bool store_oldest(int lane) {
         const int slot = tail % n_slots;
@@ -906,8 +915,10 @@ struct CachePump {
         // (one slot of slack: all but the latest store have been read out of shared memory)
         ptx::bulk_wait_read<1>();
         __syncwarp();
-        const int n = min(per_unit, min(run - i, left));
-        const bool ok = row >= 0 && row < live_rows && row > before;
+        const int n = min(min(per_unit, win + 32 - i), min(run - i, left));
+        const int at = min(i - win + lane, 31);
+        const int my_row = __shfl_sync(0xffffffffu, row, at), ahead = __shfl_sync(0xffffffffu, before, at);
+        const bool ok = my_row >= 0 && my_row < live_rows && my_row > ahead;
         if (lane < n && !ok) record_status(p->dev_status, REGIONE_DEV_BOUNDS);
         const uint32_t valid = __ballot_sync(0xffffffffu, lane < n && ok);
         const int slot = head % n_slots;
@@ -924,13 +935,20 @@ struct CachePump {
         __syncwarp();
         if (bytes > 0)
             ptx::bulk_load(slots + slot * slot_bytes + lane * item_bytes,
-                           sp->src[x] + ((size_t)b * sp->src_cap + row) * row_bytes + off, bytes, bar);
+                           sp->src[x] + ((size_t)b * sp->src_cap + my_row) * row_bytes + off, bytes, bar);
         ++head;
         left -= n;
         i += n;
         if (left > 0) {
-            if (i >= run) open_run();
-            fetch(lane);
+            if (i >= run) {
+                open_run();
+                open_window(lane);
+            } else if (i == win + 32) {
+                win = i;
+                row = row_next;
+                before = before_next;
+                fetch(win + 32, lane, row_next, before_next);
+            }
         }
     }
     // Moves the CTA's rows: through a corner of shared memory beside the walks, through the idle tiles once they are
@@ -1627,7 +1645,8 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
     const int rc = prepare_kernel<D, STORE>(&fitting);
     if (rc != REGIONE_OK) return rc;
     prm.cluster = choose_cluster(fitting, prm, nt_cap);
-    if (prm.cluster > 0) grid = prm.B * prm.H * prm.P_cap * prm.cluster;
+    // (a refreshing launch takes every cluster that fits: those without an item copy rows of the cache)
+    if (prm.cluster > 0) grid = (STORE ? fitting[prm.cluster] : prm.B * prm.H * prm.P_cap) * prm.cluster;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kAttnThreads);
