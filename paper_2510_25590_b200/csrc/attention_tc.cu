@@ -85,7 +85,7 @@ constexpr int kBM = 128;                 // query rows per tile
 constexpr int kBN = 128;                 // key rows per shared-memory tile
 constexpr int kBH = 64;                  // key rows per chunk (half a tile): the logits one thread holds
 constexpr float kOutgrownSum = 1.152921504606846976e18f;   // 2^60: chunk sum at which a reference maximum is renewed
-constexpr int kCopySlots = 8;             // cache refresh: at most so many units of rows in flight
+constexpr int kCopySlots = 2;             // cache refresh: batches of rows under way at once, at most
 constexpr int kHalfBytes = 128 * 64 * 2; // one 128-row x 64-column bf16 box (128-byte rows)
 constexpr long long kTimeoutCycles = 4000000000LL;   // default bound of every wait (about 2 s)
 
@@ -819,8 +819,10 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& p, const SegInfo
 // ran them from the producer warp between its loads: every wait for a slot delayed a key tile, and 194 MB of copies
 // cost the attention of 819 queries as much as a store kernel ahead of it.)  The launch's rows (K of every request,
 // then V) are cut into equal contiguous shares, one per CTA, whatever attention work the CTA has.  An item is one
-// row, or a slot's length of it where a row is longer than that; a unit is up to `per_unit` consecutive items of one
-// request, lane i moving item i.
+// row, or a slot's length of it where a row is longer than that; a batch is up to `per_unit` consecutive items of one
+// request, lane i moving item i.  Beside the walks one batch at a time fills the corner of shared memory that is left
+// (5 rows of 24 x 128): the warp gets few issue slots there, and several slots of a row each with the same number of
+// rows in flight took 2660 cycles a row.  Over the idle tiles two batches alternate.
 struct CachePump {
     const StoreParams* sp;
     const int32_t* n_rows;
@@ -842,6 +844,7 @@ struct CachePump {
         if (report && blockIdx.x == 0) record_status(p->dev_status, REGIONE_DEV_BOUNDS);
         return nk < 0 ? 0 : sp->store_cap;
     }
+    __device__ __forceinline__ int row_of(int item) const { return per_row > 1 ? item / per_row : item; }
     // from an item index behind the runs x, b to the run that holds it (a request without rows stores nothing)
     __device__ __forceinline__ void open_run() {
         for (;;) {
@@ -857,7 +860,7 @@ struct CachePump {
         r = ahead = -1;
         if (first + lane < min(run, i + left)) {
             const int32_t* keep = sp->keep_rows + (size_t)b * sp->store_cap;
-            const int j = (first + lane) / per_row;
+            const int j = row_of(first + lane);
             r = keep[j];
             if (j > 0) ahead = keep[j - 1];
         }
@@ -867,11 +870,11 @@ struct CachePump {
         fetch(win, lane, row, before);
         fetch(win + 32, lane, row_next, before_next);
     }
-    // slots of one item each for long rows, of `unit` bytes for short ones, in `bytes` of shared memory
-    __device__ __forceinline__ void use_slots(uint32_t at, int bytes, int unit, int lane) {
+    // `n` slots in `bytes` of shared memory
+    __device__ __forceinline__ void use_slots(uint32_t at, int bytes, int n, int lane) {
         slots = at;
-        slot_bytes = max(unit, (item_bytes + 127) & ~127);
-        n_slots = min(kCopySlots, bytes / slot_bytes);
+        n_slots = n;
+        slot_bytes = (bytes / n) & ~127;
         per_unit = min(32, slot_bytes / item_bytes);
         head = tail = 0;
         if (lane < n_slots) ptx::mbar_init(ptx::smem_addr(&ctrl->copy_full[lane]), 1);
@@ -898,12 +901,12 @@ struct CachePump {
         }
     }
     __device__ __forceinline__ bool store_oldest(int lane) {
-        const int slot = tail % n_slots;
-        const bool landed = wait_bar(ptx::smem_addr(&ctrl->copy_full[slot]), (tail / n_slots) & 1, &ctrl->abort_flag,
+        const int slot = n_slots > 1 ? tail & 1 : 0;
+        const bool landed = wait_bar(ptx::smem_addr(&ctrl->copy_full[slot]), (n_slots > 1 ? tail >> 1 : tail) & 1, &ctrl->abort_flag,
                                      p->dev_status, p->timeout_cycles);
         if (!__all_sync(0xffffffffu, landed)) return false;
         if ((ctrl->copy_valid[slot] >> lane) & 1u) {
-            const int at = ctrl->copy_item[slot] + lane, j = at / per_row, off = (at - j * per_row) * item_bytes;
+            const int at = ctrl->copy_item[slot] + lane, j = row_of(at), off = (at - j * per_row) * item_bytes;
             ptx::bulk_store(ctrl->copy_dst[slot] + (size_t)j * row_bytes + off, slots + slot * slot_bytes + lane * item_bytes,
                             min(item_bytes, row_bytes - off));
         }
@@ -912,8 +915,8 @@ struct CachePump {
         return true;
     }
     __device__ __forceinline__ void load_next(int lane) {
-        // (one slot of slack: all but the latest store have been read out of shared memory)
-        ptx::bulk_wait_read<1>();
+        // (the batch that this slot held last has been read out of shared memory)
+        ptx::bulk_wait_read<0>();
         __syncwarp();
         const int n = min(min(per_unit, win + 32 - i), min(run - i, left));
         const int at = min(i - win + lane, 31);
@@ -921,9 +924,9 @@ struct CachePump {
         const bool ok = my_row >= 0 && my_row < live_rows && my_row > ahead;
         if (lane < n && !ok) record_status(p->dev_status, REGIONE_DEV_BOUNDS);
         const uint32_t valid = __ballot_sync(0xffffffffu, lane < n && ok);
-        const int slot = head % n_slots;
+        const int slot = n_slots > 1 ? head & 1 : 0;
         const uint32_t bar = ptx::smem_addr(&ctrl->copy_full[slot]);
-        const int off = ((i + lane) % per_row) * item_bytes;
+        const int off = (i + lane - row_of(i + lane) * per_row) * item_bytes;
         const int bytes = (valid >> lane) & 1u ? min(item_bytes, row_bytes - off) : 0;
         const int unit_bytes = __reduce_add_sync(0xffffffffu, bytes);
         if (lane == 0) {
@@ -957,7 +960,7 @@ struct CachePump {
     __device__ __forceinline__ bool run_all(uint32_t smem, int lane) {
         using Cfg = AttnCfg<D>;
         bool wide = false;
-        if (left > 0) use_slots(smem + Cfg::kCopyAt, Cfg::kCopyBytes, Cfg::kCopyBytes / kCopySlots, lane);
+        if (left > 0) use_slots(smem + Cfg::kCopyAt, Cfg::kCopyBytes, 1, lane);
         while (left > 0) {
             if (!wide && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&ctrl->walks_done) != 0)) {
                 while (tail < head)
@@ -968,10 +971,10 @@ struct CachePump {
                 __syncwarp();
                 if (lane < n_slots) ptx::mbar_inval(ptx::smem_addr(&ctrl->copy_full[lane]));
                 __syncwarp();
-                use_slots(smem, Cfg::kTailBytes, Cfg::kTailBytes / kCopySlots, lane);
+                use_slots(smem, Cfg::kTailBytes, kCopySlots, lane);
                 wide = true;
             }
-            if (head - tail < n_slots - 1) load_next(lane);
+            if (head - tail < n_slots) load_next(lane);
             else if (!store_oldest(lane)) return false;
         }
         while (tail < head)
