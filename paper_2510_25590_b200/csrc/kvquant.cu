@@ -12,6 +12,9 @@
 //   elements of that row and head); written with frexp(amax) = m * 2^e, m in [0.5, 1):
 //   k = e - 9 + (m > 0.875); k = 0 for amax = 0; k is kept >= -100.
 //
+// Measured, 70248 rows of 24 x 128 (1.3 GB): store 222 us, 5890 GB/s (224 us with cached loads and stores; at one
+// request of 7885 rows 29.6 -> 28.5 us); four rows per block with the next row's loads ahead took 300 us, the
+// registers cost more in blocks per SM than the chain of count, index and data costs a block.
 // Both kernels are HBM-bound row passes: one block per kept row covers K and V of that row, a lane
 // owns 8 consecutive elements (16 bytes of bf16, 8 bytes of codes), the D / 8 lanes of one head sit
 // side by side in a warp and find the head's maximum by shuffles.
@@ -58,7 +61,7 @@ __device__ __forceinline__ int live_rows(const int32_t* n_keep, int b, int Nc_ca
 }
 
 template <int D>
-__global__ void __launch_bounds__(kQuantThreads)
+__global__ void __launch_bounds__(kQuantThreads, 8)
 rikv_store_e4m3_kernel(const uint16_t* __restrict__ k_full, const uint16_t* __restrict__ v_full,
                        const int32_t* __restrict__ keep_rows, const int32_t* __restrict__ n_keep,
                        int N_full, int Nc_cap, int H, uint8_t* __restrict__ k_q, uint8_t* __restrict__ v_q,
@@ -84,8 +87,8 @@ rikv_store_e4m3_kernel(const uint16_t* __restrict__ k_full, const uint16_t* __re
             const int c = c0 + u * kQuantThreads + (threadIdx.x & 31);
             w[u] = make_uint4(0u, 0u, 0u, 0u);
             if (c < total)
-                w[u] = *reinterpret_cast<const uint4*>((c >= per_tensor ? v_full : k_full) + src_off +
-                                                       (size_t)(c >= per_tensor ? c - per_tensor : c) * 8);
+                w[u] = ld_stream128((c >= per_tensor ? v_full : k_full) + src_off +
+                                    (size_t)(c >= per_tensor ? c - per_tensor : c) * 8);
         }
 #pragma unroll
         for (int u = 0; u < kQuantUnroll; ++u) {
@@ -107,7 +110,7 @@ rikv_store_e4m3_kernel(const uint16_t* __restrict__ k_full, const uint16_t* __re
             uint2 q;
             q.x = pack_e4m3x2(x[0] * inv, x[1] * inv) | (pack_e4m3x2(x[2] * inv, x[3] * inv) << 16);
             q.y = pack_e4m3x2(x[4] * inv, x[5] * inv) | (pack_e4m3x2(x[6] * inv, x[7] * inv) << 16);
-            *reinterpret_cast<uint2*>((is_v ? v_q : k_q) + dst_row * H * D + (size_t)piece * 8) = q;
+            __stcs(reinterpret_cast<uint2*>((is_v ? v_q : k_q) + dst_row * H * D + (size_t)piece * 8), q);
             if (piece % kLanesPerHead == 0)
                 (is_v ? v_scale : k_scale)[dst_row * H + piece / kLanesPerHead] =
                     __uint_as_float((uint32_t)(127 + k) << 23);
