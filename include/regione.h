@@ -335,8 +335,9 @@ int regione_region_attention_scatter(const regione_bf16* q,
  *   regione_region_step_workspace(plan) bytes; dev_status i32 [1] or NULL.
  * x_t, v, ref bf16 [B, N, C]; q_full, k_full, v_full bf16 [B, n_full, H, D]; t, scale, dt, dt_unedited host
  * arrays [B] (NaN: the request sits that operation out, as in the single calls).
- * store_cache != 0: the attention reads K and V where they are (fresh and cached rows together are all of
- * them), the cache receives its rows in the same launch, k_fresh and v_fresh are not written.
+ * store_cache != 0: with enough queries beside the keys the attention reads K and V where they are (fresh and
+ * cached rows together are all of them), the cache receives its rows in the same launch, and k_fresh and v_fresh
+ * are not written; with fewer the rows are copied ahead of it.  Both parts have to be called with the same value.
  * parts: REGIONE_STEP_MOVES (everything up to the attention) | REGIONE_STEP_ATTENTION.
  */
 typedef struct {

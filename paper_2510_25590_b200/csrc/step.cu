@@ -19,6 +19,15 @@
 
 namespace regione {
 
+// Whether the attention of a step that refreshes the cache reads K and V where they are and takes the rows of the
+// cache along, or reads [cache | fresh] as a step that keeps the cache does, with the rows copied ahead of it.  The
+// copies need the attention's time to hide behind, which grows with the queries; and only with enough queries beside
+// the keys does the other order of the keys stay a matter of rounding in the scattered buffer (see choose_cluster).
+// Measured, rows ahead -> along, us: 8704 rows of 24 heads, 128 queries 76 -> 82, 256 84 -> 84, 512 104 -> 90, 1536
+// 169 -> 145; four requests of 18944, 512 queries 700 -> 622, 1408 1372 -> 1178.  So the line is the rounding's: below
+// a sixteenth single elements of the scattered buffer moved by up to 0.1 of its rms, from there on by 0.05.
+static bool takes_rows_along(int q_cap, int n_full) { return 16LL * (q_cap - 64) >= n_full; }
+
 struct LatentMove {
     const uint4 *x, *v;             // [B, N, C] current latent and velocity
     const int32_t* slot;            // [B, N] place of an edited token in X^E, negative: unedited
@@ -67,14 +76,17 @@ __device__ __forceinline__ void move_latents(const LatentMove& a, int b, unsigne
     if (merge) a.x_out[at] = y;
 }
 
-// blockIdx.x: blocks of the latent update, then of each gathered tensor; blockIdx.y = request of this launch.
+// blockIdx.x: blocks of the latent update, then of each gathered tensor, then of K and V of the rows that go to the
+// cache (where the attention does not take them along); blockIdx.y = request of this launch.
 // Bound by launch and one or two memory round trips at the sizes of the paper's editors (4 to 5 us); the row gathers
 // run at the bandwidth of HBM where they are large, and the latent blocks, which come first, hide behind them.
 __global__ void __launch_bounds__(kCopyThreads)
 region_step_move_kernel(const LatentMove lat, const __grid_constant__ PerRequestF neg_dt_scale,
                         const __grid_constant__ PerRequestF neg_dt_u, int b0, int lat_blocks,
-                        const __grid_constant__ RowCopyPairs rows, int row_blocks, const int32_t* __restrict__ query_rows,
-                        const int32_t* __restrict__ n_q, int n_full, int q_cap, int row_cpr, int32_t* dev_status) {
+                        const __grid_constant__ RowCopyPairs rows, int n_pairs, int row_blocks,
+                        const int32_t* __restrict__ query_rows, const int32_t* __restrict__ n_q, int n_full, int q_cap,
+                        int row_cpr, const __grid_constant__ RowCopyPairs kept, int kept_blocks,
+                        const int32_t* __restrict__ cache_rows, const int32_t* __restrict__ n_cache, int32_t* dev_status) {
     grid_dependency_wait();
     grid_launch_dependents();
     const int b = b0 + blockIdx.y;
@@ -83,9 +95,15 @@ region_step_move_kernel(const LatentMove lat, const __grid_constant__ PerRequest
         move_latents(lat, b, blk, neg_dt_scale.v[blockIdx.y], neg_dt_u.v[blockIdx.y], dev_status);
         return;
     }
-    const int pair = (blk - lat_blocks) / row_blocks;
-    copy_rows<true>(rows.p[pair], b, blk - lat_blocks - pair * row_blocks, query_rows, n_q, n_full, q_cap, q_cap, row_cpr,
-                    dev_status);
+    int at = blk - lat_blocks;
+    if (at < n_pairs * row_blocks) {
+        const int pair = at / row_blocks;
+        copy_rows<true>(rows.p[pair], b, at - pair * row_blocks, query_rows, n_q, n_full, q_cap, q_cap, row_cpr, dev_status);
+        return;
+    }
+    at -= n_pairs * row_blocks;
+    const int pair = at / kept_blocks;
+    copy_rows<true>(kept.p[pair], b, at - pair * kept_blocks, cache_rows, n_cache, n_full, n_full, n_full, row_cpr, dev_status);
 }
 
 }  // namespace regione
@@ -127,6 +145,7 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
         return REGIONE_UNSUPPORTED;
     if (B == 0) return REGIONE_OK;
     cudaStream_t st = (cudaStream_t)stream;
+    const bool along = store_cache && q_cap > 0 && takes_rows_along(q_cap, n_full);
 
     if (parts & REGIONE_STEP_MOVES) {
         const int rc = regione_partition_rows(x_t, v, ref, B, N, C, t, p->metric, p->threshold, p->mask, p->edit_idx,
@@ -138,12 +157,17 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
         lm.x = (const uint4*)x_t; lm.v = (const uint4*)v; lm.slot = p->slot; lm.n_edit = p->n_edit;
         lm.x_e = (uint4*)p->x_e; lm.v_e = (uint4*)p->v_e; lm.v_avd = (uint4*)p->v_avd; lm.x_out = (uint4*)p->x_out;
         lm.N = N; lm.Ne_cap = p->ne_cap; lm.cpr = C / 8;
-        // a step that refreshes the cache attends over K and V themselves: only the queries are gathered
+        // rows taken along: the attention reads K and V themselves, only the queries are gathered
         RowCopyPairs rows = {};
         rows.p[0] = RowCopyPair{(const uint4*)q_full, (uint4*)p->q_e};
         rows.p[1] = RowCopyPair{(const uint4*)k_full, (uint4*)p->k_fresh};
         rows.p[2] = RowCopyPair{(const uint4*)v_full, (uint4*)p->v_fresh};
-        const int n_pairs = q_cap == 0 ? 0 : store_cache ? 1 : 3;
+        const int n_pairs = q_cap == 0 ? 0 : along ? 1 : 3;
+        RowCopyPairs kept = {};
+        kept.p[0] = RowCopyPair{(const uint4*)k_full, (uint4*)p->k_cache};
+        kept.p[1] = RowCopyPair{(const uint4*)v_full, (uint4*)p->v_cache};
+        const int n_kept = store_cache && !along ? 2 : 0;
+        const int kept_blocks = (int)((n_full * row_cpr + per_block - 1) / per_block);
         const int lat_blocks = (int)((lat_chunks + kCopyThreads - 1) / kCopyThreads);
         const int row_blocks = (int)((q_cap * row_cpr + per_block - 1) / per_block);
         cudaError_t e = cudaSuccess;
@@ -154,22 +178,21 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
                 a.v[i] = -(dt[b0 + i] * scale[b0 + i]);      // x - (dt * scale) * v, the product formed in fp32 first
                 u.v[i] = -dt_unedited[b0 + i];
             }
-            e = launch_overlapped(region_step_move_kernel, dim3(lat_blocks + n_pairs * row_blocks, nb), dim3(kCopyThreads), 0,
-                                  st, lm, a, u, b0, lat_blocks, rows, row_blocks > 0 ? row_blocks : 1, p->query_rows, p->n_q,
-                                  n_full, q_cap, (int)row_cpr, p->dev_status);
+            e = launch_overlapped(region_step_move_kernel, dim3(lat_blocks + n_pairs * row_blocks + n_kept * kept_blocks, nb),
+                                  dim3(kCopyThreads), 0,
+                                  st, lm, a, u, b0, lat_blocks, rows, n_pairs, row_blocks > 0 ? row_blocks : 1, p->query_rows,
+                                  p->n_q, n_full, q_cap, (int)row_cpr, kept, kept_blocks, p->cache_rows, p->n_cache,
+                                  p->dev_status);
         }
         if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
     }
     if (parts & REGIONE_STEP_ATTENTION) {
-        if (q_cap == 0)                                       // no query can exist: the cache alone is refreshed
-            return store_cache ? regione_rikv_store(k_full, v_full, p->cache_rows, p->n_cache, B, n_full, n_full, H, D,
-                                                    p->k_cache, p->v_cache, p->dev_status, stream)
-                               : REGIONE_OK;
+        if (q_cap == 0) return REGIONE_OK;                    // no query can exist
         const size_t need = regione_region_step_workspace(p);
         if (need > 0 && (!p->workspace || (reinterpret_cast<uintptr_t>(p->workspace) & 255u))) return REGIONE_INVALID_ARG;
         if (p->workspace_bytes < need) return REGIONE_WORKSPACE_TOO_SMALL;
         const float sm = 1.0f / sqrtf((float)D);
-        if (store_cache) {
+        if (along) {
             CacheStore cs;
             cs.keep_rows = p->cache_rows; cs.n_keep = p->n_cache; cs.cap = n_full;
             cs.k_cache = p->k_cache; cs.v_cache = p->v_cache;
