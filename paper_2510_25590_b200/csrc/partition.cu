@@ -280,8 +280,13 @@ partition_kernel(const uint16_t* __restrict__ x_t, const uint16_t* __restrict__ 
     const int total = block_popc_scan(bits, prefix, nwords, warp_tot);
     if (threadIdx.x == 0) cta_count = total;
     cluster.sync();
-    int edit_base = 0;
-    for (int r = 0; r < rank; ++r) edit_base += *cluster.map_shared_rank(&cta_count, r);
+    // Lane r of every warp reads rank r's count, so all counts come in one round trip through distributed
+    // shared memory (read one after the other by each thread they were a third of a short request's launch).
+    static_assert(kPartMaxCluster <= 32, "one lane per rank");
+    const int theirs = lane < csize ? *cluster.map_shared_rank(&cta_count, lane) : 0;
+    const int edit_base = __reduce_add_sync(0xffffffffu, lane < rank ? theirs : 0);
+    const int ne_all = __reduce_add_sync(0xffffffffu, theirs);
+    cluster.barrier_arrive();                    // the counts are read: peers may leave once all have said so
     const int keep_base = start - edit_base;     // every token before `start` exists (start <= N)
 
     // ---- phase 3: coalesced per-token writes --------------------------------------------
@@ -298,8 +303,6 @@ partition_kernel(const uint16_t* __restrict__ x_t, const uint16_t* __restrict__ 
     if (lists) {
         // rows that do not depend on the mask: the text rows and the reference rows, spread over
         // the cluster's threads; the request's totals come from every rank's count
-        int ne_all = 0;
-        for (int r = 0; r < csize; ++r) ne_all += *cluster.map_shared_rank(&cta_count, r);
         const int nu_all = N - ne_all;
         const int stride = csize * blockDim.x;
         for (int i = rank * blockDim.x + threadIdx.x; i < rl.n_text; i += stride) {
@@ -317,7 +320,7 @@ partition_kernel(const uint16_t* __restrict__ x_t, const uint16_t* __restrict__ 
             rl.n_cache[b] = min(nc, rl.c_cap);
         }
     }
-    cluster.sync();                              // peers may still be reading cta_count
+    cluster.barrier_wait();                      // peers may still be reading cta_count
 }
 
 // ---- morphological opening + closing, then compaction (one CTA per request) -------------
@@ -433,10 +436,11 @@ static cudaError_t launch_partition(int csize, int B, int share, cudaStream_t st
                                     int32_t* n_edit, float* score, const RowLists& rl,
                                     int32_t* dev_status) {
     cudaLaunchConfig_t cfg = {};
-    // enough warps per CTA to keep the loads of a large share in flight (a cluster is at most 8
-    // CTAs, so a long request cannot get its memory parallelism from the grid); 512 threads let
-    // two CTAs share an SM, which measured faster than one CTA of 1024
-    const int threads = share >= 2048 ? 512 : 256;
+    // A warp per mask word while the words are few, so that a short request waits for its loads once; and
+    // enough warps to keep the loads of a large share in flight (a cluster is at most 8 CTAs, so a long
+    // request cannot get its memory parallelism from the grid).  512 threads let two CTAs share an SM,
+    // which measured faster than one CTA of 1024.
+    const int threads = share > 256 ? 512 : 256;
     cfg.gridDim = dim3(csize, B, 1);
     cfg.blockDim = dim3(threads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)(share >> 5) * 8;

@@ -9,7 +9,7 @@ namespace regione {
 // blockIdx.z picks the tensor pair.
 template <bool GATHER>
 __global__ void __launch_bounds__(kCopyThreads)
-row_copy_kernel(const RowCopyPairs pairs, const int32_t* __restrict__ idx,
+row_copy_kernel(const __grid_constant__ RowCopyPairs pairs, const int32_t* __restrict__ idx,
                 const int32_t* __restrict__ n, long long idx_rows, long long idx_stride,
                 long long cap, int cpr, int32_t* dev_status) {
     grid_dependency_wait();
