@@ -463,6 +463,15 @@ int regione_velocity_decay(const regione_bf16* v_in, const float* scale, const f
                            int B, int Ne_cap, int C, int32_t* dev_status, void* stream);
 
 /*
+ * n_steps (1 .. 128) of these updates with one velocity in one launch, x_e rounded to bf16 after each, as
+ * n_steps calls leave it: a recomputed step and the steps behind it that reuse its velocity.
+ * scale, dt : host f32 [n_steps, B]; a request whose first dt * scale is NaN sits the call out.
+ */
+int regione_velocity_decay_run(const regione_bf16* v_in, const float* scale, const float* dt, int n_steps,
+                               regione_bf16* x_e, regione_bf16* v_cache_out, const int32_t* n_edit,
+                               int B, int Ne_cap, int C, int32_t* dev_status, void* stream);
+
+/*
  * Merge of the two regions at the end of a run of region steps (Sec. 4, one-step
  * estimation equation applied to the unedited tokens; Algorithm 1, the one-step
  * line before the inner loop and the gather line after it):

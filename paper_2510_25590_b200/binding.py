@@ -65,6 +65,7 @@ SIGNATURES = {
     "regione_avd_step": (c_int, [POINTER(c_double), c_double, c_double, c_double, POINTER(c_int)]),
     "regione_gamma_fit": (c_int, [_P, c_int, c_int, c_int64, _P, _P, _P, _P]),
     "regione_velocity_decay": (c_int, [_P, _P, _P, _P, _P, _P, c_int, c_int, c_int, _P, _P]),
+    "regione_velocity_decay_run": (c_int, [_P, _P, _P, c_int, _P, _P, _P, c_int, c_int, c_int, _P, _P]),
     "regione_merge": (c_int, [_P, _P, _P, _P, _P, c_int, c_int, c_int, c_int, _P, _P, _P]),
     "regione_crosscheck_region_attention": (c_int, [_P] * 8 + [c_int] * 6 + [c_float, _P, _P, _P]),
     "regione_selftest_bounded_wait": (c_int, [c_longlong, _P, _P, _P]),

@@ -11,16 +11,18 @@ namespace regione {
 
 constexpr int kLatThreads = 256;
 
-// x_e <- x_e - dt * (scale * v_in); optionally v_cache_out <- v_in.  One thread = 8 channels.
+// x_e <- x_e - dt * (scale * v_in), n_steps times with the steps' own dt and scale and the rounding to bf16
+// between them; optionally v_cache_out <- v_in.  One thread = 8 channels.  A launch of 1 to 2 us bounds the small
+// latents of a sampler loop, so the steps that reuse a velocity ride with the step that computed it.
 __global__ void __launch_bounds__(kLatThreads)
-velocity_decay_kernel(const uint4* __restrict__ v_in, const PerRequestF neg_dt_scale_v, int b0,
+velocity_decay_kernel(const uint4* __restrict__ v_in, const __grid_constant__ PerRequestF neg_dt_scale, int n_steps, int b0,
                       uint4* __restrict__ x_e, uint4* __restrict__ v_cache_out,
                       const int32_t* __restrict__ n_edit, int Ne_cap, int cpr, int32_t* dev_status) {
     grid_dependency_wait();
     grid_launch_dependents();
     const int b = b0 + blockIdx.y;                       // requests b0 .. b0 + gridDim.y of the batch
-    const float neg_dt_scale = neg_dt_scale_v.v[blockIdx.y];
-    if (neg_dt_scale != neg_dt_scale) return;            // NaN: this request sits the call out
+    const float* a = neg_dt_scale.v + blockIdx.y * n_steps;
+    if (a[0] != a[0]) return;                            // NaN: this request sits the call out
     int ne = n_edit[b];
     if (ne < 0 || ne > Ne_cap) {
         if (threadIdx.x == 0 && blockIdx.x == 0) record_status(dev_status, REGIONE_DEV_BOUNDS);
@@ -31,8 +33,9 @@ velocity_decay_kernel(const uint4* __restrict__ v_in, const PerRequestF neg_dt_s
     if (e >= live) return;
     const size_t off = (size_t)b * Ne_cap * cpr + e;
     const uint4 v = ld_stream128(v_in + off);
-    const uint4 x = x_e[off];
-    x_e[off] = axpy8(x, v, neg_dt_scale);
+    uint4 x = x_e[off];
+    for (int i = 0; i < n_steps; ++i) x = axpy8(x, v, a[i]);
+    x_e[off] = x;
     if (v_cache_out != nullptr) v_cache_out[off] = v;
 }
 
@@ -98,21 +101,32 @@ extern "C" int regione_velocity_decay(const regione_bf16* v_in, const float* sca
                                       regione_bf16* x_e, regione_bf16* v_cache_out,
                                       const int32_t* n_edit, int B, int Ne_cap, int C,
                                       int32_t* dev_status, void* stream) {
+    return regione_velocity_decay_run(v_in, scale, dt, 1, x_e, v_cache_out, n_edit, B, Ne_cap, C, dev_status, stream);
+}
+
+extern "C" int regione_velocity_decay_run(const regione_bf16* v_in, const float* scale, const float* dt, int n_steps,
+                                          regione_bf16* x_e, regione_bf16* v_cache_out, const int32_t* n_edit, int B,
+                                          int Ne_cap, int C, int32_t* dev_status, void* stream) {
     if (!v_in || !x_e || !n_edit || !scale || !dt) return REGIONE_INVALID_ARG;
-    if (B < 0 || Ne_cap < 0 || C < 1) return REGIONE_INVALID_ARG;
+    if (B < 0 || Ne_cap < 0 || C < 1 || n_steps < 1 || n_steps > kReqChunk) return REGIONE_INVALID_ARG;
     if (!aligned16(v_in) || !aligned16(x_e) || !aligned16(v_cache_out)) return REGIONE_INVALID_ARG;
     if ((C & 7) != 0 || B > 65535) return REGIONE_UNSUPPORTED;
     const long long cpr = C / 8, total = (long long)Ne_cap * cpr;
     if (total + kLatThreads >= 0x7fffffffLL) return REGIONE_UNSUPPORTED;
     if (B == 0 || Ne_cap == 0) return REGIONE_OK;
     cudaError_t e = cudaSuccess;
-    for (int b0 = 0; b0 < B && e == cudaSuccess; b0 += kReqChunk) {
-        const int nb = B - b0 < kReqChunk ? B - b0 : kReqChunk;
+    const int chunk = kReqChunk / n_steps;   // a launch carries kReqChunk scalars
+    for (int b0 = 0; b0 < B && e == cudaSuccess; b0 += chunk) {
+        const int nb = B - b0 < chunk ? B - b0 : chunk;
         PerRequestF a;                       // x - (dt * scale) * v, the product formed in fp32 first
-        for (int i = 0; i < nb; ++i) a.v[i] = -(dt[b0 + i] * scale[b0 + i]);
+        for (int i = 0; i < nb; ++i)
+            for (int k = 0; k < n_steps; ++k) {
+                const size_t at = (size_t)k * B + b0 + i;
+                a.v[i * n_steps + k] = -(dt[at] * scale[at]);
+            }
         dim3 grid((unsigned)((total + kLatThreads - 1) / kLatThreads), nb);
         e = launch_overlapped(velocity_decay_kernel, grid, dim3(kLatThreads), 0, (cudaStream_t)stream,
-                              (const uint4*)v_in, a, b0, (uint4*)x_e, (uint4*)v_cache_out, n_edit,
+                              (const uint4*)v_in, a, n_steps, b0, (uint4*)x_e, (uint4*)v_cache_out, n_edit,
                               Ne_cap, (int)cpr, dev_status);
     }
     return launch_status(e);
