@@ -45,13 +45,14 @@
 // Scheduling: the kernel is persistent, one CTA per SM.  A "step" is one key tile of one
 // (request, head, query pair) item; all steps of the launch form one sequence, item after item,
 // laid out on a cost axis (a step of a pair with one live query tile costs half a step of a full
-// pair, and every item starts with a fixed cost for draining and refilling the pipeline), which is cut into equal contiguous shares, one per CTA (a stream-K decomposition:
-// the grid is always one balanced wave, whatever the number of items).  A CTA's share is a few
-// segments, each a run of key tiles of one item.  A segment that covers its item completely writes
-// the output rows directly; otherwise it writes its unnormalised output and (max, sum) pair to a
-// slot of the caller's workspace and a small second kernel merges the slots of such items (the
-// attention kernel leaves it a table of the items that its share boundaries cut).  The share
-// length is bounded below so that no item is spread over more slots than the workspace holds.
+// pair, and every item starts with a fixed cost for draining and refilling the pipeline), which is cut into
+// equal contiguous shares, one per CTA (a stream-K decomposition: the grid is always one balanced wave,
+// whatever the number of items).  A CTA's share is a few segments, each a run of key tiles of one item.  A segment
+// that covers its item completely writes the output rows directly; otherwise its unnormalised output and
+// (max, sum) pairs go to a slot of the caller's workspace, and either the item's first share merges the slots into its
+// own rows (kMergeHere) or a small second kernel does (kMergeKernel; the attention kernel leaves it a table of the items
+// that its share boundaries cut): see merges_here.  The share length is bounded below so that no item is spread over
+// more slots than the workspace holds.
 // Where the capacities allow only few items (choose_cluster), an item is shared by a cluster of 2 to 8 CTAs instead, an
 // equal run of its key tiles each; they leave their partial rows in shared memory, where the cluster's CTAs read
 // them (distributed shared memory) and write the output: no workspace, no second kernel, no plan to derive.  Measured,
@@ -69,6 +70,8 @@
 #include <type_traits>
 
 #include <algorithm>
+#include <atomic>
+#include <chrono>
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
@@ -169,6 +172,10 @@ struct alignas(16) CutItem {
     int valid, b, h, qp, n_slots, nq, pad0, pad1;
 };
 
+// Who puts the parts of an item together that several CTAs work on: a merge kernel behind this one, the item's
+// first share, or the CTAs of a cluster.  (Instantiations of their own: the code of one form costs the others 1 to 2 %.)
+enum MergeForm { kMergeKernel, kMergeHere, kMergeCluster };
+
 struct AttnParams {
     const int32_t* n_q;
     const int32_t* n_fresh;
@@ -181,10 +188,12 @@ struct AttnParams {
     const int32_t* out_rows;   // nullptr: query row i goes to out row i; else to row out_rows[b, i]
     int out_cap;         // rows per request of `out` (Nq_cap without out_rows)
     int32_t* dev_status;
-    float* part_o;       // [B, H, P_cap, max_slots, 256, D] unnormalised outputs
+    float* part_o;       // [B, H, P_cap, max_slots, 256, D] unnormalised outputs; kMergeHere: [..., D / 4, 256, 4]
     float2* part_ml;     // [B, H, P_cap, max_slots, 256]    (running max in the exp2 domain, sum)
-    int cluster;         // > 0: every item is shared by a cluster of so many CTAs, no workspace, no merge kernel
-    CutItem* cut;        // [grid] the item that the start of each share cuts, for the merge kernel
+    int cluster;         // kMergeCluster: CTAs that share an item; no workspace
+    CutItem* cut;        // kMergeKernel: [grid] the item that the start of each share cuts
+    unsigned long long* ready;       // kMergeHere: [grid] `epoch`: the share's partial rows are in its slot (0: merged)
+    unsigned long long epoch;        // of this launch: what lies in the workspace otherwise is not equal to it
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
 };
 
@@ -501,7 +510,32 @@ __device__ __forceinline__ VLanding v_landing(AttnCtrl* ctrl, bool split, int n_
 enum WalkMode { kWalk, kMaxOnly, kExact };
 
 // ---- softmax / epilogue of one segment: thread = (query row, 64-key chunk) ----------------------------
-template <int D, bool STORE, bool CLUSTER>
+// Share of a CTA on the cost axis.  The first share of an item waits for the later ones, so shares are dealt
+// from the last block to the first: blocks become resident in the order of their indexes, and a block waits
+// only for blocks ahead of it, whatever else runs on the GPU.
+__device__ __forceinline__ int my_share() { return (int)gridDim.x - 1 - (int)blockIdx.x; }
+
+// Bounded wait of a warp for the partial rows of the n shares behind this CTA's (true: they are there).
+__device__ __forceinline__ bool wait_shares(const AttnParams& p, int n, int lane, volatile int* abort_flag) {
+    bool there = lane >= n, gave_up = false;
+    if (!there) {
+        const unsigned long long* const flag = p.ready + my_share() + 1 + lane;
+        const long long t0 = clock64();
+        while (!(there = ptx::ld_acquire_u64(flag) == p.epoch) && !gave_up) {
+            gave_up = *abort_flag != 0;
+            if (clock64() - t0 > p.timeout_cycles) {
+                *abort_flag = 1;
+                record_status(p.dev_status, REGIONE_DEV_TIMEOUT);
+                gave_up = true;
+            }
+        }
+    }
+    there = __all_sync(0xffffffffu, there);
+    __syncwarp();                          // (the polling lanes' acquire holds for the whole warp)
+    return there;
+}
+
+template <int D, bool STORE, int FORM>
 __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it, uint8_t* smem_gen,
                                                 const uint32_t tmem, const int warp, const int lane, const int mode,
                                                 float& m_known) {
@@ -650,7 +684,9 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             l = exch[0] + exch[kBM];
         }
     }
-    constexpr bool shared = CLUSTER;
+    // the rows stay in shared memory: of an item shared by a cluster, and of the first share of a cut item, which
+    // merges the later shares' rows into them (merge_shares)
+    const bool shared = FORM == kMergeCluster || (FORM == kMergeHere && it.n_slots > 1 && it.slot == 0);
     if (shared && n_tiles > 0 && pair && ok) {
         // (the partial rows go over the tiles that the other query tile's products may still read)
         ok = wait_bar(ptx::smem_addr(&ctrl->o_final[1 - t]), 0, abort_flag, p.dev_status, p.timeout_cycles);
@@ -661,11 +697,11 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
     const int per = split ? (kPieces >= 4 ? 1 : (t == 0 ? 1 : 0)) : kPieces / 2;
     const int pc0 = split ? (kPieces >= 4 ? 2 * ck + t : ck) : ck * per, pc1 = pc0 + per;
     const uint32_t tO = tmem + lane_sel + 256 + (split ? 0 : t * D);
+    const size_t prow = ((size_t)it.item * p.max_slots + it.slot) * (2 * kBM) + qt * kBM + row;     // row in the slot
     const float inv = l > 0.f ? 1.f / l : 0.f;
     uint8_t* const stage = smem_gen + Cfg::kStageAt + warp * 4096;
     const size_t out_stride = (size_t)p.H * D * 2;
     uint8_t* const out0 = reinterpret_cast<uint8_t*>(p.out) + (((size_t)it.b * p.out_cap) * p.H + it.h) * D * 2;
-    const size_t prow_w = ((size_t)it.item * p.max_slots + it.slot) * (2 * kBM) + qt * kBM + ((warp & 3) << 5);
     if (direct && (dst_row >= p.out_cap || (dst_row < 0 && live))) {     // destination out of range: dropped
         record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         dst_row = -1;
@@ -676,11 +712,10 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
     }
     if (shared && n_tiles == 0) {
     } else if (n_tiles == 0) {
-        // no keys: zero rows, or an empty slot
+        // no keys: zero rows (an item without keys is one step and never cut)
         if (ck == 0 && direct && dst_row >= 0)
             for (int q = 0; q < D / 8; ++q)
                 reinterpret_cast<uint4*>(out0 + dst_row * out_stride)[q] = make_uint4(0, 0, 0, 0);
-        if (ck == 0 && !direct && live) p.part_ml[prow_w + lane] = make_float2(-INFINITY, 0.f);
     } else if (ok) {
 #pragma unroll 1
         for (int pc = pc0; pc < pc1; ++pc) {
@@ -727,22 +762,34 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
                     if (to >= 0) *reinterpret_cast<uint4*>(out0 + to * out_stride + pc * 64 + q * 16) = x;
                 }
             } else {
-                // unnormalised O of this segment -> its workspace slot: 128-byte pieces, 4 rows per instruction
+                if constexpr (FORM == kMergeHere) {
+                    // unnormalised O of this segment -> its workspace slot: a warp writes 512 contiguous bytes per store
+                    float4* const o = reinterpret_cast<float4*>(p.part_o) + ((size_t)it.item * p.max_slots + it.slot) * (2 * kBM) * (D / 4) +
+                                      (size_t)pc * 8 * (2 * kBM) + qt * kBM + row;
+                    if (live) {
 #pragma unroll
-                for (int q = 0; q < 8; ++q) mine[q ^ (lane & 7)] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-                __syncwarp();
-                uint8_t* const g0 = reinterpret_cast<uint8_t*>(p.part_o + prow_w * D) + pc * 128;
-                const int n_live = it.nq - wrow0;
+                        for (int q = 0; q < 8; ++q)
+                            o[q * (2 * kBM)] = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+                                                           __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
+                    }
+                } else {
+                    // unnormalised O of this segment -> its workspace slot: 128-byte pieces, 4 rows per instruction
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int rr = i * 4 + (lane >> 3), q = lane & 7;
-                    const uint4 x = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((q ^ (rr & 7)) << 4));
-                    if (rr < n_live) *reinterpret_cast<uint4*>(g0 + (size_t)rr * D * 4 + q * 16) = x;
+                    for (int q = 0; q < 8; ++q) mine[q ^ (lane & 7)] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                    __syncwarp();
+                    uint8_t* const g0 = reinterpret_cast<uint8_t*>(p.part_o + (prow - lane) * D) + pc * 128;
+                    const int n_live = it.nq - wrow0;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int rr = i * 4 + (lane >> 3), q = lane & 7;
+                        const uint4 x = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((q ^ (rr & 7)) << 4));
+                        if (rr < n_live) *reinterpret_cast<uint4*>(g0 + (size_t)rr * D * 4 + q * 16) = x;
+                    }
                 }
             }
             __syncwarp();
         }
-        if (!shared && !direct && live && ck == 0 && (!split || t == 0)) p.part_ml[prow_w + lane] = make_float2(m, l);
+        if (!shared && !direct && live && ck == 0 && (!split || t == 0)) p.part_ml[prow] = make_float2(m, l);
     }
     ptx::fence_proxy_async_smem();      // the next segment's query tile arrives by TMA
 }
@@ -809,6 +856,93 @@ __device__ __forceinline__ void merge_cluster(const AttnParams& p, const SegInfo
             o.x = pack_bf16x2(acc[0] * inv, acc[1] * inv); o.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
             o.z = pack_bf16x2(acc[4] * inv, acc[5] * inv); o.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
             *reinterpret_cast<uint4*>(p.out + (((size_t)it.b * p.out_cap + dst_row) * p.H + it.h) * D + col) = o;
+        }
+    }
+}
+
+// ---- cut item: its first share merges the later shares' partial rows into its own (softmax warps) -----------------
+//     out = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s
+// Its own rows are in shared memory, the others in their slots of the workspace.  The first share reaches the item at
+// the end of its range and the others begin with it, so it rarely waits.  A warp merges pieces of 32 columns of 32 rows,
+// a lane owns one row; the loads of the usual single other share are all under way before the first use.  The output
+// goes through the piece's own place in shared memory, so that stores cover whole sectors (a lane storing its own
+// row's chunks: 12600 cycles for a pair of tiles, this way 6500).
+template <int D>
+__device__ __forceinline__ void merge_shares(const AttnParams& p, const SegInfo& it, uint8_t* smem_gen, const int warp,
+                                             const int lane, volatile int* abort_flag) {
+    using Cfg = AttnCfg<D>;
+    const int n = it.n_slots, rb = warp >> 1;
+    const int row = rb * 32 + lane, qrow = it.q0 + row;
+    const bool live = qrow < it.nq;                // (dead rows' entries are not written and may hold anything)
+    int dst_row = -1;
+    if (live) dst_row = p.out_rows != nullptr ? p.out_rows[(size_t)it.b * p.Nq_cap + qrow] : qrow;
+    if (live && (dst_row < 0 || dst_row >= p.out_cap)) {       // destination out of range: dropped
+        if ((warp & 1) == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
+        dst_row = -1;
+    }
+    const float2 own = *(reinterpret_cast<const float2*>(smem_gen + Cfg::kPartialMlAt) + row);
+    const size_t slot1 = (size_t)it.item * p.max_slots + 1;
+    const float2* const others_ml = p.part_ml + slot1 * (2 * kBM) + row;
+    uint8_t* const out0 = reinterpret_cast<uint8_t*>(p.out) + (((size_t)it.b * p.out_cap) * p.H + it.h) * D * 2;
+    const size_t out_stride = (size_t)p.H * D * 2;
+    if (!wait_shares(p, n - 1, lane, abort_flag)) return;
+    if (rb * 32 >= it.nq - it.q0) return;
+#pragma unroll 1
+    for (int pc = (warp & 1) * (D / 64); pc < ((warp & 1) + 1) * (D / 64); ++pc) {
+        const float4* const others = reinterpret_cast<const float4*>(p.part_o) + (slot1 * (D / 4) + pc * 8) * (2 * kBM) + row;
+        uint8_t* const place = smem_gen + (rb * (D / 4) + pc * 8) * 512;      // 32 columns of 32 rows, fp32
+        float4 x[8], acc[8];
+        float2 ml = __ldcg(others_ml);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) x[q] = __ldcg(others + q * (2 * kBM));
+        // (a share without live keys in a row carries no weight)
+        float M = own.y > 0.f ? own.x : -INFINITY;
+        if (ml.y > 0.f) M = fmaxf(M, ml.x);
+        for (int sl = 1; sl < n - 1; ++sl) {
+            const float2 o = __ldcg(others_ml + sl * (2 * kBM));
+            if (o.y > 0.f) M = fmaxf(M, o.x);
+        }
+        float w = own.y > 0.f ? fast_exp2(own.x - M) : 0.f;
+        float L = w > 0.f ? w * own.y : 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 o = reinterpret_cast<const float4*>(place)[q * 32 + lane];
+            acc[q] = w > 0.f ? make_float4(w * o.x, w * o.y, w * o.z, w * o.w) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll 1
+        for (int sl = 1;; ++sl) {
+            if (ml.y > 0.f) {
+                w = fast_exp2(ml.x - M);
+                L = fmaf(w, ml.y, L);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    acc[q].x = fmaf(w, x[q].x, acc[q].x);
+                    acc[q].y = fmaf(w, x[q].y, acc[q].y);
+                    acc[q].z = fmaf(w, x[q].z, acc[q].z);
+                    acc[q].w = fmaf(w, x[q].w, acc[q].w);
+                }
+            }
+            if (sl >= n - 1) break;
+            ml = __ldcg(others_ml + sl * (2 * kBM));
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = __ldcg(others + ((size_t)sl * (D / 4) + q) * (2 * kBM));
+        }
+        const float inv = L > 0.f ? 1.f / L : 0.f;
+        __syncwarp();                              // (every lane has read its own rows' chunks)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            reinterpret_cast<uint4*>(place)[lane * 4 + (q ^ ((lane >> 1) & 3))] =
+                make_uint4(pack_bf16x2(acc[2 * q].x * inv, acc[2 * q].y * inv),
+                           pack_bf16x2(acc[2 * q].z * inv, acc[2 * q].w * inv),
+                           pack_bf16x2(acc[2 * q + 1].x * inv, acc[2 * q + 1].y * inv),
+                           pack_bf16x2(acc[2 * q + 1].z * inv, acc[2 * q + 1].w * inv));
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {              // 64 bytes of a row, 8 rows per instruction
+            const int rr = i * 8 + (lane >> 2), q = lane & 3;
+            const uint4 v = reinterpret_cast<const uint4*>(place)[rr * 4 + (q ^ ((rr >> 1) & 3))];
+            const int to = __shfl_sync(0xffffffffu, dst_row, rr);
+            if (to >= 0) *reinterpret_cast<uint4*>(out0 + to * out_stride + pc * 64 + q * 16) = v;
         }
     }
 }
@@ -1166,16 +1300,17 @@ struct ShareCursor {
         out->item = 0; out->slot = rank; out->n_slots = p.cluster;
     }
     // The next live segment of the share into *out (out->live = 0 when the share ends).
+    template <int FORM>
     __device__ __forceinline__ void next(const AttnParams& p, SegInfo* out, const int lane) {
         while (pos < hi) {
-            const Segment it = pl.whole_items ? segment_whole(p, pos) : segment_ticks(p, pl, pos, (int)blockIdx.x);
-            if (first && lane == 0) {
+            const Segment it = pl.whole_items ? segment_whole(p, pos) : segment_ticks(p, pl, pos, my_share());
+            if (FORM == kMergeKernel && first && lane == 0) {
                 // tell the merge kernel which item the start of this share cuts
                 CutItem ci;
                 ci.valid = (!pl.whole_items && it.r.np > 0 && it.n_slots >= 2 && it.slot == 1) ? 1 : 0;
                 ci.b = it.b; ci.h = it.h; ci.qp = it.qp; ci.n_slots = it.n_slots; ci.nq = it.r.nq;
                 ci.pad0 = ci.pad1 = 0;
-                p.cut[blockIdx.x] = ci;
+                p.cut[my_share()] = ci;
             }
             first = false;
             pos = pl.whole_items ? pos + gridDim.x : it.next;
@@ -1190,14 +1325,14 @@ struct ShareCursor {
             return;
         }
         if (lane == 0) {
-            if (first) p.cut[blockIdx.x].valid = 0;
+            if (FORM == kMergeKernel && first) p.cut[my_share()].valid = 0;
             out->live = 0;
         }
         first = false;
     }
 };
 
-template <int D, bool STORE, bool CLUSTER>
+template <int D, bool STORE, int FORM>
 __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, const CUtensorMap& tm_kf,
                                                       const CUtensorMap& tm_vf, const CUtensorMap& tm_kc,
                                                       const CUtensorMap& tm_vc, const AttnParams& p,
@@ -1214,14 +1349,14 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         ptx::tmem_relinquish();
     }
     grid_dependency_wait();                             // (everything below reads the launch's inputs)
-    grid_launch_dependents();                           // the merge kernel may queue up behind this CTA
+    grid_launch_dependents();                           // the next kernel may queue up behind this CTA
     ShareCursor cur;
     if (warp == kWarpS) {
         // this CTA's share [pos, hi) of the item sequence or of the cost axis
         // (whole items are dealt round-robin, so that the CTAs running at any one time work on
         // neighbouring items, which share K/V tiles in L2; a share of steps is one contiguous range)
         bool bad = false;
-        if constexpr (CLUSTER) {
+        if constexpr (FORM == kMergeCluster) {
             cur.of_cluster(p, &ctrl->seg[0], lane, &bad);
             if (lane == 0) {
                 ctrl->seg[1].live = 0;
@@ -1231,10 +1366,10 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             }
         } else {
         cur.pl = plan_shares(p, gridDim.x, &bad);
-        cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)blockIdx.x * cur.pl.chunk;
-        cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
+        cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)my_share() * cur.pl.chunk;
         cur.first = true;
-        cur.next(p, &ctrl->seg[0], lane);
+        cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
+        cur.next<FORM>(p, &ctrl->seg[0], lane);
         }
         if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         if (lane == 0) ctrl->abort_flag = 0;
@@ -1282,7 +1417,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     };
     if (STORE && threadIdx.x == 0) ctrl->walks_done = 0;
     __syncwarp();
-    if (CLUSTER) ptx::cluster_sync();             // (the peers' barriers are initialised)
+    if (FORM == kMergeCluster) ptx::cluster_sync();             // (the peers' barriers are initialised)
     __syncthreads();
     const uint32_t tmem = ctrl->tmem_base;
     int k = 0, mode = kWalk;
@@ -1309,7 +1444,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             } else if (warp == kWarpS) {
                 issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
                 // (the next segment is planned behind the last product, ahead of the end of this one)
-                if (!CLUSTER && mode == kWalk) cur.next(p, &ctrl->seg[k ^ 1], lane);
+                if (FORM != kMergeCluster && mode == kWalk) cur.next<FORM>(p, &ctrl->seg[k ^ 1], lane);
             } else {
                 issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, lane, mode);
             }
@@ -1319,16 +1454,38 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     } else {
         ptx::reg_alloc<104>();
         float m_known = -INFINITY;
+        bool publish = false, merges = false;   // the last segment's rows: (thread 0) in the workspace, the first share
+                                                // not told yet; in shared memory, to be merged with the later shares'
+        auto tell = [&]() {
+            // (every warp's rows are ordered before this by the barriers of tear_down and repeat)
+            if (publish && !*abort_flag) ptx::st_release_u64(p.ready + my_share(), p.epoch);
+            publish = false;
+        };
         while (ctrl->seg[k].live && !*abort_flag) {
             set_up(ctrl->seg[k]);
-            softmax_segment<D, STORE, CLUSTER>(p, ctrl, ctrl->seg[k], smem_raw, tmem, warp, lane, mode, m_known);
+            if (FORM == kMergeHere) tell();                   // (while the first key tiles are on their way)
+            softmax_segment<D, STORE, FORM>(p, ctrl, ctrl->seg[k], smem_raw, tmem, warp, lane, mode, m_known);
             tear_down();
-            if (!repeat(mode)) k ^= 1;
+            const bool cut = FORM == kMergeHere && ctrl->seg[k].n_slots > 1, head = ctrl->seg[k].slot == 0;
+            if (!repeat(mode)) {
+                publish = cut && !head && threadIdx.x == 0;
+                merges = cut && head;               // (the item goes on behind this share: nothing follows here)
+                k ^= 1;
+            }
+        }
+        if (FORM == kMergeHere) tell();
+        if (FORM == kMergeHere && merges) {
+            const SegInfo& it = ctrl->seg[k ^ 1];
+            if (!*abort_flag) merge_shares<D>(p, it, smem_raw, warp, lane, abort_flag);
+            // every warp has seen the flags: they are left as no launch's epoch (a graph replays the launch with the
+            // one it has)
+            named_barrier(3, 32 * kSoftmaxWarps);
+            if (threadIdx.x < it.n_slots - 1) p.ready[my_share() + 1 + threadIdx.x] = 0;
         }
     }
 
     // ================= item shared by a cluster =================
-    if (CLUSTER && ctrl->seg[0].live) {
+    if (FORM == kMergeCluster && ctrl->seg[0].live) {
         // (tear_down's barrier has ordered every warp's partial rows before this)
         const uint32_t ready = ptx::smem_addr(&ctrl->peers_ready), done = ptx::smem_addr(&ctrl->peers_done);
         if (warp == 0 && lane < p.cluster && !*abort_flag) ptx::mbar_arrive_cluster(ptx::map_rank(ready, lane));
@@ -1365,7 +1522,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
 
 // The attention kernel, and the one that also refreshes the cache (one parameter more); each also in the form
 // whose items are shared by clusters (instantiations of their own: the code of one form costs the other 1 %).
-template <int D, bool CLUSTER>
+template <int D, int FORM>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 region_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                            const __grid_constant__ CUtensorMap tm_kf,
@@ -1373,9 +1530,9 @@ region_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                            const __grid_constant__ CUtensorMap tm_kc,
                            const __grid_constant__ CUtensorMap tm_vc, const AttnParams p) {
     const StoreParams none = {};
-    attention_kernel_body<D, false, CLUSTER>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, none);
+    attention_kernel_body<D, false, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, none);
 }
-template <int D, bool CLUSTER>
+template <int D, int FORM>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_kf,
@@ -1383,7 +1540,7 @@ region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_kc,
                               const __grid_constant__ CUtensorMap tm_vc, const AttnParams p,
                               const __grid_constant__ StoreParams sp) {
-    attention_kernel_body<D, true, CLUSTER>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, sp);
+    attention_kernel_body<D, true, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, sp);
 }
 
 // Merges the workspace slots of the items that were spread over several shares:
@@ -1572,13 +1729,13 @@ size_t region_attention_tc_workspace(int B, int Nq_cap, int Nf_cap, int Nc_cap, 
     const LaunchPlan lp = plan_launch(B, Nq_cap, Nf_cap, Nc_cap, H);
     const size_t rows = slot_rows(lp, B, H);
     return ((rows * D * sizeof(float) + 255) & ~(size_t)255) +
-           ((rows * sizeof(float2) + 255) & ~(size_t)255) + (size_t)lp.grid * sizeof(CutItem);
+           ((rows * sizeof(float2) + 255) & ~(size_t)255) + (size_t)lp.grid * (sizeof(CutItem) + sizeof(unsigned long long));
 }
 
-template <int D, bool STORE, bool CLUSTER>
+template <int D, bool STORE, int FORM>
 static auto main_kernel() {
-    if constexpr (STORE) return region_attention_store_kernel<D, CLUSTER>;
-    else return region_attention_tc_kernel<D, CLUSTER>;
+    if constexpr (STORE) return region_attention_store_kernel<D, FORM>;
+    else return region_attention_tc_kernel<D, FORM>;
 }
 
 // Once per device: the opt-in to large dynamic shared memory, and how many clusters of each size fit the GPU.
@@ -1589,9 +1746,11 @@ static int prepare_kernel(const int** fitting) {
     const int dev = current_device();
     if (dev < 0) return REGIONE_CUDA_ERROR;
     if (!__atomic_load_n(&configured[dev], __ATOMIC_ACQUIRE)) {
-        if (cudaFuncSetAttribute(main_kernel<D, STORE, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(main_kernel<D, STORE, kMergeKernel>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  AttnCfg<D>::kSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(main_kernel<D, STORE, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(main_kernel<D, STORE, kMergeHere>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 AttnCfg<D>::kSmemBytes) != cudaSuccess ||
+            cudaFuncSetAttribute(main_kernel<D, STORE, kMergeCluster>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  AttnCfg<D>::kSmemBytes) != cudaSuccess)
             return REGIONE_CUDA_ERROR;
         for (int n = 2; n <= kMaxCluster; ++n) {
@@ -1605,7 +1764,7 @@ static int prepare_kernel(const int** fitting) {
             cfg.attrs = attr;
             cfg.numAttrs = 1;
             int fit = 0;
-            if (cudaOccupancyMaxActiveClusters(&fit, main_kernel<D, STORE, true>(), &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&fit, main_kernel<D, STORE, kMergeCluster>(), &cfg) != cudaSuccess) {
                 (void)cudaGetLastError();
                 fit = 0;
             }
@@ -1617,6 +1776,14 @@ static int prepare_kernel(const int** fitting) {
     return REGIONE_OK;
 }
 
+// Rows that are put back into a joint sequence many times their number keep the cuts of the cost axis with kTickStart:
+// where an item is cut decides which reference maximum its probabilities are rounded against, and seen against the rms
+// of the whole buffer, mostly rows that were not recomputed, another rounding moves single elements by up to 0.1 (by
+// 0.04 from a twelfth of the rows on).
+static bool keeps_cuts(const AttnParams& p) {
+    return p.out_rows != nullptr && 12LL * (p.Nq_cap - kBM / 2) < (long long)p.Nf_cap + p.Nc_cap;
+}
+
 // How many CTAs share an item through a cluster, 0: shares of the cost axis with a merge kernel behind them.
 // Few items (at most one cluster of two per pair of SMs) are better off in clusters: the shares of the cost axis are
 // balanced to a step, but every cut item's rows go through the workspace (7300 cycles per pair of tiles, all
@@ -1624,11 +1791,7 @@ static int prepare_kernel(const int** fitting) {
 // kTickCluster for a merge through distributed shared memory.  Both sides' ticks from the capacities:
 constexpr int kTickMerge = 125, kTickCluster = 45;
 static int choose_cluster(const int* fitting, const AttnParams& p, int nt) {
-    // Rows that are put back into a joint sequence many times their number keep the cuts of the cost axis: where an
-    // item is cut decides which reference maximum its probabilities are rounded against, and seen against the rms of
-    // the whole buffer, mostly rows that were not recomputed, another rounding moves single elements by up to 0.1
-    // (by 0.04 from a twelfth of the rows on).
-    if (p.out_rows != nullptr && 12LL * (p.Nq_cap - kBM / 2) < (long long)p.Nf_cap + p.Nc_cap) return 0;
+    if (keeps_cuts(p)) return 0;
     const long long items = (long long)p.B * p.H * p.P_cap;
     const bool lone_last = ((p.Nq_cap + kBM - 1) / kBM) % 2 == 1;
     const long long w_max = p.P_cap == 1 && lone_last ? kTickSingle : kTickPair;
@@ -1645,6 +1808,18 @@ static int choose_cluster(const int* fitting, const AttnParams& p, int nt) {
         if (cost < best) { best = cost; n_best = n; }
     }
     return n_best;
+}
+
+// Who merges cut items.  The first share takes about as long for one other share's rows (6500 cycles and a wait of 1000)
+// as the merge kernel does for all of them (8 us behind the attention), but off the path of the shares that it waits
+// for, without the write and the read of its own rows and without a launch.  Measured, merge kernel -> first share, us
+// (plain calls with what precedes them, stores as region steps): 2048 of 8448 rows, 24 heads, refreshed 252.7 -> 244.2;
+// four requests with 1382 of 18944 1395 -> 1378; 1075 queries x 8448 keys 149.3 -> 147.7; 819 x 8704 129.2 -> 129.4, behind
+// an 8-bit decode 137.4 -> 136.4; D = 64, 2048 x 6048 118.6 -> 110.2.  Not where an item is spread over many shares, whose
+// rows one CTA would read one after the other (205 x 8448 keys, 6 shares: 53.4 -> 63.3), nor where whole items outnumber
+// the cut ones (8704 x 8704, 816 items, at the power limit: 856 -> 868).
+static bool merges_here(const AttnParams& p, int grid) {
+    return p.max_slots <= 3 && (long long)p.B * p.H * p.P_cap <= 4LL * grid;
 }
 
 template <int D, bool STORE>
@@ -1673,11 +1848,14 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
         if constexpr (STORE) return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm, sp);
         else return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
     };
-    e = prm.cluster > 0 ? launch(main_kernel<D, STORE, true>()) : launch(main_kernel<D, STORE, false>());
+    const int form = prm.cluster > 0 ? kMergeCluster : merges_here(prm, grid) ? kMergeHere : kMergeKernel;
+    e = form == kMergeCluster ? launch(main_kernel<D, STORE, kMergeCluster>())
+        : form == kMergeHere  ? launch(main_kernel<D, STORE, kMergeHere>())
+                              : launch(main_kernel<D, STORE, kMergeKernel>());
     if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
     // the merge kernel may become resident while the attention kernel drains (it waits for that
     // kernel's completion before it reads a slot)
-    if (grid < 2 || prm.cluster > 0) return launch_status(cudaGetLastError());     // nothing is cut
+    if (grid < 2 || form != kMergeKernel) return launch_status(cudaGetLastError());     // nothing is cut
     const dim3 cgrid((unsigned)(grid - 1), (2 * kBM) / 8, 1);
     if (prm.max_slots <= 2)
         e = launch_overlapped(region_attention_combine_kernel<D, 2>, cgrid, dim3(256), 0, st, prm);
@@ -1689,6 +1867,16 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
         e = launch_overlapped(region_attention_combine_kernel<D, 8>, cgrid, dim3(256), 0, st, prm);
     if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
     return launch_status(cudaGetLastError());
+}
+
+// A number that no other launch has and that memory does not hold by chance: a count, scattered over 64 bits.
+static unsigned long long next_epoch() {
+    static std::atomic<unsigned long long> count{
+        (unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count()};
+    unsigned long long z = count.fetch_add(1, std::memory_order_relaxed) * 0x9E3779B97F4A7C15ull;     // (odd: a bijection)
+    z = (z ^ (z >> 31)) * 0xD6E8FEB86659FD93ull;
+    z ^= z >> 32;
+    return z != 0 ? z : 1;
 }
 
 int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const uint16_t* v_fresh,
@@ -1731,6 +1919,8 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
     const size_t off_ml = (rows * D * sizeof(float) + 255) & ~(size_t)255;
     prm.part_ml = reinterpret_cast<float2*>(ws + off_ml);
     prm.cut = reinterpret_cast<CutItem*>(ws + off_ml + ((rows * sizeof(float2) + 255) & ~(size_t)255));
+    prm.ready = reinterpret_cast<unsigned long long*>(prm.cut + lp.grid);
+    prm.epoch = next_epoch();
     prm.cluster = 0;
     const int nt_cap = std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN);
     if (store != nullptr)

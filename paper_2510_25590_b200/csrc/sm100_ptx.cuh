@@ -280,6 +280,16 @@ __device__ __forceinline__ uint64_t smem_desc_join(uint32_t lo, uint32_t hi) {
     return ((uint64_t)hi << 32) | lo;
 }
 
+// Hand-over of data between CTAs through global memory.
+__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // Instruction descriptor for kind::f16 with bf16 operands and an fp32 accumulator.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, bool b_mn_major) {
     return (1u << 4)                        // D format = F32
