@@ -1816,10 +1816,12 @@ static int choose_cluster(const int* fitting, const AttnParams& p, int nt) {
 // (plain calls with what precedes them, stores as region steps): 2048 of 8448 rows, 24 heads, refreshed 252.7 -> 244.2;
 // four requests with 1382 of 18944 1395 -> 1378; 1075 queries x 8448 keys 149.3 -> 147.7; 819 x 8704 129.2 -> 129.4, behind
 // an 8-bit decode 137.4 -> 136.4; D = 64, 2048 x 6048 118.6 -> 110.2.  Not where an item is spread over many shares, whose
-// rows one CTA would read one after the other (205 x 8448 keys, 6 shares: 53.4 -> 63.3), nor where whole items outnumber
-// the cut ones (8704 x 8704, 816 items, at the power limit: 856 -> 868).
-static bool merges_here(const AttnParams& p, int grid) {
-    return p.max_slots <= 3 && (long long)p.B * p.H * p.P_cap <= 4LL * grid;
+// rows one CTA would read one after the other (205 x 8448 keys, 6 shares: 53.4 -> 63.3), nor where a share is short
+// beside the merge (three requests, 250 x 4650, 16 heads, 26 steps a share: 60.3 -> 63.8), nor where whole items
+// outnumber the cut ones (8704 x 8704, 816 items, at the power limit: 856 -> 868).
+static bool merges_here(const AttnParams& p, int grid, int nt) {
+    const long long items = (long long)p.B * p.H * p.P_cap;
+    return p.max_slots <= 3 && items <= 4LL * grid && items * nt >= 40LL * grid;
 }
 
 template <int D, bool STORE>
@@ -1848,7 +1850,7 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
         if constexpr (STORE) return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm, sp);
         else return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
     };
-    const int form = prm.cluster > 0 ? kMergeCluster : merges_here(prm, grid) ? kMergeHere : kMergeKernel;
+    const int form = prm.cluster > 0 ? kMergeCluster : merges_here(prm, grid, nt_cap) ? kMergeHere : kMergeKernel;
     e = form == kMergeCluster ? launch(main_kernel<D, STORE, kMergeCluster>())
         : form == kMergeHere  ? launch(main_kernel<D, STORE, kMergeHere>())
                               : launch(main_kernel<D, STORE, kMergeKernel>());
