@@ -5,7 +5,7 @@ A "step" is one pass of the whole hot path over one batch of synthetic input of
 the FLUX-Kontext-shaped workload (4096 image + 4096 reference + 512 text tokens,
 24 heads x 128, two-ellipse 20 % edit mask): partition, row lists, gathers, RIKV
 store, region attention with its rows scattered back, velocity decay + Euler, merge (one library call,
-4 kernel launches).
+3 or 4 kernel launches).
 
 Prints ONE JSON line (rank 0).  `value` = region-attention FLOPs of the step
 divided by the whole step's device time (inputs resident in HBM).  `roofline`
@@ -282,7 +282,7 @@ def hbm_sweep(torch, binding, step, d, flush_l2, peak_gbs, iters=10):
 
 def ratio_sweep(torch, binding, synth, flush_l2, to_dev, steps=20):
     """Denoise-step time against the edit-mask ratio on the Qwen-Image-Edit-shaped workload (config 3):
-    one region step (one library call, 4 launches) and its attention call per ratio, CUDA events, L2
+    one region step (one library call, 3 or 4 launches) and its attention call per ratio, CUDA events, L2
     flushed per step."""
     from paper_2510_25590_b200.step import RegionStep, StepShapes, plan_capacity
     wl = synth.WORKLOADS[3]
@@ -367,7 +367,7 @@ def per_config_rows(torch, binding, synth, flush_l2, to_dev, peaks, steps=12):
         reuse_us = float(np.mean([a.elapsed_time(b) for a, b in reuse]) * 1e3)
         graph_us = None
         if cfg == 1:
-            # the tiny layer's step is launch-bound (8 kernels of a few microseconds each): the same step
+            # the tiny layer's step is launch-bound (3 kernels of a few microseconds each): the same step
             # captured once into a CUDA graph and replayed shows the device time without the host's
             # launch path in between
             side = torch.cuda.Stream()

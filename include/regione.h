@@ -325,7 +325,7 @@ int regione_region_attention_scatter(const regione_bf16* q,
 /*
  * One whole region-aware step of one attention layer: regione_partition_rows, the gather of X^E and v,
  * regione_velocity_decay, regione_merge, the gather of Q / K / V, regione_rikv_store (with store_cache) and
- * regione_region_attention_scatter, with the results those calls leave, in four kernel launches.
+ * regione_region_attention_scatter, with the results those calls leave, in three or four kernel launches.
  * The plan names the sizes and the buffers that the step owns (device pointers; layouts as in those
  * calls, c_cap = n_full = n_text + N + n_ref, q_cap = ne_cap, plus n_text under REGIONE_ROWS_PAPER):
  *   mask u8 [B, N]; edit_idx, keep_idx, slot i32 [B, N]; n_edit, n_q, n_cache i32 [B];
@@ -367,9 +367,8 @@ int regione_region_step(const regione_step_plan* plan, const regione_bf16* x_t, 
  *     regione_region_attention(q, k, v, NULL, NULL, n_rows, n_rows, 0, ...)     (plain joint attention)
  *     regione_rikv_store(k, v, keep_rows, n_keep, ...)
  * do one after the other, bit for bit the same cache and the same output, but K and V are read from
- * device memory once: the attention kernel stages every K / V tile of a head in shared memory anyway,
- * and the thread block that walks the first query rows of a (request, head) writes the retained
- * rows of each tile from there to their slots in the cache.
+ * device memory by one launch: a warp of every thread block copies its share of the retained rows to
+ * their slots in the cache while the block's other warps attend.
  *
  * q, k, v, out : dev bf16 [B, N_cap, H, D];  n_rows dev int32 [B] live rows (queries = keys)
  * keep_rows    : dev int32 [B, Nc_cap], strictly ascending per request (as regione_region_rows

@@ -1,20 +1,20 @@
-// One region-aware step of one attention layer as a sequence of four launches (Algorithm 1, one iteration of
+// One region-aware step of one attention layer as a sequence of three or four launches (Algorithm 1, one iteration of
 // the region loop for one layer):
 //   1 partition with the joint-sequence row lists
 //   2 everything that moves rows between the partition and the attention: the latent update and the gathers
 //   3 region attention, its rows written at their joint-sequence positions; in a step that refreshes the
 //     cache the copies to the cache travel in the same launch
-//   4 merge of the attention's shared items
+//   4 merge of the items that the attention cut, where it does not do that itself
 //
 // Why one launch for all the moves: the kernels it replaces (gather of X^E and v, velocity decay, merge, gather
 // of Q / K / V) take 2 to 5 us each, most of it launch and one memory round trip, and had two streams to be forked
 // and joined.  Why the cache store rides with the attention: the rows of a step that refreshes the cache from its own
 // K and V are, fresh and cached together, all rows of K and V, so the attention reads those directly and nothing
 // waits for the cache.  Measured, one pass among others with its host work (seven calls on two streams -> one call):
-//   256 of 1024 tokens, 4 heads x 64, cache refreshed       107 -> 31 us
-//   205 of 4096 tokens, 24 heads x 128, cache read           95 -> 55 us
-//   819 of 4096 tokens, 24 heads x 128, cache read          136 -> 128 us (power-capped attention)
-//   2048 of 4096 tokens, 24 heads x 128, cache refreshed    285 -> 272 us (power-capped attention)
+//   256 of 1024 tokens, 4 heads x 64, cache refreshed       108 -> 24 us
+//   205 of 4096 tokens, 24 heads x 128, cache read           95 -> 54 us
+//   819 of 4096 tokens, 24 heads x 128, cache read          135 -> 128 us (power-capped attention)
+//   2048 of 4096 tokens, 24 heads x 128, cache refreshed    281 -> 243 us (power-capped attention)
 #include "rowcopy.cuh"
 
 namespace regione {

@@ -85,7 +85,7 @@ class RegionStep:
         self.workspace = torch.empty(max(binding.region_step_workspace(self._step_plan()), 256), dtype=torch.uint8,
                                      device=device)
         self.launches = 0                 # operations of the sequence run so far (8 per step, 7 without the store)
-        self.kernel_launches = 0          # kernels launched so far (batches of up to 128 requests)
+        self.kernel_launches = 0          # kernels launched so far, at least (a fourth merges cut items in some shapes)
         self.attention_events = None      # optional (start, stop) pair recorded around the attention
 
     _BUFFERS = ("mask", "edit_idx", "keep_idx", "slot", "n_edit", "query_rows", "n_q", "cache_rows", "n_cache", "n_rows",
@@ -123,5 +123,5 @@ class RegionStep:
             binding.region_step(*args, parts=binding.STEP_ATTENTION, stream=stream)
             self.attention_events[1].record(stream)
         self.launches += 8 if store_cache else 7
-        self.kernel_launches += 4
+        self.kernel_launches += 3
         return self.x_out
