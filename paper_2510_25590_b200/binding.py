@@ -8,6 +8,7 @@ if the shared library is missing or a call fails, a ``RegionEError`` is raised.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 from ctypes import POINTER, c_char_p, c_double, c_float, c_int, c_int64, c_longlong, c_size_t, c_void_p
 
@@ -123,6 +124,11 @@ def _ptr(t, dtype=None, name="tensor"):
     """Device address of a contiguous CUDA tensor (an int: ctypes converts it), None for None."""
     if t is None:
         return None
+    try:
+        if t.is_cuda and (dtype is None or t.dtype == dtype) and t.is_contiguous():
+            return t.data_ptr()
+    except AttributeError:
+        pass
     if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise RegionEError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
@@ -217,20 +223,16 @@ def region_rows(edit_idx, keep_idx, n_edit, n_text, n_ref, membership, query_row
 
 
 def _row_bytes(t):
-    rb = t.element_size()
-    for d in t.shape[2:]:
-        rb *= d
-    return rb
+    return t.element_size() * math.prod(t.shape[2:])
 
 
 def gather(src, idx, n, dst, dev_status=None, stream=None):
     """dst[b, j] = src[b, idx[b, j]], j < n[b].  src [B, rows, ...], dst [B, cap, ...]."""
-    torch = _torch()
-    B = src.shape[0]
+    i32, shape = _torch().int32, src.shape
     _check(load().regione_gather(
-        _ptr(src, None, "src"), _ptr(idx, torch.int32, "idx"), _ptr(n, torch.int32, "n"), B,
-        src.shape[1], idx.shape[1], dst.shape[1], _row_bytes(src), _ptr(dst, src.dtype, "dst"),
-        _ptr(dev_status, torch.int32), _stream(stream)), "regione_gather")
+        _ptr(src, None, "src"), _ptr(idx, i32, "idx"), _ptr(n, i32, "n"), shape[0], shape[1], idx.shape[1],
+        dst.shape[1], src.element_size() * math.prod(shape[2:]), _ptr(dst, src.dtype, "dst"), _ptr(dev_status, i32),
+        _stream(stream)), "regione_gather")
 
 
 def gather_multi(srcs, idx, n, dsts, dev_status=None, stream=None):
