@@ -850,7 +850,7 @@ def run_ours(args):
     achieved = flops / (attn_us * 1e-6) / 1e12
     roofline = dict(bound="tensor", achieved=achieved, peak=peaks["bf16_tflops"], unit="TFLOP/s",
                     frac=achieved / peaks["bf16_tflops"], traffic=recorded_traffic(cfg),
-                    kernel=f"region_attention_tc_kernel<{wl.head_dim}> (+ merge of shared items)",
+                    kernel=f"region_attention_store_kernel<{wl.head_dim}> (attention with the cache copies in the same launch)",
                     us_per_launch=attn_us,
                     peak_source=f"bf16_tflops (burst) of {peaks['source']}",
                     frac_of_nominal_2250=achieved / NOMINAL_BF16_TFLOPS)
