@@ -337,7 +337,9 @@ int regione_region_attention_scatter(const regione_bf16* q,
  * arrays [B] (NaN: the request sits that operation out, as in the single calls).
  * store_cache != 0: with enough queries beside the keys the attention reads K and V where they are (fresh and
  * cached rows together are all of them), the cache receives its rows in the same launch, and k_fresh and v_fresh
- * are not written; with fewer the rows are copied ahead of it.  Both parts have to be called with the same value.
+ * are not written; with fewer the rows are copied ahead of it.  A request whose edited tokens exceed the capacity
+ * (REGIONE_DEV_BOUNDS) has its rows copied ahead too: the dropped tokens' keys are in neither list, so nothing attends
+ * to them.  Both parts have to be called with the same value.
  * parts: REGIONE_STEP_MOVES (everything up to the attention) | REGIONE_STEP_ATTENTION.
  */
 typedef struct {

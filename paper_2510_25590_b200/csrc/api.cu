@@ -139,7 +139,7 @@ extern "C" int regione_full_attention_store(
         if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return REGIONE_INVALID_ARG;
         if (workspace_bytes < need) return REGIONE_WORKSPACE_TOO_SMALL;
     }
-    CacheStore store;
+    CacheStore store = {};
     store.keep_rows = keep_rows; store.n_keep = n_keep; store.cap = Nc_cap;
     store.k_cache = k_cache; store.v_cache = v_cache;
     // no cached segment: n_cache = nullptr stands for "zero rows" in every request

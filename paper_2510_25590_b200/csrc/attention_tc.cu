@@ -128,6 +128,7 @@ struct SegInfo {
     int j_first, n_tiles;       // key tiles [j_first, j_first + n_tiles) of the item
     int nt_c, nt, nc, nf;       // cached key tiles, all key tiles, live keys of the two segments
     int item, slot, n_slots;    // item index within the launch, slot among the shares that touch it
+    int apart;                  // (launch that refreshes the cache) fresh rows are not in K and V themselves: see ReqShape
 };
 
 struct AttnCtrl {
@@ -187,6 +188,7 @@ struct AttnParams {
     uint16_t* out;       // [B, out_cap, H, D]
     const int32_t* out_rows;   // nullptr: query row i goes to out row i; else to row out_rows[b, i]
     int out_cap;         // rows per request of `out` (Nq_cap without out_rows)
+    int all_rows;        // > 0: query and cached rows of a request are parts of its K and V of this many rows (see ReqShape)
     int32_t* dev_status;
     float* part_o;       // [B, H, P_cap, max_slots, 256, D] unnormalised outputs; kMergeHere: [..., D / 4, 256, 4]
     float2* part_ml;     // [B, H, P_cap, max_slots, 256]    (running max in the exp2 domain, sum)
@@ -224,6 +226,8 @@ struct ReqShape {
     int nt_c, nt;        // cached key tiles, all key tiles
     long long items;     // H * np
     int steps;           // steps of an item: max(nt, 1) (an item without keys writes zeros in one step)
+    bool apart;          // AttnParams::all_rows: the query and cached rows are not all rows (more tokens were edited than
+                         // the capacity holds), so the request attends over [cached | fresh] as copied ahead of the launch
     int w_last;          // ticks per step of the last query pair
     long long ticks_full, ticks_last, head_ticks, ticks;   // per full-pair item, last item, head, request
 };
@@ -231,11 +235,17 @@ struct ReqShape {
 __device__ __forceinline__ ReqShape req_shape(const AttnParams& p, int b, bool* bad = nullptr) {
     ReqShape r;
     int nq = p.n_q[b], nf = p.n_fresh[b], nc = p.n_cache == nullptr ? 0 : p.n_cache[b];      // (nullptr: no cached segment)
-    if (nq < 0 || nq > p.Nq_cap || nf < 0 || nf > p.Nf_cap || nc < 0 || nc > p.Nc_cap) {
+    const int c_cap = p.all_rows > 0 ? p.all_rows : p.Nc_cap;
+    if (nq < 0 || nq > p.Nq_cap || nf < 0 || nf > p.Nf_cap || nc < 0 || nc > c_cap) {
         if (bad) *bad = true;
         nq = max(0, min(nq, p.Nq_cap));
         nf = max(0, min(nf, p.Nf_cap));
-        nc = max(0, min(nc, p.Nc_cap));
+        nc = max(0, min(nc, c_cap));
+    }
+    r.apart = p.all_rows > 0 && rows_apart(nq, nc, p.Nq_cap, p.all_rows);
+    if (p.all_rows > 0) {
+        nf = r.apart ? nq : p.all_rows;
+        nc = r.apart ? nc : 0;
     }
     r.nq = nq; r.nf = nf; r.nc = nc;
     r.np = (nq + 2 * kBM - 1) / (2 * kBM);
@@ -959,7 +969,6 @@ __device__ __forceinline__ void merge_shares(const AttnParams& p, const SegInfo&
 // rows in flight took 2660 cycles a row.  Over the idle tiles two batches alternate.
 struct CachePump {
     const StoreParams* sp;
-    const int32_t* n_rows;
     AttnCtrl* ctrl;
     const AttnParams* p;
     int row_bytes, item_bytes, per_row; // items per row
@@ -974,15 +983,19 @@ struct CachePump {
 
     __device__ __forceinline__ int kept(int req, bool report) const {
         const int nk = sp->n_keep[req];
+        if (p->all_rows > 0 && rows_apart(p->n_q[req], nk, p->Nq_cap, p->all_rows)) return 0;      // (copied ahead)
         if (nk >= 0 && nk <= sp->store_cap) return nk;
         if (report && blockIdx.x == 0) record_status(p->dev_status, REGIONE_DEV_BOUNDS);
         return nk < 0 ? 0 : sp->store_cap;
+    }
+    __device__ __forceinline__ int source_rows(int req) const {
+        return p->all_rows > 0 ? p->all_rows : min(p->n_fresh[req], sp->src_cap);
     }
     __device__ __forceinline__ int row_of(int item) const { return per_row > 1 ? item / per_row : item; }
     // from an item index behind the runs x, b to the run that holds it (a request without rows stores nothing)
     __device__ __forceinline__ void open_run() {
         for (;;) {
-            live_rows = min(n_rows[b], sp->src_cap);
+            live_rows = source_rows(b);
             run = live_rows > 0 ? kept(b, false) * per_row : 0;
             if (i < run) return;
             i -= run;
@@ -1016,14 +1029,14 @@ struct CachePump {
         __syncwarp();
     }
     __device__ __forceinline__ void begin(const AttnParams& prm, const StoreParams& s, AttnCtrl* c, int d, int longest, int lane) {
-        sp = &s; n_rows = prm.n_fresh; ctrl = c; p = &prm;
+        sp = &s; ctrl = c; p = &prm;
         row_bytes = prm.H * d * 2;
         per_row = (row_bytes + longest - 1) / longest;
         item_bytes = min(row_bytes, longest);
         long long total = 0;
         for (int r = 0; r < prm.B; ++r) {
             const int nk = kept(r, lane == 0);
-            if (n_rows[r] > 0) total += 2LL * nk * per_row;
+            if (source_rows(r) > 0) total += 2LL * nk * per_row;
         }
         const long long per = (total + gridDim.x - 1) / gridDim.x, first = per * blockIdx.x;
         left = (int)max(0LL, min(per, total - first));
@@ -1120,8 +1133,9 @@ struct CachePump {
 // ---- TMA producer of one segment (whole warp; lane 0 issues) ----------------------------------------------
 template <int D, bool STORE>
 __device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUtensorMap* tm_kf, const CUtensorMap* tm_vf,
-                                             const CUtensorMap* tm_kc, const CUtensorMap* tm_vc, const AttnParams& p,
-                                             AttnCtrl* ctrl, const SegInfo& it, const uint32_t smem, const int lane) {
+                                             const CUtensorMap* tm_kc, const CUtensorMap* tm_vc, const CUtensorMap* tm_ka,
+                                             const CUtensorMap* tm_va, const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it,
+                                             const uint32_t smem, const int lane) {
     using Cfg = AttnCfg<D>;
     constexpr int kTileBytes = Cfg::kTileBytes;
     const int n_tiles = it.n_tiles;
@@ -1131,6 +1145,7 @@ __device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUte
     const int n_stages = split ? Cfg::lone_stages(STORE) : Cfg::kStages;
     const uint32_t ring = smem + (split ? 1 : 2) * kTileBytes;
     const int nt_c = it.nt_c, j_first = it.j_first, h = it.h, b = it.b;
+    if (STORE && it.apart) { tm_kf = tm_ka; tm_vf = tm_va; }
     if (lane == 0) {
         ptx::prefetch_tensormap(tm_q);
         ptx::prefetch_tensormap(j_first < nt_c ? tm_kc : tm_kf);
@@ -1297,7 +1312,7 @@ struct ShareCursor {
         out->nq = r.nq; out->nt_c = r.nt_c; out->nt = r.nt; out->nc = r.nc; out->nf = r.nf;
         out->j_first = rank * r.nt / p.cluster;
         out->n_tiles = (rank + 1) * r.nt / p.cluster - out->j_first;
-        out->item = 0; out->slot = rank; out->n_slots = p.cluster;
+        out->item = 0; out->slot = rank; out->n_slots = p.cluster; out->apart = r.apart;
     }
     // The next live segment of the share into *out (out->live = 0 when the share ends).
     template <int FORM>
@@ -1320,6 +1335,7 @@ struct ShareCursor {
                 out->j_first = it.j_first; out->n_tiles = it.r.nt == 0 ? 0 : it.n_steps;
                 out->nt_c = it.r.nt_c; out->nt = it.r.nt; out->nc = it.r.nc; out->nf = it.r.nf;
                 out->item = (it.b * p.H + it.h) * p.P_cap + it.qp; out->slot = it.slot; out->n_slots = it.n_slots;
+                out->apart = it.r.apart;
                 out->live = 1;
             }
             return;
@@ -1335,8 +1351,8 @@ struct ShareCursor {
 template <int D, bool STORE, int FORM>
 __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, const CUtensorMap& tm_kf,
                                                       const CUtensorMap& tm_vf, const CUtensorMap& tm_kc,
-                                                      const CUtensorMap& tm_vc, const AttnParams& p,
-                                                      const StoreParams& sp) {
+                                                      const CUtensorMap& tm_vc, const CUtensorMap& tm_ka,
+                                                      const CUtensorMap& tm_va, const AttnParams& p, const StoreParams& sp) {
     using Cfg = AttnCfg<D>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t smem = ptx::smem_addr(smem_raw);     // 2 query tiles, then the ring of K/V stages
@@ -1440,7 +1456,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             const SegInfo& it = ctrl->seg[k];
             set_up(it);
             if (warp == kWarpLoad) {
-                load_segment<D, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, p, ctrl, it, smem, lane);
+                load_segment<D, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, &tm_ka, &tm_va, p, ctrl, it, smem, lane);
             } else if (warp == kWarpS) {
                 issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
                 // (the next segment is planned behind the last product, ahead of the end of this one)
@@ -1520,7 +1536,8 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     }
 }
 
-// The attention kernel, and the one that also refreshes the cache (one parameter more); each also in the form
+// The attention kernel, and the one that also refreshes the cache (its parameters, and the fresh rows of requests that
+// do not attend over K and V in place: ReqShape::apart); each also in the form
 // whose items are shared by clusters (instantiations of their own: the code of one form costs the other 1 %).
 template <int D, int FORM>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -1530,7 +1547,7 @@ region_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                            const __grid_constant__ CUtensorMap tm_kc,
                            const __grid_constant__ CUtensorMap tm_vc, const AttnParams p) {
     const StoreParams none = {};
-    attention_kernel_body<D, false, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, none);
+    attention_kernel_body<D, false, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_kf, tm_vf, p, none);
 }
 template <int D, int FORM>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -1538,9 +1555,11 @@ region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_kf,
                               const __grid_constant__ CUtensorMap tm_vf,
                               const __grid_constant__ CUtensorMap tm_kc,
-                              const __grid_constant__ CUtensorMap tm_vc, const AttnParams p,
+                              const __grid_constant__ CUtensorMap tm_vc,
+                              const __grid_constant__ CUtensorMap tm_ka,
+                              const __grid_constant__ CUtensorMap tm_va, const AttnParams p,
                               const __grid_constant__ StoreParams sp) {
-    attention_kernel_body<D, true, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, p, sp);
+    attention_kernel_body<D, true, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_ka, tm_va, p, sp);
 }
 
 // Merges the workspace slots of the items that were spread over several shares:
@@ -1847,7 +1866,7 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
     cfg.numAttrs = prm.cluster > 0 ? 2 : 1;
     cudaError_t e;
     auto launch = [&](auto kernel) {
-        if constexpr (STORE) return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm, sp);
+        if constexpr (STORE) return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6], prm, sp);
         else return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
     };
     const int form = prm.cluster > 0 ? kMergeCluster : merges_here(prm, grid, nt_cap) ? kMergeHere : kMergeKernel;
@@ -1889,15 +1908,19 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
                                size_t workspace_bytes, int32_t* dev_status, cudaStream_t st,
                                const CacheStore* store) {
     (void)workspace_bytes;
-    CUtensorMap maps[5];
+    CUtensorMap maps[7];
+    const int all_rows = store != nullptr ? store->all_rows : 0;
     // an absent segment still needs a valid (never dereferenced) base address
     const void* kf = Nf_cap > 0 ? (const void*)k_fresh : (const void*)q;
     const void* vf = Nf_cap > 0 ? (const void*)v_fresh : (const void*)q;
-    const void* kc = Nc_cap > 0 ? (const void*)k_cache : (const void*)q;
-    const void* vc = Nc_cap > 0 ? (const void*)v_cache : (const void*)q;
+    const void* kc = all_rows > 0 ? store->k_cache : Nc_cap > 0 ? (const void*)k_cache : (const void*)q;
+    const void* vc = all_rows > 0 ? store->v_cache : Nc_cap > 0 ? (const void*)v_cache : (const void*)q;
     if (!make_map(&maps[0], q, B, Nq_cap, H, D) || !make_map(&maps[1], kf, B, Nf_cap, H, D) ||
-        !make_map(&maps[2], vf, B, Nf_cap, H, D) || !make_map(&maps[3], kc, B, Nc_cap, H, D) ||
-        !make_map(&maps[4], vc, B, Nc_cap, H, D))
+        !make_map(&maps[2], vf, B, Nf_cap, H, D) || !make_map(&maps[3], kc, B, all_rows > 0 ? all_rows : Nc_cap, H, D) ||
+        !make_map(&maps[4], vc, B, all_rows > 0 ? all_rows : Nc_cap, H, D))
+        return REGIONE_CUDA_ERROR;
+    if (store != nullptr && (!make_map(&maps[5], all_rows > 0 ? store->k_apart : q, B, Nq_cap, H, D) ||
+                             !make_map(&maps[6], all_rows > 0 ? store->v_apart : q, B, Nq_cap, H, D)))
         return REGIONE_CUDA_ERROR;
     const LaunchPlan lp = plan_launch(B, Nq_cap, Nf_cap, Nc_cap, H);
     AttnParams prm;
@@ -1908,6 +1931,7 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
     prm.out = out; prm.dev_status = dev_status;
     prm.out_rows = out_rows;
     prm.out_cap = out_rows != nullptr ? out_cap : Nq_cap;
+    prm.all_rows = all_rows;
     prm.timeout_cycles = kTimeoutCycles;
     StoreParams sp = {};
     if (store != nullptr) {

@@ -97,7 +97,19 @@ struct CacheStore {
     int cap;
     uint16_t* k_cache;          // dev [B, cap, H, D]
     uint16_t* v_cache;
+    // > 0 (the region step): the queries' rows and the kept rows are parts of K and V of this many rows.  A request whose
+    // two lists name all of them attends over K and V in place; any other (see rows_apart) over the rows of its lists,
+    // which the caller has copied to k_cache / v_cache and to k_apart / v_apart [B, Nq_cap, H, D].
+    int all_rows;
+    const uint16_t* k_apart;
+    const uint16_t* v_apart;
 };
+
+// Whether the recomputed and the cached rows of a request are not all of its rows: more tokens were edited than the
+// capacity holds (the others are dropped), or the request has no partition yet.
+__device__ __forceinline__ bool rows_apart(int n_q, int n_cache, int q_cap, int all_rows) {
+    return max(0, min(n_q, q_cap)) + max(0, min(n_cache, all_rows)) != all_rows;
+}
 
 // The attention's host side (defined in attention_tc.cu).  n_cache = nullptr: no cached rows in any request;
 // store != nullptr: the rows store->keep_rows of k_fresh / v_fresh go to the cache in the same launch.

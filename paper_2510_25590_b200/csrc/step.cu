@@ -28,6 +28,8 @@ namespace regione {
 // a sixteenth single elements of the scattered buffer moved by up to 0.1 of its rms, from there on by 0.05.
 static bool takes_rows_along(int q_cap, int n_full) { return 16LL * (q_cap - 64) >= n_full; }
 
+constexpr int kApartBlocks = 64;      // blocks of a request that copy rows only where rows_apart says so
+
 struct LatentMove {
     const uint4 *x, *v;             // [B, N, C] current latent and velocity
     const int32_t* slot;            // [B, N] place of an edited token in X^E, negative: unedited
@@ -76,8 +78,10 @@ __device__ __forceinline__ void move_latents(const LatentMove& a, int b, unsigne
     if (merge) a.x_out[at] = y;
 }
 
-// blockIdx.x: blocks of the latent update, then of each gathered tensor, then of K and V of the rows that go to the
-// cache (where the attention does not take them along); blockIdx.y = request of this launch.
+// blockIdx.x: blocks of the latent update, then of each of the n_pairs tensors whose recomputed rows are gathered, then
+// of K and V of the rows that go to the cache; blockIdx.y = request of this launch.  Where the attention reads K and V
+// in place (along), only the queries are gathered for certain: a request whose lists do not name all rows needs its
+// other rows as well (rows_apart), which is rare, so that a few blocks stride over them.
 // Bound by launch and one or two memory round trips at the sizes of the paper's editors (4 to 5 us); the row gathers
 // run at the bandwidth of HBM where they are large, and the latent blocks, which come first, hide behind them.
 __global__ void __launch_bounds__(kCopyThreads)
@@ -85,7 +89,7 @@ region_step_move_kernel(const LatentMove lat, const __grid_constant__ PerRequest
                         const __grid_constant__ PerRequestF neg_dt_u, int b0, int lat_blocks,
                         const __grid_constant__ RowCopyPairs rows, int n_pairs, int row_blocks,
                         const int32_t* __restrict__ query_rows, const int32_t* __restrict__ n_q, int n_full, int q_cap,
-                        int row_cpr, const __grid_constant__ RowCopyPairs kept, int kept_blocks,
+                        int row_cpr, const __grid_constant__ RowCopyPairs kept, int kept_blocks, bool along, int tail_blocks,
                         const int32_t* __restrict__ cache_rows, const int32_t* __restrict__ n_cache, int32_t* dev_status) {
     grid_dependency_wait();
     grid_launch_dependents();
@@ -102,8 +106,17 @@ region_step_move_kernel(const LatentMove lat, const __grid_constant__ PerRequest
         return;
     }
     at -= n_pairs * row_blocks;
-    const int pair = at / kept_blocks;
-    copy_rows<true>(kept.p[pair], b, at - pair * kept_blocks, cache_rows, n_cache, n_full, n_full, n_full, row_cpr, dev_status);
+    if (along && !rows_apart(n_q[b], n_cache[b], q_cap, n_full)) return;
+    const int fresh = along ? 2 * row_blocks : 0;              // K and V, pairs 1 and 2 of `rows`
+    for (; at < fresh + 2 * kept_blocks; at += tail_blocks) {
+        const int pair = at < fresh ? at / row_blocks : (at - fresh) / kept_blocks;
+        if (at < fresh)
+            copy_rows<true>(rows.p[1 + pair], b, at - pair * row_blocks, query_rows, n_q, n_full, q_cap, q_cap, row_cpr,
+                            dev_status);
+        else
+            copy_rows<true>(kept.p[pair], b, at - fresh - pair * kept_blocks, cache_rows, n_cache, n_full, n_full, n_full,
+                            row_cpr, dev_status);
+    }
 }
 
 }  // namespace regione
@@ -157,7 +170,7 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
         lm.x = (const uint4*)x_t; lm.v = (const uint4*)v; lm.slot = p->slot; lm.n_edit = p->n_edit;
         lm.x_e = (uint4*)p->x_e; lm.v_e = (uint4*)p->v_e; lm.v_avd = (uint4*)p->v_avd; lm.x_out = (uint4*)p->x_out;
         lm.N = N; lm.Ne_cap = p->ne_cap; lm.cpr = C / 8;
-        // rows taken along: the attention reads K and V themselves, only the queries are gathered
+        // rows taken along: the attention reads K and V themselves, only the queries are gathered (see the kernel)
         RowCopyPairs rows = {};
         rows.p[0] = RowCopyPair{(const uint4*)q_full, (uint4*)p->q_e};
         rows.p[1] = RowCopyPair{(const uint4*)k_full, (uint4*)p->k_fresh};
@@ -166,10 +179,10 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
         RowCopyPairs kept = {};
         kept.p[0] = RowCopyPair{(const uint4*)k_full, (uint4*)p->k_cache};
         kept.p[1] = RowCopyPair{(const uint4*)v_full, (uint4*)p->v_cache};
-        const int n_kept = store_cache && !along ? 2 : 0;
         const int kept_blocks = (int)((n_full * row_cpr + per_block - 1) / per_block);
         const int lat_blocks = (int)((lat_chunks + kCopyThreads - 1) / kCopyThreads);
         const int row_blocks = (int)((q_cap * row_cpr + per_block - 1) / per_block);
+        const int tail_blocks = !store_cache ? 0 : !along ? 2 * kept_blocks : kApartBlocks;
         cudaError_t e = cudaSuccess;
         for (int b0 = 0; b0 < B && e == cudaSuccess; b0 += kReqChunk) {
             const int nb = B - b0 < kReqChunk ? B - b0 : kReqChunk;
@@ -178,11 +191,11 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
                 a.v[i] = -(dt[b0 + i] * scale[b0 + i]);      // x - (dt * scale) * v, the product formed in fp32 first
                 u.v[i] = -dt_unedited[b0 + i];
             }
-            e = launch_overlapped(region_step_move_kernel, dim3(lat_blocks + n_pairs * row_blocks + n_kept * kept_blocks, nb),
+            e = launch_overlapped(region_step_move_kernel, dim3(lat_blocks + n_pairs * row_blocks + tail_blocks, nb),
                                   dim3(kCopyThreads), 0,
                                   st, lm, a, u, b0, lat_blocks, rows, n_pairs, row_blocks > 0 ? row_blocks : 1, p->query_rows,
-                                  p->n_q, n_full, q_cap, (int)row_cpr, kept, kept_blocks, p->cache_rows, p->n_cache,
-                                  p->dev_status);
+                                  p->n_q, n_full, q_cap, (int)row_cpr, kept, kept_blocks, along, tail_blocks, p->cache_rows,
+                                  p->n_cache, p->dev_status);
         }
         if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
     }
@@ -193,10 +206,11 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
         if (p->workspace_bytes < need) return REGIONE_WORKSPACE_TOO_SMALL;
         const float sm = 1.0f / sqrtf((float)D);
         if (along) {
-            CacheStore cs;
+            CacheStore cs = {};
             cs.keep_rows = p->cache_rows; cs.n_keep = p->n_cache; cs.cap = n_full;
             cs.k_cache = p->k_cache; cs.v_cache = p->v_cache;
-            return launch_region_attention_tc(p->q_e, k_full, v_full, nullptr, nullptr, p->n_q, p->n_rows, nullptr, B, q_cap,
+            cs.all_rows = n_full; cs.k_apart = p->k_fresh; cs.v_apart = p->v_fresh;
+            return launch_region_attention_tc(p->q_e, k_full, v_full, nullptr, nullptr, p->n_q, p->n_q, p->n_cache, B, q_cap,
                                               n_full, 0, H, D, sm, p->o_full, p->query_rows, n_full, p->workspace,
                                               p->workspace_bytes, p->dev_status, st, &cs);
         }

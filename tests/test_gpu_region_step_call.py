@@ -83,3 +83,30 @@ def test_requests_that_sit_out_and_requests_in_a_batch_of_three():
         for name in ("mask", "slot", "n_edit", "x_e", "v_e", "v_avd", "x_out", "k_cache", "v_cache"):
             assert torch.equal(getattr(one, name), getattr(sep, name)), name
         assert_close(host_f64(one.o_full), host_f64(sep.o_full), "attention rows")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("H,grid,n_text,ne_cap", [
+    (3, (24, 24), 20, 256),      # few items: shared by clusters
+    (24, (30, 30), 30, 512),     # shares of the cost axis
+])
+@pytest.mark.parametrize("membership", [binding.ROWS_EDITED_QUERIES, binding.ROWS_PAPER])
+def test_storing_step_with_more_edited_tokens_than_the_capacity_holds(D, H, grid, n_text, ne_cap, membership):
+    """A request whose edited tokens do not fit attends over the rows of its lists alone (the dropped tokens' keys are
+    neither fresh nor cached), beside one that fits and attends over K and V in place."""
+    import torch
+    wl, lat, x, qkv = _inputs(2, grid, n_text, H, D, 0.9)
+    x[0][1, 200:] = x[2][1, 200:]                # request 1: the tokens from 200 on equal their reference, v = 0
+    x[1][1, 200:] = 0
+    shp = StepShapes(2, wl.n_img, n_text, wl.n_ref, wl.channels, H, D, ne_cap, binding.METRIC_COSINE, wl.threshold, membership)
+    assert 16 * (shp.q_cap - 64) >= shp.n_full   # the attention reads K and V in place
+    one, sep = RegionStep(shp), RegionStep(shp)
+    one.run(*x, *qkv, lat["t"], 0.97, 0.1, 0.2)
+    _separate(sep, x, qkv, lat["t"], 0.97, 0.1, 0.2, True)
+    torch.cuda.synchronize()
+    assert int(one.n_edit[0]) > ne_cap >= int(one.n_edit[1]) > 0
+    assert int(one.dev_status[0]) == int(sep.dev_status[0]) == binding.DEV_BOUNDS
+    for name in ("n_q", "n_cache", "query_rows", "cache_rows", "k_cache", "v_cache", "q_e", "x_out"):
+        assert torch.equal(getattr(one, name), getattr(sep, name)), name
+    for b in range(2):
+        assert_close(host_f64(one.o_full[b]), host_f64(sep.o_full[b]), f"attention rows, request {b}")
