@@ -336,8 +336,8 @@ int regione_region_attention_scatter(const regione_bf16* q,
  * x_t, v, ref bf16 [B, N, C]; q_full, k_full, v_full bf16 [B, n_full, H, D]; t, scale, dt, dt_unedited host
  * arrays [B] (NaN: the request sits that operation out, as in the single calls).
  * store_cache != 0: with enough queries beside the keys the attention reads K and V where they are (fresh and
- * cached rows together are all of them), the cache receives its rows in the same launch, and k_fresh and v_fresh
- * are not written; with fewer the rows are copied ahead of it.  A request whose edited tokens exceed the capacity
+ * cached rows together are all of them), and the cache, k_fresh and v_fresh receive their rows in the same launch;
+ * with fewer the rows are copied ahead of it.  A request whose edited tokens exceed the capacity
  * (REGIONE_DEV_BOUNDS) has its rows copied ahead too: the dropped tokens' keys are in neither list, so nothing attends
  * to them.  Both parts have to be called with the same value.
  * parts: REGIONE_STEP_MOVES (everything up to the attention) | REGIONE_STEP_ATTENTION.

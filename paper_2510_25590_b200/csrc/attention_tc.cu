@@ -199,15 +199,17 @@ struct AttnParams {
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
 };
 
-// Cache refresh fused into a full step: the rows keep_rows[b, 0..n_keep[b]) (ascending) of the K and V
-// that the launch attends over are also written to k_store / v_store [B, store_cap, H, D].  A parameter of
-// its own, of the kernel that refreshes the cache only: the plain attention kernel's parameters do not grow.
+// Cache refresh fused into a full step: the rows rows[l][b, 0..n[l][b]) (ascending) of the K and V that the launch
+// attends over are also written to dst[2l], dst[2l + 1] [B, cap[l], H, D], l < n_lists: the rows that the cache
+// retains, and in a region step the recomputed rows.  A parameter of its own, of the kernel that refreshes the cache
+// only: the plain attention kernel's parameters do not grow.
 struct StoreParams {
-    const int32_t* keep_rows;
-    const int32_t* n_keep;
-    int store_cap, src_cap;             // rows per request of the cache and of the sources
+    const int32_t* rows[2];
+    const int32_t* n[2];
+    int cap[2];
+    int n_lists, src_cap;               // (rows per request of the sources)
     const uint8_t* src[2];              // K, V [B, src_cap, H, D]
-    uint8_t* dst[2];
+    uint8_t* dst[4];
 };
 
 // ---- the plan every CTA (and the merge kernel) derives from the device-side counts ------------
@@ -962,7 +964,7 @@ __device__ __forceinline__ void merge_shares(const AttnParams& p, const SegInfo&
 // no registers, few issue slots and no time of the tensor cores, and the warp may block on them.  (A first version
 // ran them from the producer warp between its loads: every wait for a slot delayed a key tile, and 194 MB of copies
 // cost the attention of 819 queries as much as a store kernel ahead of it.)  The launch's rows (K of every request,
-// then V) are cut into equal contiguous shares, one per CTA, whatever attention work the CTA has.  An item is one
+// then V, of one list and then the other) are cut into equal contiguous shares, one per CTA, whatever attention work the CTA has.  An item is one
 // row, or a slot's length of it where a row is longer than that; a batch is up to `per_unit` consecutive items of one
 // request, lane i moving item i.  Beside the walks one batch at a time fills the corner of shared memory that is left
 // (5 rows of 24 x 128): the warp gets few issue slots there, and several slots of a row each with the same number of
@@ -974,19 +976,19 @@ struct CachePump {
     int row_bytes, item_bytes, per_row; // items per row
     uint32_t slots;                     // shared-memory address of slot 0
     int n_slots, slot_bytes, per_unit;
-    int x, b, i, run, live_rows;        // cursor of the loads: tensor, request, item, items of the run, source rows
+    int x, b, i, run, live_rows;        // cursor of the loads: destination, request, item, items of the run, source rows
     int left;                           // items not yet loaded
     int head, tail;                     // units loaded / stored through the present slots
     int win;                            // first item of the window of list entries held, one per lane:
     int row, before;                    // the entry of item win + lane and the one ahead of it,
     int row_next, before_next;          // the same for the window behind it (fetched long before it is needed)
 
-    __device__ __forceinline__ int kept(int req, bool report) const {
-        const int nk = sp->n_keep[req];
-        if (p->all_rows > 0 && rows_apart(p->n_q[req], nk, p->Nq_cap, p->all_rows)) return 0;      // (copied ahead)
-        if (nk >= 0 && nk <= sp->store_cap) return nk;
+    __device__ __forceinline__ int kept(int list, int req, bool report) const {
+        if (p->all_rows > 0 && rows_apart(p->n_q[req], sp->n[0][req], p->Nq_cap, p->all_rows)) return 0;   // (copied ahead)
+        const int nk = sp->n[list][req], cap = sp->cap[list];
+        if (nk >= 0 && nk <= cap) return nk;
         if (report && blockIdx.x == 0) record_status(p->dev_status, REGIONE_DEV_BOUNDS);
-        return nk < 0 ? 0 : sp->store_cap;
+        return nk < 0 ? 0 : cap;
     }
     __device__ __forceinline__ int source_rows(int req) const {
         return p->all_rows > 0 ? p->all_rows : min(p->n_fresh[req], sp->src_cap);
@@ -996,7 +998,7 @@ struct CachePump {
     __device__ __forceinline__ void open_run() {
         for (;;) {
             live_rows = source_rows(b);
-            run = live_rows > 0 ? kept(b, false) * per_row : 0;
+            run = live_rows > 0 ? kept(x >> 1, b, false) * per_row : 0;
             if (i < run) return;
             i -= run;
             if (++b == p->B) { b = 0; ++x; }
@@ -1006,7 +1008,7 @@ struct CachePump {
     __device__ __forceinline__ void fetch(int first, int lane, int& r, int& ahead) const {
         r = ahead = -1;
         if (first + lane < min(run, i + left)) {
-            const int32_t* keep = sp->keep_rows + (size_t)b * sp->store_cap;
+            const int32_t* keep = sp->rows[x >> 1] + (size_t)b * sp->cap[x >> 1];
             const int j = row_of(first + lane);
             r = keep[j];
             if (j > 0) ahead = keep[j - 1];
@@ -1034,10 +1036,11 @@ struct CachePump {
         per_row = (row_bytes + longest - 1) / longest;
         item_bytes = min(row_bytes, longest);
         long long total = 0;
-        for (int r = 0; r < prm.B; ++r) {
-            const int nk = kept(r, lane == 0);
-            if (source_rows(r) > 0) total += 2LL * nk * per_row;
-        }
+        for (int l = 0; l < s.n_lists; ++l)
+            for (int r = 0; r < prm.B; ++r) {
+                const int nk = kept(l, r, lane == 0);
+                if (source_rows(r) > 0) total += 2LL * nk * per_row;
+            }
         const long long per = (total + gridDim.x - 1) / gridDim.x, first = per * blockIdx.x;
         left = (int)max(0LL, min(per, total - first));
         x = b = 0;
@@ -1079,13 +1082,13 @@ struct CachePump {
         if (lane == 0) {
             ctrl->copy_valid[slot] = valid;
             ctrl->copy_item[slot] = i;
-            ctrl->copy_dst[slot] = sp->dst[x] + (size_t)b * sp->store_cap * row_bytes;
+            ctrl->copy_dst[slot] = sp->dst[x] + (size_t)b * sp->cap[x >> 1] * row_bytes;
             ptx::mbar_arrive_expect_tx(bar, unit_bytes);
         }
         __syncwarp();
         if (bytes > 0)
             ptx::bulk_load(slots + slot * slot_bytes + lane * item_bytes,
-                           sp->src[x] + ((size_t)b * sp->src_cap + my_row) * row_bytes + off, bytes, bar);
+                           sp->src[x & 1] + ((size_t)b * sp->src_cap + my_row) * row_bytes + off, bytes, bar);
         ++head;
         left -= n;
         i += n;
@@ -1935,9 +1938,15 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
     prm.timeout_cycles = kTimeoutCycles;
     StoreParams sp = {};
     if (store != nullptr) {
-        sp.keep_rows = store->keep_rows; sp.n_keep = store->n_keep; sp.store_cap = store->cap; sp.src_cap = Nf_cap;
+        sp.rows[0] = store->keep_rows; sp.n[0] = store->n_keep; sp.cap[0] = store->cap; sp.src_cap = Nf_cap;
         sp.src[0] = reinterpret_cast<const uint8_t*>(k_fresh); sp.src[1] = reinterpret_cast<const uint8_t*>(v_fresh);
         sp.dst[0] = reinterpret_cast<uint8_t*>(store->k_cache); sp.dst[1] = reinterpret_cast<uint8_t*>(store->v_cache);
+        sp.n_lists = 1;
+        if (all_rows > 0) {
+            sp.rows[1] = out_rows; sp.n[1] = n_q; sp.cap[1] = Nq_cap;
+            sp.dst[2] = reinterpret_cast<uint8_t*>(store->k_apart); sp.dst[3] = reinterpret_cast<uint8_t*>(store->v_apart);
+            sp.n_lists = 2;
+        }
     }
     const size_t rows = slot_rows(lp, B, H);
     prm.part_o = reinterpret_cast<float*>(workspace);

@@ -97,12 +97,13 @@ struct CacheStore {
     int cap;
     uint16_t* k_cache;          // dev [B, cap, H, D]
     uint16_t* v_cache;
-    // > 0 (the region step): the queries' rows and the kept rows are parts of K and V of this many rows.  A request whose
-    // two lists name all of them attends over K and V in place; any other (see rows_apart) over the rows of its lists,
-    // which the caller has copied to k_cache / v_cache and to k_apart / v_apart [B, Nq_cap, H, D].
+    // > 0 (the region step): the queries' rows (out_rows, ascending) and the kept rows are parts of K and V of this many
+    // rows.  A request whose two lists name all of them attends over K and V in place, and the launch copies the rows
+    // of both lists; any other (see rows_apart) attends over the rows of its lists, which the caller has copied to
+    // k_cache / v_cache and to k_apart / v_apart [B, Nq_cap, H, D].
     int all_rows;
-    const uint16_t* k_apart;
-    const uint16_t* v_apart;
+    uint16_t* k_apart;
+    uint16_t* v_apart;
 };
 
 // Whether the recomputed and the cached rows of a request are not all of its rows: more tokens were edited than the

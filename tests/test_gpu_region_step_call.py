@@ -106,7 +106,29 @@ def test_storing_step_with_more_edited_tokens_than_the_capacity_holds(D, H, grid
     torch.cuda.synchronize()
     assert int(one.n_edit[0]) > ne_cap >= int(one.n_edit[1]) > 0
     assert int(one.dev_status[0]) == int(sep.dev_status[0]) == binding.DEV_BOUNDS
-    for name in ("n_q", "n_cache", "query_rows", "cache_rows", "k_cache", "v_cache", "q_e", "x_out"):
+    for name in ("n_q", "n_cache", "query_rows", "cache_rows", "k_cache", "v_cache", "q_e", "x_out", "k_fresh",
+                 "v_fresh"):
         assert torch.equal(getattr(one, name), getattr(sep, name)), name
     for b in range(2):
         assert_close(host_f64(one.o_full[b]), host_f64(sep.o_full[b]), f"attention rows, request {b}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("H,grid,n_text,ratio", [(2, (24, 24), 20, 0.3), (24, (30, 30), 30, 0.5), (70, (16, 16), 16, 1.0)])
+@pytest.mark.parametrize("membership", [binding.ROWS_EDITED_QUERIES, binding.ROWS_PAPER])
+def test_storing_step_leaves_its_fresh_rows_too(D, H, grid, n_text, ratio, membership):
+    """k_fresh and v_fresh after a step whose attention reads K and V in place: rows of this step, those behind the
+    live ones as they were.  Row lengths below and above what one copy moves."""
+    import torch
+    wl, lat, x, qkv = _inputs(2, grid, n_text, H, D, ratio)
+    shp = StepShapes(2, wl.n_img, n_text, wl.n_ref, wl.channels, H, D, wl.n_img, binding.METRIC_COSINE, wl.threshold, membership)
+    assert 16 * (shp.q_cap - 64) >= shp.n_full
+    one, sep = RegionStep(shp), RegionStep(shp)
+    for s in (one, sep):
+        s.k_fresh.fill_(-3.0); s.v_fresh.fill_(-3.0)
+    one.run(*x, *qkv, lat["t"], 0.97, 0.1, 0.2)
+    _separate(sep, x, qkv, lat["t"], 0.97, 0.1, 0.2, True)
+    torch.cuda.synchronize()
+    assert int(one.dev_status[0]) == 0
+    for name in ("k_fresh", "v_fresh", "k_cache", "v_cache", "q_e"):
+        assert torch.equal(getattr(one, name), getattr(sep, name)), name
