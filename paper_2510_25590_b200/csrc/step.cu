@@ -150,12 +150,15 @@ extern "C" int regione_region_step(const regione_step_plan* p, const regione_bf1
     for (const void* a : wide)
         if (!aligned16(a)) return REGIONE_INVALID_ARG;
     if ((D != 64 && D != 128) || (C & 7) != 0 || B > 65535 || H > 65535) return REGIONE_UNSUPPORTED;
-    const int n_full = p->n_text + N + p->n_ref;
-    const int q_cap = p->ne_cap + (p->membership == REGIONE_ROWS_PAPER ? p->n_text : 0);
+    const long long n_full_ll = (long long)p->n_text + N + p->n_ref;
+    const long long q_cap_ll = (long long)p->ne_cap + (p->membership == REGIONE_ROWS_PAPER ? p->n_text : 0);
     const long long lat_chunks = (long long)N * (C / 8), row_cpr = (long long)H * D / 8;
     const long long per_block = (long long)kCopyThreads * kUnroll;
-    if (lat_chunks + kCopyThreads >= 0x7fffffffLL || (long long)n_full * row_cpr + per_block >= 0x7fffffffLL)
+    // (the copies index the chunks of a request's rows in 32 bits; ne_cap may exceed N, so neither bounds the other)
+    if (lat_chunks + kCopyThreads >= 0x7fffffffLL || (long long)p->ne_cap * (C / 8) >= 0x7fffffffLL ||
+        (n_full_ll > q_cap_ll ? n_full_ll : q_cap_ll) * row_cpr + per_block >= 0x7fffffffLL)
         return REGIONE_UNSUPPORTED;
+    const int n_full = (int)n_full_ll, q_cap = (int)q_cap_ll;
     if (B == 0) return REGIONE_OK;
     cudaStream_t st = (cudaStream_t)stream;
     const bool along = store_cache && q_cap > 0 && takes_rows_along(q_cap, n_full);

@@ -119,3 +119,21 @@ def test_avd_step_matches_oracle():
             assert r_lib == r_orc and abs(p_lib - p_orc) < 1e-15
     with pytest.raises(binding.RegionEError):
         binding._check(binding.load().regione_avd_step(None, 0.1, 1.0, 0.1, None), "avd")
+
+
+def test_region_step_refuses_sizes_its_copies_cannot_index():
+    """The copies index the 16-byte chunks of a request's rows in 32 bits: the query capacity, which may exceed the
+    number of image tokens, is bounded like the joint sequence.  (Fake addresses: nothing may be launched.)"""
+    def plan(**sizes):
+        p = binding.StepPlan(**{**dict(B=1, N=64, n_text=4, n_ref=64, C=16, H=24, D=128, ne_cap=64), **sizes})
+        for name, kind in binding.StepPlan._fields_:
+            if kind is ctypes.c_void_p:
+                setattr(p, name, 4096)
+        return p
+    t1, fake = (ctypes.c_float * 1)(0.5), [4096] * 6
+    call = lambda p: binding.load().regione_region_step(p, *fake, t1, t1, t1, t1, 1, 1, None)
+    assert call(plan(ne_cap=5_600_000)) == binding.UNSUPPORTED          # 5.6e6 * 384 chunks > 2^31
+    assert call(plan(ne_cap=2 ** 31 - 1, membership=1)) == binding.UNSUPPORTED
+    assert call(plan(n_ref=5_600_000)) == binding.UNSUPPORTED
+    assert call(plan(N=2 ** 30, C=16)) == binding.UNSUPPORTED
+    assert call(plan(C=12)) == binding.UNSUPPORTED
