@@ -77,6 +77,10 @@ class RegionEError(RuntimeError):
     pass
 
 
+class ShapeError(RegionEError):
+    """A tensor whose shape is not the one that a plan was made for."""
+
+
 _lib = None
 
 
@@ -370,7 +374,7 @@ def _shaped(t, shape, name):
     """Address of a contiguous bf16 CUDA tensor of the given shape."""
     p = _ptr(t, _torch().bfloat16, name)
     if t.shape != shape:
-        raise RegionEError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
+        raise ShapeError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     return p
 
 

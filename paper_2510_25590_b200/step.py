@@ -81,12 +81,12 @@ class RegionStep:
         self.x_out = z(B, N, C)
         self.dev_status = z(1, dt=i32)
         self.n_rows = torch.full((B,), shp.n_full, dtype=i32, device=device)
-        self.workspace = None
-        self.workspace = torch.empty(max(binding.region_step_workspace(self._step_plan()), 256), dtype=torch.uint8,
+        self.workspace = torch.empty(max(binding.region_step_workspace(self._new_plan()), 256), dtype=torch.uint8,
                                      device=device)
         self.launches = 0                 # operations of the sequence run so far (8 per step, 7 without the store)
         self.kernel_launches = 0          # kernels launched so far, at least (a fourth merges cut items in some shapes)
         self.attention_events = None      # optional (start, stop) pair recorded around the attention
+        self._step_plan()
 
     _BUFFERS = ("mask", "edit_idx", "keep_idx", "slot", "n_edit", "query_rows", "n_q", "cache_rows", "n_cache", "n_rows",
                 "x_e", "v_e", "v_avd", "x_out", "q_e", "k_fresh", "v_fresh", "k_cache", "v_cache", "o_full", "workspace",
@@ -95,33 +95,108 @@ class RegionStep:
     def __setattr__(self, name, value):
         object.__setattr__(self, name, value)
         if name in self._BUFFERS or name == "shp":
-            object.__setattr__(self, "_plan", None)      # the plan names this object's buffers: made anew
+            object.__setattr__(self, "_plan_of", None)   # the plan names this object's buffers: made anew
+
+    def _forms(self):
+        """Type and shape of every buffer as the plan lays them out (the workspace's size is the plan's own)."""
+        import torch
+        s = self.shp
+        i32, bf = torch.int32, torch.bfloat16
+        per_token, per_request = (s.B, s.N), (s.B,)
+        lat_e, rows_q, rows = (s.B, s.ne_cap, s.C), (s.B, s.q_cap, s.H, s.D), (s.B, s.n_full, s.H, s.D)
+        return dict(mask=(torch.uint8, per_token), edit_idx=(i32, per_token), keep_idx=(i32, per_token),
+                    slot=(i32, per_token), n_edit=(i32, per_request), n_q=(i32, per_request), n_cache=(i32, per_request),
+                    n_rows=(i32, per_request), query_rows=(i32, (s.B, s.q_cap)), cache_rows=(i32, (s.B, s.n_full)),
+                    x_e=(bf, lat_e), v_e=(bf, lat_e), v_avd=(bf, lat_e), x_out=(bf, (s.B, s.N, s.C)), q_e=(bf, rows_q),
+                    k_fresh=(bf, rows_q), v_fresh=(bf, rows_q), k_cache=(bf, rows), v_cache=(bf, rows), o_full=(bf, rows))
+
+    def _new_plan(self):
+        s = self.shp
+        return binding.StepPlan(s.B, s.N, s.n_text, s.n_ref, s.C, s.H, s.D, s.ne_cap, int(s.metric), int(s.membership),
+                                float(s.threshold))
 
     def _step_plan(self):
-        if self._plan is None:
-            s = self.shp
-            p = binding.StepPlan(s.B, s.N, s.n_text, s.n_ref, s.C, s.H, s.D, s.ne_cap, int(s.metric), int(s.membership),
-                                 float(s.threshold))
-            for name in self._BUFFERS:
-                t = getattr(self, name)
-                setattr(p, name, None if t is None else t.data_ptr())
-            p.workspace_bytes = 0 if self.workspace is None else self.workspace.numel()
-            object.__setattr__(self, "_plan", p)
-        self._plan.metric, self._plan.threshold = int(self.shp.metric), self.shp.threshold
+        """The plan of the one-call step, or None where a buffer is not of the form it stands for.  It holds addresses,
+        so it is compared with the buffers and the sizes as they are now, and made anew when one of them has changed."""
+        s, d = self.shp, self.__dict__
+        of = ([None if d[n] is None else d[n].data_ptr() for n in self._BUFFERS],
+              (s.B, s.N, s.n_text, s.n_ref, s.C, s.H, s.D, s.ne_cap, s.membership))
+        if self._plan_of != of:
+            plan = None
+            if all(d[n] is not None and d[n].is_cuda and d[n].dtype == dtype and tuple(d[n].shape) == shape and
+                   d[n].is_contiguous() for n, (dtype, shape) in self._forms().items()) and \
+               all(d[n] is None or d[n].is_cuda and d[n].is_contiguous() for n in ("workspace", "dev_status")):
+                plan = self._new_plan()
+                for name, at in zip(self._BUFFERS, of[0]):
+                    setattr(plan, name, at)
+                ws = self.workspace
+                plan.workspace_bytes = 0 if ws is None else ws.numel() * ws.element_size()
+            object.__setattr__(self, "_plan", plan)
+            object.__setattr__(self, "_plan_of", of)
+        if self._plan is not None:
+            self._plan.metric, self._plan.threshold = int(s.metric), s.threshold
         return self._plan
 
     def run(self, x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, stream=None,
             store_cache=True):
         """One region-aware step.  ``store_cache=False`` leaves the cache as the last storing call wrote
         it (Algorithm 1 refreshes it at full steps only; valid while the partition is unchanged)."""
-        args = (self._step_plan(), x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, store_cache)
-        if self.attention_events is None:
-            binding.region_step(*args, stream=stream)
-        else:
-            binding.region_step(*args, parts=binding.STEP_MOVES, stream=stream)
-            self.attention_events[0].record(stream)
-            binding.region_step(*args, parts=binding.STEP_ATTENTION, stream=stream)
-            self.attention_events[1].record(stream)
+        args = (x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, store_cache)
+        plan, B, events = self._step_plan(), binding, self.attention_events
+        if plan is None:
+            return self._run_calls(*args, stream)
+        try:
+            B.region_step(plan, *args, parts=B.STEP_MOVES | (0 if events else B.STEP_ATTENTION), stream=stream)
+        except B.ShapeError:                             # (nothing has been launched)
+            s, rows = self.shp, lambda t: len(t.shape) > 2 and t.shape[0] == s.B and t.shape[2:].numel() == s.H * s.D
+            if x_t.shape != (s.B, s.N, s.C) or v.shape != x_t.shape or ref.numel() != x_t.numel() or \
+                    not (rows(q_full) and rows(k_full) and rows(v_full)):
+                raise
+            return self._run_calls(*args, stream)
+        if events:
+            events[0].record(stream)
+            B.region_step(plan, *args, parts=B.STEP_ATTENTION, stream=stream)
+            events[1].record(stream)
         self.launches += 8 if store_cache else 7
         self.kernel_launches += 3
+        return self.x_out
+
+    # buffers that may hold another number of rows per request than planned, those that share it together
+    _ROWS = (("x_e", "v_e", "v_avd"), ("q_e", "k_fresh", "v_fresh", "query_rows"), ("k_cache", "v_cache", "cache_rows"),
+             ("o_full",))
+
+    def _check_shapes(self):
+        free = {n: group[0] for group in self._ROWS for n in group}
+        for n, (_, shape) in self._forms().items():
+            got = tuple(getattr(self, n).shape)
+            if n in free and len(got) == len(shape) and (n != "cache_rows" or self.shp.B > 1):
+                shape = (shape[0], getattr(self, free[n]).shape[1], *shape[2:])
+            if got != shape and (n != "cache_rows" or len(got) != 2 or got[0] != shape[0] or self.shp.B > 1):
+                raise binding.RegionEError(f"{n} must have shape {shape}, got {got}")
+
+    def _run_calls(self, x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, store_cache, stream):
+        """The step as separate library calls, which take their sizes from the tensors: for inputs and buffers of other
+        shapes than the plan's (rows as one dimension, a larger output, a cache that holds fewer rows)."""
+        s, st, b = self.shp, self.dev_status, binding
+        self._check_shapes()
+        b.partition_rows(x_t, v, ref, t, s.metric, s.threshold, self.mask, self.edit_idx, self.keep_idx, self.slot,
+                         self.n_edit, s.n_text, s.n_ref, s.membership, self.query_rows, self.n_q, self.cache_rows,
+                         self.n_cache, dev_status=st, stream=stream)
+        b.gather_multi([x_t, v], self.edit_idx, self.n_edit, [self.x_e, self.v_e], dev_status=st, stream=stream)
+        b.velocity_decay(self.v_e, scale, dt, self.x_e, self.n_edit, v_cache_out=self.v_avd, dev_status=st, stream=stream)
+        b.merge(x_t, v, self.x_e, self.slot, dt_unedited, self.x_out, dev_status=st, stream=stream)
+        if store_cache:
+            b.rikv_store(k_full, v_full, self.cache_rows, self.n_cache, self.k_cache, self.v_cache, dev_status=st,
+                         stream=stream)
+        b.gather_multi([q_full, k_full, v_full], self.query_rows, self.n_q, [self.q_e, self.k_fresh, self.v_fresh],
+                       dev_status=st, stream=stream)
+        if self.attention_events is not None:
+            self.attention_events[0].record(stream)
+        b.region_attention_scatter(self.q_e, self.k_fresh, self.v_fresh, self.k_cache, self.v_cache, self.n_q, self.n_q,
+                                   self.n_cache, self.o_full, self.query_rows, workspace=self.workspace, dev_status=st,
+                                   stream=stream)
+        if self.attention_events is not None:
+            self.attention_events[1].record(stream)
+        self.launches += 8 if store_cache else 7
+        self.kernel_launches += 7 if store_cache else 6
         return self.x_out
