@@ -148,7 +148,7 @@ struct AttnCtrl {
     int redo;                   // a row outgrew the reference maximum of its first key tile
     SegInfo seg[2];
     uint64_t peers_ready;       // item shared by a cluster: every CTA's partial rows are in its shared memory
-    uint64_t peers_done;        // ... and have been read by every CTA
+    uint64_t peers_done;        // ... and have been read by every CTA (launch that refreshes the cache)
     int walks_done;             // cache refresh: the walks are over, every tile of shared memory is idle
     // cache refresh: a slot's rows have landed; where they go, and which of them are to be stored
     uint64_t copy_full[kCopySlots];
@@ -1513,10 +1513,12 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             if (ok) ok = wait_bar_cluster(ready, abort_flag, p.dev_status, p.timeout_cycles);
             if (ok) merge_cluster<D>(p, ctrl->seg[0], smem, warp, lane);
         }
-        walk_sync();
-        if (warp == 0 && lane < p.cluster && !*abort_flag) ptx::mbar_arrive_cluster(ptx::map_rank(done, lane));
-        // (a CTA's shared memory stays until every peer has read it)
-        if (!*abort_flag) wait_bar_cluster(done, abort_flag, p.dev_status, p.timeout_cycles);
+        if (STORE) {
+            // (the copies of rows take the tiles over, once every peer has read them)
+            walk_sync();
+            if (warp == 0 && lane < p.cluster && !*abort_flag) ptx::mbar_arrive_cluster(ptx::map_rank(done, lane));
+            if (!*abort_flag) wait_bar_cluster(done, abort_flag, p.dev_status, p.timeout_cycles);
+        }
     }
 
     // ================= teardown =================
@@ -1536,6 +1538,12 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     if (STORE && threadIdx.x == 0) {
         __threadfence_block();
         *reinterpret_cast<volatile int*>(&ctrl->walks_done) = 1;
+    }
+    // A CTA's shared memory stays until no peer reads it or arrives on its barriers any more, also where a wait has run
+    // out: every wait above is bounded, so that all of the cluster's threads come here or have ended (the copying warp).
+    if (FORM == kMergeCluster) {
+        __syncwarp();
+        ptx::cluster_sync();
     }
 }
 
