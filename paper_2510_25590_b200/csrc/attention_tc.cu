@@ -150,6 +150,8 @@ struct AttnCtrl {
     uint64_t peers_ready;       // item shared by a cluster: every CTA's partial rows are in its shared memory
     uint64_t peers_done;        // ... and have been read by every CTA (launch that refreshes the cache)
     int walks_done;             // cache refresh: the walks are over, every tile of shared memory is idle
+    int copy_abort;             // cache refresh: a copy did not land in time.  Not abort_flag: that one changes only
+                                // while every role is between two barriers of a segment, so that all leave together
     // cache refresh: a slot's rows have landed; where they go, and which of them are to be stored
     uint64_t copy_full[kCopySlots];
     uint8_t* copy_dst[kCopySlots];
@@ -1052,7 +1054,7 @@ struct CachePump {
     }
     __device__ __forceinline__ bool store_oldest(int lane) {
         const int slot = n_slots > 1 ? tail & 1 : 0;
-        const bool landed = wait_bar(ptx::smem_addr(&ctrl->copy_full[slot]), (n_slots > 1 ? tail >> 1 : tail) & 1, &ctrl->abort_flag,
+        const bool landed = wait_bar(ptx::smem_addr(&ctrl->copy_full[slot]), (n_slots > 1 ? tail >> 1 : tail) & 1, &ctrl->copy_abort,
                                      p->dev_status, p->timeout_cycles);
         if (!__all_sync(0xffffffffu, landed)) return false;
         if ((ctrl->copy_valid[slot] >> lane) & 1u) {
@@ -1445,6 +1447,8 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         if (warp == kWarpCopy) {
             if constexpr (STORE) {
                 CachePump pump;
+                if (lane == 0) ctrl->copy_abort = 0;
+                __syncwarp();
                 pump.begin(p, sp, ctrl, D, Cfg::kCopyBytes / 4, lane);
                 if (!pump.run_all<D>(smem, lane)) {
                     // give copies that are still in flight time to land before shared memory is given back
