@@ -1425,7 +1425,8 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         ptx::tc_fence_before_sync();
         walk_sync();
         ptx::tc_fence_after_sync();
-        if (threadIdx.x < kNumBarriers) ptx::mbar_inval(ptx::smem_addr(&ctrl->q_full + threadIdx.x));
+        // (after a wait that ran out, loads and products may still be on their way to their barriers: those stay)
+        if (threadIdx.x < kNumBarriers && !*abort_flag) ptx::mbar_inval(ptx::smem_addr(&ctrl->q_full + threadIdx.x));
     };
     // what to do after a walk: repeat the segment (new mode) or go on
     auto repeat = [&](int& mode) {
