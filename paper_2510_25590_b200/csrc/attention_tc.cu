@@ -236,18 +236,21 @@ struct ReqShape {
     long long ticks_full, ticks_last, head_ticks, ticks;   // per full-pair item, last item, head, request
 };
 
+// (IN_PLACE: the launch may read K and V in place, see ReqShape::apart; 0.5 us a call for the launches that never do)
+template <bool IN_PLACE>
 __device__ __forceinline__ ReqShape req_shape(const AttnParams& p, int b, bool* bad = nullptr) {
     ReqShape r;
     int nq = p.n_q[b], nf = p.n_fresh[b], nc = p.n_cache == nullptr ? 0 : p.n_cache[b];      // (nullptr: no cached segment)
-    const int c_cap = p.all_rows > 0 ? p.all_rows : p.Nc_cap;
+    const bool in_place = IN_PLACE && p.all_rows > 0;
+    const int c_cap = in_place ? p.all_rows : p.Nc_cap;
     if (nq < 0 || nq > p.Nq_cap || nf < 0 || nf > p.Nf_cap || nc < 0 || nc > c_cap) {
         if (bad) *bad = true;
         nq = max(0, min(nq, p.Nq_cap));
         nf = max(0, min(nf, p.Nf_cap));
         nc = max(0, min(nc, c_cap));
     }
-    r.apart = p.all_rows > 0 && rows_apart(nq, nc, p.Nq_cap, p.all_rows);
-    if (p.all_rows > 0) {
+    r.apart = in_place && rows_apart(nq, nc, p.Nq_cap, p.all_rows);
+    if (in_place) {
         nf = r.apart ? nq : p.all_rows;
         nc = r.apart ? nc : 0;
     }
@@ -276,11 +279,12 @@ struct Plan {
     long long total, chunk;
 };
 
+template <bool IN_PLACE>
 __device__ __forceinline__ Plan plan_shares(const AttnParams& p, int grid, bool* bad = nullptr) {
     Plan pl;
     long long items = 0, ticks = 0, span = 0;      // span: first tick of an item's last step, at most
     for (int b = 0; b < p.B; ++b) {
-        const ReqShape r = req_shape(p, b, bad);
+        const ReqShape r = req_shape<IN_PLACE>(p, b, bad);
         items += r.items;
         ticks += r.ticks;
         if (r.np > 0) span = max(span, (long long)(r.np > 1 ? kTickPair : r.w_last) * (r.steps - 1));
@@ -327,15 +331,16 @@ __device__ __forceinline__ void item_slots(const Plan& pl, long long first_tick,
 }
 
 // Whole-item plan: the item with index `idx`.
+template <bool IN_PLACE>
 __device__ __forceinline__ Segment segment_whole(const AttnParams& p, long long idx) {
     Segment sg;
     long long base = 0;
     int b = 0;
-    ReqShape r = req_shape(p, 0);
+    ReqShape r = req_shape<IN_PLACE>(p, 0);
     while (idx >= base + r.items && b + 1 < p.B) {
         base += r.items;
         ++b;
-        r = req_shape(p, b);
+        r = req_shape<IN_PLACE>(p, b);
     }
     const long long item = idx - base;
     sg.b = b; sg.r = r;
@@ -349,16 +354,17 @@ __device__ __forceinline__ Segment segment_whole(const AttnParams& p, long long 
 }
 
 // Tick plan: the item that contains tick `pos`, and the steps of it that share `c` owns.
+template <bool IN_PLACE>
 __device__ __forceinline__ Segment segment_ticks(const AttnParams& p, const Plan& pl, long long pos,
                                                  int c) {
     Segment sg;
     long long base = 0;
     int b = 0;
-    ReqShape r = req_shape(p, 0);
+    ReqShape r = req_shape<IN_PLACE>(p, 0);
     while (pos >= base + r.ticks && b + 1 < p.B) {
         base += r.ticks;
         ++b;
-        r = req_shape(p, b);
+        r = req_shape<IN_PLACE>(p, b);
     }
     sg.b = b; sg.r = r;
     if (r.np == 0) {                                  // nothing left behind the last live request
@@ -1297,14 +1303,15 @@ struct ShareCursor {
     bool first;
     // The only segment of a CTA whose item is shared by a cluster: rank r of n takes the key tiles
     // [r * nt / n, (r + 1) * nt / n) (possibly none) and reads back its part of the rows.
+    template <bool IN_PLACE>
     __device__ __forceinline__ void of_cluster(const AttnParams& p, SegInfo* out, const int lane, bool* bad) {
         int idx = blockIdx.x / p.cluster;
         const int rank = blockIdx.x - idx * p.cluster;
-        ReqShape r = req_shape(p, 0, bad);
+        ReqShape r = req_shape<IN_PLACE>(p, 0, bad);
         int b = 0;
         while (b + 1 < p.B && idx >= p.H * r.np) {
             idx -= p.H * r.np;
-            r = req_shape(p, ++b, bad);
+            r = req_shape<IN_PLACE>(p, ++b, bad);
         }
         pos = hi = 0;
         first = false;
@@ -1317,13 +1324,14 @@ struct ShareCursor {
         out->nq = r.nq; out->nt_c = r.nt_c; out->nt = r.nt; out->nc = r.nc; out->nf = r.nf;
         out->j_first = rank * r.nt / p.cluster;
         out->n_tiles = (rank + 1) * r.nt / p.cluster - out->j_first;
-        out->item = 0; out->slot = rank; out->n_slots = p.cluster; out->apart = r.apart;
+        out->item = 0; out->slot = rank; out->n_slots = p.cluster;
+        if (IN_PLACE) out->apart = r.apart;
     }
     // The next live segment of the share into *out (out->live = 0 when the share ends).
-    template <int FORM>
+    template <int FORM, bool IN_PLACE>
     __device__ __forceinline__ void next(const AttnParams& p, SegInfo* out, const int lane) {
         while (pos < hi) {
-            const Segment it = pl.whole_items ? segment_whole(p, pos) : segment_ticks(p, pl, pos, my_share());
+            const Segment it = pl.whole_items ? segment_whole<IN_PLACE>(p, pos) : segment_ticks<IN_PLACE>(p, pl, pos, my_share());
             if (FORM == kMergeKernel && first && lane == 0) {
                 // tell the merge kernel which item the start of this share cuts
                 CutItem ci;
@@ -1340,7 +1348,7 @@ struct ShareCursor {
                 out->j_first = it.j_first; out->n_tiles = it.r.nt == 0 ? 0 : it.n_steps;
                 out->nt_c = it.r.nt_c; out->nt = it.r.nt; out->nc = it.r.nc; out->nf = it.r.nf;
                 out->item = (it.b * p.H + it.h) * p.P_cap + it.qp; out->slot = it.slot; out->n_slots = it.n_slots;
-                out->apart = it.r.apart;
+                if (IN_PLACE) out->apart = it.r.apart;
                 out->live = 1;
             }
             return;
@@ -1378,7 +1386,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         // neighbouring items, which share K/V tiles in L2; a share of steps is one contiguous range)
         bool bad = false;
         if constexpr (FORM == kMergeCluster) {
-            cur.of_cluster(p, &ctrl->seg[0], lane, &bad);
+            cur.of_cluster<STORE>(p, &ctrl->seg[0], lane, &bad);
             if (lane == 0) {
                 ctrl->seg[1].live = 0;
                 ptx::mbar_init(ptx::smem_addr(&ctrl->peers_ready), p.cluster);
@@ -1386,11 +1394,11 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
                 ptx::fence_barrier_init();
             }
         } else {
-        cur.pl = plan_shares(p, gridDim.x, &bad);
+        cur.pl = plan_shares<STORE>(p, gridDim.x, &bad);
         cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)my_share() * cur.pl.chunk;
         cur.first = true;
         cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
-        cur.next<FORM>(p, &ctrl->seg[0], lane);
+        cur.next<FORM, STORE>(p, &ctrl->seg[0], lane);
         }
         if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         if (lane == 0) ctrl->abort_flag = 0;
@@ -1468,7 +1476,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             } else if (warp == kWarpS) {
                 issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
                 // (the next segment is planned behind the last product, ahead of the end of this one)
-                if (FORM != kMergeCluster && mode == kWalk) cur.next<FORM>(p, &ctrl->seg[k ^ 1], lane);
+                if (FORM != kMergeCluster && mode == kWalk) cur.next<FORM, STORE>(p, &ctrl->seg[k ^ 1], lane);
             } else {
                 issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, lane, mode);
             }
