@@ -281,9 +281,13 @@ int regione_rikv_load_e4m3(const uint8_t* k_q, const uint8_t* v_q, const float* 
  * workspace       : dev, 256-byte aligned, at least
  *                   regione_region_attention_workspace(...) bytes.  It holds the
  *                   partial results of (request, head, query-tile pair) items whose
- *                   key range was shared between thread blocks, and a small table
- *                   naming those items; its contents need not be initialised and
- *                   mean nothing after the call.
+ *                   key range was shared between thread blocks, a small table
+ *                   naming those items and the flags by which the blocks hand them
+ *                   over; its contents need not be initialised and mean nothing
+ *                   after the call.  One exception: a call that recorded
+ *                   REGIONE_DEV_TIMEOUT and is repeated by a CUDA graph records it
+ *                   again, its results incomplete, until the graph is captured
+ *                   anew or the workspace is overwritten.
  * D must be 64 or 128.  bf16 inputs, fp32 accumulation, probabilities rounded
  * to bf16 before the second product.  With no key at all a row is zero.
  * The call enqueues two kernels (attention, then the merge of shared items; the

@@ -196,7 +196,8 @@ struct AttnParams {
     float2* part_ml;     // [B, H, P_cap, max_slots, 256]    (running max in the exp2 domain, sum)
     int cluster;         // kMergeCluster: CTAs that share an item; no workspace
     CutItem* cut;        // kMergeKernel: [grid] the item that the start of each share cuts
-    unsigned long long* ready;       // kMergeHere: [grid] `epoch`: the share's partial rows are in its slot (0: merged)
+    unsigned long long* ready;       // kMergeHere: [grid] `epoch`: the share's partial rows are in its slot (0: merged),
+                                     // and a word behind them, `epoch`: a launch of this epoch has timed out
     unsigned long long epoch;        // of this launch: what lies in the workspace otherwise is not equal to it
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
 };
@@ -531,19 +532,24 @@ enum WalkMode { kWalk, kMaxOnly, kExact };
 
 // ---- softmax / epilogue of one segment: thread = (query row, 64-key chunk) ----------------------------
 // Share of a CTA on the cost axis.  The first share of an item waits for the later ones, so shares are dealt
-// from the last block to the first: blocks become resident in the order of their indexes, and a block waits
-// only for blocks ahead of it, whatever else runs on the GPU.
+// from the last block to the first: blocks become resident in the order of their indexes on this GPU, and a block
+// waits only for blocks ahead of it, whatever else runs.  CUDA does not promise that order; were it another, a wait
+// for a block that cannot start would end with its bound and REGIONE_DEV_TIMEOUT.
 __device__ __forceinline__ int my_share() { return (int)gridDim.x - 1 - (int)blockIdx.x; }
 
-// Bounded wait of a warp for the partial rows of the n shares behind this CTA's (true: they are there).
+// Bounded wait of a warp for the partial rows of the n shares behind this CTA's (true: they are there).  A launch that
+// has timed out may have left flags of its epoch behind, and a graph repeats the launch with that epoch: the repetition
+// gives up as well, instead of merging what the flags no longer stand for.  (Asked here, beside the flags: at the start
+// of the launch the question cost 819 queries x 8704 keys 1.5 us.)
 __device__ __forceinline__ bool wait_shares(const AttnParams& p, int n, int lane, volatile int* abort_flag) {
-    bool there = lane >= n, gave_up = false;
+    const bool asks_failed = lane == 31;   // (the word behind the flags; n < 31)
+    bool there = lane >= n && !asks_failed, gave_up = false;
     if (!there) {
-        const unsigned long long* const flag = p.ready + my_share() + 1 + lane;
+        const unsigned long long* const word = p.ready + (asks_failed ? (int)gridDim.x : my_share() + 1 + lane);
         const long long t0 = clock64();
-        while (!(there = ptx::ld_acquire_u64(flag) == p.epoch) && !gave_up) {
+        while (!(there = (ptx::ld_acquire_u64(word) == p.epoch) != asks_failed) && !gave_up) {
             gave_up = *abort_flag != 0;
-            if (clock64() - t0 > p.timeout_cycles) {
+            if (asks_failed || clock64() - t0 > p.timeout_cycles) {
                 *abort_flag = 1;
                 record_status(p.dev_status, REGIONE_DEV_TIMEOUT);
                 gave_up = true;
@@ -1536,6 +1542,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
 
     // ================= teardown =================
     if (*abort_flag) {
+        if (FORM == kMergeHere && threadIdx.x == 0) p.ready[gridDim.x] = p.epoch;
         // give copies and MMAs that are still in flight time to land before tensor memory and
         // shared memory are given back
         const long long t0 = clock64();
@@ -1772,7 +1779,8 @@ size_t region_attention_tc_workspace(int B, int Nq_cap, int Nf_cap, int Nc_cap, 
     const LaunchPlan lp = plan_launch(B, Nq_cap, Nf_cap, Nc_cap, H);
     const size_t rows = slot_rows(lp, B, H);
     return ((rows * D * sizeof(float) + 255) & ~(size_t)255) +
-           ((rows * sizeof(float2) + 255) & ~(size_t)255) + (size_t)lp.grid * (sizeof(CutItem) + sizeof(unsigned long long));
+           ((rows * sizeof(float2) + 255) & ~(size_t)255) + (size_t)lp.grid * (sizeof(CutItem) + sizeof(unsigned long long)) +
+           sizeof(unsigned long long);
 }
 
 template <int D, bool STORE, int FORM>

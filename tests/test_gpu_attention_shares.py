@@ -60,3 +60,56 @@ def test_any_workspace_content_graphs_and_streams():
     assert int(status[0]) == 0
     for o in outs[1:]:
         assert torch.equal(o, outs[0])
+
+
+def _captured_epoch(graph):
+    """The number that tells a captured launch's flags from others': in the kernel's parameters, ahead of the bound of
+    its waits (4e9 cycles)."""
+    import ctypes
+    from cuda.bindings import driver
+    err, _, n = driver.cuGraphGetNodes(driver.CUgraph(graph.raw_cuda_graph()), 0)
+    assert int(err) == 0
+    err, nodes, n = driver.cuGraphGetNodes(driver.CUgraph(graph.raw_cuda_graph()), n)
+    assert int(err) == 0
+    kernels = [k for k in nodes if driver.cuGraphNodeGetType(k)[1] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL]
+    assert len(kernels) == 1                                   # merged by the first shares: no second kernel
+    err, params = driver.cuGraphKernelNodeGetParams(kernels[0])
+    assert int(err) == 0
+    at = (ctypes.c_void_p * 6).from_address(int(params.kernelParams))[5]      # (five tensor maps ahead of it)
+    words = (ctypes.c_uint64 * 18).from_address(at)
+    assert words[17] == 4_000_000_000
+    return words[16]
+
+
+def test_a_launch_that_timed_out_is_not_repeated_over_its_leftovers():
+    """A repetition by a graph has the epoch of the launch that timed out: told so by the workspace's last word, it
+    records the time-out again and merges nothing, whatever flags lie there; with the word overwritten it works as before."""
+    import torch
+    rng = np.random.default_rng(6)
+    H, D, n_q, n_c = 24, 128, 1000, 8000
+    r = lambda n: dev_bf16(_rand_bf16(rng, (1, n, H, D)))
+    q, kf, vf, kc, vc = r(n_q), r(n_q), r(n_q), r(n_c), r(n_c)
+    nq, nc = dev_i32([n_q]), dev_i32([n_c])
+    status, out = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros_like(q)
+    ws = torch.zeros(binding.region_attention_workspace(1, n_q, n_q, n_c, H, D), dtype=torch.uint8, device="cuda")
+    call = lambda: binding.region_attention(q, kf, vf, kc, vc, nq, nq, nc, out, workspace=ws, dev_status=status)
+    call()
+    want = out.clone()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    epoch = _captured_epoch(graph)
+    graph.instantiate()
+    last = torch.frombuffer(bytearray(int(epoch).to_bytes(8, "little")), dtype=torch.uint8).cuda()
+    for failed in (False, True, False):
+        out.fill_(-3.0)
+        status.zero_()
+        ws[-8:] = last if failed else 0
+        graph.replay()
+        torch.cuda.synchronize()
+        assert int(status[0]) == (binding.DEV_TIMEOUT if failed else 0)
+        assert failed or torch.equal(out, want)
+        rows = ((out == -3.0).all(-1) | (out == want).all(-1))                 # left out or as they should be
+        assert bool(rows.all()) and (not failed or bool((out == -3.0).all(-1).any()))
+    call()                                                     # (a launch of its own has another epoch)
+    assert torch.equal(out, want)
