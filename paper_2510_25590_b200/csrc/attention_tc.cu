@@ -242,17 +242,17 @@ template <bool IN_PLACE>
 __device__ __forceinline__ ReqShape req_shape(const AttnParams& p, int b, bool* bad = nullptr) {
     ReqShape r;
     int nq = p.n_q[b], nf = p.n_fresh[b], nc = p.n_cache == nullptr ? 0 : p.n_cache[b];      // (nullptr: no cached segment)
-    const bool in_place = IN_PLACE && p.all_rows > 0;
-    const int c_cap = in_place ? p.all_rows : p.Nc_cap;
+    const int all_rows = IN_PLACE ? p.all_rows : 0;
+    const int c_cap = all_rows > 0 ? all_rows : p.Nc_cap;
     if (nq < 0 || nq > p.Nq_cap || nf < 0 || nf > p.Nf_cap || nc < 0 || nc > c_cap) {
         if (bad) *bad = true;
         nq = max(0, min(nq, p.Nq_cap));
         nf = max(0, min(nf, p.Nf_cap));
         nc = max(0, min(nc, c_cap));
     }
-    r.apart = in_place && rows_apart(nq, nc, p.Nq_cap, p.all_rows);
-    if (in_place) {
-        nf = r.apart ? nq : p.all_rows;
+    r.apart = all_rows > 0 && nq + nc != all_rows;
+    if (all_rows > 0) {
+        nf = r.apart ? nq : all_rows;
         nc = r.apart ? nc : 0;
     }
     r.nq = nq; r.nf = nf; r.nc = nc;
