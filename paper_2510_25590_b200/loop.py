@@ -98,6 +98,22 @@ class _Group:
     have_cache: bool = False
 
 
+def _velocity(v, shape, name, region=False):
+    """Address of a velocity that the model returned.  One of all tokens may come without the batch dimension of a single
+    request; one of a region step holds its rows at the beginning of each request's, for a single request as many as it
+    likes (at least the edited tokens)."""
+    p = binding._ptr(v, binding._torch().bfloat16, name)
+    got = v.shape
+    if got != shape:
+        if region:
+            fits = shape[0] == 1 or got.numel() == shape[0] * shape[1] * shape[2]
+        else:
+            fits = got.numel() == shape[0] * shape[1] * shape[2] and shape[max(3 - len(got), 0):] == got
+        if not fits:
+            raise binding.RegionEError(f"{name} must have shape {shape}, got {tuple(got)}")
+    return p
+
+
 _NAN = float("nan")
 _MAX_RUN = 16                        # sampler steps that one update of X^E applies
 
@@ -150,12 +166,6 @@ class RegionELoop:
         p_all, p_st = self.n_all.data_ptr(), st.data_ptr()
         if x.shape != shape:
             raise b.RegionEError(f"x must have shape {shape}, got {tuple(x.shape)}")
-
-        def velocity(v, name):
-            p = ptr(v, bf, name)
-            if v.shape != shape:
-                raise b.RegionEError(f"{name} must have shape {shape}, got {tuple(v.shape)}")
-            return p
 
         def decay(p_v, scale, dts, p_target, p_keep, p_n):
             check(lib.regione_velocity_decay(p_v, floats(scale, B, "scale"), floats(dts, B, "dt"), p_target, p_keep, p_n,
@@ -236,7 +246,7 @@ class RegionELoop:
                                 t_full[r] = ts[g.k]
                     v = model.full(x, t_full, store)
                 tr.model_full_calls += 1
-                p_v = velocity(v, "v")
+                p_v = _velocity(v, shape, "v")
                 dts = spread([(g, ts[g.k] - ts[g.k + 1]) for g in full])
                 if hook is not None:
                     hook("euler_in", k0, dict(x=x, v=v, dt=listed(dts), active=members(full)))
@@ -289,7 +299,7 @@ class RegionELoop:
                                     t_e[r] = ts[g.k]
                             v_e = model.region(self.x_e, t_e, self.edit_idx, self.n_edit)
                         tr.model_region_calls += 1
-                        p_v, p_keep = velocity(v_e, "v_e"), p_vc
+                        p_v, p_keep = _velocity(v_e, shape, "v_e", region=True), p_vc
                     if hook is not None:
                         hook("decay_in", k0, dict(v=v_e, x_e=self.x_e, scale=listed(scale), dt=listed(dts),
                                                   n_edit=self.n_edit, active=members(gs)))
@@ -343,9 +353,7 @@ class RegionELoop:
                 last_before = k + 1 == after
                 v = model.full(x, t, partitioned or last_before)
                 full_calls += 1
-                p_v = ptr(v, bf, "v")
-                if v.shape != shape:
-                    raise b.RegionEError(f"v must have shape {shape}, got {tuple(v.shape)}")
+                p_v = _velocity(v, shape, "v")
                 check(decay(p_v, unit, one(*[t - t_next] * B), p_x, p_vl, p_all, B, N, C, p_st, s), "regione_velocity_decay")
                 launches += 1
                 if last_before:
@@ -365,9 +373,7 @@ class RegionELoop:
                 t_run = ts[k]
             v_e = model.region(self.x_e, ts[k], self.edit_idx, self.n_edit)
             region_calls += 1
-            p_v = ptr(v_e, bf, "v_e")
-            if v_e.shape != shape:
-                raise b.RegionEError(f"v_e must have shape {shape}, got {tuple(v_e.shape)}")
+            p_v = _velocity(v_e, shape, "v_e", region=True)
             log.append((k, "R", "compute", 1.0))
             scales, dts, product, again = [1.0] * B, [ts[k] - ts[k + 1]] * B, 1.0, True
             first, keep, k = k, p_vc, k + 1

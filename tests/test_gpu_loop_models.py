@@ -1,0 +1,51 @@
+"""What the sampler loop takes from its velocity model: velocities of other shapes that hold the same rows, and streams
+that the model makes current."""
+import pytest
+
+from gpu_util import dev_bf16
+from paper_2510_25590_b200 import binding, loop as gloop
+from test_gpu_loop import TorchStraightLine, _case
+
+pytestmark = pytest.mark.gpu
+
+
+class _Shaped(TorchStraightLine):
+    def __init__(self, target, full=lambda v: v, region=lambda v: v):
+        super().__init__(target)
+        self.shape_full, self.shape_region = full, region
+
+    def full(self, x, t, store):
+        return self.shape_full(super().full(x, t, store))
+
+    def region(self, x_e, t, edit_idx, n_edit):
+        return self.shape_region(super().region(x_e, t, edit_idx, n_edit))
+
+
+def _loop(noise):
+    kinds, after = gloop.alternating_schedule()
+    T = len(kinds)
+    cfg = gloop.LoopConfig(kinds, after, [1.0 - k / T for k in range(T + 1)], [1.0] * (T + 1), 0.05, binding.METRIC_COSINE, 0.9)
+    return gloop.RegionELoop(*noise.shape, cfg)
+
+
+@pytest.mark.parametrize("hooked", [False, True])
+def test_velocities_of_other_shapes_with_the_same_rows(hooked):
+    import torch
+    def run(B, **shapes):
+        _, ref, _, target, noise = _case(B=B)
+        lp = _loop(noise)
+        lp.hook = (lambda *a: None) if hooked else None
+        x, _ = lp.run(dev_bf16(noise), dev_bf16(ref), _Shaped(dev_bf16(target), **shapes))
+        torch.cuda.synchronize()
+        assert int(lp.dev_status[0]) == 0
+        return x, int(lp.n_edit.max())
+    want, n = run(1)
+    # one request: without its dimension; only the rows of the edited tokens; more rows than tokens
+    for region in (lambda v: v[:, :n].contiguous(), lambda v: v[0, :n + 3].contiguous(), lambda v: torch.cat([v, v], 1)):
+        assert torch.equal(run(1, full=lambda v: v[0], region=region)[0], want)
+    want, _ = run(2)
+    assert torch.equal(run(2, region=lambda v: v.flatten(0, 1))[0], want)
+    for shapes in (dict(full=lambda v: v[:1]), dict(full=lambda v: v[0]), dict(region=lambda v: v[:, :n].contiguous()),
+                   dict(full=lambda v: v.float()), dict(region=lambda v: v.transpose(0, 1))):
+        with pytest.raises(binding.RegionEError):
+            run(2, **shapes)
