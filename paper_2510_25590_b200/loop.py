@@ -123,7 +123,7 @@ class RegionELoop:
     optionally shifted against each other by ``offsets``).
 
     The loop's own work is launch-bound (kernels of 2 to 3 us), so its host side is kept short: addresses
-    and the stream are looked up once per run, requests that move together share their bookkeeping and
+    are looked up once per run (the buffers are the loop's while it runs, ``x`` included), requests that move together share their bookkeeping and
     their calls, a full step's velocity is kept by the Euler update that reads it, and the steps that reuse a
     region step's velocity are applied by that step's update (nothing reads X^E between them)."""
 
@@ -160,7 +160,7 @@ class RegionELoop:
 
         # ---- the library calls of the loop, over the whole batch (NaN scalar: a request sits a call out) ----
         lib, check, ptr, floats = b.load(), b._check, b._ptr, b._per_request
-        bf, shape, s = torch.bfloat16, (B, N, C), b._stream(stream)
+        bf, shape = torch.bfloat16, (B, N, C)
         p_x, p_xe, p_vl, p_vc = ptr(x, bf, "x"), self.x_e.data_ptr(), self.v_last_full.data_ptr(), self.v_cache.data_ptr()
         p_idx, p_slot, p_ne = self.edit_idx.data_ptr(), self.slot.data_ptr(), self.n_edit.data_ptr()
         p_all, p_st = self.n_all.data_ptr(), st.data_ptr()
@@ -168,6 +168,7 @@ class RegionELoop:
             raise b.RegionEError(f"x must have shape {shape}, got {tuple(x.shape)}")
 
         def decay(p_v, scale, dts, p_target, p_keep, p_n):
+            s = b._stream(stream)                           # (the model may have made another stream current)
             check(lib.regione_velocity_decay(p_v, floats(scale, B, "scale"), floats(dts, B, "dt"), p_target, p_keep, p_n,
                                              B, N, C, p_st, s), "regione_velocity_decay")
             tr.launches += 1
@@ -195,7 +196,7 @@ class RegionELoop:
             # velocity over the whole run (x has not changed since the run began, so it is merged in place)
             if hook is None:
                 check(lib.regione_merge(p_x, p_vl, p_xe, p_slot, floats(spread([(g, g.t_run - t) for g, t in ending]), B, "dt"),
-                                        B, N, N, C, p_x, p_st, s), "regione_merge")
+                                        B, N, N, C, p_x, p_st, b._stream(stream)), "regione_merge")
                 tr.launches += 1
             for g, t in ending:
                 g.in_run = False
@@ -210,7 +211,7 @@ class RegionELoop:
 
         def start_runs(starting):
             if uniform:
-                check(lib.regione_gather(p_x, p_idx, p_ne, B, N, N, N, 2 * C, p_xe, p_st, s), "regione_gather")
+                check(lib.regione_gather(p_x, p_idx, p_ne, B, N, N, N, 2 * C, p_xe, p_st, b._stream(stream)), "regione_gather")
                 tr.launches += 1
             for g in starting:
                 g.in_run, g.t_run, g.product, g.have_cache = True, ts[g.k], 1.0, False
@@ -328,7 +329,7 @@ class RegionELoop:
         kinds, after, gammas, delta = cfg.kinds, cfg.partition_after, cfg.gammas, cfg.delta
         T, B, N, C = len(kinds), self.B, self.N, self.C
         lib, check, ptr, avd_step = b.load(), b._check, b._ptr, b.avd_step
-        bf, shape, s = torch.bfloat16, (B, N, C), b._stream(stream)
+        bf, shape, s = torch.bfloat16, (B, N, C), b._stream(stream)     # (s: looked up again behind each call of the model)
         p_x, p_xe, p_vl, p_vc = ptr(x, bf, "x"), self.x_e.data_ptr(), self.v_last_full.data_ptr(), self.v_cache.data_ptr()
         p_slot, p_ne, p_all, p_st = (t.data_ptr() for t in (self.slot, self.n_edit, self.n_all, self.dev_status))
         if x.shape != shape:
@@ -352,6 +353,7 @@ class RegionELoop:
                 t, t_next = ts[k], ts[k + 1]
                 last_before = k + 1 == after
                 v = model.full(x, t, partitioned or last_before)
+                s = b._stream(stream)
                 full_calls += 1
                 p_v = _velocity(v, shape, "v")
                 check(decay(p_v, unit, one(*[t - t_next] * B), p_x, p_vl, p_all, B, N, C, p_st, s), "regione_velocity_decay")
@@ -372,6 +374,7 @@ class RegionELoop:
                 launches += 1
                 t_run = ts[k]
             v_e = model.region(self.x_e, ts[k], self.edit_idx, self.n_edit)
+            s = b._stream(stream)
             region_calls += 1
             p_v = _velocity(v_e, shape, "v_e", region=True)
             log.append((k, "R", "compute", 1.0))

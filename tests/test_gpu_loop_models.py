@@ -49,3 +49,33 @@ def test_velocities_of_other_shapes_with_the_same_rows(hooked):
                    dict(full=lambda v: v.float()), dict(region=lambda v: v.transpose(0, 1))):
         with pytest.raises(binding.RegionEError):
             run(2, **shapes)
+
+
+@pytest.mark.parametrize("hooked", [False, True])
+def test_loop_follows_the_stream_that_the_model_makes_current(hooked):
+    """A model that leaves another stream current, its velocity still being computed there when it returns."""
+    import torch
+    class Elsewhere(TorchStraightLine):
+        def switch(self):
+            old, new = torch.cuda.current_stream(), torch.cuda.Stream()
+            new.wait_stream(old)
+            torch.cuda.set_stream(new)
+            torch.cuda._sleep(200_000)
+        def full(self, x, t, store):
+            self.switch()
+            return super().full(x, t, store)
+        def region(self, x_e, t, edit_idx, n_edit):
+            self.switch()
+            return super().region(x_e, t, edit_idx, n_edit)
+    _, ref, _, target, noise = _case()
+    first, done = torch.cuda.current_stream(), []
+    for model in (TorchStraightLine, Elsewhere):
+        lp = _loop(noise)
+        lp.hook = (lambda *a: None) if hooked else None
+        try:
+            done.append(lp.run(dev_bf16(noise), dev_bf16(ref), model(dev_bf16(target)))[0])
+            torch.cuda.synchronize()
+        finally:
+            torch.cuda.set_stream(first)
+        done.append(lp.x_e)
+    assert torch.equal(done[0], done[2]) and torch.equal(done[1], done[3])
