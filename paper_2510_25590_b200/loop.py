@@ -98,20 +98,13 @@ class _Group:
     have_cache: bool = False
 
 
-def _velocity(v, shape, name, region=False):
-    """Address of a velocity that the model returned.  One of all tokens may come without the batch dimension of a single
+def _check_rows(got, shape, name, region=False):
+    """A velocity of another shape than [B, N, C]: one of all tokens may come without the batch dimension of a single
     request; one of a region step holds its rows at the beginning of each request's, for a single request as many as it
     likes (at least the edited tokens)."""
-    p = binding._ptr(v, binding._torch().bfloat16, name)
-    got = v.shape
-    if got != shape:
-        if region:
-            fits = shape[0] == 1 or got.numel() == shape[0] * shape[1] * shape[2]
-        else:
-            fits = got.numel() == shape[0] * shape[1] * shape[2] and shape[max(3 - len(got), 0):] == got
-        if not fits:
-            raise binding.RegionEError(f"{name} must have shape {shape}, got {tuple(got)}")
-    return p
+    same = got.numel() == shape[0] * shape[1] * shape[2]
+    if not (same or shape[0] == 1 if region else same and shape[max(3 - len(got), 0):] == got):
+        raise binding.RegionEError(f"{name} must have shape {shape}, got {tuple(got)}")
 
 
 _NAN = float("nan")
@@ -247,7 +240,9 @@ class RegionELoop:
                                 t_full[r] = ts[g.k]
                     v = model.full(x, t_full, store)
                 tr.model_full_calls += 1
-                p_v = _velocity(v, shape, "v")
+                p_v = ptr(v, bf, "v")
+                if v.shape != shape:
+                    _check_rows(v.shape, shape, "v")
                 dts = spread([(g, ts[g.k] - ts[g.k + 1]) for g in full])
                 if hook is not None:
                     hook("euler_in", k0, dict(x=x, v=v, dt=listed(dts), active=members(full)))
@@ -300,7 +295,9 @@ class RegionELoop:
                                     t_e[r] = ts[g.k]
                             v_e = model.region(self.x_e, t_e, self.edit_idx, self.n_edit)
                         tr.model_region_calls += 1
-                        p_v, p_keep = _velocity(v_e, shape, "v_e", region=True), p_vc
+                        p_v, p_keep = ptr(v_e, bf, "v_e"), p_vc
+                        if v_e.shape != shape:
+                            _check_rows(v_e.shape, shape, "v_e", region=True)
                     if hook is not None:
                         hook("decay_in", k0, dict(v=v_e, x_e=self.x_e, scale=listed(scale), dt=listed(dts),
                                                   n_edit=self.n_edit, active=members(gs)))
@@ -329,7 +326,9 @@ class RegionELoop:
         kinds, after, gammas, delta = cfg.kinds, cfg.partition_after, cfg.gammas, cfg.delta
         T, B, N, C = len(kinds), self.B, self.N, self.C
         lib, check, ptr, avd_step = b.load(), b._check, b._ptr, b.avd_step
-        bf, shape, s = torch.bfloat16, (B, N, C), b._stream(stream)     # (s: looked up again behind each call of the model)
+        bf, shape, s = torch.bfloat16, (B, N, C), b._stream(stream)
+        # (the model may make another stream current: looked up again behind each of its calls)
+        follow, stream_of, device = stream is None, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
         p_x, p_xe, p_vl, p_vc = ptr(x, bf, "x"), self.x_e.data_ptr(), self.v_last_full.data_ptr(), self.v_cache.data_ptr()
         p_slot, p_ne, p_all, p_st = (t.data_ptr() for t in (self.slot, self.n_edit, self.n_all, self.dev_status))
         if x.shape != shape:
@@ -353,9 +352,12 @@ class RegionELoop:
                 t, t_next = ts[k], ts[k + 1]
                 last_before = k + 1 == after
                 v = model.full(x, t, partitioned or last_before)
-                s = b._stream(stream)
+                if follow:
+                    s = stream_of(device())
                 full_calls += 1
-                p_v = _velocity(v, shape, "v")
+                p_v = ptr(v, bf, "v")
+                if v.shape != shape:
+                    _check_rows(v.shape, shape, "v")
                 check(decay(p_v, unit, one(*[t - t_next] * B), p_x, p_vl, p_all, B, N, C, p_st, s), "regione_velocity_decay")
                 launches += 1
                 if last_before:
@@ -374,9 +376,12 @@ class RegionELoop:
                 launches += 1
                 t_run = ts[k]
             v_e = model.region(self.x_e, ts[k], self.edit_idx, self.n_edit)
-            s = b._stream(stream)
+            if follow:
+                s = stream_of(device())
             region_calls += 1
-            p_v = _velocity(v_e, shape, "v_e", region=True)
+            p_v = ptr(v_e, bf, "v_e")
+            if v_e.shape != shape:
+                _check_rows(v_e.shape, shape, "v_e", region=True)
             log.append((k, "R", "compute", 1.0))
             scales, dts, product, again = [1.0] * B, [ts[k] - ts[k + 1]] * B, 1.0, True
             first, keep, k = k, p_vc, k + 1
