@@ -73,6 +73,9 @@ enum { REGIONE_ROPE_INTERLEAVED = 0, REGIONE_ROPE_HALF = 1 };
 /* Library version (major*10000 + minor*100 + patch) and status names. */
 int regione_version(void);
 const char* regione_status_string(int status);
+/* Kernels that the calling thread has launched through the entry points below (the cross-check and self-test ones
+ * excepted) since it started.  Which of its forms a call took shows in how many it launched. */
+unsigned long long regione_kernel_launches(void);
 
 /*
  * Adaptive Region Partition (Sec. 4, "Adaptive Region Partition"; Algorithm 1,

@@ -10,7 +10,7 @@ from __future__ import annotations
 import ctypes
 import math
 import os
-from ctypes import POINTER, c_char_p, c_double, c_float, c_int, c_int64, c_longlong, c_size_t, c_void_p
+from ctypes import POINTER, c_char_p, c_double, c_float, c_int, c_int64, c_longlong, c_size_t, c_ulonglong, c_void_p
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libregione.so")
@@ -39,6 +39,7 @@ _P = c_void_p
 SIGNATURES = {
     "regione_version": (c_int, []),
     "regione_status_string": (c_char_p, [c_int]),
+    "regione_kernel_launches": (c_ulonglong, []),
     "regione_partition": (c_int, [_P, _P, _P, c_int, c_int, c_int, _P, c_int, c_float,
                                   _P, _P, _P, _P, _P, _P, _P, _P]),
     "regione_partition_rows": (c_int, [_P, _P, _P, c_int, c_int, c_int, _P, c_int, c_float,
@@ -165,6 +166,11 @@ def _per_request(value, B, name):
         if len(vals) != B:
             raise RegionEError(f"{name} must be one number or {B} numbers, got {len(vals)}")
     return (_FLOATS.get(B) or _FLOATS.setdefault(B, c_float * max(B, 1)))(*vals)
+
+
+def kernel_launches() -> int:
+    """Kernels that this thread has launched through the library so far."""
+    return load().regione_kernel_launches()
 
 
 def version() -> int:

@@ -9,9 +9,15 @@ int launch_region_attention_simt(const uint16_t*, const uint16_t*, const uint16_
                                  const uint16_t*, const int32_t*, const int32_t*, const int32_t*,
                                  int, int, int, int, int, int, float, uint16_t*, int32_t*,
                                  cudaStream_t);
+unsigned long long& launch_count() {
+    static thread_local unsigned long long count = 0;
+    return count;
+}
 }  // namespace regione
 
 using namespace regione;
+
+extern "C" unsigned long long regione_kernel_launches(void) { return launch_count(); }
 
 extern "C" int regione_version(void) { return 200; }
 

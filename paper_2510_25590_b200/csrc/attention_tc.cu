@@ -1898,8 +1898,8 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
     cfg.numAttrs = prm.cluster > 0 ? 2 : 1;
     cudaError_t e;
     auto launch = [&](auto kernel) {
-        if constexpr (STORE) return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6], prm, sp);
-        else return cudaLaunchKernelEx(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
+        if constexpr (STORE) return launch_counted(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6], prm, sp);
+        else return launch_counted(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
     };
     const int form = prm.cluster > 0 ? kMergeCluster : merges_here(prm, grid, nt_cap) ? kMergeHere : kMergeKernel;
     e = form == kMergeCluster ? launch(main_kernel<D, STORE, kMergeCluster>())

@@ -64,6 +64,16 @@ __device__ __forceinline__ void grid_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Kernels that the calling thread has launched through the product entry points (defined in api.cu).
+unsigned long long& launch_count();
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_counted(const cudaLaunchConfig_t* cfg, void (*kernel)(Params...), Args&&... args) {
+    const cudaError_t e = cudaLaunchKernelEx(cfg, kernel, static_cast<Args&&>(args)...);
+    if (e == cudaSuccess) ++launch_count();
+    return e;
+}
+
 // Launches `kernel` with programmatic stream serialization (see grid_dependency_wait).
 template <typename... Params, typename... Args>
 inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
@@ -78,7 +88,7 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    return launch_counted(&cfg, kernel, static_cast<Params>(args)...);
 }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

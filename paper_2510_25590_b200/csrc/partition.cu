@@ -454,7 +454,7 @@ static cudaError_t launch_partition(int csize, int B, int share, cudaStream_t st
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, partition_kernel<L, FROM_MASK>, x_t, v, ref, N, C, share, tv, b0, metric,
+    return launch_counted(&cfg, partition_kernel<L, FROM_MASK>, x_t, v, ref, N, C, share, tv, b0, metric,
                               thr, mask, edit_idx, keep_idx, slot, n_edit, score, rl, dev_status);
 }
 

@@ -83,8 +83,9 @@ class RegionStep:
         self.n_rows = torch.full((B,), shp.n_full, dtype=i32, device=device)
         self.workspace = torch.empty(max(binding.region_step_workspace(self._new_plan()), 256), dtype=torch.uint8,
                                      device=device)
-        self.launches = 0                 # operations of the sequence run so far (8 per step, 7 without the store)
-        self.kernel_launches = 0          # kernels launched so far, at least (a fourth merges cut items in some shapes)
+        self.launches = 0                 # operations of the sequence run so far (8 per step, 7 without the store), however
+                                          # many kernels they took
+        self.kernel_launches = 0          # kernels launched so far, as the library counts them
         self.attention_events = None      # optional (start, stop) pair recorded around the attention
         self._step_plan()
 
@@ -142,7 +143,7 @@ class RegionStep:
         """One region-aware step.  ``store_cache=False`` leaves the cache as the last storing call wrote
         it (Algorithm 1 refreshes it at full steps only; valid while the partition is unchanged)."""
         args = (x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, store_cache)
-        plan, B, events = self._step_plan(), binding, self.attention_events
+        plan, B, events, before = self._step_plan(), binding, self.attention_events, binding.kernel_launches()
         if plan is None:
             return self._run_calls(*args, stream)
         try:
@@ -158,7 +159,7 @@ class RegionStep:
             B.region_step(plan, *args, parts=B.STEP_ATTENTION, stream=stream)
             events[1].record(stream)
         self.launches += 8 if store_cache else 7
-        self.kernel_launches += 3
+        self.kernel_launches += B.kernel_launches() - before
         return self.x_out
 
     # buffers that may hold another number of rows per request than planned, those that share it together
@@ -177,7 +178,7 @@ class RegionStep:
     def _run_calls(self, x_t, v, ref, q_full, k_full, v_full, t, scale, dt, dt_unedited, store_cache, stream):
         """The step as separate library calls, which take their sizes from the tensors: for inputs and buffers of other
         shapes than the plan's (rows as one dimension, a larger output, a cache that holds fewer rows)."""
-        s, st, b = self.shp, self.dev_status, binding
+        s, st, b, before = self.shp, self.dev_status, binding, binding.kernel_launches()
         self._check_shapes()
         b.partition_rows(x_t, v, ref, t, s.metric, s.threshold, self.mask, self.edit_idx, self.keep_idx, self.slot,
                          self.n_edit, s.n_text, s.n_ref, s.membership, self.query_rows, self.n_q, self.cache_rows,
@@ -198,5 +199,5 @@ class RegionStep:
         if self.attention_events is not None:
             self.attention_events[1].record(stream)
         self.launches += 8 if store_cache else 7
-        self.kernel_launches += 7 if store_cache else 6
+        self.kernel_launches += b.kernel_launches() - before
         return self.x_out
