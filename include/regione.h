@@ -515,14 +515,15 @@ int regione_crosscheck_region_attention(const regione_bf16* q,
                                         int32_t* dev_status, void* stream);
 
 /*
- * Lets a bounded wait run out, in the harmless form (the paper has no counterpart; this covers
- * the convention above that a wait that expires ends in REGIONE_DEV_TIMEOUT).  One thread of one
- * thread block waits, through the very routine the attention kernel's roles wait with, on a
- * barrier that nothing ever arrives on, with no copy and no tensor-core operation in flight.
- * After limit_cycles SM clock cycles (1 .. 10^8) the wait gives up, REGIONE_DEV_TIMEOUT is
+ * Lets the bounded waits run out, in the harmless form (the paper has no counterpart; this covers
+ * the convention above that a wait that expires ends in REGIONE_DEV_TIMEOUT).  One warp
+ * waits, through the very routines the attention kernel's roles wait with, on a barrier that
+ * nothing ever arrives on, for a peer's arrival on it, and for another block's flags, which nothing sets,
+ * with no copy and no tensor-core operation in flight.
+ * After limit_cycles SM clock cycles (1 .. 10^8) each gives up, REGIONE_DEV_TIMEOUT is
  * recorded in dev_status and the kernel ends normally; the context stays usable.
- * out : dev int64 [3], nullable: {1 if the wait claimed completion (must be 0), cycles spent
- *       waiting, the abort flag the other roles would have seen (must be 1)}.
+ * out : dev int64 [3], nullable: {1 if a wait claimed completion (must be 0), cycles spent in the
+ *       shortest wait, 1 if each raised the abort flag the other roles would have seen (must be 1)}.
  */
 int regione_selftest_bounded_wait(long long limit_cycles, int32_t* dev_status, long long* out,
                                   void* stream);

@@ -1669,25 +1669,43 @@ region_attention_combine_kernel(const AttnParams p) {
         *reinterpret_cast<uint32_t*>(orow) = packed[0];
 }
 
-// Self-test of the bounded wait: one thread waits, through the same wait_bar the attention
-// kernel's roles use, on an mbarrier that nobody ever arrives on.  No copy and no tensor-core
-// operation is in flight, so giving up is all that happens: the wait must return false after
-// `limit` cycles with REGIONE_DEV_TIMEOUT recorded, and the kernel ends normally.
-// out[0] = 1 if the wait reported a completed phase (it must not), out[1] = cycles spent waiting.
+// Self-test of the bounded waits: a warp waits, through the same routines that the attention kernel's roles wait with,
+// on an mbarrier that nobody ever arrives on, for a peer's arrival on it, and for flags that nothing sets.  No copy and
+// no tensor-core operation is in flight, so giving up is all that happens: each wait must return false after `limit`
+// cycles with REGIONE_DEV_TIMEOUT recorded, and the kernel ends normally.
+// out[0] = 1 if a wait reported a completed phase (it must not), out[1] = cycles spent in the shortest wait,
+// out[2] = 1 if each of them raised its abort flag.
+__device__ unsigned long long g_unset_flags[33];
 __global__ void bounded_wait_selftest_kernel(long long limit, int32_t* dev_status, long long* out) {
     __shared__ uint64_t bar;
-    __shared__ int abort_flag;
-    if (threadIdx.x == 0) {
-        abort_flag = 0;
+    __shared__ int abort_flag[3];
+    const int lane = threadIdx.x;
+    if (lane < 3) abort_flag[lane] = 0;
+    if (lane == 0) {
         ptx::mbar_init(ptx::smem_addr(&bar), 1);
         ptx::fence_barrier_init();
+    }
+    __syncwarp();
+    AttnParams p = {};
+    p.dev_status = dev_status; p.timeout_cycles = limit;
+    p.ready = g_unset_flags; p.epoch = 1;
+    bool done = false;
+    long long shortest = 0x7fffffffffffffffLL;
+    for (int i = 0; i < 3; ++i) {
         const long long t0 = clock64();
-        const bool done = wait_bar(ptx::smem_addr(&bar), 0, &abort_flag, dev_status, limit);
+        if (i == 2) done |= wait_shares(p, 1, lane, &abort_flag[2]);             // (a wait of the whole warp)
+        else if (lane == 0)
+            done |= i == 0 ? wait_bar(ptx::smem_addr(&bar), 0, &abort_flag[0], dev_status, limit)
+                           : wait_bar_cluster(ptx::smem_addr(&bar), &abort_flag[1], dev_status, limit);
         const long long spent = clock64() - t0;
+        shortest = spent < shortest ? spent : shortest;
+        __syncwarp();
+    }
+    if (lane == 0) {
         if (out != nullptr) {
             out[0] = done ? 1 : 0;
-            out[1] = spent;
-            out[2] = abort_flag;
+            out[1] = shortest;
+            out[2] = abort_flag[0] && abort_flag[1] && abort_flag[2];
         }
         ptx::mbar_inval(ptx::smem_addr(&bar));
     }
