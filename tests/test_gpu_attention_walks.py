@@ -103,3 +103,30 @@ def test_items_shared_by_clusters(D, counts):
     kf, vf = _rand_bf16(rng, (B, cap_f, H, D)), _rand_bf16(rng, (B, cap_f, H, D))
     kc, vc = _rand_bf16(rng, (B, cap_c, H, D)), _rand_bf16(rng, (B, cap_c, H, D))
     check(q, kf, vf, kc, vc, [c[0] for c in counts], [c[1] for c in counts], [c[2] for c in counts], what=f"clusters {counts}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("H,n_q,n_f,n_c", [(3, 300, 300, 2000), (40, 100, 0, 1500), (24, 819, 819, 7000)])
+def test_rows_that_one_key_dominates_are_exact_to_the_rounding_of_the_output(D, H, n_q, n_f, n_c):
+    """Each query meets one key, anywhere in the sequence, whose logit is 15 (the others' deviate by 1 / 4): its weight is
+    above 0.99.  Whatever reference the probabilities are rounded against, that key's rounding cancels between the
+    product and the sum, and what is left is the rounding of the output to bf16, which the exact result shows when it is
+    rounded.  1.1 of that leaves room for the other keys; a rounding that does not cancel gives 1.17 to 2.3."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(D + H)
+    r = lambda n: torch.randn((1, n, H, D), generator=g, device="cuda").bfloat16()
+    q, k, v = r(n_q), r(n_f + n_c) * 0.25, r(n_f + n_c)
+    at = torch.randperm(n_f + n_c, generator=torch.Generator().manual_seed(D)).cuda()[:n_q]
+    k[0, at] = (q[0].float() * (15.0 * D ** 0.5 / q[0].float().pow(2).sum(-1, keepdim=True))).bfloat16()
+    out, status = torch.zeros_like(q), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ws = torch.empty(max(binding.region_attention_workspace(1, n_q, n_f, n_c, H, D), 256), dtype=torch.uint8, device="cuda")
+    kf, vf = (k[:, :n_f].contiguous(), v[:, :n_f].contiguous()) if n_f else (None, None)
+    binding.region_attention(q, kf, vf, k[:, n_f:].contiguous(), v[:, n_f:].contiguous(), dev_i32([n_q]), dev_i32([n_f]),
+                             dev_i32([n_c]), out, workspace=ws, dev_status=status)
+    want = torch.empty(q.shape, dtype=torch.float64, device="cuda")
+    for h in range(H):
+        s = q[0, :, h].double() @ k[0, :, h].double().T * D ** -0.5
+        want[0, :, h] = torch.softmax(s, -1) @ v[0, :, h].double()
+    assert int(status[0]) == 0
+    error = lambda a: float((a.double() - want).norm() / want.norm())
+    assert error(out) <= 1.1 * error(want.bfloat16()), (error(out), error(want.bfloat16()))
