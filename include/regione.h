@@ -293,8 +293,8 @@ int regione_rikv_load_e4m3(const uint8_t* k_q, const uint8_t* v_q, const float* 
  *                   anew or the workspace is overwritten.
  * D must be 64 or 128.  bf16 inputs, fp32 accumulation, probabilities rounded
  * to bf16 before the second product.  With no key at all a row is zero.
- * The call enqueues two kernels (attention, then the merge of shared items; the
- * second is launched with programmatic stream serialization, i.e. it may become
+ * The call enqueues one kernel, or two where a kernel of its own merges the shared
+ * items (launched with programmatic stream serialization, i.e. it may become
  * resident while the first drains and waits for its completion on the device).
  */
 size_t regione_region_attention_workspace(int B, int Nq_cap, int Nf_cap, int Nc_cap, int H, int D);

@@ -29,17 +29,20 @@
 // What bounds the loop: per key tile and query pair the tensor cores need 2048 cycles and the special-function
 // unit 2048 (32768 exponentials, 16 a cycle); the dependency chain  S -> registers -> exponentials -> P -> product
 // hides behind neither.  Two threads per row (four softmax warps per scheduler instead of two), no row maximum
-// after the first key tile and packed fp32 arithmetic shorten the chain: 2860 cycles per key tile and pair,
-// against 3250 with one thread per row, a maximum per key tile and scalar arithmetic.  Measured, one box, L2 warm:
+// after the first key tile and packed fp32 arithmetic shorten the chain: 2690 cycles per key tile and pair, 2540 with
+// D = 64 (active cycles of 64 key tiles less those of 32, one item a CTA; 19000 more are fill, drain and epilogue).
+// Measured, one box, L2 warm, against one thread per row, a maximum per key tile and scalar arithmetic:
 // 8704 queries x 8704 keys x 24 heads 763 -> 720 us in isolation (1292 TFLOP/s), 889 -> 848 us under the power
 // cap; 4 x 1382 queries x 18944 keys 1141 -> 1056 us; 2048 queries x 8448 keys 189 -> 180 us; D = 64 127 -> 114 us;
 // 205 queries x 8448 keys, where the fill and the drain of the pipeline dominate, 42.3 -> 43.2 us.
 //
 // Online softmax in the exp2 domain without a running maximum: a row's reference is its maximum over the
 // segment's first key tile.  Any reference within a factor of 2^60 of the true maximum gives the same relative
-// accuracy (probabilities are bf16, sums fp32).  A row whose chunk sum reaches 2^60 makes the CTA walk the
-// segment twice more, once for the rows' true maxima and once with them; that costs three times the segment,
-// for inputs whose logits spread over more than 41 nats.  Keys past a segment's live count are masked in the
+// accuracy (probabilities are bf16, their sums fp32: see chunk_probabilities).  A row whose chunk sum reaches 2^60 (a
+// later logit above the first key tile's by 37 nats if a chunk holds 64 of them, by 42 if it is alone) makes the CTA
+// walk the segment twice more, once for the rows' true maxima and once with them.  That costs up to three times the
+// segment: 819 queries x 8704 keys 97 -> 213 us with one such row a head, 8704 x 8704 718 -> 1056 us, with every row
+// 1944 us.  Keys past a segment's live count are masked in the
 // softmax and their V rows zeroed in shared memory, so garbage (even NaN) behind the live prefix cannot leak.
 //
 // Scheduling: the kernel is persistent, one CTA per SM.  A "step" is one key tile of one
@@ -113,10 +116,11 @@ struct AttnCfg {
     static constexpr int kSmemBytes = kExtraAt + (D == 128 ? 0 : kSoftmaxWarps * 4096 + kCopyBytes);
     static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
     __host__ __device__ static constexpr int lone_stages(bool store) { return kStages + (D == 128 && store ? 0 : 2); }
-    // slots of the copies that are left when the walks are over and all tiles are idle
-    // an item shared by a cluster: its CTAs leave their partial rows, chunk by chunk, and (max, sum) pairs here
+    // partial rows that stay in shared memory, chunk by chunk, and their (max, sum) pairs: of an item shared by a
+    // cluster, and of the first share of a cut item
     static constexpr int kPartialMlAt = 2 * kBM * D * 4;
     static_assert(kPartialMlAt + 2 * kBM * 8 <= kSmemTiles, "partial rows");
+    // slots of the copies that are left when the walks are over and all tiles are idle
     static constexpr int kTailBytes = (D == 128) ? 3 * 65536 : 3 * 40960;
     static_assert(kTailBytes <= kSmemTiles, "tail slots");
 };
@@ -478,9 +482,9 @@ __device__ __forceinline__ float add_bf16(float c, uint16_t a) {
 // deviation 1 / 2 / 4 / 8, relative error 2.33 / 2.27 / 2.29 / 2.27e-3, this way 2.33 / 2.21 / 1.91 / 1.76e-3, with a
 // running maximum 2.32 / 2.25 / 1.96 / 1.74e-3.  The mixed additions cost 0.5 to 0.9 % of a call, widening the rounded
 // values and adding them in pairs 2.3 %.)  The exponentials replace the logits in place and leave in pieces of 8 columns, so that
-// a thread's 104 registers hold the chunk.  All of them run on the special-function unit: with four softmax
-// warps per scheduler it is busy 70 % of the time, and moving a quarter or an eighth of them to the FMA pipe
-// (a cubic) made the call 4 % and 0 % slower.
+// a thread's 104 registers hold the chunk.  All of them run on the special-function unit: it is busy 2048 of the
+// loop's 2690 cycles, and moving a quarter or an eighth of them to the FMA pipe (a cubic) made the call 4 % and 0 %
+// slower.
 __device__ __forceinline__ float chunk_probabilities(uint32_t tP, uint32_t* s, float c, float m) {
     const uint64_t c2 = pack2(c, c), m2 = pack2(-m, -m);
     float sum[4] = {0.f, 0.f, 0.f, 0.f};
@@ -534,7 +538,6 @@ __device__ __forceinline__ VLanding v_landing(AttnCtrl* ctrl, bool split, int n_
 // kMaxOnly finds the rows' maxima, kExact repeats the pass with them.
 enum WalkMode { kWalk, kMaxOnly, kExact };
 
-// ---- softmax / epilogue of one segment: thread = (query row, 64-key chunk) ----------------------------
 // Share of a CTA on the cost axis.  The first share of an item waits for the later ones, so shares are dealt
 // from the last block to the first: blocks become resident in the order of their indexes on this GPU, and a block
 // waits only for blocks ahead of it, whatever else runs.  CUDA does not promise that order; were it another, a wait
@@ -565,6 +568,7 @@ __device__ __forceinline__ bool wait_shares(const AttnParams& p, int n, int lane
     return there;
 }
 
+// ---- softmax / epilogue of one segment: thread = (query row, 64-key chunk) ----------------------------
 template <int D, bool STORE, int FORM>
 __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* ctrl, const SegInfo& it, uint8_t* smem_gen,
                                                 const uint32_t tmem, const int warp, const int lane, const int mode,
@@ -1404,11 +1408,11 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
                 ptx::fence_barrier_init();
             }
         } else {
-        cur.pl = plan_shares<STORE>(p, gridDim.x, &bad);
-        cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)my_share() * cur.pl.chunk;
-        cur.first = true;
-        cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
-        cur.next<FORM, STORE>(p, &ctrl->seg[0], lane);
+            cur.pl = plan_shares<STORE>(p, gridDim.x, &bad);
+            cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)my_share() * cur.pl.chunk;
+            cur.first = true;
+            cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
+            cur.next<FORM, STORE>(p, &ctrl->seg[0], lane);
         }
         if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         if (lane == 0) ctrl->abort_flag = 0;
@@ -1849,10 +1853,12 @@ static int prepare_kernel(const int** fitting) {
     return REGIONE_OK;
 }
 
-// Rows that are put back into a joint sequence many times their number keep the cuts of the cost axis with kTickStart:
-// where an item is cut decides which reference maximum its probabilities are rounded against, and seen against the rms
-// of the whole buffer, mostly rows that were not recomputed, another rounding moves single elements by up to 0.1 (by
-// 0.04 from a twelfth of the rows on).
+// Rows that are put back into a joint sequence many times their number keep the cuts of the cost axis with kTickStart.
+// This line is neither the faster side's nor the more accurate one's: where an item is cut decides which reference
+// maximum its probabilities are rounded against, and against the rms of the whole buffer, mostly rows that were not
+// recomputed, the two forms differ from each other by up to 0.1 in single elements (by 0.04 from a twelfth of the rows
+// on).  Against 64 bits, over the recomputed rows, clusters / cost axis: 64 of 8448 rows rel 2.32 / 2.31e-3, 32.7 / 36.4 us;
+// 128 2.31 / 2.31e-3, 33.6 / 38.7 us; 205 2.32 / 2.32e-3, 42.7 / 43.6 us; 704 2.33 / 2.33e-3, 74.4 / 79.8 us.
 static bool keeps_cuts(const AttnParams& p) {
     return p.out_rows != nullptr && 12LL * (p.Nq_cap - kBM / 2) < (long long)p.Nf_cap + p.Nc_cap;
 }
@@ -1944,13 +1950,12 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
     return launch_status(cudaGetLastError());
 }
 
-// A number that no other launch has and that memory does not hold by chance: a count, scattered over 64 bits.
+// A number that no other launch has and that memory does not hold by chance: a count, spread over 64 bits by
+// multiplication with 2^64 / golden ratio (Fibonacci hashing, Knuth, The Art of Computer Programming 3, 6.4).
 static unsigned long long next_epoch() {
     static std::atomic<unsigned long long> count{
         (unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count()};
-    unsigned long long z = count.fetch_add(1, std::memory_order_relaxed) * 0x9E3779B97F4A7C15ull;     // (odd: a bijection)
-    z = (z ^ (z >> 31)) * 0xD6E8FEB86659FD93ull;
-    z ^= z >> 32;
+    const unsigned long long z = count.fetch_add(1, std::memory_order_relaxed) * 0x9E3779B97F4A7C15ull;   // (odd: a bijection)
     return z != 0 ? z : 1;
 }
 
@@ -2072,8 +2077,8 @@ extern "C" int regione_region_attention_static(
     const int rc = static_scratch_address(&scratch);
     if (rc != REGIONE_OK) return rc;
     const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)D);
-    // Nothing in the scratch has to start at zero: every word that is merged is written
-    // by the attention kernel of the same call, so the previous call's contents are harmless.
+    // Nothing in the scratch has to start at zero: every row that is merged is written by the attention kernel of the
+    // same call, and the flags that say so are compared with a number that only this call has.
     return launch_region_attention_tc(q, k_fresh, v_fresh, k_cache, v_cache, n_q, n_fresh, n_cache,
                                       B, Nq_cap, Nf_cap, Nc_cap, H, D, scale, out, nullptr, 0, scratch,
                                       kStaticScratchBytes, dev_status, (cudaStream_t)stream, nullptr);

@@ -14,18 +14,18 @@
 //   256 of 1024 tokens, 4 heads x 64, cache refreshed       108 -> 24 us
 //   205 of 4096 tokens, 24 heads x 128, cache read           95 -> 54 us
 //   819 of 4096 tokens, 24 heads x 128, cache read          135 -> 128 us (power-capped attention)
-//   2048 of 4096 tokens, 24 heads x 128, cache refreshed    281 -> 243 us (power-capped attention)
+//   2048 of 4096 tokens, 24 heads x 128, cache refreshed    281 -> 246 us (power-capped attention)
 #include "rowcopy.cuh"
 
 namespace regione {
 
 // Whether the attention of a step that refreshes the cache reads K and V where they are and takes the rows of the
 // cache along, or reads [cache | fresh] as a step that keeps the cache does, with the rows copied ahead of it.  The
-// copies need the attention's time to hide behind, which grows with the queries; and only with enough queries beside
-// the keys does the other order of the keys stay a matter of rounding in the scattered buffer (see choose_cluster).
-// Measured, rows ahead -> along, us: 8704 rows of 24 heads, 128 queries 76 -> 82, 256 84 -> 84, 512 104 -> 90, 1536
-// 169 -> 145; four requests of 18944, 512 queries 700 -> 622, 1408 1372 -> 1178.  So the line is the rounding's: below
-// a sixteenth single elements of the scattered buffer moved by up to 0.1 of its rms, from there on by 0.05.
+// copies need the attention's time to hide behind, which grows with the queries.  Measured, a whole step with the rows
+// copied ahead -> along, us: 8704 rows of 24 heads, 128 queries 81 -> 83, 256 89 -> 90, 512 104 -> 93, 819 143 -> 132, 1536
+// 168 -> 143; four requests of 18944, 512 queries 758 -> 612, 1382 1537 -> 1274.  The line lies above the point where
+// the two meet: it is where the other order of the keys moves single elements of the scattered buffer by 0.05 of its
+// rms, not by 0.1 as below (see keeps_cuts: a difference between two roundings, not an error of either).
 static bool takes_rows_along(int q_cap, int n_full) { return 16LL * (q_cap - 64) >= n_full; }
 
 constexpr int kApartBlocks = 64;      // blocks of a request that copy rows only where rows_apart says so
