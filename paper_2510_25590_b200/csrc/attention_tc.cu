@@ -38,7 +38,7 @@
 //
 // Online softmax in the exp2 domain without a running maximum: a row's reference is its maximum over the
 // segment's first key tile.  Any reference within a factor of 2^60 of the true maximum gives the same relative
-// accuracy (probabilities are bf16, their sums fp32: see chunk_probabilities).  A row whose chunk sum reaches 2^60 (a
+// accuracy (probabilities are bf16, their sums fp32: see chunk_sum).  A row whose chunk sum reaches 2^60 (a
 // later logit above the first key tile's by 37 nats if a chunk holds 64 of them, by 42 if it is alone) makes the CTA
 // walk the segment twice more, once for the rows' true maxima and once with them.  That costs up to three times the
 // segment: 819 queries x 8704 keys 97 -> 213 us with one such row a head, 8704 x 8704 718 -> 1056 us, with every row
@@ -476,18 +476,13 @@ __device__ __forceinline__ float add_bf16(float c, uint16_t a) {
     return r;
 }
 
-// p = 2^(s*c - m) for 64 logits, written to tensor memory at `tP` (32 columns) as packed bf16; returns
-// the fp32 sum of what is written.  (The sum of the unrounded values leaves the rounding of a key that dominates its row
-// in the result, unless the reference m is that key's own logit: against 64 bits, 512 x 8448 x 128 with logits of
-// deviation 1 / 2 / 4 / 8, relative error 2.33 / 2.27 / 2.29 / 2.27e-3, this way 2.33 / 2.21 / 1.91 / 1.76e-3, with a
-// running maximum 2.32 / 2.25 / 1.96 / 1.74e-3.  The mixed additions cost 0.5 to 0.9 % of a call, widening the rounded
-// values and adding them in pairs 2.3 %.)  The exponentials replace the logits in place and leave in pieces of 8 columns, so that
+// p = 2^(s*c - m) for 64 logits, written to tensor memory at `tP` (32 columns) as packed bf16; the packed pairs are left
+// in s[0..31] for chunk_sum.  The exponentials replace the logits in place and leave in pieces of 8 columns, so that
 // a thread's 104 registers hold the chunk.  All of them run on the special-function unit: it is busy 2048 of the
 // loop's 2690 cycles, and moving a quarter or an eighth of them to the FMA pipe (a cubic) made the call 4 % and 0 %
 // slower.
-__device__ __forceinline__ float chunk_probabilities(uint32_t tP, uint32_t* s, float c, float m) {
+__device__ __forceinline__ void chunk_probabilities(uint32_t tP, uint32_t* s, float c, float m) {
     const uint64_t c2 = pack2(c, c), m2 = pack2(-m, -m);
-    float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < kBH; i += 2) {
         float a, b;
@@ -499,13 +494,25 @@ __device__ __forceinline__ float chunk_probabilities(uint32_t tP, uint32_t* s, f
     for (int g = 0; g < kBH; g += 16) {
         uint32_t pk[8];
 #pragma unroll
-        for (int i = g; i < g + 16; i += 2) {
-            const uint32_t w = pack_bf16x2(__uint_as_float(s[i]), __uint_as_float(s[i + 1]));
-            sum[i & 3] = add_bf16(sum[i & 3], (uint16_t)w);
-            sum[(i + 1) & 3] = add_bf16(sum[(i + 1) & 3], (uint16_t)(w >> 16));
-            pk[(i - g) >> 1] = w;
-        }
+        for (int i = g; i < g + 16; i += 2)
+            s[i >> 1] = pk[(i - g) >> 1] = pack_bf16x2(__uint_as_float(s[i]), __uint_as_float(s[i + 1]));
         ptx::tmem_st8(tP + (g >> 1), pk);
+    }
+}
+
+// fp32 sum of a chunk's probabilities as they were written.  (The sum of the unrounded values leaves the rounding of a key
+// that dominates its row in the result, unless the reference m is that key's own logit: against 64 bits, 512 x 8448 x 128
+// with logits of deviation 1 / 2 / 4 / 8, relative error 2.33 / 2.27 / 2.29 / 2.27e-3, this way 2.33 / 2.21 / 1.91 /
+// 1.76e-3, with a running maximum 2.32 / 2.25 / 1.96 / 1.74e-3.)  Nothing waits for it, so it follows the chunk's arrival:
+// beside the exponentials, ahead of the arrival, the 64 additions cost 205 queries x 8448 keys 1.1 us (step 55.1 -> 54.0),
+// 8704 x 8704 15 us (854 -> 839); the launches that copy rows beside it +-0.6 %.  Widening the pairs and adding them two
+// at a time: step 54.8 us, 857 us.
+__device__ __forceinline__ float chunk_sum(const uint32_t* w) {
+    float sum[4] = {};
+#pragma unroll
+    for (int i = 0; i < kBH; i += 2) {
+        sum[i & 3] = add_bf16(sum[i & 3], (uint16_t)w[i >> 1]);
+        sum[(i + 1) & 3] = add_bf16(sum[(i + 1) & 3], (uint16_t)(w[i >> 1] >> 16));
     }
     return (sum[0] + sum[1]) + (sum[2] + sum[3]);
 }
@@ -644,9 +651,7 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             // (a second chunk without live keys waits and arrives like any other, so that every barrier goes
             // through one phase per key tile; it writes nothing and no product reads it)
             if (live_keys > 0) {
-                const float sum = chunk_probabilities(tP, s, c, m);
-                outgrown |= !(sum < kOutgrownSum);
-                l += sum;
+                chunk_probabilities(tP, s, c, m);
                 ptx::tmem_wait_st();
             }
             if (valid < kBN && ck == 0) {
@@ -669,6 +674,11 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             ptx::tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(bar_p);
+            if (live_keys > 0) {
+                const float sum = chunk_sum(s);
+                outgrown |= !(sum < kOutgrownSum);
+                l += sum;
+            }
         }
     }
     if (mode == kMaxOnly) {
