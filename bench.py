@@ -48,7 +48,7 @@ def measured_peaks():
 
 # DRAM bytes per attention launch on config 2 (dram__bytes_read.sum + dram__bytes_write.sum of one ncu
 # capture of this workload), valid for the kernel source with this digest only.
-ATTENTION_TRAFFIC = dict(source_sha256_16="5ecff76da22c4a5e", config=2, dram_bytes_per_launch=453.6e6)
+ATTENTION_TRAFFIC = dict(source_sha256_16="768093a2c5902e22", config=2, dram_bytes_per_launch=470.2e6)
 
 
 def recorded_traffic(cfg):

@@ -29,7 +29,7 @@
 // What bounds the loop: per key tile and query pair the tensor cores need 2048 cycles and the special-function
 // unit 2048 (32768 exponentials, 16 a cycle); the dependency chain  S -> registers -> exponentials -> P -> product
 // hides behind neither.  Two threads per row (four softmax warps per scheduler instead of two), no row maximum
-// after the first key tile and packed fp32 arithmetic shorten the chain: 2690 cycles per key tile and pair, 2540 with
+// after the first key tile and packed fp32 arithmetic shorten the chain: 2640 cycles per key tile and pair, 2460 with
 // D = 64 (active cycles of 64 key tiles less those of 32, one item a CTA; 19000 more are fill, drain and epilogue).
 // Measured, one box, L2 warm, against one thread per row, a maximum per key tile and scalar arithmetic:
 // 8704 queries x 8704 keys x 24 heads 763 -> 720 us in isolation (1292 TFLOP/s), 889 -> 848 us under the power
@@ -479,7 +479,7 @@ __device__ __forceinline__ float add_bf16(float c, uint16_t a) {
 // p = 2^(s*c - m) for 64 logits, written to tensor memory at `tP` (32 columns) as packed bf16; the packed pairs are left
 // in s[0..31] for chunk_sum.  The exponentials replace the logits in place and leave in pieces of 8 columns, so that
 // a thread's 104 registers hold the chunk.  All of them run on the special-function unit: it is busy 2048 of the
-// loop's 2690 cycles, and moving a quarter or an eighth of them to the FMA pipe (a cubic) made the call 4 % and 0 %
+// loop's 2640 cycles, and moving a quarter or an eighth of them to the FMA pipe (a cubic) made the call 4 % and 0 %
 // slower.
 __device__ __forceinline__ void chunk_probabilities(uint32_t tP, uint32_t* s, float c, float m) {
     const uint64_t c2 = pack2(c, c), m2 = pack2(-m, -m);

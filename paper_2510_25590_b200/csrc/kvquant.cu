@@ -12,8 +12,8 @@
 //   elements of that row and head); written with frexp(amax) = m * 2^e, m in [0.5, 1):
 //   k = e - 9 + (m > 0.875); k = 0 for amax = 0; k is kept >= -100.
 //
-// Measured, 70248 rows of 24 x 128 (1.3 GB): store 222 us, 5890 GB/s (224 us with cached loads and stores; at one
-// request of 7885 rows 29.6 -> 28.5 us); four rows per block with the next row's loads ahead took 300 us, the
+// Measured, 70248 rows of 24 x 128 (1.3 GB): store 222 us, 5890 GB/s (the same within the noise of two runs
+// with cached loads and stores); four rows per block with the next row's loads ahead took 300 us, the
 // registers cost more in blocks per SM than the chain of count, index and data costs a block.
 // Both kernels are HBM-bound row passes: one block per kept row covers K and V of that row, a lane
 // owns 8 consecutive elements (16 bytes of bf16, 8 bytes of codes), the D / 8 lanes of one head sit

@@ -7,7 +7,8 @@ library's kernels.  The sequence follows Algorithm 1 of the paper for one layer:
   the one-step-predicted unedited tokens; gather of the recomputed rows of Q (K, V) -> region attention
   writing its rows back at their joint-sequence positions, the RIKV store in the same launch
 
-(four kernel launches: partition, moves, attention, merge of the attention's shared items).
+(three kernel launches: partition, moves, attention; a fourth where a kernel of its own merges the attention's shared
+items.  `regione_kernel_launches` counts them).
 
 No step needs a host round trip: per-request counts stay in device memory.
 Capacities are host integers chosen by the caller (``plan_capacity`` reads the
