@@ -101,10 +101,12 @@ class _Group:
 def _check_rows(got, shape, name, region=False):
     """A velocity of another shape than [B, N, C]: one of all tokens may come without the batch dimension of a single
     request; one of a region step holds its rows at the beginning of each request's, for a single request as many as it
-    likes (at least the edited tokens)."""
+    likes.  Returns how many rows of a request may be read: edited tokens beyond them are reported as
+    REGIONE_DEV_BOUNDS and keep their place (only a single request can have fewer than N, so strides stay N)."""
     same = got.numel() == shape[0] * shape[1] * shape[2]
     if not (same or shape[0] == 1 if region else same and shape[max(3 - len(got), 0):] == got):
         raise binding.RegionEError(f"{name} must have shape {shape}, got {tuple(got)}")
+    return shape[1] if same else min(shape[1], got.numel() // shape[2])
 
 
 _NAN = float("nan")
@@ -160,10 +162,10 @@ class RegionELoop:
         if x.shape != shape:
             raise b.RegionEError(f"x must have shape {shape}, got {tuple(x.shape)}")
 
-        def decay(p_v, scale, dts, p_target, p_keep, p_n):
+        def decay(p_v, scale, dts, p_target, p_keep, p_n, rows=N):
             s = b._stream(stream)                           # (the model may have made another stream current)
             check(lib.regione_velocity_decay(p_v, floats(scale, B, "scale"), floats(dts, B, "dt"), p_target, p_keep, p_n,
-                                             B, N, C, p_st, s), "regione_velocity_decay")
+                                             B, rows, C, p_st, s), "regione_velocity_decay")
             tr.launches += 1
 
         def spread(values):
@@ -284,7 +286,7 @@ class RegionELoop:
                         continue
                     scale = spread([(g, g.product if kind == "reuse" else 1.0) for g in gs])
                     dts = spread([(g, ts[g.k] - ts[g.k + 1]) for g in gs])
-                    v_e, p_v, p_keep = self.v_cache, p_vc, None
+                    v_e, p_v, p_keep, rows = self.v_cache, p_vc, None, N
                     if kind == "compute":
                         if uniform:
                             v_e = model.region(self.x_e, ts[gs[0].k], self.edit_idx, self.n_edit)
@@ -297,11 +299,11 @@ class RegionELoop:
                         tr.model_region_calls += 1
                         p_v, p_keep = ptr(v_e, bf, "v_e"), p_vc
                         if v_e.shape != shape:
-                            _check_rows(v_e.shape, shape, "v_e", region=True)
+                            rows = _check_rows(v_e.shape, shape, "v_e", region=True)
                     if hook is not None:
                         hook("decay_in", k0, dict(v=v_e, x_e=self.x_e, scale=listed(scale), dt=listed(dts),
                                                   n_edit=self.n_edit, active=members(gs)))
-                    decay(p_v, scale, dts, p_xe, p_keep, p_ne)
+                    decay(p_v, scale, dts, p_xe, p_keep, p_ne, rows)
                     if hook is not None:
                         hook("decay_out", k0, dict(x_e=self.x_e, active=members(gs)))
                     for g in gs:
@@ -379,9 +381,9 @@ class RegionELoop:
             if follow:
                 s = stream_of(device())
             region_calls += 1
-            p_v = ptr(v_e, bf, "v_e")
+            p_v, rows = ptr(v_e, bf, "v_e"), N
             if v_e.shape != shape:
-                _check_rows(v_e.shape, shape, "v_e", region=True)
+                rows = _check_rows(v_e.shape, shape, "v_e", region=True)
             log.append((k, "R", "compute", 1.0))
             scales, dts, product, again = [1.0] * B, [ts[k] - ts[k + 1]] * B, 1.0, True
             first, keep, k = k, p_vc, k + 1
@@ -397,11 +399,11 @@ class RegionELoop:
                     continue
                 # (a run that is longer than one update carries goes on in the next, from the kept velocity)
                 n = k - first
-                check(run(p_v, (c_float * (n * B))(*scales), (c_float * (n * B))(*dts), n, p_xe, keep, p_ne, B, N, C, p_st, s),
+                check(run(p_v, (c_float * (n * B))(*scales), (c_float * (n * B))(*dts), n, p_xe, keep, p_ne, B, rows, C, p_st, s),
                       "regione_velocity_decay_run")
                 launches += 1
                 if again:
                     log.append((k, "R", "reuse", product))
-                    p_v, keep, first, scales, dts = p_vc, None, k, [product] * B, [ts[k] - ts[k + 1]] * B
+                    p_v, rows, keep, first, scales, dts = p_vc, N, None, k, [product] * B, [ts[k] - ts[k + 1]] * B
                     k += 1
         return x, LoopTrace(log, [list(log) for _ in range(B)], full_calls, region_calls, launches)

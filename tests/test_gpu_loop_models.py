@@ -52,6 +52,26 @@ def test_velocities_of_other_shapes_with_the_same_rows(hooked):
 
 
 @pytest.mark.parametrize("hooked", [False, True])
+def test_a_region_velocity_with_too_few_rows_is_reported(hooked):
+    """A single request's velocity of fewer rows than it has edited tokens: its rows are applied, none is read behind them."""
+    import torch
+    _, ref, _, target, noise = _case(B=1)
+    before = []
+    class Model(_Shaped):
+        def region(self, x_e, t, edit_idx, n_edit):
+            before.append(x_e[0].clone())
+            return super().region(x_e, t, edit_idx, n_edit)
+    lp = _loop(noise)
+    lp.hook = (lambda *a: None) if hooked else None
+    lp.run(dev_bf16(noise), dev_bf16(ref), Model(dev_bf16(target), region=lambda v: v[:, :5].contiguous()))
+    torch.cuda.synchronize()
+    n = int(lp.n_edit[0])
+    assert n > 5 and int(lp.dev_status[0]) == binding.DEV_BOUNDS
+    assert torch.equal(lp.x_e[0, 5:n], before[-1][5:n]) and not torch.equal(lp.x_e[0, :5], before[-1][:5])
+    assert not lp.v_cache[0, 5:].any()
+
+
+@pytest.mark.parametrize("hooked", [False, True])
 def test_loop_follows_the_stream_that_the_model_makes_current(hooked):
     """A model that leaves another stream current, its velocity still being computed there when it returns."""
     import torch
