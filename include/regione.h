@@ -495,8 +495,8 @@ int regione_merge(const regione_bf16* x_full, const regione_bf16* v_last_full,
 
 /* ------------------------------------------------------------------------------------------
  * Cross-check and self-test entry points.  Test infrastructure that has to live inside the
- * library because it runs on the device; no product entry point above calls either of them,
- * and both are ordinary (not dependency-wait) launches.
+ * library because it runs the library's own device code; no product entry point above calls any of
+ * them, the launches are ordinary (not dependency-wait) ones, and the last one runs on the host.
  * ------------------------------------------------------------------------------------------ */
 
 /*
@@ -527,6 +527,22 @@ int regione_crosscheck_region_attention(const regione_bf16* q,
  */
 int regione_selftest_bounded_wait(long long limit_cycles, int32_t* dev_status, long long* out,
                                   void* stream);
+
+/*
+ * How the attention kernel cuts the work of one call into shares, one per block: the functions that
+ * the kernel's planning warps run, run on the host.  n_q, n_fresh, n_cache: host int32 [B].  all_rows: 0, or
+ * the rows of K and V of which the query and cached rows are parts.  spread: plan of the calls whose K and V
+ * are more than L2 keeps.  sms: SMs of the GPU.
+ * shape    : host int32 [4], {blocks, query pairs per head at capacity, workspace slots per item, team}
+ * segments : host int32 [cap, 12], one row per run of key tiles, block after block in the order of the walk:
+ *            {block, request, head, query pair, first key tile, key tiles, slot among the item's shares, shares
+ *            of the item, workspace index of its slot 1, distance of the later ones, distance of its shares,
+ *            plan (0 whole items, 1 cost axis, 2 cost axis behind waves, 3 teams, -1 dealt in a wave)}
+ * Returns the number of segments (which may exceed cap), -1 for invalid arguments.
+ */
+int regione_selftest_attention_plan(const int32_t* n_q, const int32_t* n_fresh, const int32_t* n_cache, int B, int Nq_cap,
+                                    int Nf_cap, int Nc_cap, int H, int all_rows, int spread, int sms, int32_t* shape,
+                                    int32_t* segments, int cap);
 
 #ifdef __cplusplus
 }

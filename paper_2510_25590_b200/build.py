@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libregione.so")
 SOURCES = ["api.cu", "partition.cu", "rowcopy.cu", "latent.cu", "gamma.cu", "kvquant.cu", "freshqkv.cu", "attention_simt.cu", "attention_tc.cu",
            "step.cu"]
-HEADERS = ["common.cuh", "rowcopy.cuh", "sm100_ptx.cuh"]
+HEADERS = ["attention_plan.cuh", "common.cuh", "rowcopy.cuh", "sm100_ptx.cuh"]
 
 
 def _nvcc() -> str:

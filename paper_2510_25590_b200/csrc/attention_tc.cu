@@ -56,6 +56,11 @@
 // own rows (kMergeHere) or a small second kernel does (kMergeKernel; the attention kernel leaves it a table of the items
 // that its share boundaries cut): see merges_here.  The share length is bounded below so that no item is spread over
 // more slots than the workspace holds.
+// On large calls the power limit sets the time, and K and V read from HBM again and again cost as much of it as all of the
+// softmax: where they are more than L2 keeps, whole pairs are dealt in waves, or teams of CTAs walk a head together
+// (plan_shares).  8704 x 8704, 24 heads: 1.18 -> 0.16 GB read from HBM, 35 -> 10 M sectors across the halves of L2, 838 -> 768
+// us at 1 kW; 8448 x 8448 refreshing the cache 819 -> 750; 2048 of 8448 rows refreshed 245 -> 227; 1075 x 8448 143 -> 134;
+// 819 x 8704 201 -> 139 MB, 127 -> 123 us.
 // Where the capacities allow only few items (choose_cluster), an item is shared by a cluster of 2 to 8 CTAs instead, an
 // equal run of its key tiles each; they leave their partial rows in shared memory, where the cluster's CTAs read
 // them (distributed shared memory) and write the output: no workspace, no second kernel, no plan to derive.  Measured,
@@ -76,6 +81,7 @@
 #include <atomic>
 #include <chrono>
 
+#include "attention_plan.cuh"
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -87,8 +93,6 @@ constexpr int kWarpLoad = kSoftmaxWarps, kWarpPv = kSoftmaxWarps + 1, kWarpCopy 
 constexpr int kAttnThreads = 32 * (kSoftmaxWarps + 4);
 constexpr int kWalkBarrier = 4, kWalkThreads = kAttnThreads - 32;   // named barrier of the warps that walk the segments
 constexpr int kMaxCluster = 8;           // CTAs that may share an item through their shared memories
-constexpr int kBM = 128;                 // query rows per tile
-constexpr int kBN = 128;                 // key rows per shared-memory tile
 constexpr int kBH = 64;                  // key rows per chunk (half a tile): the logits one thread holds
 constexpr float kOutgrownSum = 1.152921504606846976e18f;   // 2^60: chunk sum at which a reference maximum is renewed
 constexpr int kCopySlots = 2;             // cache refresh: batches of rows under way at once, at most
@@ -131,7 +135,9 @@ struct SegInfo {
     int b, h, q0, nq;           // request, head, first query row, live query rows of the request
     int j_first, n_tiles;       // key tiles [j_first, j_first + n_tiles) of the item
     int nt_c, nt, nc, nf;       // cached key tiles, all key tiles, live keys of the two segments
-    int item, slot, n_slots;    // item index within the launch, slot among the shares that touch it
+    int slot, n_slots;          // slot among the shares that touch the item
+    int slot_at, slot_step;     // where slot 1 lies in the workspace, and how far apart the later ones do (slot 0: slot_at - 1)
+    int share_step;             // how far apart the shares are that touch the item
     int apart;                  // (launch that refreshes the cache) fresh rows are not in K and V themselves: see ReqShape
 };
 
@@ -176,34 +182,30 @@ static_assert(offsetof(AttnCtrl, kv_empty) == kBarKvEmpty * 8 && offsetof(AttnCt
 // What share c tells the merge kernel: the item that the boundary between shares c - 1 and c
 // cuts, if c is the second share of that item (so every cut item is named exactly once).
 struct alignas(16) CutItem {
-    int valid, b, h, qp, n_slots, nq, pad0, pad1;
+    int valid, b, h, qp, n_slots, nq, slot_at, slot_step;
 };
 
 // Who puts the parts of an item together that several CTAs work on: a merge kernel behind this one, the item's
-// first share, or the CTAs of a cluster.  (Instantiations of their own: the code of one form costs the others 1 to 2 %.)
+// first share, or the CTAs of a cluster; and whether the plan minds the order in which K and V are read (see plan_shares).
+// (Instantiations of their own: the code of one form costs the others 1 to 2 %; the plan of the spread forms 205 queries x
+// 8448 keys 7 %.)
 enum MergeForm { kMergeKernel, kMergeHere, kMergeCluster };
+enum KernelForm { kFormKernel, kFormHere, kFormCluster, kFormSpreadKernel, kFormSpreadHere };
 
-struct AttnParams {
-    const int32_t* n_q;
-    const int32_t* n_fresh;
-    const int32_t* n_cache;
-    int B, Nq_cap, Nf_cap, Nc_cap, H;
-    int P_cap;           // query pairs per (request, head) at capacity
-    int max_slots;       // workspace slots per item (>= 2)
+struct AttnParams : PlanInput {
     float scale_log2e;
+    int out_cap;         // rows per request of `out` (Nq_cap without out_rows)
     uint16_t* out;       // [B, out_cap, H, D]
     const int32_t* out_rows;   // nullptr: query row i goes to out row i; else to row out_rows[b, i]
-    int out_cap;         // rows per request of `out` (Nq_cap without out_rows)
-    int all_rows;        // > 0: query and cached rows of a request are parts of its K and V of this many rows (see ReqShape)
     int32_t* dev_status;
-    float* part_o;       // [B, H, P_cap, max_slots, 256, D] unnormalised outputs; kMergeHere: [..., D / 4, 256, 4]
-    float2* part_ml;     // [B, H, P_cap, max_slots, 256]    (running max in the exp2 domain, sum)
-    int cluster;         // kMergeCluster: CTAs that share an item; no workspace
+    float* part_o;       // [B * H * P_cap * max_slots, 256, D] unnormalised outputs; kMergeHere: [..., D / 4, 256, 4]
+    float2* part_ml;     // [B * H * P_cap * max_slots, 256]    (running max in the exp2 domain, sum)
     CutItem* cut;        // kMergeKernel: [grid] the item that the start of each share cuts
     unsigned long long* ready;       // kMergeHere: [grid] `epoch`: the share's partial rows are in its slot (0: merged),
                                      // and a word behind them, `epoch`: a launch of this epoch has timed out
     unsigned long long epoch;        // of this launch: what lies in the workspace otherwise is not equal to it
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
+    int cluster;         // kMergeCluster: CTAs that share an item; no workspace
 };
 
 // Cache refresh fused into a full step: the rows rows[l][b, 0..n[l][b]) (ascending) of the K and V that the launch
@@ -218,187 +220,6 @@ struct StoreParams {
     const uint8_t* src[2];              // K, V [B, src_cap, H, D]
     uint8_t* dst[4];
 };
-
-// ---- the plan every CTA (and the merge kernel) derives from the device-side counts ------------
-// Shares are cut on a cost axis measured in ticks, not in steps, so that they take about the same
-// time: a key tile of a full query pair costs kTickPair, a key tile of a pair with one live query
-// tile kTickSingle (its even and odd key tiles run side by side on the two tile roles; measured per
-// thread block against its share's composition: 0.55 to 0.56 of a pair's step, not half), and every
-// item starts with kTickStart ticks that stand for the drain of the previous segment and the fill of
-// the new one (measured the same way: 3.5 to 6 pair steps depending on the workload, 5 with 819 x 8704 and
-// 1075 x 8448 keys, 24 heads of 128; 100, 120 and 140 ticks for items that a first share merges: 0 to +3 %).
-constexpr int kTickPair = 16, kTickSingle = 9, kTickStart = 80;
-
-struct ReqShape {
-    int nq, nf, nc;      // clamped counts
-    int np;              // live query pairs
-    int nt_c, nt;        // cached key tiles, all key tiles
-    long long items;     // H * np
-    int steps;           // steps of an item: max(nt, 1) (an item without keys writes zeros in one step)
-    bool apart;          // AttnParams::all_rows: the query and cached rows are not all rows (more tokens were edited than
-                         // the capacity holds), so the request attends over [cached | fresh] as copied ahead of the launch
-    int w_last;          // ticks per step of the last query pair
-    long long ticks_full, ticks_last, head_ticks, ticks;   // per full-pair item, last item, head, request
-};
-
-// (IN_PLACE: the launch may read K and V in place, see ReqShape::apart; 0.5 us a call for the launches that never do)
-template <bool IN_PLACE>
-__device__ __forceinline__ ReqShape req_shape(const AttnParams& p, int b, bool* bad = nullptr) {
-    ReqShape r;
-    int nq = p.n_q[b], nf = p.n_fresh[b], nc = p.n_cache == nullptr ? 0 : p.n_cache[b];      // (nullptr: no cached segment)
-    const int all_rows = IN_PLACE ? p.all_rows : 0;
-    const int c_cap = all_rows > 0 ? all_rows : p.Nc_cap;
-    if (nq < 0 || nq > p.Nq_cap || nf < 0 || nf > p.Nf_cap || nc < 0 || nc > c_cap) {
-        if (bad) *bad = true;
-        nq = max(0, min(nq, p.Nq_cap));
-        nf = max(0, min(nf, p.Nf_cap));
-        nc = max(0, min(nc, c_cap));
-    }
-    r.apart = all_rows > 0 && nq + nc != all_rows;
-    if (all_rows > 0) {
-        nf = r.apart ? nq : all_rows;
-        nc = r.apart ? nc : 0;
-    }
-    r.nq = nq; r.nf = nf; r.nc = nc;
-    r.np = (nq + 2 * kBM - 1) / (2 * kBM);
-    r.nt_c = (nc + kBN - 1) / kBN;
-    r.nt = r.nt_c + (nf + kBN - 1) / kBN;
-    r.items = (long long)p.H * r.np;
-    r.steps = max(r.nt, 1);
-    r.w_last = (nq - (r.np - 1) * 2 * kBM > kBM) ? kTickPair : kTickSingle;
-    r.ticks_full = kTickStart + (long long)kTickPair * r.steps;
-    r.ticks_last = kTickStart + (long long)r.w_last * r.steps;
-    r.head_ticks = r.np > 0 ? (r.np - 1) * r.ticks_full + r.ticks_last : 0;
-    r.ticks = p.H * r.head_ticks;
-    return r;
-}
-
-// How the launch's work is cut into shares, one per CTA.
-//  - whole items: when handing out whole items wastes at most 6 % of the grid's last round, items
-//    are dealt round-robin and never split (no workspace traffic, no merge): positions count items.
-//  - otherwise positions count ticks and CTA c owns the steps whose first tick lies in
-//    [c * chunk, (c + 1) * chunk); shares may cut items.  The share length is bounded below so
-//    that an item never meets more than max_slots shares.
-struct Plan {
-    bool whole_items;
-    long long total, chunk;
-};
-
-template <bool IN_PLACE>
-__device__ __forceinline__ Plan plan_shares(const AttnParams& p, int grid, bool* bad = nullptr) {
-    Plan pl;
-    long long items = 0, ticks = 0, span = 0;      // span: first tick of an item's last step, at most
-    for (int b = 0; b < p.B; ++b) {
-        const ReqShape r = req_shape<IN_PLACE>(p, b, bad);
-        items += r.items;
-        ticks += r.ticks;
-        if (r.np > 0) span = max(span, (long long)(r.np > 1 ? kTickPair : r.w_last) * (r.steps - 1));
-    }
-    const long long per = (items + grid - 1) / grid;
-    pl.whole_items = per * grid * 100 <= items * 106;
-    if (pl.whole_items) {
-        pl.total = items;
-        pl.chunk = max(per, 1LL);
-    } else {
-        pl.total = ticks;
-        pl.chunk = (ticks + grid - 1) / grid;
-        // an item meets at most span / chunk + 2 shares: keep that within max_slots; and a share is
-        // at least one step long, so that every share between an item's first and last holds a
-        // step of it (and writes its slot)
-        const long long floor_len = max(span / (p.max_slots - 1) + 1, (long long)kTickPair);
-        if (pl.chunk < floor_len) pl.chunk = floor_len;
-    }
-    return pl;
-}
-
-// The part of one item that a CTA works on.
-struct Segment {
-    int b, h, qp;
-    ReqShape r;
-    int j_first, n_steps;   // steps [j_first, j_first + n_steps) of the item; n_steps may be 0
-    int slot, n_slots;      // this share's slot among the shares that hold steps of the item
-    long long next;         // position behind the item
-};
-
-// a / b for non-negative a and positive b; positions fit 32 bits in every realistic launch, and a
-// 32-bit division is several times shorter than a 64-bit one (the lookups below sit between two
-// segments, on every thread's path).
-__device__ __forceinline__ long long div_pos(long long a, long long b) {
-    if (((a | b) >> 32) == 0) return (long long)((unsigned)a / (unsigned)b);
-    return a / b;
-}
-
-// Shares that hold steps of the item whose step 0 starts at tick `first_tick`.
-__device__ __forceinline__ void item_slots(const Plan& pl, long long first_tick, int w, int steps,
-                                           int& c_first, int& n_slots) {
-    c_first = (int)div_pos(first_tick, pl.chunk);
-    n_slots = (int)div_pos(first_tick + (long long)w * (steps - 1), pl.chunk) - c_first + 1;
-}
-
-// Whole-item plan: the item with index `idx`.
-template <bool IN_PLACE>
-__device__ __forceinline__ Segment segment_whole(const AttnParams& p, long long idx) {
-    Segment sg;
-    long long base = 0;
-    int b = 0;
-    ReqShape r = req_shape<IN_PLACE>(p, 0);
-    while (idx >= base + r.items && b + 1 < p.B) {
-        base += r.items;
-        ++b;
-        r = req_shape<IN_PLACE>(p, b);
-    }
-    const long long item = idx - base;
-    sg.b = b; sg.r = r;
-    sg.h = r.np > 0 ? (int)(item / r.np) : 0;
-    sg.qp = (int)(item - (long long)sg.h * r.np);
-    sg.j_first = 0;
-    sg.n_steps = r.np > 0 ? r.steps : 0;
-    sg.slot = 0; sg.n_slots = 1;
-    sg.next = idx + 1;
-    return sg;
-}
-
-// Tick plan: the item that contains tick `pos`, and the steps of it that share `c` owns.
-template <bool IN_PLACE>
-__device__ __forceinline__ Segment segment_ticks(const AttnParams& p, const Plan& pl, long long pos,
-                                                 int c) {
-    Segment sg;
-    long long base = 0;
-    int b = 0;
-    ReqShape r = req_shape<IN_PLACE>(p, 0);
-    while (pos >= base + r.ticks && b + 1 < p.B) {
-        base += r.ticks;
-        ++b;
-        r = req_shape<IN_PLACE>(p, b);
-    }
-    sg.b = b; sg.r = r;
-    if (r.np == 0) {                                  // nothing left behind the last live request
-        sg.h = sg.qp = sg.j_first = sg.n_steps = sg.slot = 0;
-        sg.n_slots = 1;
-        sg.next = pl.total;
-        return sg;
-    }
-    const long long rel = pos - base;
-    sg.h = (int)div_pos(rel, r.head_ticks);
-    const long long rem = rel - (long long)sg.h * r.head_ticks;
-    sg.qp = (int)min(div_pos(rem, r.ticks_full), (long long)(r.np - 1));
-    const long long t0 = base + (long long)sg.h * r.head_ticks + (long long)sg.qp * r.ticks_full;
-    const bool last = sg.qp == r.np - 1;
-    const int w = last ? r.w_last : kTickPair;
-    const long long first_tick = t0 + kTickStart;
-    const long long lo = (long long)c * pl.chunk, hi = lo + pl.chunk;
-    long long s_lo = lo <= first_tick ? 0 : div_pos(lo - first_tick + w - 1, w);
-    long long s_hi = hi <= first_tick ? 0 : div_pos(hi - first_tick + w - 1, w);
-    s_lo = min(s_lo, (long long)r.steps);
-    s_hi = min(s_hi, (long long)r.steps);
-    sg.j_first = (int)s_lo;
-    sg.n_steps = (int)(s_hi - s_lo);
-    int c_first;
-    item_slots(pl, first_tick, w, r.steps, c_first, sg.n_slots);
-    sg.slot = c - c_first;
-    sg.next = t0 + (last ? r.ticks_last : r.ticks_full);
-    return sg;
-}
 
 // Bounded wait on phase `parity` of an mbarrier: true when the phase completed, false when another
 // role has already given up or `limit` cycles have passed (then the abort flag is raised and
@@ -545,21 +366,15 @@ __device__ __forceinline__ VLanding v_landing(AttnCtrl* ctrl, bool split, int n_
 // kMaxOnly finds the rows' maxima, kExact repeats the pass with them.
 enum WalkMode { kWalk, kMaxOnly, kExact };
 
-// Share of a CTA on the cost axis.  The first share of an item waits for the later ones, so shares are dealt
-// from the last block to the first: blocks become resident in the order of their indexes on this GPU, and a block
-// waits only for blocks ahead of it, whatever else runs.  CUDA does not promise that order; were it another, a wait
-// for a block that cannot start would end with its bound and REGIONE_DEV_TIMEOUT.
-__device__ __forceinline__ int my_share() { return (int)gridDim.x - 1 - (int)blockIdx.x; }
-
-// Bounded wait of a warp for the partial rows of the n shares behind this CTA's (true: they are there).  A launch that
+// Bounded wait of a warp for the partial rows of the n shares behind this CTA's, `step` apart (true: they are there).  A launch that
 // has timed out may have left flags of its epoch behind, and a graph repeats the launch with that epoch: the repetition
 // gives up as well, instead of merging what the flags no longer stand for.  (Asked here, beside the flags: at the start
 // of the launch the question cost 819 queries x 8704 keys 1.5 us.)
-__device__ __forceinline__ bool wait_shares(const AttnParams& p, int n, int lane, volatile int* abort_flag) {
+__device__ __forceinline__ bool wait_shares(const AttnParams& p, int n, int step, int lane, volatile int* abort_flag) {
     const bool asks_failed = lane == 31;   // (the word behind the flags; n < 31)
     bool there = lane >= n && !asks_failed, gave_up = false;
     if (!there) {
-        const unsigned long long* const word = p.ready + (asks_failed ? (int)gridDim.x : my_share() + 1 + lane);
+        const unsigned long long* const word = p.ready + (asks_failed ? (int)gridDim.x : share_of(gridDim.x, blockIdx.x) + (1 + lane) * step);
         const long long t0 = clock64();
         while (!(there = (ptx::ld_acquire_u64(word) == p.epoch) != asks_failed) && !gave_up) {
             gave_up = *abort_flag != 0;
@@ -741,7 +556,8 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
     const int per = split ? (kPieces >= 4 ? 1 : (t == 0 ? 1 : 0)) : kPieces / 2;
     const int pc0 = split ? (kPieces >= 4 ? 2 * ck + t : ck) : ck * per, pc1 = pc0 + per;
     const uint32_t tO = tmem + lane_sel + 256 + (split ? 0 : t * D);
-    const size_t prow = ((size_t)it.item * p.max_slots + it.slot) * (2 * kBM) + qt * kBM + row;     // row in the slot
+    const size_t slot_at = (size_t)(it.slot > 0 ? it.slot_at + (it.slot - 1) * it.slot_step : it.slot_at - 1);
+    const size_t prow = slot_at * (2 * kBM) + qt * kBM + row;           // row in the slot
     const float inv = l > 0.f ? 1.f / l : 0.f;
     uint8_t* const stage = smem_gen + Cfg::kStageAt + warp * 4096;
     const size_t out_stride = (size_t)p.H * D * 2;
@@ -808,7 +624,7 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, AttnCtrl* c
             } else {
                 if constexpr (FORM == kMergeHere) {
                     // unnormalised O of this segment -> its workspace slot: a warp writes 512 contiguous bytes per store
-                    float4* const o = reinterpret_cast<float4*>(p.part_o) + ((size_t)it.item * p.max_slots + it.slot) * (2 * kBM) * (D / 4) +
+                    float4* const o = reinterpret_cast<float4*>(p.part_o) + slot_at * (2 * kBM) * (D / 4) +
                                       (size_t)pc * 8 * (2 * kBM) + qt * kBM + row;
                     if (live) {
 #pragma unroll
@@ -925,11 +741,11 @@ __device__ __forceinline__ void merge_shares(const AttnParams& p, const SegInfo&
         dst_row = -1;
     }
     const float2 own = *(reinterpret_cast<const float2*>(smem_gen + Cfg::kPartialMlAt) + row);
-    const size_t slot1 = (size_t)it.item * p.max_slots + 1;
+    const size_t slot1 = (size_t)it.slot_at, step = (size_t)it.slot_step * (2 * kBM);
     const float2* const others_ml = p.part_ml + slot1 * (2 * kBM) + row;
     uint8_t* const out0 = reinterpret_cast<uint8_t*>(p.out) + (((size_t)it.b * p.out_cap) * p.H + it.h) * D * 2;
     const size_t out_stride = (size_t)p.H * D * 2;
-    if (!wait_shares(p, n - 1, lane, abort_flag)) return;
+    if (!wait_shares(p, n - 1, it.share_step, lane, abort_flag)) return;
     if (rb * 32 >= it.nq - it.q0) return;
 #pragma unroll 1
     for (int pc = (warp & 1) * (D / 64); pc < ((warp & 1) + 1) * (D / 64); ++pc) {
@@ -943,7 +759,7 @@ __device__ __forceinline__ void merge_shares(const AttnParams& p, const SegInfo&
         float M = own.y > 0.f ? own.x : -INFINITY;
         if (ml.y > 0.f) M = fmaxf(M, ml.x);
         for (int sl = 1; sl < n - 1; ++sl) {
-            const float2 o = __ldcg(others_ml + sl * (2 * kBM));
+            const float2 o = __ldcg(others_ml + sl * step);
             if (o.y > 0.f) M = fmaxf(M, o.x);
         }
         float w = own.y > 0.f ? fast_exp2(own.x - M) : 0.f;
@@ -967,9 +783,9 @@ __device__ __forceinline__ void merge_shares(const AttnParams& p, const SegInfo&
                 }
             }
             if (sl >= n - 1) break;
-            ml = __ldcg(others_ml + sl * (2 * kBM));
+            ml = __ldcg(others_ml + sl * step);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) x[q] = __ldcg(others + ((size_t)sl * (D / 4) + q) * (2 * kBM));
+            for (int q = 0; q < 8; ++q) x[q] = __ldcg(others + sl * step * (D / 4) + q * (2 * kBM));
         }
         const float inv = L > 0.f ? 1.f / L : 0.f;
         __syncwarp();                              // (every lane has read its own rows' chunks)
@@ -1321,13 +1137,12 @@ __device__ __forceinline__ void issue_pv_segment(const AttnParams& p, AttnCtrl* 
 }
 
 // ---- the share of one CTA: plan and next segment (one warp computes them, the others read SegInfo) --------
+template <bool IN_PLACE, bool SPREAD>
 struct ShareCursor {
-    Plan pl;
-    long long pos, hi;
+    ShareWalk<IN_PLACE, SPREAD> walk;
     bool first;
     // The only segment of a CTA whose item is shared by a cluster: rank r of n takes the key tiles
     // [r * nt / n, (r + 1) * nt / n) (possibly none) and reads back its part of the rows.
-    template <bool IN_PLACE>
     __device__ __forceinline__ void of_cluster(const AttnParams& p, SegInfo* out, const int lane, bool* bad) {
         int idx = blockIdx.x / p.cluster;
         const int rank = blockIdx.x - idx * p.cluster;
@@ -1337,7 +1152,6 @@ struct ShareCursor {
             idx -= p.H * r.np;
             r = req_shape<IN_PLACE>(p, ++b, bad);
         }
-        pos = hi = 0;
         first = false;
         if (lane != 0) return;
         out->live = idx < p.H * r.np;
@@ -1348,44 +1162,52 @@ struct ShareCursor {
         out->nq = r.nq; out->nt_c = r.nt_c; out->nt = r.nt; out->nc = r.nc; out->nf = r.nf;
         out->j_first = rank * r.nt / p.cluster;
         out->n_tiles = (rank + 1) * r.nt / p.cluster - out->j_first;
-        out->item = 0; out->slot = rank; out->n_slots = p.cluster;
+        out->slot = rank; out->n_slots = p.cluster; out->slot_at = 1; out->slot_step = out->share_step = 1;
         if (IN_PLACE) out->apart = r.apart;
     }
+    // This CTA's share of the plan.
+    __device__ __forceinline__ void of_plan(const AttnParams& p, bool* bad) {
+        walk.begin(p, gridDim.x, blockIdx.x, bad);
+        first = true;
+    }
     // The next live segment of the share into *out (out->live = 0 when the share ends).
-    template <int FORM, bool IN_PLACE>
+    template <int FORM>
     __device__ __forceinline__ void next(const AttnParams& p, SegInfo* out, const int lane) {
-        while (pos < hi) {
-            const Segment it = pl.whole_items ? segment_whole<IN_PLACE>(p, pos) : segment_ticks<IN_PLACE>(p, pl, pos, my_share());
-            if (FORM == kMergeKernel && first && lane == 0) {
+        Segment it;
+        while (walk.next(p, gridDim.x, blockIdx.x, it)) {
+            if (FORM == kMergeKernel && first && !it.in_wave) {
                 // tell the merge kernel which item the start of this share cuts
-                CutItem ci;
-                ci.valid = (!pl.whole_items && it.r.np > 0 && it.n_slots >= 2 && it.slot == 1) ? 1 : 0;
-                ci.b = it.b; ci.h = it.h; ci.qp = it.qp; ci.n_slots = it.n_slots; ci.nq = it.r.nq;
-                ci.pad0 = ci.pad1 = 0;
-                p.cut[my_share()] = ci;
+                if (lane == 0) {
+                    CutItem ci;
+                    ci.valid = (it.n_steps > 0 && it.n_slots >= 2 && it.slot == 1) ? 1 : 0;
+                    ci.b = it.b; ci.h = it.h; ci.qp = it.qp; ci.n_slots = it.n_slots; ci.nq = it.r.nq;
+                    ci.slot_at = it.slot_at; ci.slot_step = it.slot_step;
+                    p.cut[share_of(gridDim.x, blockIdx.x)] = ci;
+                }
+                first = false;
             }
-            first = false;
-            pos = pl.whole_items ? pos + gridDim.x : it.next;
             if (it.n_steps == 0) continue;
             if (lane == 0) {
                 out->b = it.b; out->h = it.h; out->q0 = it.qp * (2 * kBM); out->nq = it.r.nq;
                 out->j_first = it.j_first; out->n_tiles = it.r.nt == 0 ? 0 : it.n_steps;
                 out->nt_c = it.r.nt_c; out->nt = it.r.nt; out->nc = it.r.nc; out->nf = it.r.nf;
-                out->item = (it.b * p.H + it.h) * p.P_cap + it.qp; out->slot = it.slot; out->n_slots = it.n_slots;
+                out->slot = it.slot; out->n_slots = it.n_slots;
+                out->slot_at = it.slot_at; out->slot_step = it.slot_step;
+                out->share_step = walk.step;
                 if (IN_PLACE) out->apart = it.r.apart;
                 out->live = 1;
             }
             return;
         }
         if (lane == 0) {
-            if (FORM == kMergeKernel && first) p.cut[my_share()].valid = 0;
+            if (FORM == kMergeKernel && first) p.cut[share_of(gridDim.x, blockIdx.x)].valid = 0;
             out->live = 0;
         }
         first = false;
     }
 };
 
-template <int D, bool STORE, int FORM>
+template <int D, bool STORE, int FORM, bool SPREAD>
 __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, const CUtensorMap& tm_kf,
                                                       const CUtensorMap& tm_vf, const CUtensorMap& tm_kc,
                                                       const CUtensorMap& tm_vc, const CUtensorMap& tm_ka,
@@ -1403,14 +1225,11 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     }
     grid_dependency_wait();                             // (everything below reads the launch's inputs)
     grid_launch_dependents();                           // the next kernel may queue up behind this CTA
-    ShareCursor cur;
+    ShareCursor<STORE, SPREAD> cur;
     if (warp == kWarpS) {
-        // this CTA's share [pos, hi) of the item sequence or of the cost axis
-        // (whole items are dealt round-robin, so that the CTAs running at any one time work on
-        // neighbouring items, which share K/V tiles in L2; a share of steps is one contiguous range)
         bool bad = false;
         if constexpr (FORM == kMergeCluster) {
-            cur.of_cluster<STORE>(p, &ctrl->seg[0], lane, &bad);
+            cur.of_cluster(p, &ctrl->seg[0], lane, &bad);
             if (lane == 0) {
                 ctrl->seg[1].live = 0;
                 ptx::mbar_init(ptx::smem_addr(&ctrl->peers_ready), p.cluster);
@@ -1418,11 +1237,8 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
                 ptx::fence_barrier_init();
             }
         } else {
-            cur.pl = plan_shares<STORE>(p, gridDim.x, &bad);
-            cur.pos = cur.pl.whole_items ? (long long)blockIdx.x : (long long)my_share() * cur.pl.chunk;
-            cur.first = true;
-            cur.hi = cur.pl.whole_items ? cur.pl.total : min(cur.pos + cur.pl.chunk, cur.pl.total);
-            cur.next<FORM, STORE>(p, &ctrl->seg[0], lane);
+            cur.of_plan(p, &bad);
+            cur.template next<FORM>(p, &ctrl->seg[0], lane);
         }
         if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         if (lane == 0) ctrl->abort_flag = 0;
@@ -1500,7 +1316,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             } else if (warp == kWarpS) {
                 issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
                 // (the next segment is planned behind the last product, ahead of the end of this one)
-                if (FORM != kMergeCluster && mode == kWalk) cur.next<FORM, STORE>(p, &ctrl->seg[k ^ 1], lane);
+                if (FORM != kMergeCluster && mode == kWalk) cur.template next<FORM>(p, &ctrl->seg[k ^ 1], lane);
             } else {
                 issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, lane, mode);
             }
@@ -1514,7 +1330,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
                                                 // not told yet; in shared memory, to be merged with the later shares'
         auto tell = [&]() {
             // (every warp's rows are ordered before this by the barriers of tear_down and repeat)
-            if (publish && !*abort_flag) ptx::st_release_u64(p.ready + my_share(), p.epoch);
+            if (publish && !*abort_flag) ptx::st_release_u64(p.ready + share_of(gridDim.x, blockIdx.x), p.epoch);
             publish = false;
         };
         while (ctrl->seg[k].live && !*abort_flag) {
@@ -1536,7 +1352,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             // every warp has seen the flags: they are left as no launch's epoch (a graph replays the launch with the
             // one it has)
             named_barrier(3, 32 * kSoftmaxWarps);
-            if (threadIdx.x < it.n_slots - 1) p.ready[my_share() + 1 + threadIdx.x] = 0;
+            if (threadIdx.x < it.n_slots - 1) p.ready[share_of(gridDim.x, blockIdx.x) + (1 + threadIdx.x) * it.share_step] = 0;
         }
     }
 
@@ -1596,7 +1412,7 @@ region_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                            const __grid_constant__ CUtensorMap tm_kc,
                            const __grid_constant__ CUtensorMap tm_vc, const AttnParams p) {
     const StoreParams none = {};
-    attention_kernel_body<D, false, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_kf, tm_vf, p, none);
+    attention_kernel_body<D, false, (FORM >= kFormSpreadKernel ? FORM - kFormSpreadKernel : FORM), (FORM >= kFormSpreadKernel)>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_kf, tm_vf, p, none);
 }
 template <int D, int FORM>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -1608,7 +1424,7 @@ region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_ka,
                               const __grid_constant__ CUtensorMap tm_va, const AttnParams p,
                               const __grid_constant__ StoreParams sp) {
-    attention_kernel_body<D, true, FORM>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_ka, tm_va, p, sp);
+    attention_kernel_body<D, true, (FORM >= kFormSpreadKernel ? FORM - kFormSpreadKernel : FORM), (FORM >= kFormSpreadKernel)>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_ka, tm_va, p, sp);
 }
 
 // Merges the workspace slots of the items that were spread over several shares:
@@ -1629,18 +1445,17 @@ region_attention_combine_kernel(const AttnParams p) {
     grid_dependency_wait();
     const int4* cp = reinterpret_cast<const int4*>(p.cut + blockIdx.x + 1);
     const int4 c0 = cp[0], c1 = cp[1];
-    const int b = c0.y, h = c0.z, qp = c0.w, n_slots = c1.x, nq = c1.y;
+    const int b = c0.y, h = c0.z, qp = c0.w, n_slots = c1.x, nq = c1.y, slot_at = c1.z, slot_step = c1.w;
     // (the fields are checked so that a table left incomplete by an aborted launch cannot send
     // this kernel out of bounds)
     if (c0.x != 1 || b < 0 || b >= p.B || h < 0 || h >= p.H || qp < 0 || qp >= p.P_cap ||
-        n_slots < 2 || n_slots > p.max_slots || n_slots > kCombineMaxSlots || nq > p.Nq_cap)
+        n_slots < 2 || n_slots > kCombineMaxSlots || nq > p.Nq_cap || slot_at < 1 || slot_step < 1 || slot_step > 2 ||
+        slot_at + (n_slots - 2) * slot_step >= p.B * p.H * p.P_cap * p.max_slots)
         return;
     const int lane = threadIdx.x & 31;
     const int r_local = blockIdx.y * 8 + (threadIdx.x >> 5);
     const int qrow = qp * (2 * kBM) + r_local;
     if (qrow >= nq) return;
-    const size_t item_idx = ((size_t)b * p.H + h) * p.P_cap + qp;
-    const size_t prow0 = item_idx * p.max_slots * (2 * kBM) + r_local;
     // (issued together with the slots' loads, used after them)
     const int dst_row = p.out_rows != nullptr ? p.out_rows[(size_t)b * p.Nq_cap + qrow] : qrow;
 
@@ -1649,7 +1464,7 @@ region_attention_combine_kernel(const AttnParams p) {
 #pragma unroll
     for (int s = 0; s < kCombineMaxSlots; ++s) {
         if (s < n_slots) {
-            const size_t prow = prow0 + (size_t)s * (2 * kBM);
+            const size_t prow = (size_t)(s > 0 ? slot_at + (s - 1) * slot_step : slot_at - 1) * (2 * kBM) + r_local;
             ml[s] = p.part_ml[prow];
             o[s] = *reinterpret_cast<const Vec*>(p.part_o + prow * D + lane * E);
         }
@@ -1711,7 +1526,7 @@ __global__ void bounded_wait_selftest_kernel(long long limit, int32_t* dev_statu
     long long shortest = 0x7fffffffffffffffLL;
     for (int i = 0; i < 3; ++i) {
         const long long t0 = clock64();
-        if (i == 2) done |= wait_shares(p, 1, lane, &abort_flag[2]);             // (a wait of the whole warp)
+        if (i == 2) done |= wait_shares(p, 1, 1, lane, &abort_flag[2]);             // (a wait of the whole warp)
         else if (lane == 0)
             done |= i == 0 ? wait_bar(ptx::smem_addr(&bar), 0, &abort_flag[0], dev_status, limit)
                            : wait_bar_cluster(ptx::smem_addr(&bar), &abort_flag[1], dev_status, limit);
@@ -1763,12 +1578,12 @@ struct LaunchPlan {
     int grid, P_cap, max_slots;
 };
 
-static LaunchPlan plan_launch(int B, int Nq_cap, int Nf_cap, int Nc_cap, int H) {
+static LaunchPlan plan_launch(int B, int Nq_cap, int Nf_cap, int Nc_cap, int H, int sms = sm_count()) {
     LaunchPlan lp;
     lp.P_cap = (Nq_cap + 2 * kBM - 1) / (2 * kBM);
     const long long nt_cap = std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN);
     const long long total_cap = (long long)B * H * lp.P_cap * nt_cap;
-    lp.grid = (int)std::min<long long>(sm_count(), std::max<long long>(total_cap, 1));
+    lp.grid = (int)std::min<long long>(sms, std::max<long long>(total_cap, 1));
     const long long share = (total_cap + lp.grid - 1) / lp.grid;
     lp.max_slots = (int)std::min<long long>(8, std::max<long long>(2, (nt_cap + share - 1) / share + 1));
     return lp;
@@ -1833,12 +1648,12 @@ static int prepare_kernel(const int** fitting) {
     const int dev = current_device();
     if (dev < 0) return REGIONE_CUDA_ERROR;
     if (!__atomic_load_n(&configured[dev], __ATOMIC_ACQUIRE)) {
-        if (cudaFuncSetAttribute(main_kernel<D, STORE, kMergeKernel>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 AttnCfg<D>::kSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(main_kernel<D, STORE, kMergeHere>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 AttnCfg<D>::kSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(main_kernel<D, STORE, kMergeCluster>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 AttnCfg<D>::kSmemBytes) != cudaSuccess)
+        auto opt_in = [](auto kernel) {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<D>::kSmemBytes) == cudaSuccess;
+        };
+        if (!opt_in(main_kernel<D, STORE, kFormKernel>()) || !opt_in(main_kernel<D, STORE, kFormHere>()) ||
+            !opt_in(main_kernel<D, STORE, kFormCluster>()) || !opt_in(main_kernel<D, STORE, kFormSpreadKernel>()) ||
+            !opt_in(main_kernel<D, STORE, kFormSpreadHere>()))
             return REGIONE_CUDA_ERROR;
         for (int n = 2; n <= kMaxCluster; ++n) {
             cudaLaunchConfig_t cfg = {};
@@ -1851,7 +1666,7 @@ static int prepare_kernel(const int** fitting) {
             cfg.attrs = attr;
             cfg.numAttrs = 1;
             int fit = 0;
-            if (cudaOccupancyMaxActiveClusters(&fit, main_kernel<D, STORE, kMergeCluster>(), &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&fit, main_kernel<D, STORE, kFormCluster>(), &cfg) != cudaSuccess) {
                 (void)cudaGetLastError();
                 fit = 0;
             }
@@ -1875,10 +1690,9 @@ static bool keeps_cuts(const AttnParams& p) {
 
 // How many CTAs share an item through a cluster, 0: shares of the cost axis with a merge kernel behind them.
 // Few items (at most one cluster of two per pair of SMs) are better off in clusters: the shares of the cost axis are
-// balanced to a step, but every cut item's rows go through the workspace (7300 cycles per pair of tiles, all
-// CTAs at once) and a second kernel (8 us behind the attention's last block), about kTickMerge ticks in all against
-// kTickCluster for a merge through distributed shared memory.  Both sides' ticks from the capacities:
-constexpr int kTickMerge = 125, kTickCluster = 45;
+// balanced to a step, but their cut items cost about kTickMerge ticks against kTickCluster for a merge through distributed
+// shared memory.  Both sides' ticks from the capacities:
+constexpr int kTickCluster = 45;
 static int choose_cluster(const int* fitting, const AttnParams& p, int nt) {
     if (keeps_cuts(p)) return 0;
     const long long items = (long long)p.B * p.H * p.P_cap;
@@ -1913,6 +1727,17 @@ static bool merges_here(const AttnParams& p, int grid, int nt) {
     return p.max_slots <= 3 && items <= 4LL * grid && items * nt >= 40LL * grid;
 }
 
+// Whether the plan minds the order in which K and V are read (see plan_shares): where they are more than L2 keeps (126 MB
+// in two halves, each of which holds what its own SMs read).  Measured, without -> with, us: 1075 queries x 8448 keys of 128,
+// 8 heads (33 MB) 57.4 -> 58.1, 12 (49 MB) 77.2 -> 79.6, 16 (66 MB) 99.1 -> 97.5, 24 (99 MB) 146.3 -> 136.9; 8704 x
+// 8704, 8 heads 268 -> 272, 12 401 -> 398, 16 561 -> 525, 24 845 -> 767; a step that refreshes 2048 of 8448 rows, 12 heads
+// 125.8 -> 127.2, 16 162.7 -> 159.6, 24 248.7 -> 229.4.
+constexpr long long kSpreadBytes = 60LL << 20;
+template <int D>
+static bool minds_order(const AttnParams& p) {
+    return !keeps_cuts(p) && 4LL * D * p.B * p.H * ((long long)p.Nf_cap + p.Nc_cap) >= kSpreadBytes;
+}
+
 template <int D, bool STORE>
 static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams& sp, int grid, int nt_cap, cudaStream_t st) {
     const int* fitting = nullptr;
@@ -1934,25 +1759,28 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = prm.cluster > 0 ? 2 : 1;
+    const bool spread = prm.cluster == 0 && minds_order<D>(prm);
+    prm.team = spread ? choose_team(prm, grid, nt_cap) : 0;
     cudaError_t e;
     auto launch = [&](auto kernel) {
         if constexpr (STORE) return launch_counted(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6], prm, sp);
         else return launch_counted(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
     };
-    const int form = prm.cluster > 0 ? kMergeCluster : merges_here(prm, grid, nt_cap) ? kMergeHere : kMergeKernel;
-    e = form == kMergeCluster ? launch(main_kernel<D, STORE, kMergeCluster>())
-        : form == kMergeHere  ? launch(main_kernel<D, STORE, kMergeHere>())
-                              : launch(main_kernel<D, STORE, kMergeKernel>());
+    const bool here = prm.cluster == 0 && merges_here(prm, grid, nt_cap);
+    if (prm.cluster > 0) e = launch(main_kernel<D, STORE, kFormCluster>());
+    else if (spread) e = here ? launch(main_kernel<D, STORE, kFormSpreadHere>()) : launch(main_kernel<D, STORE, kFormSpreadKernel>());
+    else e = here ? launch(main_kernel<D, STORE, kFormHere>()) : launch(main_kernel<D, STORE, kFormKernel>());
     if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
     // the merge kernel may become resident while the attention kernel drains (it waits for that
     // kernel's completion before it reads a slot)
-    if (grid < 2 || form != kMergeKernel) return launch_status(cudaGetLastError());     // nothing is cut
+    if (grid < 2 || prm.cluster > 0 || here) return launch_status(cudaGetLastError());     // nothing is cut
     const dim3 cgrid((unsigned)(grid - 1), (2 * kBM) / 8, 1);
-    if (prm.max_slots <= 2)
+    const int most_slots = spread ? std::max(prm.max_slots, kWaveSlots) : prm.max_slots;
+    if (most_slots <= 2)
         e = launch_overlapped(region_attention_combine_kernel<D, 2>, cgrid, dim3(256), 0, st, prm);
-    else if (prm.max_slots <= 3)
+    else if (most_slots <= 3)
         e = launch_overlapped(region_attention_combine_kernel<D, 3>, cgrid, dim3(256), 0, st, prm);
-    else if (prm.max_slots <= 4)
+    else if (most_slots <= 4)
         e = launch_overlapped(region_attention_combine_kernel<D, 4>, cgrid, dim3(256), 0, st, prm);
     else
         e = launch_overlapped(region_attention_combine_kernel<D, 8>, cgrid, dim3(256), 0, st, prm);
@@ -2031,6 +1859,26 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
                    : launch_tc<128, false>(maps, prm, sp, lp.grid, nt_cap, st);
 }
 
+// The segments of every block of a launch, as the planning warps walk them (host).
+template <bool IN_PLACE, bool SPREAD>
+static int list_segments(const PlanInput& p, int grid, int32_t* out, int cap) {
+    int n = 0;
+    for (int block = 0; block < grid; ++block) {
+        ShareWalk<IN_PLACE, SPREAD> walk;
+        bool bad = false;
+        walk.begin(p, grid, block, &bad);
+        Segment it;
+        while (walk.next(p, grid, block, it)) {
+            if (it.n_steps == 0) continue;
+            const int32_t row[12] = {block,   it.b,       it.h,       it.qp,        it.j_first, it.n_steps,
+                                     it.slot, it.n_slots, it.slot_at, it.slot_step, walk.step,  it.in_wave ? -1 : (int)walk.pl.kind};
+            if (n < cap) std::copy(row, row + 12, out + 12 * (size_t)n);
+            ++n;
+        }
+    }
+    return n;
+}
+
 // ---- variant with library-owned scratch -----------------------------------------------------
 // The split-KV partials of regione_region_attention_static live here instead of in a caller
 // workspace.  The array is part of the library image: every GPU that loads the library keeps
@@ -2068,6 +1916,25 @@ extern "C" int regione_selftest_bounded_wait(long long limit_cycles, int32_t* de
     if (limit_cycles < 1 || limit_cycles > 100000000LL) return REGIONE_INVALID_ARG;
     bounded_wait_selftest_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(limit_cycles, dev_status, out);
     return launch_status(cudaGetLastError());
+}
+
+extern "C" int regione_selftest_attention_plan(const int32_t* n_q, const int32_t* n_fresh, const int32_t* n_cache, int B, int Nq_cap,
+                                               int Nf_cap, int Nc_cap, int H, int all_rows, int spread, int sms, int32_t* shape,
+                                               int32_t* segments, int cap) {
+    using namespace regione;
+    if (!n_q || !n_fresh || !n_cache || !shape || (!segments && cap > 0) || B < 1 || H < 1 || Nq_cap < 1 || Nf_cap < 0 || Nc_cap < 0 ||
+        all_rows < 0 || sms < 1 || cap < 0)
+        return -1;
+    const LaunchPlan lp = plan_launch(B, Nq_cap, Nf_cap, Nc_cap, H, sms);
+    PlanInput p = {};
+    p.n_q = n_q; p.n_fresh = n_fresh; p.n_cache = n_cache;
+    p.B = B; p.Nq_cap = Nq_cap; p.Nf_cap = Nf_cap; p.Nc_cap = Nc_cap; p.H = H;
+    p.P_cap = lp.P_cap; p.max_slots = lp.max_slots; p.all_rows = all_rows;
+    p.team = spread ? choose_team(p, lp.grid, std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN)) : 0;
+    shape[0] = lp.grid; shape[1] = lp.P_cap; shape[2] = lp.max_slots; shape[3] = p.team;
+    if (all_rows > 0)
+        return spread ? list_segments<true, true>(p, lp.grid, segments, cap) : list_segments<true, false>(p, lp.grid, segments, cap);
+    return spread ? list_segments<false, true>(p, lp.grid, segments, cap) : list_segments<false, false>(p, lp.grid, segments, cap);
 }
 
 extern "C" int regione_region_attention_static(
