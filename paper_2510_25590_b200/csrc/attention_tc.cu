@@ -206,6 +206,7 @@ struct AttnParams : PlanInput {
     unsigned long long epoch;        // of this launch: what lies in the workspace otherwise is not equal to it
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
     int cluster;         // kMergeCluster: CTAs that share an item; no workspace
+    int kv_once;         // every key tile is read by one CTA: it need not stay in L2
 };
 
 // Cache refresh fused into a full step: the rows rows[l][b, 0..n[l][b]) (ascending) of the K and V that the launch
@@ -1019,9 +1020,12 @@ __device__ __forceinline__ void load_segment(const CUtensorMap* tm_q, const CUte
             const CUtensorMap* map = cached ? (is_v ? tm_vc : tm_kc) : (is_v ? tm_vf : tm_kf);
             const uint32_t bar = is_v ? v_landing(ctrl, split, n_stages, i >> 1).bar : ptx::smem_addr(&ctrl->kv_full[stage]);
             ptx::mbar_arrive_expect_tx(bar, kTileBytes);
-            for (int hf = 0; hf < Cfg::kHalves; ++hf)
-                ptx::tma_load_4d(ring + stage * kTileBytes + hf * kHalfBytes, map, bar, hf * 64, h,
-                                 (cached ? j : j - nt_c) * kBN, b);
+            const int row = (cached ? j : j - nt_c) * kBN;
+            for (int hf = 0; hf < Cfg::kHalves; ++hf) {
+                const uint32_t dst = ring + stage * kTileBytes + hf * kHalfBytes;
+                if (p.kv_once) ptx::tma_load_4d_once(dst, map, bar, hf * 64, h, row, b);
+                else ptx::tma_load_4d(dst, map, bar, hf * 64, h, row, b);
+            }
         }
         __syncwarp();
         if (++stage == n_stages) { stage = 0; ++use; }
@@ -1733,9 +1737,20 @@ static bool merges_here(const AttnParams& p, int grid, int nt) {
 // 8704, 8 heads 268 -> 272, 12 401 -> 398, 16 561 -> 525, 24 845 -> 767; a step that refreshes 2048 of 8448 rows, 12 heads
 // 125.8 -> 127.2, 16 162.7 -> 159.6, 24 248.7 -> 229.4.
 constexpr long long kSpreadBytes = 60LL << 20;
+static long long kv_bytes(const AttnParams& p, int d) { return 4LL * d * p.B * p.H * ((long long)p.Nf_cap + p.Nc_cap); }
 template <int D>
 static bool minds_order(const AttnParams& p) {
-    return !keeps_cuts(p) && 4LL * D * p.B * p.H * ((long long)p.Nf_cap + p.Nc_cap) >= kSpreadBytes;
+    return !keeps_cuts(p) && kv_bytes(p, D) >= kSpreadBytes;
+}
+
+// Whether K and V are told to leave L2 first: where a head has one query pair, so that they pass through once, and are more
+// than L2 keeps.  What the next launches read (lists, latents, partial rows, code) stays then.  A step with 205 of 8448 rows
+// 54.1 -> 52.2 us, four requests of 92 x 4736 74.9 -> 69.9 (other K and V in every call).  Not where several pairs read
+// them (four requests of 1382 x 18944 +7 %, 1075 x 8448 +1 to 2 %, 819 x 8704 -1 %), nor where they fit L2 (two requests of
+// 102 x 2176, 8 heads of 64, +2 to 4 %), nor in calls without a row list, whose cache an 8-bit decode may just have
+// left in L2 (205 x 8448 behind one 67.3 -> 69.5).
+static bool reads_once(const AttnParams& p, int d) {
+    return p.P_cap == 1 && p.out_rows != nullptr && kv_bytes(p, d) >= kSpreadBytes;
 }
 
 template <int D, bool STORE>
@@ -1851,6 +1866,7 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
     prm.ready = reinterpret_cast<unsigned long long*>(prm.cut + lp.grid);
     prm.epoch = next_epoch();
     prm.cluster = 0;
+    prm.kv_once = reads_once(prm, D);
     const int nt_cap = std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN);
     if (store != nullptr)
         return D == 64 ? launch_tc<64, true>(maps, prm, sp, lp.grid, nt_cap, st)

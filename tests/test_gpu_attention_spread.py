@@ -43,3 +43,23 @@ def test_spread_plans(D, H, n_q, n_f, n_c):
     for b, n in enumerate(n_q):
         if n > 0:
             assert_close(host_f64(out[b, :n]), host_f64(want[b, :n]), f"request {b}")
+
+
+def test_one_pair_a_head_behind_a_row_list():
+    """K and V that pass through once (told to leave L2 first): rows of a ragged pair at their places."""
+    import torch
+    H, D, n_q, n_c = 24, 128, 205, 5400
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = lambda n: torch.randn((1, n, H, D), generator=g, device="cuda", dtype=torch.bfloat16)
+    q, kf, vf, kc, vc = r(n_q), r(n_q), r(n_q), r(n_c), r(n_c)
+    rows = torch.randperm(n_q + n_c, device="cuda", generator=g)[:n_q].int()[None].contiguous()
+    nq, nc = dev_i32([n_q]), dev_i32([n_c])
+    assert 4 * D * H * (n_q + n_c) >= 60 << 20
+    ws = torch.empty(binding.region_attention_workspace(1, n_q, n_q, n_c, H, D), dtype=torch.uint8, device="cuda")
+    status, want = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros_like(q)
+    full = torch.zeros((1, n_q + n_c, H, D), dtype=torch.bfloat16, device="cuda")
+    binding.region_attention_scatter(q, kf, vf, kc, vc, nq, nq, nc, full, rows, workspace=ws, dev_status=status)
+    binding.crosscheck_region_attention(q, kf, vf, kc, vc, nq, nq, nc, want)
+    torch.cuda.synchronize()
+    assert int(status[0]) == 0
+    assert_close(host_f64(full[0, rows[0].long()]), host_f64(want[0]), "rows")
