@@ -493,6 +493,28 @@ int regione_merge(const regione_bf16* x_full, const regione_bf16* v_last_full,
                   int B, int N, int Ne_cap, int C, regione_bf16* x_out,
                   int32_t* dev_status, void* stream);
 
+/*
+ * The latent updates of Algorithm 1's loop over buffers that stay the same from step to step (Sec. 3, the Euler sampler
+ * equation; Sec. 4, the case equation of the AVDCache and the one-step estimation equation), each in one launch
+ * with what the loop does next to the same rows.  Layouts as above with Ne_cap = N.
+ */
+typedef struct {
+    int B, N, C;                       /* requests, tokens, channels (a multiple of 8) */
+    regione_bf16* x;                   /* [B, N, C] latent */
+    regione_bf16 *x_e, *v_last, *v_cache; /* [B, N, C] X^E, the last full step's velocity, the last region step's */
+    const int32_t *slot, *n_edit;      /* [B, N], [B] as the partition left them */
+    int32_t* dev_status;               /* nullable */
+} regione_loop_plan;
+
+/* x <- x - dt v, v_last <- v; with starts_run also x_e[slot[n]] <- x[n] (what regione_gather with the partition's list
+ * leaves): a run of region steps follows.  v dev bf16 [B, N, C], dt host f32 [B]; NaN: the request sits the call out. */
+int regione_loop_full_step(const regione_loop_plan* plan, const regione_bf16* v, const float* dt, int starts_run, void* stream);
+
+/* regione_velocity_decay_run on x_e with v_e (kept in v_cache) or, v_e = NULL, with v_cache; dt_unedited (host f32 [B],
+ * nullable): the run of region steps ends here, and regione_merge of x_e and v_last into x is part of the launch. */
+int regione_loop_region_steps(const regione_loop_plan* plan, const regione_bf16* v_e, const float* scale, const float* dt,
+                              int n_steps, const float* dt_unedited, void* stream);
+
 /* ------------------------------------------------------------------------------------------
  * Cross-check and self-test entry points.  Test infrastructure that has to live inside the
  * library because it runs the library's own device code; no product entry point above calls any of

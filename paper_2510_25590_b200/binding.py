@@ -34,6 +34,12 @@ class StepPlan(ctypes.Structure):
                 [("workspace_bytes", c_size_t), ("dev_status", c_void_p)])
 
 
+class LoopPlan(ctypes.Structure):
+    """``regione_loop_plan``: sizes and buffers of a sampler loop."""
+    _fields_ = ([(n, c_int) for n in ("B", "N", "C")] +
+                [(n, c_void_p) for n in ("x", "x_e", "v_last", "v_cache", "slot", "n_edit", "dev_status")])
+
+
 # every symbol include/regione.h declares: name -> (restype, argtypes)
 _P = c_void_p
 SIGNATURES = {
@@ -68,6 +74,8 @@ SIGNATURES = {
     "regione_gamma_fit": (c_int, [_P, c_int, c_int, c_int64, _P, _P, _P, _P]),
     "regione_velocity_decay": (c_int, [_P, _P, _P, _P, _P, _P, c_int, c_int, c_int, _P, _P]),
     "regione_velocity_decay_run": (c_int, [_P, _P, _P, c_int, _P, _P, _P, c_int, c_int, c_int, _P, _P]),
+    "regione_loop_full_step": (c_int, [POINTER(LoopPlan), _P, _P, c_int, _P]),
+    "regione_loop_region_steps": (c_int, [POINTER(LoopPlan), _P, _P, _P, c_int, _P, _P]),
     "regione_merge": (c_int, [_P, _P, _P, _P, _P, c_int, c_int, c_int, c_int, _P, _P, _P]),
     "regione_crosscheck_region_attention": (c_int, [_P] * 8 + [c_int] * 6 + [c_float, _P, _P, _P]),
     "regione_selftest_bounded_wait": (c_int, [c_longlong, _P, _P, _P]),

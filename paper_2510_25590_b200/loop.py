@@ -321,8 +321,9 @@ class RegionELoop:
 
     def _run_together(self, x, ref, model, stream, ts):
         """All steps of requests that take them at the same time, without a hook: what ``run`` does then, with one
-        set of scalars for the batch.  Host-bound (28 steps of 4096 tokens, 16 of them full: 112 us of kernels;
-        347 us with the bookkeeping per group and a call per step, 247 us this way)."""
+        set of scalars for the batch.  Host-bound (28 steps of 4096 tokens, 12 of them full: about 6 us a
+        launch, 253 us with a launch for each of the loop's operations, 214 us this way), so an update and what the loop does next to the same rows are one call: a full step and the gather of X^E behind
+        it, the last update of a run of region steps and the merge."""
         import torch
         cfg, b = self.cfg, binding
         kinds, after, gammas, delta = cfg.kinds, cfg.partition_after, cfg.gammas, cfg.delta
@@ -332,16 +333,16 @@ class RegionELoop:
         # (the model may make another stream current: looked up again behind each of its calls)
         follow, stream_of, device = stream is None, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
         p_x, p_xe, p_vl, p_vc = ptr(x, bf, "x"), self.x_e.data_ptr(), self.v_last_full.data_ptr(), self.v_cache.data_ptr()
-        p_slot, p_ne, p_all, p_st = (t.data_ptr() for t in (self.slot, self.n_edit, self.n_all, self.dev_status))
+        p_slot, p_ne, p_st = (t.data_ptr() for t in (self.slot, self.n_edit, self.dev_status))
         if x.shape != shape:
             raise b.RegionEError(f"x must have shape {shape}, got {tuple(x.shape)}")
-        one, decay, run = c_float * B, lib.regione_velocity_decay, lib.regione_velocity_decay_run
-        unit = one(*[1.0] * B)
+        plan = b.LoopPlan(B, N, C, p_x, p_xe, p_vl, p_vc, p_slot, p_ne, p_st)
+        one, full_step, region_steps = c_float * B, lib.regione_loop_full_step, lib.regione_loop_region_steps
         log, launches, full_calls, region_calls = [], 0, 0, 0
         partitioned, t_run, k = False, None, 0               # t_run: time at which the present run of region steps began
 
         while k < T or t_run is not None:
-            if t_run is not None and (k == T or kinds[k] == "F"):
+            if t_run is not None and (k == T or kinds[k] == "F"):     # (a region velocity of other rows came last)
                 # x has not changed since the run began: edited tokens from X^E, the others by one step of the last
                 # full velocity over the whole run
                 check(lib.regione_merge(p_x, p_vl, p_xe, p_slot, one(*[t_run - ts[k]] * B), B, N, N, C, p_x, p_st, s),
@@ -360,8 +361,11 @@ class RegionELoop:
                 p_v = ptr(v, bf, "v")
                 if v.shape != shape:
                     _check_rows(v.shape, shape, "v")
-                check(decay(p_v, unit, one(*[t - t_next] * B), p_x, p_vl, p_all, B, N, C, p_st, s), "regione_velocity_decay")
+                starts = partitioned and k + 1 < T and kinds[k + 1] == "R"
+                check(full_step(plan, p_v, one(*[t - t_next] * B), starts, s), "regione_loop_full_step")
                 launches += 1
+                if starts:
+                    t_run = t_next
                 if last_before:
                     b.partition(x, v, ref, t_next, cfg.metric, cfg.threshold, self.mask, self.edit_idx, self.keep_idx,
                                 self.slot, self.n_edit, dev_status=self.dev_status, stream=stream)
@@ -386,7 +390,7 @@ class RegionELoop:
                 rows = _check_rows(v_e.shape, shape, "v_e", region=True)
             log.append((k, "R", "compute", 1.0))
             scales, dts, product, again = [1.0] * B, [ts[k] - ts[k + 1]] * B, 1.0, True
-            first, keep, k = k, p_vc, k + 1
+            first, k = k, k + 1
             while again:
                 again = False
                 if k < T and kinds[k] == "R":
@@ -399,11 +403,19 @@ class RegionELoop:
                     continue
                 # (a run that is longer than one update carries goes on in the next, from the kept velocity)
                 n = k - first
-                check(run(p_v, (c_float * (n * B))(*scales), (c_float * (n * B))(*dts), n, p_xe, keep, p_ne, B, rows, C, p_st, s),
-                      "regione_velocity_decay_run")
+                many = c_float * (n * B)
+                if rows == N:
+                    ends = not again and (k == T or kinds[k] == "F")
+                    check(region_steps(plan, p_v, many(*scales), many(*dts), n, one(*[t_run - ts[k]] * B) if ends else None, s),
+                          "regione_loop_region_steps")
+                    if ends:
+                        t_run = None
+                else:
+                    check(lib.regione_velocity_decay_run(p_v, many(*scales), many(*dts), n, p_xe, p_vc, p_ne, B, rows, C, p_st, s),
+                          "regione_velocity_decay_run")
                 launches += 1
                 if again:
                     log.append((k, "R", "reuse", product))
-                    p_v, rows, keep, first, scales, dts = p_vc, N, None, k, [product] * B, [ts[k] - ts[k + 1]] * B
+                    p_v, rows, first, scales, dts = None, N, k, [product] * B, [ts[k] - ts[k + 1]] * B
                     k += 1
         return x, LoopTrace(log, [list(log) for _ in range(B)], full_calls, region_calls, launches)
