@@ -116,6 +116,11 @@ struct Plan {
     int waves;
     int team, n_teams;
 };
+// Items dealt round-robin are walked in step too.  Percent of the mean share up to which they are, where the grid's last round
+// also is full by kWhole's rule: at the power limit CTAs that end early leave their power to the others, and nothing is
+// merged.  Waves -> whole items, us: four requests of 1382 x 18944, 24 heads (10.6 % above the mean) 1424 -> 1376, three of
+// 4916 x 4916 (4.8 %) 868 -> 841.
+constexpr int kWholeWaste = 112;
 constexpr int kWaveSlots = 4;    // kWaves: shares that a cut item may meet
 
 template <bool IN_PLACE, bool SPREAD>
@@ -137,13 +142,14 @@ REGIONE_HD Plan plan_shares(const PlanInput& p, int grid, bool* bad = nullptr) {
         }
     }
     const long long per = div_pos(items + grid - 1, grid);
+    const bool whole = per * grid * 100 <= items * 106;
     if (SPREAD) {
         pl.origin = 0;
         pl.waves = 0;
         const long long pair_ticks = kTickStart + (long long)kTickPair * steps, fair = div_pos(ticks + grid - 1, grid);
         // (whole items need no merge, and no second start)
         const bool spread = steps > 0 && per * pair_ticks > fair + kTickStart + kTickMerge;
-        if (spread && p.team == 0 && pairs >= 2 * grid) {
+        if (spread && p.team == 0 && pairs >= 2 * grid && !(whole && per * pair_ticks * 100 <= fair * kWholeWaste)) {
             pl.kind = kWaves;
             pl.waves = (int)div_pos(pairs, grid);
             long long left = pairs - (long long)pl.waves * grid;
@@ -179,7 +185,7 @@ REGIONE_HD Plan plan_shares(const PlanInput& p, int grid, bool* bad = nullptr) {
             }
         }
     }
-    if (per * grid * 100 <= items * 106) {
+    if (whole) {
         pl.kind = kWhole;
         pl.total = items;
         pl.chunk = max(per, 1LL);
