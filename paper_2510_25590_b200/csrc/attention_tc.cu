@@ -1550,31 +1550,6 @@ __global__ void bounded_wait_selftest_kernel(long long limit, int32_t* dev_statu
 
 // ---- host side ---------------------------------------------------------------------------------
 
-constexpr int kMaxDevices = 64;
-
-// Ordinal of the current device, or -1 (no device / an ordinal beyond the per-device caches).
-static int current_device() {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return -1;
-    return dev;
-}
-
-// SM count of the current device (cached per device; 148 when it cannot be read).
-static int sm_count() {
-    static int cached[kMaxDevices] = {};
-    const int dev = current_device();
-    if (dev < 0) return 148;
-    int n = __atomic_load_n(&cached[dev], __ATOMIC_ACQUIRE);
-    if (n == 0) {
-        int v = 0;
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-            return 148;
-        n = v;
-        __atomic_store_n(&cached[dev], n, __ATOMIC_RELEASE);
-    }
-    return n;
-}
-
 // Launch shape from the capacities alone (so the workspace query and the launch agree): a
 // persistent grid of one CTA per SM (fewer if there are fewer steps), and enough workspace slots
 // per item that the longest item can be spread over the shares it meets at that grid size.

@@ -91,6 +91,31 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
     return launch_counted(&cfg, kernel, static_cast<Params>(args)...);
 }
 
+constexpr int kMaxDevices = 64;
+
+// Ordinal of the current device, or -1 (no device / an ordinal beyond the per-device caches).
+inline int current_device() {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return -1;
+    return dev;
+}
+
+// SM count of the current device (cached per device; 148 when it cannot be read).
+inline int sm_count() {
+    static int cached[kMaxDevices] = {};
+    const int dev = current_device();
+    if (dev < 0) return 148;
+    int n = __atomic_load_n(&cached[dev], __ATOMIC_ACQUIRE);
+    if (n == 0) {
+        int v = 0;
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
+            return 148;
+        n = v;
+        __atomic_store_n(&cached[dev], n, __ATOMIC_RELEASE);
+    }
+    return n;
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Per-request scalars (sampler time, step length, decay product) reach a kernel by value, a chunk
