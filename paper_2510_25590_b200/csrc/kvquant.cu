@@ -19,7 +19,8 @@
 // (1.3 GB) 246.9 -> 242.4 us (5.4 TB/s), two requests of 5882 rows of 24 x 64 28.5 -> 23.2.  (Four rows per block with
 // the next row's loads ahead in registers took 1.3 times as long as one.)
 // Load: one block per kept row covers K and V of that row, a lane owns 8 consecutive elements (8 bytes of codes, 16 bytes of
-// bf16).
+// bf16); the codes of kQuantUnroll pieces are on their way before the first is widened, and are the first to leave L2.  7885
+// rows of 24 x 128 and the attention behind them, one piece at a time -> three: 128.8 -> 128.0 us.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -28,6 +29,7 @@
 namespace regione {
 
 constexpr int kQuantThreads = 256;
+constexpr int kQuantUnroll = 3;
 
 // Two fp32 -> two E4M3 codes (round to nearest even, saturating); `lo` lands in bits [7:0].
 __device__ __forceinline__ uint32_t pack_e4m3x2(float lo, float hi) {
@@ -233,17 +235,30 @@ rikv_load_e4m3_kernel(const uint8_t* __restrict__ k_q, const uint8_t* __restrict
     if (j >= live_rows(n_keep, b, Nc_cap, threadIdx.x == 0 && j == 0, dev_status)) return;
     const size_t dst_row = (size_t)b * Nc_cap + j;
     const int per_tensor = H * kLanesPerHead, total = 2 * per_tensor;
-    for (int c = threadIdx.x; c < total; c += kQuantThreads) {
-        const int is_v = c >= per_tensor, piece = c - (is_v ? per_tensor : 0);
-        const uint2 q = *reinterpret_cast<const uint2*>((is_v ? v_q : k_q) + dst_row * H * D + (size_t)piece * 8);
-        const float s = (is_v ? v_scale : k_scale)[dst_row * H + piece / kLanesPerHead];
-        // (code value) * 2^k is exact in bf16: 4 significant bits, exponent well inside the range
-        const float2 a = unpack_e4m3x2(q.x), c2 = unpack_e4m3x2(q.x >> 16);
-        const float2 e = unpack_e4m3x2(q.y), g = unpack_e4m3x2(q.y >> 16);
-        uint4 w;
-        w.x = pack_bf16x2(a.x * s, a.y * s); w.y = pack_bf16x2(c2.x * s, c2.y * s);
-        w.z = pack_bf16x2(e.x * s, e.y * s); w.w = pack_bf16x2(g.x * s, g.y * s);
-        *reinterpret_cast<uint4*>((is_v ? v_cache : k_cache) + dst_row * H * D + (size_t)piece * 8) = w;
+    for (int c0 = threadIdx.x; c0 < total; c0 += kQuantUnroll * kQuantThreads) {
+        uint2 q[kQuantUnroll];
+        float s[kQuantUnroll];
+#pragma unroll
+        for (int u = 0; u < kQuantUnroll; ++u) {
+            const int c = c0 + u * kQuantThreads;
+            if (c >= total) break;
+            const int is_v = c >= per_tensor, piece = c - (is_v ? per_tensor : 0);
+            q[u] = __ldcs(reinterpret_cast<const uint2*>((is_v ? v_q : k_q) + dst_row * H * D + (size_t)piece * 8));
+            s[u] = (is_v ? v_scale : k_scale)[dst_row * H + piece / kLanesPerHead];
+        }
+#pragma unroll
+        for (int u = 0; u < kQuantUnroll; ++u) {
+            const int c = c0 + u * kQuantThreads;
+            if (c >= total) break;
+            const int is_v = c >= per_tensor, piece = c - (is_v ? per_tensor : 0);
+            // (code value) * 2^k is exact in bf16: 4 significant bits, exponent well inside the range
+            const float2 a = unpack_e4m3x2(q[u].x), c2 = unpack_e4m3x2(q[u].x >> 16);
+            const float2 e = unpack_e4m3x2(q[u].y), g = unpack_e4m3x2(q[u].y >> 16);
+            uint4 w;
+            w.x = pack_bf16x2(a.x * s[u], a.y * s[u]); w.y = pack_bf16x2(c2.x * s[u], c2.y * s[u]);
+            w.z = pack_bf16x2(e.x * s[u], e.y * s[u]); w.w = pack_bf16x2(g.x * s[u], g.y * s[u]);
+            *reinterpret_cast<uint4*>((is_v ? v_cache : k_cache) + dst_row * H * D + (size_t)piece * 8) = w;
+        }
     }
 }
 
