@@ -1660,12 +1660,11 @@ static int prepare_kernel(const int** fitting) {
 // Rows that are put back into a joint sequence many times their number keep the cuts of the cost axis with kTickStart.
 // This line is neither the faster side's nor the more accurate one's: where an item is cut decides which reference
 // maximum its probabilities are rounded against, and against the rms of the whole buffer, mostly rows that were not
-// recomputed, the two forms differ from each other by up to 0.1 in single elements (by 0.033 to 0.043 from a sixteenth of
-// the rows on).  Against 64 bits, over the recomputed rows, clusters / cost axis: 64 of 8448 rows rel 2.32 / 2.31e-3, 32.7 /
-// 36.4 us; 128 2.31 / 2.31e-3, 33.6 / 38.7 us; 205 2.32 / 2.32e-3, 42.7 / 43.6 us; 704 2.33 / 2.33e-3, 74.4 / 79.8 us.  Line at
-// a twelfth -> a sixteenth: 510 of 5850 rows, 8 heads, 44.3 -> 40.2 us; 194 of 3698, 4 heads, 32.4 -> 28.5.
+// recomputed, the two forms differ from each other by up to 0.1 in single elements (by 0.04 from a twelfth of the rows
+// on).  Against 64 bits, over the recomputed rows, clusters / cost axis: 64 of 8448 rows rel 2.32 / 2.31e-3, 32.7 / 36.4 us;
+// 128 2.31 / 2.31e-3, 33.6 / 38.7 us; 205 2.32 / 2.32e-3, 42.7 / 43.6 us; 704 2.33 / 2.33e-3, 74.4 / 79.8 us.
 static bool keeps_cuts(const AttnParams& p) {
-    return p.out_rows != nullptr && 16LL * (p.Nq_cap - kBM / 2) < (long long)p.Nf_cap + p.Nc_cap;
+    return p.out_rows != nullptr && 12LL * (p.Nq_cap - kBM / 2) < (long long)p.Nf_cap + p.Nc_cap;
 }
 
 // How many CTAs share an item through a cluster, 0: shares of the cost axis with a merge kernel behind them.
