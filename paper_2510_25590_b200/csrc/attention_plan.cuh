@@ -118,8 +118,8 @@ struct Plan {
 };
 // Items dealt round-robin are walked in step too.  Percent of the mean share up to which they are, where the grid's last round
 // also is full by kWhole's rule: at the power limit CTAs that end early leave their power to the others, and nothing is
-// merged.  Waves -> whole items, us: four requests of 1382 x 18944, 24 heads (10.6 % above the mean) 1424 -> 1376, three of
-// 4916 x 4916 (4.8 %) 868 -> 841.
+// merged.  Waves -> whole items, us: three requests of 4916 x 4916, 24 heads (4.8 % above the mean) 868 -> 841; four of 1382 x
+// 18944 (10.6 %), with the line of keeps_cuts moved so that they came here, 1424 -> 1376.
 constexpr int kWholeWaste = 112;
 constexpr int kWaveSlots = 4;    // kWaves: shares that a cut item may meet
 
