@@ -80,6 +80,7 @@ def check(n_q, n_fresh, n_cache, caps, H, all_rows=0, spread=1, sms=148):
     ("2048 of 8448", [2048], 8448, (2048, 8448, 0), 24, 8448, TEAMS),
     ("1075 of 8448", [1075], 8448, (1075, 1075, 7373), 24, 0, TEAMS),
     ("eight pairs more than two waves: one wave", [256 * 38], 2048, (256 * 38, 2048, 0), 8, 0, WAVES),
+    ("three of 4916 x 4916: whole items fill the rounds", [4916] * 3, 4916, (4916, 4916, 0), 24, 0, WHOLE),
     ("requests whose key tiles differ", [819, 600], 8704, (896, 896, 8704), 24, 0, TICKS),
 ])
 def test_plans_of_known_shapes(name, n_q, n_keys, caps, H, all_rows, kind):
