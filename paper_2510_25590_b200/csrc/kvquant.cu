@@ -12,12 +12,10 @@
 //   elements of that row and head); written with frexp(amax) = m * 2^e, m in [0.5, 1):
 //   k = e - 9 + (m > 0.875); k = 0 for amax = 0; k is kept >= -100.
 //
-// Both kernels are HBM-bound row passes.
-// Store: a block per row read its count, its index and its data one after the other, and an SM had too few reads in flight
-// meanwhile; now every warp runs a ring of bulk copies (below), with 16 elements to a lane instead of 8 (three shuffles for a
-// maximum instead of four) and the scale taken from the maximum's bits.  Block per row -> rings: 70248 rows of 24 x 128
-// (1.3 GB) 246.9 -> 242.4 us (5.4 TB/s), two requests of 5882 rows of 24 x 64 28.5 -> 23.2.  (Four rows per block with
-// the next row's loads ahead in registers took 1.3 times as long as one.)
+// All kernels are HBM-bound row passes.
+// Store: a block per row reads its count, its index and its data one after the other, and an SM has few reads in flight
+// meanwhile unless the rows are long; in rings of bulk copies, one per warp, the chain is off the path.  See takes_rows for
+// which of the two takes a call.
 // Load: one block per kept row covers K and V of that row, a lane owns 8 consecutive elements (8 bytes of codes, 16 bytes of
 // bf16); the codes of kQuantUnroll pieces are on their way before the first is widened, and are the first to leave L2.  7885
 // rows of 24 x 128 and the attention behind them, one piece at a time -> three: 128.8 -> 128.0 us.
@@ -30,6 +28,7 @@ namespace regione {
 
 constexpr int kQuantThreads = 256;
 constexpr int kQuantUnroll = 3;
+constexpr int kRowBlocks = 8;                        // store, a block per row: blocks an SM
 
 // Two fp32 -> two E4M3 codes (round to nearest even, saturating); `lo` lands in bits [7:0].
 __device__ __forceinline__ uint32_t pack_e4m3x2(float lo, float hi) {
@@ -67,15 +66,75 @@ __device__ __forceinline__ int live_rows(const int32_t* n_keep, int b, int Nc_ca
     return live < 0 ? 0 : Nc_cap;
 }
 
-// ---- store -----------------------------------------------------------------------------------------
-// Every warp works for itself: it takes pieces of rows (one tensor, as many heads as make at most 8 KB), each fetched by
-// one bulk copy into a ring of its own, so that the chain of count, index and data is off the path of the arithmetic and
-// an SM has 100 to 200 KB of reads in flight whatever its warps are doing.
+// ---- store, a block per row ------------------------------------------------------------------------
+// A block covers K and V of its row, a lane owns 8 consecutive elements (16 bytes), the D / 8 lanes of one head sit side
+// by side in a warp; whole warps walk the pieces so that every shuffle has its 32 lanes, kQuantUnroll loads are issued
+// before the first is used.
+template <int D>
+__global__ void __launch_bounds__(kQuantThreads, kRowBlocks)
+rikv_store_e4m3_rows_kernel(const uint16_t* __restrict__ k_full, const uint16_t* __restrict__ v_full,
+                            const int32_t* __restrict__ keep_rows, const int32_t* __restrict__ n_keep, int N_full, int Nc_cap,
+                            int H, uint8_t* __restrict__ k_q, uint8_t* __restrict__ v_q, float* __restrict__ k_scale,
+                            float* __restrict__ v_scale, int32_t* dev_status) {
+    grid_dependency_wait();
+    grid_launch_dependents();
+    constexpr int kLanesPerHead = D / 8;                // 16 or 8: divides the warp
+    const int b = blockIdx.y, j = blockIdx.x;
+    if (j >= live_rows(n_keep, b, Nc_cap, threadIdx.x == 0 && j == 0, dev_status)) return;
+    const int row = keep_rows[(size_t)b * Nc_cap + j];
+    if (row < 0 || row >= N_full) {
+        if (threadIdx.x == 0) record_status(dev_status, REGIONE_DEV_BOUNDS);
+        return;
+    }
+    const size_t src_off = ((size_t)b * N_full + row) * H * D, dst_row = (size_t)b * Nc_cap + j;
+    const int per_tensor = H * kLanesPerHead, total = 2 * per_tensor;     // 16-byte pieces of K, then of V
+    for (int c0 = (threadIdx.x & ~31); c0 < total; c0 += kQuantUnroll * kQuantThreads) {
+        uint4 w[kQuantUnroll];
+#pragma unroll
+        for (int u = 0; u < kQuantUnroll; ++u) {
+            const int c = c0 + u * kQuantThreads + (threadIdx.x & 31);
+            w[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (c < total)
+                w[u] = ld_stream128((c >= per_tensor ? v_full : k_full) + src_off +
+                                    (size_t)(c >= per_tensor ? c - per_tensor : c) * 8);
+        }
+#pragma unroll
+        for (int u = 0; u < kQuantUnroll; ++u) {
+            const int c = c0 + u * kQuantThreads + (threadIdx.x & 31);
+            const bool live = c < total;
+            const int is_v = live && c >= per_tensor, piece = c - (is_v ? per_tensor : 0);
+            const float x[8] = {bf16_lo(w[u].x), bf16_hi(w[u].x), bf16_lo(w[u].y), bf16_hi(w[u].y),
+                                bf16_lo(w[u].z), bf16_hi(w[u].z), bf16_lo(w[u].w), bf16_hi(w[u].w)};
+            float amax = 0.f;                           // (as floats: as packed bf16 the row takes 4 % longer)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(x[e]));   // (a NaN element is ignored here)
+#pragma unroll
+            for (int d = kLanesPerHead / 2; d > 0; d >>= 1)
+                amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
+            const int k = scale_exponent(__float_as_uint(amax) >> 16);
+            const float inv = __uint_as_float((uint32_t)(127 - k) << 23);  // 2^-k, exact
+            if (!live) continue;
+            uint2 q;
+            q.x = pack_e4m3x2(x[0] * inv, x[1] * inv) | (pack_e4m3x2(x[2] * inv, x[3] * inv) << 16);
+            q.y = pack_e4m3x2(x[4] * inv, x[5] * inv) | (pack_e4m3x2(x[6] * inv, x[7] * inv) << 16);
+            __stcs(reinterpret_cast<uint2*>((is_v ? v_q : k_q) + dst_row * H * D + (size_t)piece * 8), q);
+            if (piece % kLanesPerHead == 0)
+                (is_v ? v_scale : k_scale)[dst_row * H + piece / kLanesPerHead] = __uint_as_float((uint32_t)(127 + k) << 23);
+        }
+    }
+}
+
+// ---- store, rings ----------------------------------------------------------------------------------
+// Every warp works for itself: it takes pieces of rows (one tensor, as many heads as make at most 4.5 KB), each fetched by
+// one bulk copy into a ring of its own of up to eight pieces, so that the chain of count, index and data is off the path of
+// the arithmetic.  An SM has three blocks of four such rings: up to 216 KB of reads in flight, less where eight pieces do not
+// fill a ring (48 KB with 4 heads of 64).  16 elements to a lane, three shuffles for a maximum.  Pieces of 24 heads of 128, three
+// to a ring -> of 12, six to a ring: 40000 rows 140 -> 120 us, four requests of 17562 241 -> 218.
 constexpr int kRingWarps = 4;
 constexpr int kRingStages = 8;                       // at most
 constexpr int kRingBytes = 72 * 1024;                // per block; three blocks an SM
 constexpr int kRingBlocks = 3;
-constexpr int kPieceBytes = 8192;
+constexpr int kPieceBytes = 4608;
 constexpr long long kRingWait = 4000000000LL;        // cycles (~2 s)
 
 struct RingPiece {                                   // what a stage holds
@@ -275,10 +334,30 @@ static int check_quant_args(const void* a, const void* b, const void* c, const v
     return REGIONE_OK;
 }
 
+// A block per row, or rings.  The block's passes of 768 pieces of 16 bytes have to be filled for it to keep up, and rings take
+// longer to start and to drain.  Measured, block per row / rings, us:
+//   passes full (24, 40, 48 heads of 128): 7885 rows 27.3 / 29.4, 44.4 / 47.0, 49.2 / 54.4
+//   filled to two thirds or three quarters (16, 18, 33, 36 heads of 128): 22.3 / 20.5, 23.6 / 23.5 (14000 rows 40.0 / 36.7),
+//   41.1 / 39.5, 42.2 / 40.0; 24 heads of 64 19.8 / 17.3
+//   one full pass, many rows (24 heads of 128): 12000 rows 40.1 / 41.2, 16000 52.6 / 52.3, 20000 64.9 / 63.8, 40000 127.4 / 119.6;
+//   two (48 heads): 20000 rows 119.7 / 132.8
+//   all rows in two rounds of resident blocks: 1000 rows of 16 x 128 7.6 / 7.9, behind a flushed L2 10.2 / 12.3; 2000 rows 7.4 / 7.7,
+//   12.3 / 14.4; 4000 rows 12.3 / 10.6, 18.5 / 18.4
+static bool takes_rows(int B, int Nc_cap, int H, int D, int sms) {
+    const long long rows = (long long)B * Nc_cap;
+    if (rows <= 2LL * kRowBlocks * sms) return true;
+    const long long pieces = 2LL * H * (D / 8), pass = kQuantUnroll * kQuantThreads, passes = (pieces + pass - 1) / pass;
+    return 5 * pieces > 4 * pass * passes && (passes > 1 || rows < 18000);
+}
+
 template <int D>
 static int launch_store(const uint16_t* k_full, const uint16_t* v_full, const int32_t* keep_rows, const int32_t* n_keep, int B,
                         int N_full, int Nc_cap, int H, uint8_t* k_q, uint8_t* v_q, float* k_scale, float* v_scale,
                         int32_t* dev_status, cudaStream_t st) {
+    const int sms = sm_count();
+    if (takes_rows(B, Nc_cap, H, D, sms))
+        return launch_status(launch_overlapped(rikv_store_e4m3_rows_kernel<D>, dim3(Nc_cap, B), dim3(kQuantThreads), 0, st, k_full,
+                                               v_full, keep_rows, n_keep, N_full, Nc_cap, H, k_q, v_q, k_scale, v_scale, dev_status));
     static int configured[kMaxDevices] = {};
     const int dev = current_device();
     if (dev < 0) return REGIONE_CUDA_ERROR;
@@ -291,7 +370,7 @@ static int launch_store(const uint16_t* k_full, const uint16_t* v_full, const in
     const int stage_bytes = heads * D * 2, stages = std::min(kRingStages, kRingBytes / (kRingWarps * stage_bytes));
     const long long blocks = ((long long)B * Nc_cap * 2 * groups + kRingWarps - 1) / kRingWarps;
     const cudaError_t e = launch_overlapped(
-        rikv_store_e4m3_kernel<D>, dim3((unsigned)std::min<long long>(blocks, (long long)kRingBlocks * sm_count())),
+        rikv_store_e4m3_kernel<D>, dim3((unsigned)std::min<long long>(blocks, (long long)kRingBlocks * sms)),
         dim3(kRingWarps * 32), (size_t)kRingWarps * stages * stage_bytes, st, k_full, v_full, keep_rows, n_keep, B, N_full, Nc_cap,
         H, heads, groups, stages, k_q, v_q, k_scale, v_scale, dev_status);
     return launch_status(e);

@@ -1,5 +1,6 @@
-"""The 8-bit cache store at the sizes where its rings of row pieces can go wrong: rows of several pieces, pieces that do not
-fill a warp's last pass, rings that wrap and batches of pieces that follow one another, counts and rows out of range."""
+"""The 8-bit cache store at the sizes where its two forms can go wrong: the ring (rows of several pieces, pieces that do not fill
+a warp's last pass, rings that wrap and batches of pieces that follow one another), the block per row (passes that are full,
+partly full or repeated), both sides of the rule between them, counts and rows out of range."""
 import numpy as np
 import pytest
 
@@ -25,8 +26,16 @@ def _store(k, v, keep, n_keep):
 @pytest.mark.parametrize("D,H,N,cap,n_keep", [
     (128, 1, 31000, 30000, [30000, 29999]),          # more than one batch of pieces a warp
     (64, 3, 9000, 8000, [8000, 1]),
-    (128, 33, 400, 300, [300, 0]),                   # two pieces of 17 and 16 heads
-    (64, 130, 200, 150, [3, 150]),                   # three pieces, the last one shorter
+    (128, 33, 400, 300, [300, 0]),                   # (few rows: a block per row, two passes, the second one short)
+    (64, 130, 200, 150, [3, 150]),
+    (128, 33, 1500, 1300, [1300, 30]),               # two pieces of 17 and 16 heads
+    (64, 73, 1500, 1300, [3, 1300]),                 # three pieces, the last one shorter
+    (128, 2, 1300, 1184, [1184, 1184]),              # 2368 rows: a block per row | rings
+    (128, 2, 1300, 1185, [1185, 1185]),
+    (64, 48, 1400, 1200, [1200, 1]),                 # full passes: a block per row
+    (128, 20, 1400, 1200, [1199, 1200]),             # passes filled to five sixths | to less than four fifths
+    (128, 19, 1400, 1200, [1199, 1200]),
+    (64, 47, 9100, 9000, [9000, 200]),               # one pass, nearly full, 18000 rows: rings
 ])
 def test_codes_and_scales(D, H, N, cap, n_keep):
     rng = np.random.default_rng(D + H)
@@ -46,18 +55,20 @@ def test_codes_and_scales(D, H, N, cap, n_keep):
             assert np.all((got[b, :n][zero] & 0x7f) == 0) and np.all(got[b, n:] == REST)
 
 
-def test_special_values_and_bounds():
+@pytest.mark.parametrize("cap", [6, 2400])           # a block per row, rings
+def test_special_values_and_bounds(cap):
     import torch
     x = torch.ones((1, 8, 2, 128), dtype=torch.bfloat16, device="cuda")
     x[0, 1, 0, 5], x[0, 1, 1, 127] = float("inf"), float("nan")
     x[0, 2, 0], x[0, 2, 1] = 2.0 ** -130, 1.75                               # subnormal; the edge of the scale rule
     x[0, 3, 0], x[0, 3, 1] = -3.3e38, -1.7578125
-    (kq, vq, ks, vs), status = _store(x, x, np.array([[1, 2, 3, 8, -1, 4]], np.int32), np.array([6], np.int32))
+    rest = [4] * (cap - 6)
+    (kq, vq, ks, vs), status = _store(x, x, np.array([[1, 2, 3, 8, -1, 4] + rest], np.int32), np.array([6], np.int32))
     assert status == binding.DEV_BOUNDS
     for q, s in ((kq, ks), (vq, vs)):
         assert np.array_equal(np.log2(s[0, :3]), [[120, -8], [-100, -8], [120, -7]])
         assert q[0, 0, 0, 5] == 0x7e and np.all(q[0, 0, 0, :5] == 0) and q[0, 0, 1, 127] & 0x7f == 0x7f
         assert np.all(q[0, 1, 0] == 0) and np.all(q[0, 1, 1] == 0x7e) and np.all(q[0, 0, 1, :127] == 0x78)
         assert np.all(q[0, 3:5] == REST) and np.all(q[0, 5] == 0x78)          # rows out of range are left out
-    (kq, *_), status = _store(x, x, np.zeros((1, 3), np.int32), np.array([4], np.int32))
+    (kq, *_), status = _store(x, x, np.zeros((1, cap), np.int32), np.array([cap + 1], np.int32))
     assert status == binding.DEV_BOUNDS and np.all(kq == 0x78)               # a count beyond the capacity is clamped
