@@ -1720,12 +1720,15 @@ static bool minds_order(const AttnParams& p) {
 
 // Whether K and V are told to leave L2 first: where a head has one query pair, so that they pass through once, and are more
 // than L2 keeps.  What the next launches read (lists, latents, partial rows, code) stays then.  A step with 205 of 8448 rows
-// 54.1 -> 52.2 us, four requests of 92 x 4736 74.9 -> 69.9 (other K and V in every call).  Not where several pairs read
+// 54.1 -> 52.2 us, behind a flushed L2 63.6 -> 58.5; four requests of 92 x 4736 74.9 -> 69.9 (other K and V in every call).  A step that
+// has just copied its rows to the cache gains as well (four requests of 116 of 3000 rows 105.7 -> 100.3), and a scattered call
+// behind an 8-bit decode loses as much as it gains (205 x 8448 64.9 -> 65.7, behind a flushed L2 72.8 -> 70.8).  Not where several pairs read
 // them (four requests of 1382 x 18944 +7 %, 1075 x 8448 +1 to 2 %, 819 x 8704 -1 %), nor where they fit L2 (two requests of
-// 102 x 2176, 8 heads of 64, +2 to 4 %), nor in calls without a row list, whose cache an 8-bit decode may just have
-// left in L2 (205 x 8448 behind one 67.3 -> 69.5).
-static bool reads_once(const AttnParams& p, int d) {
-    return p.P_cap == 1 && p.out_rows != nullptr && kv_bytes(p, d) >= kSpreadBytes;
+// 102 x 2176, 8 heads of 64, +2 to 4 %), nor in calls without a row list behind a decode (205 x 8448 67.3 -> 69.5), nor in a launch
+// whose copying warps read the rows of the cache a second time (four requests of 256 of 2148 rows refreshed 92.4 -> 94.1, of
+// 246 of 2988 109.4 -> 111.2).
+static bool reads_once(const AttnParams& p, int d, bool refreshes) {
+    return p.P_cap == 1 && !refreshes && p.out_rows != nullptr && kv_bytes(p, d) >= kSpreadBytes;
 }
 
 template <int D, bool STORE>
@@ -1841,7 +1844,7 @@ int launch_region_attention_tc(const uint16_t* q, const uint16_t* k_fresh, const
     prm.ready = reinterpret_cast<unsigned long long*>(prm.cut + lp.grid);
     prm.epoch = next_epoch();
     prm.cluster = 0;
-    prm.kv_once = reads_once(prm, D);
+    prm.kv_once = reads_once(prm, D, store != nullptr);
     const int nt_cap = std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN);
     if (store != nullptr)
         return D == 64 ? launch_tc<64, true>(maps, prm, sp, lp.grid, nt_cap, st)
