@@ -555,7 +555,7 @@ int regione_selftest_bounded_wait(long long limit_cycles, int32_t* dev_status, l
  * the kernel's planning warps run, run on the host.  n_q, n_fresh, n_cache: host int32 [B].  all_rows: 0, or
  * the rows of K and V of which the query and cached rows are parts.  spread: plan of the calls whose K and V
  * are more than L2 keeps.  sms: SMs of the GPU.
- * shape    : host int32 [4], {blocks, query pairs per head at capacity, workspace slots per item, team}
+ * shape    : host int32 [4], {blocks, query pairs per head at capacity, workspace slots per item, team (plan 3)}
  * segments : host int32 [cap, 12], one row per run of key tiles, block after block in the order of the walk:
  *            {block, request, head, query pair, first key tile, key tiles, slot among the item's shares, shares
  *            of the item, workspace index of its slot 1, distance of the later ones, distance of its shares,
@@ -565,6 +565,14 @@ int regione_selftest_bounded_wait(long long limit_cycles, int32_t* dev_status, l
 int regione_selftest_attention_plan(const int32_t* n_q, const int32_t* n_fresh, const int32_t* n_cache, int B, int Nq_cap,
                                     int Nf_cap, int Nc_cap, int H, int all_rows, int spread, int sms, int32_t* shape,
                                     int32_t* segments, int cap);
+
+/*
+ * The form of the attention kernel that a call of these capacities launches on the current device.  out_cap: 0, or the rows
+ * of the buffer that a row list scatters into.  refreshes: the call also writes rows of K and V to the cache.
+ * Returns 0 merge kernel behind, 1 first share merges, 2 cluster, 3 and 4 as 0 and 1 with a plan that minds the order of
+ * the keys; -1 for invalid arguments or without a GPU.
+ */
+int regione_selftest_attention_form(int B, int Nq_cap, int Nf_cap, int Nc_cap, int H, int D, int out_cap, int refreshes);
 
 #ifdef __cplusplus
 }

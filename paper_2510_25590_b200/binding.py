@@ -80,6 +80,7 @@ SIGNATURES = {
     "regione_crosscheck_region_attention": (c_int, [_P] * 8 + [c_int] * 6 + [c_float, _P, _P, _P]),
     "regione_selftest_bounded_wait": (c_int, [c_longlong, _P, _P, _P]),
     "regione_selftest_attention_plan": (c_int, [_P, _P, _P] + [c_int] * 8 + [_P, _P, c_int]),
+    "regione_selftest_attention_form": (c_int, [c_int] * 8),
 }
 
 

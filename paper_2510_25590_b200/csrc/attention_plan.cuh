@@ -6,8 +6,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <algorithm>
-
 #define REGIONE_HD __host__ __device__ __forceinline__
 
 namespace regione {
@@ -23,7 +21,6 @@ struct PlanInput {
     int P_cap;           // query pairs per (request, head) at capacity
     int max_slots;       // workspace slots per item (>= 2)
     int all_rows;        // > 0: query and cached rows of a request are parts of its K and V of this many rows (see ReqShape)
-    int team;            // (SPREAD) 0: whole pairs in waves; else CTAs that walk a head's keys together (see plan_shares)
 };
 
 // Shares are cut on a cost axis measured in ticks, not in steps, so that they take about the same
@@ -105,7 +102,8 @@ REGIONE_HD long long div_pos(long long a, long long b) {
 //    into shares as above.
 //  - kTeams: `team` CTAs walk the same keys of a head at the same time, each for a full pair of its own.  The axis counts the
 //    ticks of one of them and is cut into one share per team; the pairs with one live query tile are an axis of their own,
-//    shared by the CTAs that are in no team, as many as make the two kinds of share equally long.
+//    shared by the CTAs that are in no team, as many as make the two kinds of share equally long.  The team is chosen from the
+//    live counts, and taken where its longest share is within 4 % of the mean.
 enum PlanKind { kWhole, kTicks, kWaves, kTeams };
 struct Plan {
     PlanKind kind;
@@ -123,12 +121,72 @@ struct Plan {
 constexpr int kWholeWaste = 112;
 constexpr int kWaveSlots = 4;    // kWaves: shares that a cut item may meet
 
+// A way to make teams: n_teams of `team` CTAs, the ticks of a member's axis, and the shares of it and of the pairs with one
+// live query tile.
+struct TeamCut {
+    int team, n_teams;
+    long long total, a, l;
+    long long cost;              // longest share, weighted (0: not possible)
+};
+
+// One team for all full pairs of a head (i = 0, 1), or for half of them where the grid divides better by that (2, 3: the
+// second reads K and V a second time, hence 1.5 %); as many teams as make their shares as long as those of the CTAs in
+// no team, or one more (odd i).  most: full pairs of a head, at most.
+REGIONE_HD TeamCut team_cut(const PlanInput& p, int grid, int i, int most, long long pair_ticks, long long lone_ticks) {
+    TeamCut c;
+    c.team = i < 2 ? most : (most + 1) >> 1;
+    long long supers = 0;
+    for (int b = 0; b < p.B; ++b) {
+        const int full = ((max(0, min(p.n_q[b], p.Nq_cap)) + kBM - 1) / kBM) >> 1;
+        supers += (long long)p.H * ((unsigned)(full + c.team - 1) / (unsigned)c.team);
+    }
+    c.total = supers * pair_ticks;
+    const long long teams = div_pos(grid * c.total, lone_ticks + c.team * c.total);
+    c.n_teams = (int)min(teams, (long long)((unsigned)grid / (unsigned)c.team)) + (i & 1);
+    const int rest = grid - c.team * c.n_teams;
+    c.a = c.l = c.cost = 0;
+    if (c.n_teams < 1 || rest < 0 || (rest == 0 && lone_ticks > 0)) return c;
+    c.a = div_pos(c.total + c.n_teams - 1, c.n_teams);
+    if (rest > 0) c.l = div_pos(lone_ticks + rest - 1, rest);
+    c.cost = max(c.a, c.l) * (i < 2 ? 1000 : 1015);
+    return c;
+}
+
+// The shortest of the four; on the GPU by the lanes of the calling warp, which has to call this as a whole.
+REGIONE_HD TeamCut best_team(const PlanInput& p, int grid, int most, long long pair_ticks, long long lone_ticks) {
+#ifdef __CUDA_ARCH__
+    const int i = threadIdx.x & 3;
+    TeamCut c = team_cut(p, grid, i, most, pair_ticks, lone_ticks);
+    int from = i;
+    long long best = c.cost;
+    for (int d = 1; d <= 2; d <<= 1) {
+        const long long cost = __shfl_xor_sync(0xffffffffu, best, d);
+        const int other = __shfl_xor_sync(0xffffffffu, from, d);
+        if (cost > 0 && (best == 0 || cost < best || (cost == best && other < from))) { best = cost; from = other; }
+    }
+    c.team = __shfl_sync(0xffffffffu, c.team, from);
+    c.n_teams = __shfl_sync(0xffffffffu, c.n_teams, from);
+    c.total = __shfl_sync(0xffffffffu, c.total, from);
+    c.a = __shfl_sync(0xffffffffu, c.a, from);
+    c.l = __shfl_sync(0xffffffffu, c.l, from);
+    c.cost = best;
+    return c;
+#else
+    TeamCut best = team_cut(p, grid, 0, most, pair_ticks, lone_ticks);
+    for (int i = 1; i < 4; ++i) {
+        const TeamCut c = team_cut(p, grid, i, most, pair_ticks, lone_ticks);
+        if (c.cost > 0 && (best.cost == 0 || c.cost < best.cost)) best = c;
+    }
+    return best;
+#endif
+}
+
 template <bool IN_PLACE, bool SPREAD>
 REGIONE_HD Plan plan_shares(const PlanInput& p, int grid, bool* bad = nullptr) {
     Plan pl;
     long long items = 0, ticks = 0, span = 0;      // span: first tick of an item's last step, at most
-    long long pairs = 0, supers = 0, lone_ticks = 0;
-    int steps = 0;                                 // steps of an item (-1: they differ)
+    long long pairs = 0, lone_ticks = 0;
+    int steps = 0, most = 0;                       // steps of an item (-1: they differ), full pairs of a head at most
     for (int b = 0; b < p.B; ++b) {
         const ReqShape r = req_shape<IN_PLACE>(p, b, bad);
         items += r.items;
@@ -136,7 +194,7 @@ REGIONE_HD Plan plan_shares(const PlanInput& p, int grid, bool* bad = nullptr) {
         if (r.np > 0) span = max(span, (long long)(r.np > 1 ? kTickPair : r.w_last) * (r.steps - 1));
         if (SPREAD && r.np > 0) {
             pairs += (long long)p.H * r.full;
-            if (p.team > 0) supers += (long long)p.H * ((r.full + p.team - 1) / p.team);
+            most = max(most, r.full);
             if (r.full < r.np) lone_ticks += p.H * r.ticks_last;
             steps = steps == 0 || steps == r.steps ? r.steps : -1;
         }
@@ -146,42 +204,34 @@ REGIONE_HD Plan plan_shares(const PlanInput& p, int grid, bool* bad = nullptr) {
     if (SPREAD) {
         pl.origin = 0;
         pl.waves = 0;
+        pl.team = 1;
         const long long pair_ticks = kTickStart + (long long)kTickPair * steps, fair = div_pos(ticks + grid - 1, grid);
         // (whole items need no merge, and no second start)
         const bool spread = steps > 0 && per * pair_ticks > fair + kTickStart + kTickMerge;
-        if (spread && p.team == 0 && pairs >= 2 * grid && !(whole && per * pair_ticks * 100 <= fair * kWholeWaste)) {
-            pl.kind = kWaves;
-            pl.waves = (int)div_pos(pairs, grid);
-            long long left = pairs - (long long)pl.waves * grid;
-            if (left > 0 && left * kWaveSlots < grid) { --pl.waves; left += grid; }       // (an item would meet too many shares)
-            pl.origin = (pairs - left) * pair_ticks;
-            pl.total = pairs * pair_ticks + lone_ticks;
-            pl.chunk = max(div_pos(pl.total - pl.origin + grid - 1, grid),
-                           max((long long)kTickPair * (steps - 1) / (kWaveSlots - 1) + 1, (long long)kTickPair));
-            return pl;
-        }
-        if (spread && p.team > 0 && supers > 0) {
-            // as many teams as make their shares as long as those of the CTAs in no team
-            const long long total = supers * pair_ticks;
-            int T = (int)min(div_pos(grid * total, lone_ticks + p.team * total), (long long)(grid / p.team));
-            const int rest = grid - p.team * T;
-            if (T > 0 && (rest > 0 || lone_ticks == 0)) {
-                long long a = div_pos(total + T - 1, T), l = rest > 0 ? div_pos(lone_ticks + rest - 1, rest) : 0;
-                if (a > l && rest > p.team) {
-                    const long long a1 = div_pos(total + T, T + 1), l1 = div_pos(lone_ticks + rest - p.team - 1, rest - p.team);
-                    if (max(a1, l1) < a) { ++T; a = a1; l = l1; }
-                }
-                if (max(a, l) * 100 <= fair * 104) {
-                    pl.kind = kTeams;
-                    pl.team = p.team;
-                    pl.n_teams = T;
-                    pl.total = total;
-                    pl.lone_total = lone_ticks;
-                    const long long floor_len = max((long long)kTickPair * (steps - 1) / (p.max_slots - 1) + 1, (long long)kTickPair);
-                    pl.chunk = max(a, floor_len);
-                    pl.lone_chunk = max(l, floor_len);
-                    return pl;
-                }
+        if (spread && pairs >= 2 * grid) {
+            if (!(whole && per * pair_ticks * 100 <= fair * kWholeWaste)) {
+                pl.kind = kWaves;
+                pl.waves = (int)div_pos(pairs, grid);
+                long long left = pairs - (long long)pl.waves * grid;
+                if (left > 0 && left * kWaveSlots < grid) { --pl.waves; left += grid; }       // (an item would meet too many shares)
+                pl.origin = (pairs - left) * pair_ticks;
+                pl.total = pairs * pair_ticks + lone_ticks;
+                pl.chunk = max(div_pos(pl.total - pl.origin + grid - 1, grid),
+                               max((long long)kTickPair * (steps - 1) / (kWaveSlots - 1) + 1, (long long)kTickPair));
+                return pl;
+            }
+        } else if (spread && pairs > 0) {
+            const TeamCut c = best_team(p, grid, most, pair_ticks, lone_ticks);
+            if (c.cost > 0 && max(c.a, c.l) * 100 <= fair * 104) {
+                pl.kind = kTeams;
+                pl.team = c.team;
+                pl.n_teams = c.n_teams;
+                pl.total = c.total;
+                pl.lone_total = lone_ticks;
+                const long long floor_len = max((long long)kTickPair * (steps - 1) / (p.max_slots - 1) + 1, (long long)kTickPair);
+                pl.chunk = max(c.a, floor_len);
+                pl.lone_chunk = max(c.l, floor_len);
+                return pl;
             }
         }
     }
@@ -214,26 +264,24 @@ struct Segment {
     long long next;         // position behind the item
 };
 
-// Whole items: the item with index `idx`, of all of them or of those with two live query tiles.
+// Whole items: the item with index `idx`.
 template <bool IN_PLACE>
-REGIONE_HD Segment segment_whole(const PlanInput& p, long long idx, bool full_only) {
+REGIONE_HD Segment segment_whole(const PlanInput& p, long long idx) {
     Segment sg;
     long long base = 0;
     int b = 0;
     ReqShape r = req_shape<IN_PLACE>(p, 0);
-    int cols = full_only ? r.full : r.np;
-    while (idx >= base + (long long)p.H * cols && b + 1 < p.B) {
-        base += (long long)p.H * cols;
+    while (idx >= base + r.items && b + 1 < p.B) {
+        base += r.items;
         ++b;
         r = req_shape<IN_PLACE>(p, b);
-        cols = full_only ? r.full : r.np;
     }
     const long long item = idx - base;
     sg.b = b; sg.r = r;
-    sg.h = cols > 0 ? (int)div_pos(item, cols) : 0;
-    sg.qp = (int)(item - (long long)sg.h * cols);
+    sg.h = r.np > 0 ? (int)div_pos(item, r.np) : 0;
+    sg.qp = (int)(item - (long long)sg.h * r.np);
     sg.j_first = 0;
-    sg.n_steps = cols > 0 ? r.steps : 0;
+    sg.n_steps = r.np > 0 ? r.steps : 0;
     sg.slot = 0; sg.n_slots = 1;
     sg.next = idx + 1;
     return sg;
@@ -286,34 +334,52 @@ REGIONE_HD Segment segment_ticks(const PlanInput& p, const Plan& pl, long long p
     return sg;
 }
 
-// Waves and teams: the axis holds the full pairs of every head, `team` of them side by side, and behind them the pairs
-// with one live query tile.  The item of the `member`th of a team that contains tick `pos`, and the steps of it that
-// share `c` of `chunk` ticks owns, the shares counted from tick `origin` on.
+// Plans of the launches that mind the order of the keys (SPREAD), one function for all of them: the code of a plan is read
+// once a launch, from memory, and what is not there is not waited for (three functions -> one: 2048 of 8448 rows with a
+// capacity a tenth above 235.6 -> 221.5 us).  `by_head`: the axis holds the pairs of a head one after the other (kTicks, kWhole).
+// Else it holds the full pairs of every head, `team` of them side by side, and behind them the pairs with one live query
+// tile.  The item of the `member`th of a team that contains position `pos`, and the steps of it that share `c` of `chunk`
+// ticks owns, the shares counted from tick `origin` on; whole: positions count items, and all steps are owned.
 template <bool IN_PLACE>
-REGIONE_HD Segment segment_spread(const PlanInput& p, long long pos, long long origin, long long chunk, int c,
-                                                  int team, int member) {
+REGIONE_HD Segment segment_spread(const PlanInput& p, long long pos, bool whole, bool by_head, long long origin, long long chunk,
+                                  int c, int team, int member) {
     Segment sg;
-    long long base = 0, col = 0;
+    long long base = 0, col = 0, head = 0;
     int b = 0, cols = 0;
     bool lone = false;
     for (;;) {
         sg.r = req_shape<IN_PLACE>(p, b);
-        cols = lone ? sg.r.np - sg.r.full : (sg.r.full + team - 1) / team;
-        col = lone ? sg.r.ticks_last : sg.r.ticks_full;
-        const long long len = p.H * cols * col;
-        if (pos < base + len || (lone && b + 1 == p.B)) break;
+        const int sides = team == 1 ? sg.r.full : (int)((unsigned)(sg.r.full + team - 1) / (unsigned)team);
+        cols = by_head ? sg.r.np : lone ? sg.r.np - sg.r.full : sides;
+        col = whole ? 1 : lone ? sg.r.ticks_last : sg.r.ticks_full;
+        head = by_head && !whole ? sg.r.head_ticks : cols * col;
+        const long long len = p.H * head;
+        if (pos < base + len || ((lone || by_head) && b + 1 == p.B)) break;
         base += len;
         if (++b == p.B) { b = 0; lone = true; }
     }
     sg.b = b;
-    const long long at = div_pos(pos - base, col);
-    sg.h = cols > 0 ? (int)div_pos(at, cols) : 0;
-    const int s = (int)(at - (long long)sg.h * cols);
-    sg.qp = lone ? sg.r.full : s * team + member;
-    const long long t0 = base + at * col;
-    cut_item(sg, chunk, t0 + kTickStart - origin, lone ? kTickSingle : kTickPair, c);
+    if (cols == 0) {                                  // nothing left behind the last live request
+        sg.h = sg.qp = sg.j_first = sg.n_steps = sg.slot = 0;
+        sg.n_slots = 1;
+        sg.next = pos + 1;
+        return sg;
+    }
+    sg.h = (int)div_pos(pos - base, head);
+    const long long h0 = base + sg.h * head;
+    const int s = (int)min(div_pos(pos - h0, col), (long long)(cols - 1));
+    const long long t0 = h0 + s * col;
+    lone |= by_head && s == cols - 1 && sg.r.full < sg.r.np;
+    sg.qp = by_head ? s : lone ? sg.r.full : s * team + member;
+    if (whole) {
+        sg.j_first = 0;
+        sg.n_steps = sg.r.steps;
+        sg.slot = 0; sg.n_slots = 1;
+    } else {
+        cut_item(sg, chunk, t0 + kTickStart - origin, lone ? kTickSingle : kTickPair, c);
+    }
     if (sg.qp >= (lone ? sg.r.np : sg.r.full)) sg.n_steps = 0;        // (a team wider than what is left of the head)
-    sg.next = t0 + col;
+    sg.next = t0 + (whole ? 1 : lone ? sg.r.ticks_last : col);
     return sg;
 }
 
@@ -364,10 +430,11 @@ struct ShareWalk {
         const bool in_wave = SPREAD && pl.kind == kWaves && wave < pl.waves;
         if (!in_wave && pos >= hi) return false;
         const bool whole = pl.kind == kWhole || in_wave;
-        it = whole ? segment_whole<IN_PLACE>(p, in_wave ? (long long)wave * grid + block : pos, in_wave)
-             : !SPREAD || pl.kind == kTicks
-                 ? segment_ticks<IN_PLACE>(p, pl, pos, share)
-                 : segment_spread<IN_PLACE>(p, pos, pl.origin, pl.chunk, share, pl.kind == kTeams ? pl.team : 1, member);
+        if constexpr (SPREAD)
+            it = segment_spread<IN_PLACE>(p, in_wave ? (long long)wave * grid + block : pos, whole,
+                                          pl.kind == kTicks || pl.kind == kWhole, pl.origin, pl.chunk, share, pl.team, member);
+        else
+            it = whole ? segment_whole<IN_PLACE>(p, pos) : segment_ticks<IN_PLACE>(p, pl, pos, share);
         it.in_wave = in_wave;
         it.slot_at = ((it.b * p.H + it.h) * p.P_cap + it.qp) * p.max_slots + 1;
         it.slot_step = 1;
@@ -380,29 +447,5 @@ struct ShareWalk {
         return true;
     }
 };
-
-// ---- host side: what is decided from the capacities -------------------------------------------------------------
-
-// CTAs of a team (0: waves).  One team for all pairs of a head, or for half of them where the grid divides better by that
-// (the second reads K and V a second time).
-inline int choose_team(const PlanInput& p, int grid, int nt) {
-    const int tiles = (p.Nq_cap + kBM - 1) / kBM, full = tiles / 2;
-    const long long heads = (long long)p.B * p.H;
-    if (heads * full >= 2LL * grid) return 0;
-    const double pair = kTickStart + (double)kTickPair * nt, lone = tiles % 2 ? heads * (kTickStart + (double)kTickSingle * nt) : 0;
-    int team = 1;
-    double best = 0;
-    for (int k = 1; k <= 2 && full > 0; ++k) {
-        const int g = (full + k - 1) / k;
-        const int T0 = (int)std::min(grid * heads * k * pair / (lone + g * heads * k * pair), (double)(grid / g));
-        for (int T = std::max(T0, 1); T <= T0 + 1 && g * T <= grid; ++T) {
-            const int rest = grid - g * T;
-            if (rest == 0 && lone > 0) continue;
-            const double cost = std::max(heads * k * pair / T, lone > 0 ? lone / rest : 0.) * (k == 2 ? 1.015 : 1.);
-            if (best == 0 || cost < best) { best = cost; team = g; }
-        }
-    }
-    return team;
-}
 
 }  // namespace regione

@@ -7,12 +7,13 @@
 //   warps 0-15  softmax and epilogue: thread = (query row, 64-key chunk of a key tile); warps 0-7 work on
 //               query tile 0, warps 8-15 on query tile 1, the first four of each on the first chunk
 //   warp  16    TMA producer: Q once, then K_j, V_j tiles (128 keys) through a ring of shared-memory stages;
-//               the cached segment and the fresh segment are two tensor maps walked one after the other
+//               the cached segment and the fresh segment are two tensor maps walked one after the other; plans the
+//               CTA's next segment
 //   warp  17    issuer of the O_t += P_t V_j products of both query tiles (the whole warp walks the loop, one
 //               elected lane issues); owns the tensor-memory allocation
 //   warp  18    in the launch that also refreshes the Region-Instruction KV cache: moves the retained rows by
 //               asynchronous bulk copies; idle otherwise
-//   warp  19    issuer of the S = Q_t K_j^T products of both query tiles; plans the CTA's next segment
+//   warp  19    issuer of the S = Q_t K_j^T products of both query tiles
 //   (warps 16-19 give registers up to the softmax warpgroups with setmaxnreg: 64 against 104 per thread)
 //
 // Tensor memory (512 columns): S | P0 | P1 | O0 | O1 = 128 + 64 + 64 + 128 + 128.
@@ -108,7 +109,7 @@ struct AttnCfg {
     // stage, the ordinary ring and the idle second query tile: kStages + 2 stages, an even number: K tiles and
     // V tiles have stages of their own)
     static constexpr int kSmemTiles = (2 + kStages + 1) * kTileBytes;
-    static constexpr int kCtrlBytes = 640;
+    static constexpr int kCtrlBytes = 768;
     static constexpr int kExchBytes = 4 * kBM * 4;         // exchange of the chunks' maxima and sums
     static constexpr int kExtraAt = kSmemTiles + kCtrlBytes + kExchBytes;
     // D = 128 fills shared memory: the epilogue stages its rows (4 KB per softmax warp) in the idle query
@@ -167,6 +168,7 @@ struct AttnCtrl {
     uint8_t* copy_dst[kCopySlots];
     int copy_item[kCopySlots];
     uint32_t copy_valid[kCopySlots];
+    alignas(8) uint8_t cursor[120];     // ShareCursor of the planning warp between two segments
 };
 
 // The barriers of AttnCtrl as one array starting at q_full.
@@ -177,7 +179,7 @@ static_assert(offsetof(AttnCtrl, kv_empty) == kBarKvEmpty * 8 && offsetof(AttnCt
               offsetof(AttnCtrl, pv_done) == kBarPvDone * 8 && offsetof(AttnCtrl, pv_half) == kBarPvHalf * 8 &&
               offsetof(AttnCtrl, s_free) == kBarSFree * 8 && offsetof(AttnCtrl, v_full) == (kBarSFree + 1) * 8 &&
               offsetof(AttnCtrl, tmem_base) == kNumBarriers * 8 &&
-              sizeof(AttnCtrl) <= 640, "barrier layout");
+              sizeof(AttnCtrl) <= AttnCfg<128>::kCtrlBytes, "barrier layout");
 
 // What share c tells the merge kernel: the item that the boundary between shares c - 1 and c
 // cuts, if c is the second share of that item (so every cut item is named exactly once).
@@ -187,14 +189,17 @@ struct alignas(16) CutItem {
 
 // Who puts the parts of an item together that several CTAs work on: a merge kernel behind this one, the item's
 // first share, or the CTAs of a cluster; and whether the plan minds the order in which K and V are read (see plan_shares).
-// (Instantiations of their own: the code of one form costs the others 1 to 2 %; the plan of the spread forms 205 queries x
-// 8448 keys 7 %.)
+// (Instantiations of their own: the code of one form costs the others 1 to 2 %, the plan of the spread forms 1 us.)
 enum MergeForm { kMergeKernel, kMergeHere, kMergeCluster };
 enum KernelForm { kFormKernel, kFormHere, kFormCluster, kFormSpreadKernel, kFormSpreadHere };
+__host__ __device__ constexpr bool is_spread(int form) { return form >= kFormSpreadKernel; }
+__host__ __device__ constexpr int merge_of(int form) { return is_spread(form) ? form - kFormSpreadKernel : form; }
 
 struct AttnParams : PlanInput {
     float scale_log2e;
     int out_cap;         // rows per request of `out` (Nq_cap without out_rows)
+    int cluster;         // kMergeCluster: CTAs that share an item; no workspace
+    int kv_once;         // every key tile is read by one CTA: it need not stay in L2
     uint16_t* out;       // [B, out_cap, H, D]
     const int32_t* out_rows;   // nullptr: query row i goes to out row i; else to row out_rows[b, i]
     int32_t* dev_status;
@@ -205,8 +210,6 @@ struct AttnParams : PlanInput {
                                      // and a word behind them, `epoch`: a launch of this epoch has timed out
     unsigned long long epoch;        // of this launch: what lies in the workspace otherwise is not equal to it
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
-    int cluster;         // kMergeCluster: CTAs that share an item; no workspace
-    int kv_once;         // every key tile is read by one CTA: it need not stay in L2
 };
 
 // Cache refresh fused into a full step: the rows rows[l][b, 0..n[l][b]) (ascending) of the K and V that the launch
@@ -1229,8 +1232,14 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
     }
     grid_dependency_wait();                             // (everything below reads the launch's inputs)
     grid_launch_dependents();                           // the next kernel may queue up behind this CTA
-    ShareCursor<STORE, SPREAD> cur;
-    if (warp == kWarpS) {
+    // The warp that loads K and V also plans: it is done with a segment well ahead of the others.  In a refreshing launch that
+    // minds the order its cursor lies in shared memory between two segments: kept in registers, its fields cost the issuing
+    // loops spills (2048 of 8448 rows refreshed 235.0 -> 230.8 us; 819 of them read 121.2 -> 124.1).
+    using Cursor = ShareCursor<STORE, SPREAD>;
+    static_assert(sizeof(Cursor) <= sizeof(ctrl->cursor), "cursor");
+    Cursor* const kept = reinterpret_cast<Cursor*>(ctrl->cursor);
+    Cursor cur;
+    if (warp == kWarpLoad) {
         bool bad = false;
         if constexpr (FORM == kMergeCluster) {
             cur.of_cluster(p, &ctrl->seg[0], lane, &bad);
@@ -1243,6 +1252,7 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
         } else {
             cur.of_plan(p, &bad);
             cur.template next<FORM>(p, &ctrl->seg[0], lane);
+            if (STORE && SPREAD && lane == 0) *kept = cur;
         }
         if (bad && blockIdx.x == 0 && lane == 0) record_status(p.dev_status, REGIONE_DEV_BOUNDS);
         if (lane == 0) ctrl->abort_flag = 0;
@@ -1317,10 +1327,19 @@ __device__ __forceinline__ void attention_kernel_body(const CUtensorMap& tm_q, c
             set_up(it);
             if (warp == kWarpLoad) {
                 load_segment<D, STORE>(&tm_q, &tm_kf, &tm_vf, &tm_kc, &tm_vc, &tm_ka, &tm_va, p, ctrl, it, smem, lane);
+                // (the next segment is planned while the last tiles are on their way and multiplied: ahead of the end of this one
+                // by the issuer of S, four requests of 205 to 1638 of 8448 rows took 432 us instead of 418)
+                if (FORM != kMergeCluster && mode == kWalk) {
+                    if (STORE && SPREAD) cur = *kept;
+                    cur.template next<FORM>(p, &ctrl->seg[k ^ 1], lane);
+                    if (STORE && SPREAD) {
+                        __syncwarp();
+                        if (lane == 0) *kept = cur;
+                        __syncwarp();
+                    }
+                }
             } else if (warp == kWarpS) {
                 issue_s_segment<D, STORE>(p, ctrl, it, smem, tmem);
-                // (the next segment is planned behind the last product, ahead of the end of this one)
-                if (FORM != kMergeCluster && mode == kWalk) cur.template next<FORM>(p, &ctrl->seg[k ^ 1], lane);
             } else {
                 issue_pv_segment<D, STORE>(p, ctrl, it, smem, tmem, lane, mode);
             }
@@ -1416,7 +1435,7 @@ region_attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q,
                            const __grid_constant__ CUtensorMap tm_kc,
                            const __grid_constant__ CUtensorMap tm_vc, const AttnParams p) {
     const StoreParams none = {};
-    attention_kernel_body<D, false, (FORM >= kFormSpreadKernel ? FORM - kFormSpreadKernel : FORM), (FORM >= kFormSpreadKernel)>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_kf, tm_vf, p, none);
+    attention_kernel_body<D, false, merge_of(FORM), is_spread(FORM)>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_kf, tm_vf, p, none);
 }
 template <int D, int FORM>
 __global__ void __launch_bounds__(kAttnThreads, 1)
@@ -1428,7 +1447,7 @@ region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
                               const __grid_constant__ CUtensorMap tm_ka,
                               const __grid_constant__ CUtensorMap tm_va, const AttnParams p,
                               const __grid_constant__ StoreParams sp) {
-    attention_kernel_body<D, true, (FORM >= kFormSpreadKernel ? FORM - kFormSpreadKernel : FORM), (FORM >= kFormSpreadKernel)>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_ka, tm_va, p, sp);
+    attention_kernel_body<D, true, merge_of(FORM), is_spread(FORM)>(tm_q, tm_kf, tm_vf, tm_kc, tm_vc, tm_ka, tm_va, p, sp);
 }
 
 // Merges the workspace slots of the items that were spread over several shares:
@@ -1438,8 +1457,8 @@ region_attention_store_kernel(const __grid_constant__ CUtensorMap tm_q,
 // is launched behind the attention kernel with programmatic serialization and reads nothing before
 // the dependency wait; all slots' loads are issued before the first use, so a warp pays one
 // memory round trip, not one per slot.
-// MAXS >= AttnParams::max_slots bounds the slots held in registers (the host knows max_slots, and
-// the smaller instantiations let more warps be resident).
+// MAXS >= the slots of an item (AttnParams::max_slots, and kWaveSlots where pairs may be dealt in waves) bounds those held in
+// registers (the host knows both, and the smaller instantiations let more warps be resident).
 template <int D, int MAXS>
 __global__ void __launch_bounds__(256)
 region_attention_combine_kernel(const AttnParams p) {
@@ -1662,7 +1681,8 @@ static int prepare_kernel(const int** fitting) {
 // maximum its probabilities are rounded against, and against the rms of the whole buffer, mostly rows that were not
 // recomputed, the two forms differ from each other by up to 0.1 in single elements (by 0.04 from a twelfth of the rows
 // on).  Against 64 bits, over the recomputed rows, clusters / cost axis: 64 of 8448 rows rel 2.32 / 2.31e-3, 32.7 / 36.4 us;
-// 128 2.31 / 2.31e-3, 33.6 / 38.7 us; 205 2.32 / 2.32e-3, 42.7 / 43.6 us; 704 2.33 / 2.33e-3, 74.4 / 79.8 us.
+// 128 2.31 / 2.31e-3, 33.6 / 38.7 us; 205 2.32 / 2.32e-3, 42.7 / 43.6 us; 704 2.33 / 2.33e-3, 74.4 / 79.8 us.  What holds it is
+// test_step_on_both_sides_of_its_rules, which counts the launches of steps with 768 and 769 rows of keys.
 static bool keeps_cuts(const AttnParams& p) {
     return p.out_rows != nullptr && 12LL * (p.Nq_cap - kBM / 2) < (long long)p.Nf_cap + p.Nc_cap;
 }
@@ -1711,19 +1731,36 @@ static bool merges_here(const AttnParams& p, int grid, int nt) {
 // 8 heads (33 MB) 57.4 -> 58.1, 12 (49 MB) 77.2 -> 79.6, 16 (66 MB) 99.1 -> 97.5, 24 (99 MB) 146.3 -> 136.9; 8704 x
 // 8704, 8 heads 268 -> 272, 12 401 -> 398, 16 561 -> 525, 24 845 -> 767; a step that refreshes 2048 of 8448 rows, 12 heads
 // 125.8 -> 127.2, 16 162.7 -> 159.6, 24 248.7 -> 229.4.
-constexpr long long kSpreadBytes = 60LL << 20;
+// Where the plan of full capacities would deal whole items or cut the cost axis after all, it is left at that: its code is the
+// shorter one (three requests of 543 of 3730 rows, 12 heads, 79.6 -> 74.0 us; of 633 x 3925 keys, 16 heads, 85.3 -> 83.2).  The plan itself
+// follows the live counts; 819, 1229 and 2048 of 8448 rows take as long with a capacity half above them as without room.
+// Requests whose counts differ by whole pairs walk the cost axis here too, and take 0 to 2.5 % longer than there (two requests
+// of 819 and 1024 of 8448 rows 246.2 / 247.1, of 410 and 1229 213.7 / 216.3, four of 205 to 1638, refreshed, 466.3 / 478.0).
+// Heads of 64 read half as many bytes for as many exponentials: only refreshing launches (1638 of 17 408 rows 266.4 -> 260.9; without the
+// refresh 250.8 -> 254.6) and waves of large sequences (16000 x 16000 1980 -> 1967, 11000 x 11000 947 -> 953) mind the order.
+constexpr long long kSpreadBytes = 60LL << 20, kSpreadBytes64 = 90LL << 20;
 static long long kv_bytes(const AttnParams& p, int d) { return 4LL * d * p.B * p.H * ((long long)p.Nf_cap + p.Nc_cap); }
 template <int D>
-static bool minds_order(const AttnParams& p) {
-    return !keeps_cuts(p) && kv_bytes(p, D) >= kSpreadBytes;
+static bool minds_order(const AttnParams& p, int grid, bool refreshes) {
+    // (a head with one pair reads its keys once, in whatever order)
+    if (keeps_cuts(p) || p.P_cap < 2 || kv_bytes(p, D) < kSpreadBytes || (long long)p.B * p.H * p.P_cap > 0x7fffffff) return false;
+    PlanInput full = p;                              // (requests alike are one with as many heads as they have together)
+    // (the rows that a row list names are those of the joint sequence, and so are the keys: together not more than its rows)
+    const int32_t cached = p.out_rows != nullptr ? std::max(0, std::min(p.Nc_cap, p.out_cap - p.Nf_cap)) : p.Nc_cap;
+    const int32_t counts[3] = {p.Nq_cap, p.Nf_cap, cached};
+    full.n_q = counts; full.n_fresh = counts + 1; full.n_cache = counts + 2;
+    full.B = 1; full.H = p.B * p.H; full.all_rows = 0;
+    const PlanKind kind = plan_shares<false, true>(full, grid).kind;
+    if (D == 64 && !refreshes) return kind == kWaves && kv_bytes(p, D) >= kSpreadBytes64;
+    return kind == kWaves || kind == kTeams;
 }
 
 // Whether K and V are told to leave L2 first: where a head has one query pair, so that they pass through once, and are more
 // than L2 keeps.  What the next launches read (lists, latents, partial rows, code) stays then.  A step with 205 of 8448 rows
-// 54.1 -> 52.2 us, behind a flushed L2 63.6 -> 58.5; four requests of 92 x 4736 74.9 -> 69.9 (other K and V in every call).  A step that
-// has just copied its rows to the cache gains as well (four requests of 116 of 3000 rows 105.7 -> 100.3), and a scattered call
-// behind an 8-bit decode loses as much as it gains (205 x 8448 64.9 -> 65.7, behind a flushed L2 72.8 -> 70.8).  Not where several pairs read
-// them (four requests of 1382 x 18944 +7 %, 1075 x 8448 +1 to 2 %, 819 x 8704 -1 %), nor where they fit L2 (two requests of
+// 54.1 -> 52.2 us, behind a flushed L2 63.6 -> 58.5; four requests of 92 x 4736 74.9 -> 69.9 (other K and V in every call).
+// A step that has just copied its rows to the cache gains as well (four requests of 116 of 3000 rows 105.7 -> 100.3), and a
+// scattered call behind an 8-bit decode loses as much as it gains (205 x 8448 64.9 -> 65.7, behind a flushed L2 72.8 -> 70.8).
+// Not where several pairs read them (four requests of 1382 x 18944 +7 %, 1075 x 8448 +1 to 2 %, 819 x 8704 -1 %), nor where they fit L2 (two requests of
 // 102 x 2176, 8 heads of 64, +2 to 4 %), nor in calls without a row list behind a decode (205 x 8448 67.3 -> 69.5), nor in a launch
 // whose copying warps read the rows of the cache a second time (four requests of 256 of 2148 rows refreshed 92.4 -> 94.1, of
 // 246 of 2988 109.4 -> 111.2).
@@ -1731,12 +1768,22 @@ static bool reads_once(const AttnParams& p, int d, bool refreshes) {
     return p.P_cap == 1 && !refreshes && p.out_rows != nullptr && kv_bytes(p, d) >= kSpreadBytes;
 }
 
+// The form of a call, and the CTAs of a cluster (prm.cluster).
+template <int D, bool STORE>
+static int choose_form(const int* fitting, AttnParams& prm, int grid, int nt_cap) {
+    prm.cluster = choose_cluster(fitting, prm, nt_cap);
+    if (prm.cluster > 0) return kFormCluster;
+    const bool here = merges_here(prm, grid, nt_cap);
+    if (minds_order<D>(prm, grid, STORE)) return here ? kFormSpreadHere : kFormSpreadKernel;
+    return here ? kFormHere : kFormKernel;
+}
+
 template <int D, bool STORE>
 static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams& sp, int grid, int nt_cap, cudaStream_t st) {
     const int* fitting = nullptr;
     const int rc = prepare_kernel<D, STORE>(&fitting);
     if (rc != REGIONE_OK) return rc;
-    prm.cluster = choose_cluster(fitting, prm, nt_cap);
+    const int form = choose_form<D, STORE>(fitting, prm, grid, nt_cap);
     // (a refreshing launch takes every cluster that fits: those without an item copy rows of the cache)
     if (prm.cluster > 0) grid = (STORE ? fitting[prm.cluster] : prm.B * prm.H * prm.P_cap) * prm.cluster;
     cudaLaunchConfig_t cfg = {};
@@ -1752,23 +1799,24 @@ static int launch_tc(const CUtensorMap* maps, AttnParams prm, const StoreParams&
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = prm.cluster > 0 ? 2 : 1;
-    const bool spread = prm.cluster == 0 && minds_order<D>(prm);
-    prm.team = spread ? choose_team(prm, grid, nt_cap) : 0;
     cudaError_t e;
     auto launch = [&](auto kernel) {
         if constexpr (STORE) return launch_counted(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], maps[6], prm, sp);
         else return launch_counted(&cfg, kernel, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
     };
-    const bool here = prm.cluster == 0 && merges_here(prm, grid, nt_cap);
-    if (prm.cluster > 0) e = launch(main_kernel<D, STORE, kFormCluster>());
-    else if (spread) e = here ? launch(main_kernel<D, STORE, kFormSpreadHere>()) : launch(main_kernel<D, STORE, kFormSpreadKernel>());
-    else e = here ? launch(main_kernel<D, STORE, kFormHere>()) : launch(main_kernel<D, STORE, kFormKernel>());
+    switch (form) {
+        case kFormCluster: e = launch(main_kernel<D, STORE, kFormCluster>()); break;
+        case kFormSpreadHere: e = launch(main_kernel<D, STORE, kFormSpreadHere>()); break;
+        case kFormSpreadKernel: e = launch(main_kernel<D, STORE, kFormSpreadKernel>()); break;
+        case kFormHere: e = launch(main_kernel<D, STORE, kFormHere>()); break;
+        default: e = launch(main_kernel<D, STORE, kFormKernel>());
+    }
     if (e != cudaSuccess) return REGIONE_CUDA_ERROR;
     // the merge kernel may become resident while the attention kernel drains (it waits for that
     // kernel's completion before it reads a slot)
-    if (grid < 2 || prm.cluster > 0 || here) return launch_status(cudaGetLastError());     // nothing is cut
+    if (grid < 2 || merge_of(form) != kMergeKernel) return launch_status(cudaGetLastError());     // nothing is cut
     const dim3 cgrid((unsigned)(grid - 1), (2 * kBM) / 8, 1);
-    const int most_slots = spread ? std::max(prm.max_slots, kWaveSlots) : prm.max_slots;
+    const int most_slots = is_spread(form) ? std::max(prm.max_slots, kWaveSlots) : prm.max_slots;
     if (most_slots <= 2)
         e = launch_overlapped(region_attention_combine_kernel<D, 2>, cgrid, dim3(256), 0, st, prm);
     else if (most_slots <= 3)
@@ -1924,11 +1972,32 @@ extern "C" int regione_selftest_attention_plan(const int32_t* n_q, const int32_t
     p.n_q = n_q; p.n_fresh = n_fresh; p.n_cache = n_cache;
     p.B = B; p.Nq_cap = Nq_cap; p.Nf_cap = Nf_cap; p.Nc_cap = Nc_cap; p.H = H;
     p.P_cap = lp.P_cap; p.max_slots = lp.max_slots; p.all_rows = all_rows;
-    p.team = spread ? choose_team(p, lp.grid, std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN)) : 0;
-    shape[0] = lp.grid; shape[1] = lp.P_cap; shape[2] = lp.max_slots; shape[3] = p.team;
+    shape[0] = lp.grid; shape[1] = lp.P_cap; shape[2] = lp.max_slots; shape[3] = 0;
+    if (spread) {
+        const Plan pl = all_rows > 0 ? plan_shares<true, true>(p, lp.grid) : plan_shares<false, true>(p, lp.grid);
+        if (pl.kind == kTeams) shape[3] = pl.team;
+    }
     if (all_rows > 0)
         return spread ? list_segments<true, true>(p, lp.grid, segments, cap) : list_segments<true, false>(p, lp.grid, segments, cap);
     return spread ? list_segments<false, true>(p, lp.grid, segments, cap) : list_segments<false, false>(p, lp.grid, segments, cap);
+}
+
+extern "C" int regione_selftest_attention_form(int B, int Nq_cap, int Nf_cap, int Nc_cap, int H, int D, int out_cap, int refreshes) {
+    using namespace regione;
+    if (B < 1 || H < 1 || Nq_cap < 1 || Nf_cap < 0 || Nc_cap < 0 || out_cap < 0 || (D != 64 && D != 128)) return -1;
+    const LaunchPlan lp = plan_launch(B, Nq_cap, Nf_cap, Nc_cap, H);
+    static const int32_t list = 0;
+    AttnParams p = {};
+    p.B = B; p.Nq_cap = Nq_cap; p.Nf_cap = Nf_cap; p.Nc_cap = Nc_cap; p.H = H;
+    p.P_cap = lp.P_cap; p.max_slots = lp.max_slots;
+    p.out_rows = out_cap > 0 ? &list : nullptr;
+    p.out_cap = out_cap > 0 ? out_cap : Nq_cap;
+    const int nt_cap = std::max(1, (Nf_cap + kBN - 1) / kBN + (Nc_cap + kBN - 1) / kBN);
+    const int* fitting = nullptr;
+    auto form = [&](auto prepared, auto choose) { return prepared(&fitting) != REGIONE_OK ? -1 : choose(fitting, p, lp.grid, nt_cap); };
+    if (refreshes)
+        return D == 64 ? form(prepare_kernel<64, true>, choose_form<64, true>) : form(prepare_kernel<128, true>, choose_form<128, true>);
+    return D == 64 ? form(prepare_kernel<64, false>, choose_form<64, false>) : form(prepare_kernel<128, false>, choose_form<128, false>);
 }
 
 extern "C" int regione_region_attention_static(

@@ -121,3 +121,31 @@ def test_plans_cover_every_step_once(seed):
             caps, all_rows = (q_cap, q_cap, c_cap), 0
         for spread in (0, 1):
             check(n_q, f, c, caps, H, all_rows, spread, sms)
+
+
+@pytest.mark.parametrize("rows", [819, 1075, 1229, 2048])
+@pytest.mark.parametrize("room", [1.1, 1.25, 1.5, 2.0])
+@pytest.mark.parametrize("refreshes", [False, True])
+def test_capacities_above_the_counts_keep_the_teams(rows, room, refreshes):
+    """The teams follow the live counts: a capacity above them changes nothing but the longest cut that its workspace holds."""
+    def teams(cap):
+        cap = -(-cap // TILE) * TILE
+        if refreshes:
+            segs, _ = check([rows], [0], [8448 - rows], (cap, 8448, 0), 24, 8448)
+        else:
+            segs, _ = check([rows], [rows], [8448 - rows], (cap, cap, 8448), 24)
+        shape = plan([rows], [0 if refreshes else rows], [8448 - rows], (cap, 8448, 0) if refreshes else (cap, cap, 8448), 24,
+                     8448 if refreshes else 0)[1]
+        return segs, shape[2], shape[3]
+    segs, slots, team = teams(rows)
+    roomy, roomy_slots, roomy_team = teams(int(rows * room))
+    assert team == roomy_team > 1 and set(roomy[:, 11]) == {TEAMS}
+    if slots == roomy_slots:
+        assert np.array_equal(segs[:, :8], roomy[:, :8])
+
+
+@pytest.mark.parametrize("n_q,kind", [([1000, 1024], TEAMS), ([4096, 3900], WAVES), ([819, 1024], TICKS)])
+def test_requests_of_other_counts(n_q, kind):
+    """Counts of the same number of pairs walk in teams; where members would idle the cost axis is the shorter plan."""
+    segs, _ = check(n_q, [0, 0], [8448 - n for n in n_q], (4096, 8448, 0), 24, 8448)
+    assert kind in segs[:, 11]
