@@ -507,11 +507,13 @@ typedef struct {
 } regione_loop_plan;
 
 /* x <- x - dt v, v_last <- v; with starts_run also x_e[slot[n]] <- x[n] (what regione_gather with the partition's list
- * leaves): a run of region steps follows.  v dev bf16 [B, N, C], dt host f32 [B]; NaN: the request sits the call out. */
+ * leaves): a run of region steps follows.  v dev bf16 [B, N, C], dt host f32 [B]; NaN: the request sits the call out.
+ * v may be x or v_last, and with starts_run may not overlap x_e. */
 int regione_loop_full_step(const regione_loop_plan* plan, const regione_bf16* v, const float* dt, int starts_run, void* stream);
 
 /* regione_velocity_decay_run on x_e with v_e (kept in v_cache) or, v_e = NULL, with v_cache; dt_unedited (host f32 [B],
- * nullable): the run of region steps ends here, and regione_merge of x_e and v_last into x is part of the launch. */
+ * nullable): the run of region steps ends here, and regione_merge of x_e and v_last into x is part of the launch.  v_e may be
+ * x_e or v_cache, and with dt_unedited may not overlap x. */
 int regione_loop_region_steps(const regione_loop_plan* plan, const regione_bf16* v_e, const float* scale, const float* dt,
                               int n_steps, const float* dt_unedited, void* stream);
 

@@ -321,9 +321,11 @@ class RegionELoop:
 
     def _run_together(self, x, ref, model, stream, ts):
         """All steps of requests that take them at the same time, without a hook: what ``run`` does then, with one
-        set of scalars for the batch.  Host-bound (28 steps of 4096 tokens, 12 of them full: about 6 us a
-        launch, 253 us with a launch for each of the loop's operations, 214 us this way), so an update and what the loop does next to the same rows are one call: a full step and the gather of X^E behind
-        it, the last update of a run of region steps and the merge."""
+        set of scalars for the batch.  Host-bound (28 steps of 4096 tokens, 12 of them full: about 6 us a launch, 237 us
+        with a launch for each of the loop's operations, 203 us this way), so an update and what the loop does next to
+        the same rows are one call: a full step and the gather of X^E behind it, the last update of a run of region
+        steps and the merge.  Not where the velocity lies in the rows that the second half writes (a model may return
+        its latent, or a buffer of the loop): other blocks may not have read it yet."""
         import torch
         cfg, b = self.cfg, binding
         kinds, after, gammas, delta = cfg.kinds, cfg.partition_after, cfg.gammas, cfg.delta
@@ -338,11 +340,12 @@ class RegionELoop:
             raise b.RegionEError(f"x must have shape {shape}, got {tuple(x.shape)}")
         plan = b.LoopPlan(B, N, C, p_x, p_xe, p_vl, p_vc, p_slot, p_ne, p_st)
         one, full_step, region_steps = c_float * B, lib.regione_loop_full_step, lib.regione_loop_region_steps
+        n_bytes = x.numel() * x.element_size()
         log, launches, full_calls, region_calls = [], 0, 0, 0
         partitioned, t_run, k = False, None, 0               # t_run: time at which the present run of region steps began
 
         while k < T or t_run is not None:
-            if t_run is not None and (k == T or kinds[k] == "F"):     # (a region velocity of other rows came last)
+            if t_run is not None and (k == T or kinds[k] == "F"):     # (not part of the last update: see above)
                 # x has not changed since the run began: edited tokens from X^E, the others by one step of the last
                 # full velocity over the whole run
                 check(lib.regione_merge(p_x, p_vl, p_xe, p_slot, one(*[t_run - ts[k]] * B), B, N, N, C, p_x, p_st, s),
@@ -361,7 +364,7 @@ class RegionELoop:
                 p_v = ptr(v, bf, "v")
                 if v.shape != shape:
                     _check_rows(v.shape, shape, "v")
-                starts = partitioned and k + 1 < T and kinds[k + 1] == "R"
+                starts = partitioned and k + 1 < T and kinds[k + 1] == "R" and abs(p_v - p_xe) >= n_bytes
                 check(full_step(plan, p_v, one(*[t - t_next] * B), starts, s), "regione_loop_full_step")
                 launches += 1
                 if starts:
@@ -386,6 +389,7 @@ class RegionELoop:
                 s = stream_of(device())
             region_calls += 1
             p_v, rows = ptr(v_e, bf, "v_e"), N
+            apart = abs(p_v - p_x) >= n_bytes
             if v_e.shape != shape:
                 rows = _check_rows(v_e.shape, shape, "v_e", region=True)
             log.append((k, "R", "compute", 1.0))
@@ -404,7 +408,7 @@ class RegionELoop:
                 # (a run that is longer than one update carries goes on in the next, from the kept velocity)
                 n = k - first
                 many = c_float * (n * B)
-                if rows == N:
+                if rows == N and apart:
                     ends = not again and (k == T or kinds[k] == "F")
                     check(region_steps(plan, p_v, many(*scales), many(*dts), n, one(*[t_run - ts[k]] * B) if ends else None, s),
                           "regione_loop_region_steps")
@@ -416,6 +420,6 @@ class RegionELoop:
                 launches += 1
                 if again:
                     log.append((k, "R", "reuse", product))
-                    p_v, rows, first, scales, dts = None, N, k, [product] * B, [ts[k] - ts[k + 1]] * B
+                    p_v, rows, apart, first, scales, dts = None, N, True, k, [product] * B, [ts[k] - ts[k + 1]] * B
                     k += 1
         return x, LoopTrace(log, [list(log) for _ in range(B)], full_calls, region_calls, launches)

@@ -99,3 +99,35 @@ def test_loop_follows_the_stream_that_the_model_makes_current(hooked):
             torch.cuda.set_stream(first)
         done.append(lp.x_e)
     assert torch.equal(done[0], done[2]) and torch.equal(done[1], done[3])
+
+
+@pytest.mark.parametrize("which", ["region velocity in x", "full velocity in x_e"])
+def test_velocities_that_lie_in_the_loop_s_buffers(which):
+    """A model whose velocity lies in rows that the loop writes next: read by every block before it is written over.
+    (65536 tokens of 64 channels are twice the blocks that are resident at once.)"""
+    import torch
+    N, C = 65536, 64
+    g = torch.Generator(device="cuda").manual_seed(11)
+    r = lambda: torch.randn((1, N, C), generator=g, device="cuda").bfloat16()
+    ref, noise, target = r(), r(), r()
+    edited = torch.rand((1, N, 1), generator=g, device="cuda") < 0.4
+    target = torch.where(edited, target, ref)
+
+    class Model(TorchStraightLine):
+        def full(self, x, t, store):
+            self.x = x
+            v = super().full(x, t, store)
+            return lp.x_e.copy_(v) if which == "full velocity in x_e" else v
+
+        def region(self, x_e, t, edit_idx, n_edit):
+            return self.x if which == "region velocity in x" else super().region(x_e, t, edit_idx, n_edit)
+
+    done = []
+    for hook in (lambda *a: None, None):                     # a call for each of the loop's operations; the short path
+        lp = _loop(noise)
+        lp.hook = hook
+        x, _ = lp.run(noise.clone(), ref, Model(target))
+        torch.cuda.synchronize()
+        assert int(lp.dev_status[0]) == 0 and 0 < int(lp.n_edit[0]) < N
+        done.append((x, lp.x_e))
+    assert all(torch.equal(a, b) for a, b in zip(*done))
