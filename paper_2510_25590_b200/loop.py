@@ -340,7 +340,7 @@ class RegionELoop:
             raise b.RegionEError(f"x must have shape {shape}, got {tuple(x.shape)}")
         plan = b.LoopPlan(B, N, C, p_x, p_xe, p_vl, p_vc, p_slot, p_ne, p_st)
         one, full_step, region_steps = c_float * B, lib.regione_loop_full_step, lib.regione_loop_region_steps
-        n_bytes = x.numel() * x.element_size()
+        n_bytes = 2 * B * N * C
         log, launches, full_calls, region_calls = [], 0, 0, 0
         partitioned, t_run, k = False, None, 0               # t_run: time at which the present run of region steps began
 
@@ -389,7 +389,6 @@ class RegionELoop:
                 s = stream_of(device())
             region_calls += 1
             p_v, rows = ptr(v_e, bf, "v_e"), N
-            apart = abs(p_v - p_x) >= n_bytes
             if v_e.shape != shape:
                 rows = _check_rows(v_e.shape, shape, "v_e", region=True)
             log.append((k, "R", "compute", 1.0))
@@ -408,8 +407,8 @@ class RegionELoop:
                 # (a run that is longer than one update carries goes on in the next, from the kept velocity)
                 n = k - first
                 many = c_float * (n * B)
-                if rows == N and apart:
-                    ends = not again and (k == T or kinds[k] == "F")
+                if rows == N:
+                    ends = not again and (k == T or kinds[k] == "F") and (p_v is None or abs(p_v - p_x) >= n_bytes)
                     check(region_steps(plan, p_v, many(*scales), many(*dts), n, one(*[t_run - ts[k]] * B) if ends else None, s),
                           "regione_loop_region_steps")
                     if ends:
@@ -420,6 +419,6 @@ class RegionELoop:
                 launches += 1
                 if again:
                     log.append((k, "R", "reuse", product))
-                    p_v, rows, apart, first, scales, dts = None, N, True, k, [product] * B, [ts[k] - ts[k + 1]] * B
+                    p_v, rows, first, scales, dts = None, N, k, [product] * B, [ts[k] - ts[k + 1]] * B
                     k += 1
         return x, LoopTrace(log, [list(log) for _ in range(B)], full_calls, region_calls, launches)
