@@ -36,9 +36,17 @@ def test_updates_leave_what_the_calls_leave(B, N, C, n_steps, new_velocity):
     plan = binding.LoopPlan(B, N, C, *(t.data_ptr() for t in (*got, slot, n, status)))
 
     binding.velocity_decay(v, [1.0] * B, dt.tolist(), want[0], n_all, v_cache_out=want[2], dev_status=status)
-    if B <= 2:                                               # (the gather knows no request that sits out)
-        binding.gather(want[0], idx, n, want[1], dev_status=status)
-    assert lib.regione_loop_full_step(plan, v.data_ptr(), host(dt), 1 if B <= 2 else 0, s) == binding.OK
+    starts = n.clone()
+    if B > 2:
+        starts[1] = 0                                        # (a request that sits out starts no run either)
+    binding.gather(want[0], idx, starts, want[1], dev_status=status)
+    assert lib.regione_loop_full_step(plan, v.data_ptr(), host(dt), 1, s) == binding.OK
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)
+    if B > 2:
+        assert torch.equal(got[1][1], x_e[1]) and not torch.equal(got[1][2], x_e[2])
+    assert lib.regione_loop_full_step(plan, v_e.data_ptr(), host(dt), 0, s) == binding.OK
+    binding.velocity_decay(v_e, [1.0] * B, dt.tolist(), want[0], n_all, v_cache_out=want[2], dev_status=status)
     for a, b in zip(want, got):
         assert torch.equal(a, b)
 
