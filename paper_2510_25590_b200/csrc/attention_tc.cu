@@ -1731,13 +1731,14 @@ static bool merges_here(const AttnParams& p, int grid, int nt) {
 // 8 heads (33 MB) 57.4 -> 58.1, 12 (49 MB) 77.2 -> 79.6, 16 (66 MB) 99.1 -> 97.5, 24 (99 MB) 146.3 -> 136.9; 8704 x
 // 8704, 8 heads 268 -> 272, 12 401 -> 398, 16 561 -> 525, 24 845 -> 767; a step that refreshes 2048 of 8448 rows, 12 heads
 // 125.8 -> 127.2, 16 162.7 -> 159.6, 24 248.7 -> 229.4.
-// Where the plan of full capacities would deal whole items or cut the cost axis after all, it is left at that: its code is the
-// shorter one (three requests of 543 of 3730 rows, 12 heads, 79.6 -> 74.0 us; of 633 x 3925 keys, 16 heads, 85.3 -> 83.2).  The plan itself
-// follows the live counts; 819, 1229 and 2048 of 8448 rows take as long with a capacity half above them as without room.
+// Where the plan of full capacities would deal whole items or cut the cost axis after all, it is left at that: its code is
+// the shorter one (three requests of 543 of 3730 rows, 12 heads, 79.6 -> 74.0 us; of 633 x 3925 keys, 16 heads, 85.3 -> 83.2).
+// The plan itself follows the live counts: 819 and 2048 of 8448 rows take as long with room for a tenth more as without.
 // Requests whose counts differ by whole pairs walk the cost axis here too, and take 0 to 2.5 % longer than there (two requests
 // of 819 and 1024 of 8448 rows 246.2 / 247.1, of 410 and 1229 213.7 / 216.3, four of 205 to 1638, refreshed, 466.3 / 478.0).
-// Heads of 64 read half as many bytes for as many exponentials: only refreshing launches (1638 of 17 408 rows 266.4 -> 260.9; without the
-// refresh 250.8 -> 254.6) and waves of large sequences (16000 x 16000 1980 -> 1967, 11000 x 11000 947 -> 953) mind the order.
+// Heads of 64 read half as many bytes for as many exponentials, and only refreshing launches mind the order (1638 of 16896
+// rows 266.4 -> 260.9; without the refresh 250.8 -> 254.6), and waves of 90 MB and more (16000 x 16000 1980 -> 1967; 11000 x
+// 11000, 67 MB, 947 -> 953).
 constexpr long long kSpreadBytes = 60LL << 20, kSpreadBytes64 = 90LL << 20;
 static long long kv_bytes(const AttnParams& p, int d) { return 4LL * d * p.B * p.H * ((long long)p.Nf_cap + p.Nc_cap); }
 template <int D>
@@ -1760,10 +1761,10 @@ static bool minds_order(const AttnParams& p, int grid, bool refreshes) {
 // 54.1 -> 52.2 us, behind a flushed L2 63.6 -> 58.5; four requests of 92 x 4736 74.9 -> 69.9 (other K and V in every call).
 // A step that has just copied its rows to the cache gains as well (four requests of 116 of 3000 rows 105.7 -> 100.3), and a
 // scattered call behind an 8-bit decode loses as much as it gains (205 x 8448 64.9 -> 65.7, behind a flushed L2 72.8 -> 70.8).
-// Not where several pairs read them (four requests of 1382 x 18944 +7 %, 1075 x 8448 +1 to 2 %, 819 x 8704 -1 %), nor where they fit L2 (two requests of
-// 102 x 2176, 8 heads of 64, +2 to 4 %), nor in calls without a row list behind a decode (205 x 8448 67.3 -> 69.5), nor in a launch
-// whose copying warps read the rows of the cache a second time (four requests of 256 of 2148 rows refreshed 92.4 -> 94.1, of
-// 246 of 2988 109.4 -> 111.2).
+// Not where several pairs read them (four requests of 1382 x 18944 +7 %, 1075 x 8448 +1 to 2 %, 819 x 8704 -1 %), nor where they
+// fit L2 (two requests of 102 x 2176, 8 heads of 64, +2 to 4 %), nor in calls without a row list behind a decode (205 x 8448
+// 67.3 -> 69.5), nor in a launch whose copying warps read the rows of the cache a second time (four requests of 256 of 2148 rows
+// refreshed 92.4 -> 94.1, of 246 of 2988 109.4 -> 111.2).
 static bool reads_once(const AttnParams& p, int d, bool refreshes) {
     return p.P_cap == 1 && !refreshes && p.out_rows != nullptr && kv_bytes(p, d) >= kSpreadBytes;
 }

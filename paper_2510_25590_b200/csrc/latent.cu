@@ -94,7 +94,8 @@ merge_kernel(const uint4* x_full, const uint4* __restrict__ v_last,
 }
 
 // The sampler loop's updates of all tokens, each with what the loop does next to the same rows: a launch of these sizes is
-// 1 to 3 us of memory round trips and 6 us of host time (28 steps of 4096 tokens: 29 launches -> 22, 253 -> 214 us with the host side).
+// 1 to 3 us of memory round trips and 6 us of host time (28 steps of 4096 tokens: 29 launches -> 22, 237 -> 203 us with the host
+// side).  The velocity may lie in the rows that the first half writes, not in those of the second: see loop.py.
 //
 // x <- x - dt * v and v_last <- v; where a run of region steps begins (slot != nullptr), the edited tokens to X^E as well.
 __global__ void __launch_bounds__(kLatThreads)
