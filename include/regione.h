@@ -556,7 +556,7 @@ int regione_selftest_bounded_wait(long long limit_cycles, int32_t* dev_status, l
  * How the attention kernel cuts the work of one call into shares, one per block: the functions that
  * the kernel's planning warps run, run on the host.  n_q, n_fresh, n_cache: host int32 [B].  all_rows: 0, or
  * the rows of K and V of which the query and cached rows are parts.  spread: plan of the calls whose K and V
- * are more than L2 keeps.  sms: SMs of the GPU.
+ * are more than L2 keeps (2: of those that refresh the cache, with heads of 128).  sms: SMs of the GPU.
  * shape    : host int32 [4], {blocks, query pairs per head at capacity, workspace slots per item, team (plan 3)}
  * segments : host int32 [cap, 12], one row per run of key tiles, block after block in the order of the walk:
  *            {block, request, head, query pair, first key tile, key tiles, slot among the item's shares, shares

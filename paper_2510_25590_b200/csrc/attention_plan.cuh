@@ -21,6 +21,7 @@ struct PlanInput {
     int P_cap;           // query pairs per (request, head) at capacity
     int max_slots;       // workspace slots per item (>= 2)
     int all_rows;        // > 0: query and cached rows of a request are parts of its K and V of this many rows (see ReqShape)
+    int single;          // ticks of a key tile of a pair with one live query tile (see kTickSingle)
 };
 
 // Shares are cut on a cost axis measured in ticks, not in steps, so that they take about the same
@@ -31,6 +32,11 @@ struct PlanInput {
 // the new one (measured the same way: 3.5 to 6 pair steps depending on the workload, 5 with 819 x 8704 and
 // 1075 x 8448 keys, 24 heads of 128; 100, 120 and 140 ticks for items that a first share merges: 0 to +3 %).
 constexpr int kTickPair = 16, kTickSingle = 9, kTickStart = 80;
+// A launch that refreshes the cache with heads of 128 has no room for the wider ring of a lone tile, whose step takes 0.75 of
+// a pair's (2320 of 3080 cycles).  It matters where lone tiles lie together, in the plans that mind the order of the keys (8211
+// x 8211 refreshed, 24 heads, 786.3 -> 737.4 us, 750.0 on the cost axis; a step that refreshes 819 of 8448 rows 138.4 -> 126.6);
+// the others deal them evenly among the pairs and keep the ticks above.
+constexpr int kTickSingleRefresh = 12;
 // What the merge of cut items costs a launch: every cut item's rows go through the workspace (7300 cycles per pair of
 // tiles, all CTAs at once) and a second kernel (8 us behind the attention's last block).
 constexpr int kTickMerge = 125;
@@ -71,7 +77,7 @@ REGIONE_HD ReqShape req_shape(const PlanInput& p, int b, bool* bad = nullptr) {
     r.nt = r.nt_c + (nf + kBN - 1) / kBN;
     r.items = (long long)p.H * r.np;
     r.steps = max(r.nt, 1);
-    r.w_last = (nq - (r.np - 1) * 2 * kBM > kBM) ? kTickPair : kTickSingle;
+    r.w_last = (nq - (r.np - 1) * 2 * kBM > kBM) ? kTickPair : p.single;
     r.full = r.w_last == kTickPair ? r.np : max(r.np - 1, 0);
     r.ticks_full = kTickStart + (long long)kTickPair * r.steps;
     r.ticks_last = kTickStart + (long long)r.w_last * r.steps;
@@ -376,7 +382,7 @@ REGIONE_HD Segment segment_spread(const PlanInput& p, long long pos, bool whole,
         sg.n_steps = sg.r.steps;
         sg.slot = 0; sg.n_slots = 1;
     } else {
-        cut_item(sg, chunk, t0 + kTickStart - origin, lone ? kTickSingle : kTickPair, c);
+        cut_item(sg, chunk, t0 + kTickStart - origin, lone ? p.single : kTickPair, c);
     }
     if (sg.qp >= (lone ? sg.r.np : sg.r.full)) sg.n_steps = 0;        // (a team wider than what is left of the head)
     sg.next = t0 + (whole ? 1 : lone ? sg.r.ticks_last : col);

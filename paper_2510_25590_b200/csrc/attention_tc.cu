@@ -198,8 +198,6 @@ __host__ __device__ constexpr int merge_of(int form) { return is_spread(form) ? 
 struct AttnParams : PlanInput {
     float scale_log2e;
     int out_cap;         // rows per request of `out` (Nq_cap without out_rows)
-    int cluster;         // kMergeCluster: CTAs that share an item; no workspace
-    int kv_once;         // every key tile is read by one CTA: it need not stay in L2
     uint16_t* out;       // [B, out_cap, H, D]
     const int32_t* out_rows;   // nullptr: query row i goes to out row i; else to row out_rows[b, i]
     int32_t* dev_status;
@@ -210,6 +208,8 @@ struct AttnParams : PlanInput {
                                      // and a word behind them, `epoch`: a launch of this epoch has timed out
     unsigned long long epoch;        // of this launch: what lies in the workspace otherwise is not equal to it
     long long timeout_cycles;   // bound of every barrier wait, in SM clock cycles
+    int cluster;         // kMergeCluster: CTAs that share an item; no workspace
+    int kv_once;         // every key tile is read by one CTA: it need not stay in L2
 };
 
 // Cache refresh fused into a full step: the rows rows[l][b, 0..n[l][b]) (ascending) of the K and V that the launch
@@ -1736,13 +1736,15 @@ static bool merges_here(const AttnParams& p, int grid, int nt) {
 // The plan itself follows the live counts: 819 and 2048 of 8448 rows take as long with room for a tenth more as without.
 // Requests whose counts differ by whole pairs walk the cost axis here too, and take 0 to 2.5 % longer than there (two requests
 // of 819 and 1024 of 8448 rows 246.2 / 247.1, of 410 and 1229 213.7 / 216.3, four of 205 to 1638, refreshed, 466.3 / 478.0).
-// Heads of 64 read half as many bytes for as many exponentials, and only refreshing launches mind the order (1638 of 16896
-// rows 266.4 -> 260.9; without the refresh 250.8 -> 254.6), and waves of 90 MB and more (16000 x 16000 1980 -> 1967; 11000 x
-// 11000, 67 MB, 947 -> 953).
+// Teams whose cut items a merge kernel puts together have short shares: 300 x 8448 59.5 -> 60.6, three requests of 552 x 6716, 12
+// heads, 97.7 -> 99.7.
+// Heads of 64 read half as many bytes for as many exponentials.  Refreshing launches mind the order (1638 of 16896 rows 266.4 ->
+// 260.9; without the refresh 250.8 -> 254.6), waves of 90 MB and more (16000 x 16000 1980 -> 1967; 11000 x 11000, 67 MB, 947 ->
+// 953), and teams where the other plan is one of whole items (four requests of 594 x 6805 178.8 -> 161.9).
 constexpr long long kSpreadBytes = 60LL << 20, kSpreadBytes64 = 90LL << 20;
 static long long kv_bytes(const AttnParams& p, int d) { return 4LL * d * p.B * p.H * ((long long)p.Nf_cap + p.Nc_cap); }
 template <int D>
-static bool minds_order(const AttnParams& p, int grid, bool refreshes) {
+static bool minds_order(const AttnParams& p, int grid, bool refreshes, int single, bool here) {
     // (a head with one pair reads its keys once, in whatever order)
     if (keeps_cuts(p) || p.P_cap < 2 || kv_bytes(p, D) < kSpreadBytes || (long long)p.B * p.H * p.P_cap > 0x7fffffff) return false;
     PlanInput full = p;                              // (requests alike are one with as many heads as they have together)
@@ -1750,10 +1752,13 @@ static bool minds_order(const AttnParams& p, int grid, bool refreshes) {
     const int32_t cached = p.out_rows != nullptr ? std::max(0, std::min(p.Nc_cap, p.out_cap - p.Nf_cap)) : p.Nc_cap;
     const int32_t counts[3] = {p.Nq_cap, p.Nf_cap, cached};
     full.n_q = counts; full.n_fresh = counts + 1; full.n_cache = counts + 2;
-    full.B = 1; full.H = p.B * p.H; full.all_rows = 0;
+    full.B = 1; full.H = p.B * p.H; full.all_rows = 0; full.single = single;
     const PlanKind kind = plan_shares<false, true>(full, grid).kind;
-    if (D == 64 && !refreshes) return kind == kWaves && kv_bytes(p, D) >= kSpreadBytes64;
-    return kind == kWaves || kind == kTeams;
+    if (D == 64 && !refreshes) {
+        if (kind == kWaves) return kv_bytes(p, D) >= kSpreadBytes64;
+        return kind == kTeams && plan_shares<false, false>(full, grid).kind == kWhole;
+    }
+    return kind == kWaves || (kind == kTeams && here);
 }
 
 // Whether K and V are told to leave L2 first: where a head has one query pair, so that they pass through once, and are more
@@ -1773,10 +1778,13 @@ static bool reads_once(const AttnParams& p, int d, bool refreshes) {
 template <int D, bool STORE>
 static int choose_form(const int* fitting, AttnParams& prm, int grid, int nt_cap) {
     prm.cluster = choose_cluster(fitting, prm, nt_cap);
+    prm.single = kTickSingle;
     if (prm.cluster > 0) return kFormCluster;
     const bool here = merges_here(prm, grid, nt_cap);
-    if (minds_order<D>(prm, grid, STORE)) return here ? kFormSpreadHere : kFormSpreadKernel;
-    return here ? kFormHere : kFormKernel;
+    constexpr int single = STORE && D == 128 ? kTickSingleRefresh : kTickSingle;
+    if (!minds_order<D>(prm, grid, STORE, single, here)) return here ? kFormHere : kFormKernel;
+    prm.single = single;
+    return here ? kFormSpreadHere : kFormSpreadKernel;
 }
 
 template <int D, bool STORE>
@@ -1973,6 +1981,7 @@ extern "C" int regione_selftest_attention_plan(const int32_t* n_q, const int32_t
     p.n_q = n_q; p.n_fresh = n_fresh; p.n_cache = n_cache;
     p.B = B; p.Nq_cap = Nq_cap; p.Nf_cap = Nf_cap; p.Nc_cap = Nc_cap; p.H = H;
     p.P_cap = lp.P_cap; p.max_slots = lp.max_slots; p.all_rows = all_rows;
+    p.single = spread == 2 ? kTickSingleRefresh : kTickSingle;
     shape[0] = lp.grid; shape[1] = lp.P_cap; shape[2] = lp.max_slots; shape[3] = 0;
     if (spread) {
         const Plan pl = all_rows > 0 ? plan_shares<true, true>(p, lp.grid) : plan_shares<false, true>(p, lp.grid);

@@ -119,7 +119,7 @@ def test_plans_cover_every_step_once(seed):
             c_cap = near(1, 9000)
             f, c = n_q, [c_cap if same else rng.randint(0, c_cap) for _ in range(B)]
             caps, all_rows = (q_cap, q_cap, c_cap), 0
-        for spread in (0, 1):
+        for spread in (0, 1, 2):
             check(n_q, f, c, caps, H, all_rows, spread, sms)
 
 
@@ -142,6 +142,22 @@ def test_capacities_above_the_counts_keep_the_teams(rows, room, refreshes):
     assert team == roomy_team > 1 and set(roomy[:, 11]) == {TEAMS}
     if slots == roomy_slots:
         assert np.array_equal(segs[:, :8], roomy[:, :8])
+
+
+@pytest.mark.parametrize("n_q,caps,all_rows", [
+    ([8211], (8211, 8211, 0), 0),                    # waves, the lone tiles behind them
+    ([6500], (6500, 6500, 0), 0),
+    ([819], (896, 8448, 0), 8448),                   # teams, the lone tiles apart
+    ([1075], (1152, 8448, 0), 8448),
+    ([1638], (1664, 8448, 0), 8448),
+])
+def test_lone_tiles_of_a_refreshing_launch_weigh_three_quarters(n_q, caps, all_rows):
+    f, c = ([0], [all_rows - n_q[0]]) if all_rows else (n_q, [0])
+    segs, grid = check(n_q, f, c, caps, 24, all_rows, spread=2)
+    assert set(segs[:, 11]) & {WAVES, TEAMS}
+    cost = 80 + segs[:, 5] * np.where(n_q[0] - segs[:, 3] * PAIR > TILE, 16, 12)
+    load = np.bincount(segs[:, 0], weights=cost, minlength=grid)
+    assert load.max() <= 1.05 * load.mean() + 32     # (teams are taken within 4 % of the mean; a step each way)
 
 
 @pytest.mark.parametrize("n_q,kind", [([1000, 1024], TEAMS), ([4096, 3900], WAVES), ([819, 1024], TICKS)])

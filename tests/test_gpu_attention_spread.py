@@ -36,9 +36,12 @@ def plan_of(n_q, n_f, n_c, caps, H):
     (128, 24, [819], [819], [7885], 400, (TEAMS, 0)),                # ... chosen from the counts
     (128, 24, [2048], [2048], [6400], 0, (TEAMS, 0)),                # teams of half a head's pairs
     (64, 24, [2048], [2048], [8300], 0, None),
-    (128, 8, [1100, 1090], [1100, 1090], [6700, 6700], 0, (TEAMS, 0)),               # two requests with the same key tiles
+    (128, 8, [1100, 1090], [1100, 1090], [6700, 6700], 0, None),                     # (short shares, merged by a kernel)
+    (128, 12, [1100, 1090], [1100, 1090], [6700, 6700], 0, (TEAMS, 0)),              # two requests with the same key tiles
     (128, 24, [1024, 1000], [1024, 1000], [5000, 5024], 0, (TEAMS, 0)),
-    (128, 8, [1100, 700], [1100, 700], [6700, 7100], 0, (TICKS, 0)),                 # other queries: some members would idle
+    (128, 8, [1100, 700], [1100, 700], [6700, 7100], 0, None),
+    (128, 12, [1100, 700], [1100, 700], [6700, 7100], 0, (TICKS, 0)),                # other queries: some members would idle
+    (64, 24, [594] * 4, [594] * 4, [6211] * 4, 0, (TEAMS, 0)),                       # (as whole items far from balanced)
     (128, 8, [1100, 0, 300], [1100, 0, 300], [6700, 0, 2000], 0, (TICKS, 0)),        # key tiles that differ, a request without queries
     (128, 24, [3584, 256, 0], [3584, 256, 0], [2000, 5328, 5584], 0, None),          # (whole items of full capacities balance)
     (128, 24, [600], [600], [6000], 700, None),
@@ -95,6 +98,8 @@ def test_one_pair_a_head_behind_a_row_list():
 
 @pytest.mark.parametrize("D,grid,ratio,ne_cap", [
     (64, (64, 80), 0.2, 1024),                       # teams, n_full = 10752
+    (128, (64, 64), 0.2, 896),                       # the lone tiles apart
+    (128, (65, 63), 0.26, 1152),
     (128, (64, 64), 0.2, 1024),                      # teams, more room than pairs
     (64, (64, 80), 0.8, 4096),                       # waves
 ])
