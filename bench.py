@@ -48,7 +48,7 @@ def measured_peaks():
 
 # DRAM bytes per attention launch on config 2 (dram__bytes_read.sum + dram__bytes_write.sum of one ncu
 # capture of this workload), valid for the kernel source with this digest only.
-ATTENTION_TRAFFIC = dict(source_sha256_16="aed07ecc2818ae47", config=2, dram_bytes_per_launch=351.7e6)
+ATTENTION_TRAFFIC = dict(source_sha256_16="be1b4250ba1a8c2a", config=2, dram_bytes_per_launch=341.4e6)
 
 
 def recorded_traffic(cfg):
